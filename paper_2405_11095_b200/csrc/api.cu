@@ -92,7 +92,27 @@ struct Plan {
     int lo[2];   // lowest index bit of each strided pass
 };
 
-Plan make_plan(int L)
+// The cut depends on L and the direction alone, never on the number of workers: the encoder's fp32 sums, and
+// with them its packed signs, are the same however the workers are batched.
+//
+// Encoder.  A strided pass costs its memory traffic up to eight stages (0.17 ms per 2^27 coordinates, nine 0.20,
+// ten 0.22), a contiguous pass its instructions (T = 12 / 13 / 14: 0.177 / 0.183 / 0.195 ms, T = 15, one block
+// per SM: 0.25).  So: T = 14 from 2^20 on, and A as small as that leaves it (2^22: 8 + 14 0.37 ms, 9 + 13 0.38,
+// 10 + 12 0.40; 2^20: 6 + 14 against 10 + 10 0.36 and 0.39 ms, and one vector of 2^20 0.018 against 0.043 ms,
+// because ten stages make only eight runs of tiles); below 2^20 the tile shrinks so that the contiguous pass still has blocks for the chip.
+// Two strided passes: eight stages each while T stays within 10..14 (2^27: 8 + 8 + 11 1.03 ms per two workers,
+// 6 + 10 + 11 1.10, 3 + 10 + 14 1.18); 2^31: 7 + 10 + 14 8.9 ms per worker against 10 + 10 + 11 10.5 ms, whose
+// top pass visits 1024 rows megabytes apart for 64 bytes each.
+//
+// Decoder.  Every value is an exact integer, so the cut is free to follow the call: `workers` summed, P planes.
+//   five workers or more, up to 2^24: tiles of 2^14, whose contiguous pass runs on the tensor cores (2^20, 128
+//     workers: 0.10 ms against 0.17 .. 0.20 on the plain ALUs at any tile); the first pass takes what is left.
+//     From 128 (tile, worker) items: below, setting up the blocks costs more (2^16, four workers: 15 against 11 us);
+//   three or four from 2^20 on: ten strided stages (on the tensor cores if there are tiles enough), short tiles;
+//   one or two, or several planes: the plain-ALU pass is fastest on short tiles (one vector of 2^30: T = 10 1.5 ms, T = 14
+//     1.95), the first pass up to eight stages (six below 2^20, to leave the contiguous pass blocks for the chip);
+//   two strided passes: the same for fp32 (2^31: T = 11 2.8 ms per worker, T = 14 4.2).
+Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1)
 {
     Plan pl{};
     pl.L = L;
@@ -101,14 +121,18 @@ Plan make_plan(int L)
         pl.ncol = 0;
         return pl;
     }
-    pl.ncol = (L - 15 + 9) / 10;
-    pl.T = L - 10 * pl.ncol;
-    if (pl.T < 10) pl.T = 10;
-    const int rest = L - pl.T;
+    pl.ncol = L <= 25 ? 1 : 2;
     if (pl.ncol == 1) {
-        pl.A[0] = rest;
+        if (L == 25) pl.T = 15;
+        else if (decoder && workers > 4 && P == 1 && (dp >> 14) * workers >= 128) pl.T = 14;
+        else if (decoder && workers > 2 && P == 1 && L >= 20) pl.T = L - 10;
+        else if (decoder) pl.T = L < 20 ? L - 6 : (L <= 22 ? (L - 8 < 12 ? 12 : L - 8) : (L == 23 && P == 1 ? 13 : 14));
+        else pl.T = L == 18 ? 11 : (L < 18 ? 12 : (L == 19 ? 13 : 14));
+        pl.A[0] = L - pl.T;
     } else {
-        pl.A[0] = rest / 2;
+        pl.T = decoder ? (L > 30 ? L - 20 : 10) : (L > 30 ? 14 : L - 16);
+        const int rest = L - pl.T;
+        pl.A[0] = decoder ? rest / 2 : (rest > 16 ? 10 : 8);
         pl.A[1] = rest - pl.A[0];
     }
     pl.lo[0] = pl.T;
@@ -156,7 +180,7 @@ struct Geometry {
     int64_t dp;
     int L;        // log2 transform length
     double rootn; // sqrt(transform length)
-    Plan plan;
+    Plan plan;    // the encoder's; both directions have strided passes, and need scratch, at the same lengths
     size_t ws_per_worker;
 };
 
@@ -166,7 +190,7 @@ bool make_geometry(int64_t d, int block_log2, Geometry* g)
     if (g->dp < 0) return false;
     g->L = block_log2 == 0 ? ilog2(g->dp) : block_log2;
     g->rootn = sqrt((double)((int64_t)1 << g->L));
-    g->plan = make_plan(g->L);
+    g->plan = make_plan(g->L, false);
     g->ws_per_worker = g->plan.ncol > 0 ? (size_t)g->dp * 4 : 0;
     return true;
 }
@@ -196,11 +220,12 @@ bool fused_encoder_enabled() { return g_fused_encoder.load(std::memory_order_rel
 int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, size_t ws_bytes,
                   cudaStream_t s)
 {
-    const Plan& pl = g.plan;
+    const Plan pl = sink == SINK_FINAL ? make_plan(g.L, true, g.dp, p.nworkers, p.P) : g.plan;
     cudaError_t e = cudaSuccess;
 #define FOSGD_CUDA_OK(call) do { e = (call); if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; } } while (0)
     if (pl.ncol == 0) {
-        FOSGD_CUDA_OK((pl.L < 10) ? traced('s', pl.L, src, sink, p, s) : traced('r', pl.T, src, sink, p, s));
+        FOSGD_CUDA_OK((pl.L < 10) ? traced('s', pl.L, src, sink, p, s)
+                                  : traced('r', pl.T, src, sink == SINK_FINAL && p.nworkers == 1 ? (int)SINK_SINGLE : sink, p, s));
         return FOSGD_OK;
     }
     if (ws == nullptr || ws_bytes < g.ws_per_worker) return FOSGD_EWORKSPACE;
@@ -222,8 +247,8 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
     const char* src0 = static_cast<const char*>(p.src);
     char* dst0 = static_cast<char*>(p.dst);
     const uint32_t id0 = p.id0;
-    // a packed one-plane source through a single strided pass stays exact in fp16 (|value| <= 2^A)
-    const bool half_path = (src == SRC_BITS && p.P == 1 && pl.ncol == 1 && pl.A[0] >= 6);
+    // a packed source through a single strided pass stays exact in fp16 (|value| <= K 2^A) for small K
+    const bool half_path = (src == SRC_BITS && pl.ncol == 1 && colh_applicable(pl.A[0], p));
     // A packed one-plane source through two strided passes (transform length above 2^25): the first pass's output
     // is still exact in fp16, so with room for it beside the fp32 intermediate (6 instead of 4 bytes per
     // coordinate and worker) the first pass writes half the bytes in 256-byte rows and the second reads half.
@@ -268,16 +293,16 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
             pc.lo_log = pl.lo[0];
             // ten stages: H_8 on packed bytes + H_128 on the tensor cores, same fp16 intermediate
             tensor_pass = pl.A[0] == 10 && tc_enabled() && tc_col_applicable(pc, tc_any_size());
-            if (tensor_pass) FOSGD_CUDA_OK(traced('t', pl.A[0], SRC_BITS, 4, pc, s));
-            else FOSGD_CUDA_OK(traced('h', pl.A[0], SRC_BITS, 4, pc, s));
+            if (tensor_pass) FOSGD_CUDA_OK(traced('t', pl.A[0], SRC_BITS, 5, pc, s));
+            else FOSGD_CUDA_OK(traced('h', pl.A[0], SRC_BITS, 5, pc, s));
         } else if (half_first) {
             PassParams pc = q;
             pc.src = srck;
             pc.dst = ws16;
             pc.dst_stride = g.dp;
             pc.lo_log = pl.lo[1];
-            if (pl.A[1] == 10 && tc_enabled() && tc_col_applicable(pc, tc_any_size())) FOSGD_CUDA_OK(traced('t', pl.A[1], SRC_BITS, 4, pc, s));
-            else FOSGD_CUDA_OK(traced('h', pl.A[1], SRC_BITS, 4, pc, s));
+            if (pl.A[1] == 10 && tc_enabled() && tc_col_applicable(pc, tc_any_size())) FOSGD_CUDA_OK(traced('t', pl.A[1], SRC_BITS, 5, pc, s));
+            else FOSGD_CUDA_OK(traced('h', pl.A[1], SRC_BITS, 5, pc, s));
             PassParams pm = q;
             pm.src = ws16;
             pm.src_stride = g.dp;
@@ -311,7 +336,8 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
         if (half_path && sink == SINK_FINAL && tc_row_enabled() && tc_row_applicable(pr, pl.T, tc_any_size()))
             FOSGD_CUDA_OK(traced('u', pl.T, SRC_WS16, sink, pr, s));
         else
-            FOSGD_CUDA_OK(traced('r', pl.T, half_path ? (int)SRC_WS16 : (int)SRC_WS, sink, pr, s));
+            FOSGD_CUDA_OK(traced('r', pl.T, half_path ? (int)SRC_WS16 : (int)SRC_WS,
+                                 sink == SINK_FINAL && m == 1 ? (int)SINK_SINGLE : sink, pr, s));
     }
 #undef FOSGD_CUDA_OK
     return FOSGD_OK;
@@ -649,7 +675,7 @@ int fosgd_amplitudes(const void* grads, int dtype, int64_t d, int64_t worker_str
                                       (cudaStream_t)stream);
     if (on) {
         cudaEventRecord(g_trace_events[2 * g_trace_count + 1], (cudaStream_t)stream);
-        g_trace_log[g_trace_count] = TraceEntry{'n', g.L, dtype == FOSGD_BF16 ? 1 : 0, 5, M, false};
+        g_trace_log[g_trace_count] = TraceEntry{'n', g.L, dtype == FOSGD_BF16 ? 1 : 0, 6, M, false};
         ++g_trace_count;
     }
     if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; }
@@ -672,10 +698,9 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
     if (g.plan.ncol > 0 && (ws == nullptr || ws_bytes < g.ws_per_worker)) return FOSGD_EWORKSPACE;
     const Plan& pl = g.plan;
     cudaStream_t s = (cudaStream_t)stream;
-    // One pass over the gradients where the strided pass can carry the sums: fp32, ten strided stages through the
-    // copy engine, and scratch for all M workers at once (the amplitude is a maximum over all of them, so every
+    // One pass over the gradients where the strided pass can carry the sums: fp32, a single strided pass, and scratch for all M workers at once (the amplitude is a maximum over all of them, so every
     // strided pass must be over before the first dither).
-    if (dtype == FOSGD_F32 && pl.ncol == 1 && pl.A[0] == 10 && ws_bytes / g.ws_per_worker >= (size_t)M) {
+    if (dtype == FOSGD_F32 && pl.ncol == 1 && ws_bytes / g.ws_per_worker >= (size_t)M) {
         PassParams pc{};
         pc.src = grads; pc.src_stride = worker_stride; pc.d = d; pc.dp = g.dp;
         pc.dst = ws; pc.dst_stride = g.dp; pc.lo_log = pl.lo[0];
@@ -683,14 +708,14 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
         bool launched = false;
         int nruns = 0;
         bool on = trace_begin(s);
-        cudaError_t e = launch_col4_norm(pc, static_cast<double*>(amp_ws), s, &launched, &nruns);
+        cudaError_t e = launch_col_norm(pl.A[0], pc, static_cast<double*>(amp_ws), s, &launched, &nruns);
         if (launched) trace_end(on, s, TraceEntry{'c', pl.A[0], SRC_G32, SINK_WS, M, false});
         if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; }
         if (launched) {
             on = trace_begin(s);
             e = launch_amplitudes_finalize(static_cast<const double*>(amp_ws), M, nruns, alpha, alpha_s,
                                            (double)((int64_t)1 << g.L), lambda_dev, lambda_s_dev, s);
-            trace_end(on, s, TraceEntry{'n', g.L, 0, 5, M, false});
+            trace_end(on, s, TraceEntry{'n', g.L, 0, 6, M, false});
             if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; }
             PassParams pr = pc;
             pr.src = ws; pr.src_stride = g.dp;
@@ -768,7 +793,7 @@ const char* fosgd_trace_label(int k)
 {
     if (k < 0 || k >= g_trace_count) return "";
     static const char* const srcs[] = {"f32", "bf16", "bits", "ws", "ws16"};
-    static const char* const sinks[] = {"ws", "pack1", "packK", "final", "ws16", "amp"};
+    static const char* const sinks[] = {"ws", "pack1", "packK", "final", "final", "ws16", "amp"};
     const TraceEntry& t = g_trace_log[k];
     char who[16];
     if (t.workers > 0) snprintf(who, sizeof who, "%d", t.workers);

@@ -1,14 +1,15 @@
 // Strided pass: A butterfly stages on the index bits [lo, lo + A) of the coordinate, lo >= 10,
 // i.e. the Kronecker factor (H_A (x) I_S) with S = 2^lo.  The vector is read as a matrix with
-// rows S apart; a warp always covers 32 consecutive columns, so global accesses are 128-byte
-// coalesced and a row segment of a packed source is exactly one word.  Sources: gradients
+// rows S apart; a warp always covers 32 or 64 consecutive columns of a row, and the row segment of a
+// packed source or of the flip vector is one or two words.  Sources: gradients
 // (pad + flip), packed bits, or the fp32 intermediate; the sink is the fp32 intermediate
 // (in place when source and sink coincide: a block reads its whole tile before writing it).
 //
-//   A <= 5: a thread holds the 2^A rows of one column in registers; no shared memory.
-//   A >  5: a block of 2^A threads owns 2^A rows x 32 columns: round F transforms the top
-//           five row bits straight from global memory, round L the remaining low row bits
-//           after one exchange through shared memory.
+//   A <= 4: a thread holds the 2^A rows of one column in registers; no shared memory.
+//   A = 5..8: col2_kernel, 2^A rows x 64 columns, two adjacent columns per thread.
+//   A = 9, 10: a tile of 2^A rows x 32 or 16 columns: round F transforms the top five row bits
+//           straight from global memory, round L the remaining low row bits after one exchange
+//           through shared memory; A = 10 from fp32 gradients: col4.cuh.
 #include <cuda.h>   // CUtensorMap and the encode entry point type; the driver is reached through the runtime
 
 #include "col4.cuh"
@@ -20,8 +21,7 @@ namespace fosgd {
 // done on 32-bit offsets from the worker's base pointer (one widening multiply-add per access
 // instead of 64-bit shifts, adds and compares).
 template <int SRC>
-__device__ __forceinline__ float col_load(const PassParams& p, const void* worker_src, uint32_t i, uint32_t d32,
-                                          uint32_t bit)
+__device__ __forceinline__ float col_load(const PassParams& p, const void* worker_src, uint32_t i, uint32_t d32)
 {
     if (SRC == SRC_G32) {
         return (i < d32) ? __ldcs(static_cast<const float*>(worker_src) + i) : 0.f;
@@ -29,10 +29,9 @@ __device__ __forceinline__ float col_load(const PassParams& p, const void* worke
         return (i < d32) ? __uint_as_float((uint32_t)__ldcs(static_cast<const uint16_t*>(worker_src) + i) << 16) : 0.f;
     } else if (SRC == SRC_WS) {
         return static_cast<const float*>(worker_src)[i];
-    } else if (SRC == SRC_WS16) {
-        return __half2float(static_cast<const __half*>(worker_src)[i]);
     } else {
-        return plane_value(static_cast<const uint32_t*>(worker_src) + (i >> 5), p.dp >> 5, p.P, p.K, bit);
+        static_assert(SRC == SRC_WS16 || SRC != SRC_BITS, "packed sources are read word by word");
+        return __half2float(static_cast<const __half*>(worker_src)[i]);
     }
 }
 
@@ -49,14 +48,15 @@ __device__ __forceinline__ float flip_shifted(float x, uint32_t word, uint32_t s
     return __uint_as_float(__float_as_uint(x) ^ ((word << sh) & 0x80000000u));
 }
 
-// One-plane packed source: the 32 columns of a row segment are one word.  Lane r fetches the
-// word of the r-th row this warp handles (one gather per warp instead of 32 broadcast loads).
-__device__ __forceinline__ uint32_t bits_row_word(const void* worker_src, uint32_t irow)
+// Packed source: the 32 columns of a row segment are one word per plane.  Lane r fetches the
+// word of the r-th row this warp handles (one gather per warp and plane instead of 32 broadcast loads:
+// 2^25 coordinates of two planes, ten stages: 174 us with every thread loading its own words).
+__device__ __forceinline__ uint32_t bits_row_word(const PassParams& p, const void* worker_src, uint32_t irow, int plane)
 {
-    return __ldg(static_cast<const uint32_t*>(worker_src) + (irow >> 5));
+    return __ldg(static_cast<const uint32_t*>(worker_src) + (irow >> 5) + (int64_t)plane * (p.dp >> 5));
 }
 
-// ---- A <= 5 -----------------------------------------------------------------------------
+// ---- A <= 4 -----------------------------------------------------------------------------
 template <int A, int SRC>
 __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
 {
@@ -72,24 +72,28 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
     const void* const wsrc = worker_source<SRC>(p, n);
 
     float v[32];
-    uint32_t myword = 0;  // flip word (gradient sources) or packed signs (one-plane bit source) of row `lane`
-    const bool one_plane = (SRC == SRC_BITS) && p.P == 1;
-    if ((int)lane < R) {
-        const uint32_t irow = (i_first - lane) + lane * step;
-        if (SRC == SRC_G32 || SRC == SRC_G16) myword = eps_word(p.rng, p.id0 + (uint32_t)n, irow >> 5);
-        if (one_plane) myword = bits_row_word(wsrc, irow);
-    }
+    if constexpr (SRC == SRC_BITS) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t i = i_first + r * step;
-        float x;
-        if (one_plane) {
-            x = ((__shfl_sync(0xFFFFFFFFu, myword, r) >> lane) & 1u) ? 1.f : -1.f;
-        } else {
-            x = col_load<SRC>(p, wsrc, i, d32, lane);
-            if (SRC == SRC_G32 || SRC == SRC_G16) x = flip_shifted(x, __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
+        for (int r = 0; r < R; ++r) v[r] = (float)(-p.K);
+        float weight = 2.f;
+        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
+            uint32_t mine = 0;
+            if ((int)lane < R) mine = bits_row_word(p, wsrc, (i_first - lane) + lane * step, pl);
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                if ((__shfl_sync(0xFFFFFFFFu, mine, r) >> lane) & 1u) v[r] += weight;
         }
-        v[r] = x;
+    } else {
+        uint32_t myword = 0;  // flip word of row `lane` (gradient sources)
+        if (SRC == SRC_G32 || SRC == SRC_G16) {
+            if ((int)lane < R) myword = eps_word(p.rng, p.id0 + (uint32_t)n, ((i_first - lane) + lane * step) >> 5);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = col_load<SRC>(p, wsrc, i_first + r * step, d32);
+        if (SRC == SRC_G32 || SRC == SRC_G16) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
+        }
     }
 #pragma unroll
     for (int r = R; r < 32; ++r) v[r] = 0.f;
@@ -99,9 +103,146 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
     for (int r = 0; r < R; ++r) dst[i_first + r * step] = v[r];
 }
 
-// ---- A > 5 ------------------------------------------------------------------------------
+// ---- A = 5..8 ----------------------------------------------------------------------------
+// 2^A rows x 64 columns, two adjacent columns x sixteen rows per thread: a warp moves 256 contiguous bytes
+// of a row per access (128 from bf16), round F has the top four row bits in registers, round L the low four.
+// Bound by memory: 2^27 coordinates of fp32 gradients take 0.17 ms at A = 8 (6.3 TB/s of the 6.5 a plain copy
+// reaches), where tiles of 16 columns (64-byte segments) took 0.21 ms; with rows megabytes apart (the top pass
+// of a 2^31 transform) the segment width decides: 5.8 ms with 64 bytes per row visit at A = 8, 2.9 ms with 256.
+// NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
+// (fp32 within a thread's tile, fp64 beyond, fixed order); blocks then take tiles gridDim.x apart.
+template <int A, int SRC, bool NORM>
+__global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams p, const uint32_t ntiles, double* const partial)
+{
+    extern __shared__ __align__(16) float2 tile2[];
+    constexpr uint32_t WARPS = 1u << (A - 4);
+    const int n = blockIdx.y;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t w = threadIdx.x >> 5;
+    const uint32_t step = 1u << p.lo_log;                         // one row
+    const uint32_t d32 = (uint32_t)p.d;
+    const void* const wsrc = worker_source<SRC>(p, n);
+    float* const dst = static_cast<float*>(p.dst) + (int64_t)n * p.dst_stride;
+    constexpr bool kGrad = SRC == SRC_G32 || SRC == SRC_G16;
+    double sumsq = 0.0;
+
+    for (uint32_t seg = blockIdx.x; seg < ntiles; seg += gridDim.x) {
+        const uint32_t lo0 = (seg << 6) & (step - 1u);
+        const uint32_t hi = (uint32_t)(((uint64_t)seg << 6) >> p.lo_log);
+        const uint32_t i_tile = (hi << (p.lo_log + A)) + lo0;     // row 0, column 0 of the tile
+        // round F: rows k = r * WARPS + w
+        const uint32_t i_f = i_tile + w * step + 2u * lane;
+        const uint32_t step_f = step * WARPS;
+        // the two words (flips, or packed signs) of row r belong to lanes 2 r and 2 r + 1
+        const uint32_t iw = i_tile + w * step + (lane >> 1) * step_f + 32u * (lane & 1u);
+        const uint32_t from = lane >> 4, bit = (2u * lane) & 31u;
+        float v[32];
+        if constexpr (SRC == SRC_BITS) {
+            const uint32_t* const words = static_cast<const uint32_t*>(wsrc) + (iw >> 5);
+            const float base = (float)(-p.K);
+#pragma unroll
+            for (int r = 0; r < 32; ++r) v[r] = base;
+            float weight = 2.f;
+            for (int pl = 0; pl < p.P; ++pl, weight += weight) {
+                const uint32_t mine = __ldg(words + (int64_t)pl * (p.dp >> 5));
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const uint32_t x = __shfl_sync(0xFFFFFFFFu, mine, 2 * r + (int)from) >> bit;
+                    if (x & 1u) v[2 * r] += weight;               // 2 c - K, bit by bit (exact)
+                    if (x & 2u) v[2 * r + 1] += weight;
+                }
+            }
+        } else if constexpr (kGrad) {
+            auto load2 = [&](uint32_t i, float& x0, float& x1) {
+                if constexpr (SRC == SRC_G32) {
+                    const float2 q = __ldcs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i));
+                    x0 = q.x; x1 = q.y;
+                } else {
+                    const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i));
+                    x0 = __uint_as_float(q << 16); x1 = __uint_as_float(q & 0xFFFF0000u);
+                }
+            };
+            // a tile whose last coordinate is inside the gradient: all sixteen loads in flight, no checks
+            if (i_tile + ((1u << A) - 1u) * step + 63u < d32) {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) load2(i_f + r * step_f, v[2 * r], v[2 * r + 1]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const uint32_t i = i_f + r * step_f;
+                    v[2 * r] = v[2 * r + 1] = 0.f;
+                    if (i + 1u < d32) load2(i, v[2 * r], v[2 * r + 1]);
+                }
+                if (d32 & 1u) {       // an odd length ends inside a pair
+#pragma unroll
+                    for (int r = 0; r < 16; ++r)
+                        if (i_f + r * step_f + 1u == d32) v[2 * r] = col_load<SRC>(p, wsrc, d32 - 1u, d32);
+                }
+            }
+            const uint32_t mine = eps_word(p.rng, p.id0 + (uint32_t)n, iw >> 5);
+            const uint32_t sh = 31u - bit;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, 2 * r + (int)from);
+                v[2 * r] = flip_shifted(v[2 * r], word, sh);
+                v[2 * r + 1] = flip_shifted(v[2 * r + 1], word, sh - 1u);
+            }
+        } else if constexpr (SRC == SRC_WS) {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const float2 q = *reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f);
+                v[2 * r] = q.x; v[2 * r + 1] = q.y;
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const float2 q = __half22float2(*reinterpret_cast<const __half2*>(static_cast<const __half*>(wsrc) + i_f + r * step_f));
+                v[2 * r] = q.x; v[2 * r + 1] = q.y;
+            }
+        }
+        if constexpr (NORM) {
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                s0 = fmaf(v[2 * r], v[2 * r], s0);
+                s1 = fmaf(v[2 * r + 1], v[2 * r + 1], s1);
+            }
+            sumsq += (double)(s0 + s1);
+        }
+        butterflies32<30>(v);
+        if (NORM) __syncthreads();                                 // readers of the previous tile
+#pragma unroll
+        for (int r = 0; r < 16; ++r) tile2[((r * WARPS + w) << 5) + lane] = make_float2(v[2 * r], v[2 * r + 1]);
+        __syncthreads();
+        // round L: rows k = w * 16 + r (the low A - 4 bits are new)
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const float2 q = tile2[((w * 16u + r) << 5) + lane];
+            v[2 * r] = q.x; v[2 * r + 1] = q.y;
+        }
+        butterflies32<((1 << (A - 4)) - 1) << 1>(v);
+        const uint32_t i_l = i_tile + (w * 16u) * step + 2u * lane;
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+            __stcg(reinterpret_cast<float2*>(dst + i_l + r * step), make_float2(v[2 * r], v[2 * r + 1]));   // L2 only: read next by another kernel
+    }
+    if constexpr (NORM) {
+        __shared__ double wsum[WARPS];
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1) sumsq += __shfl_xor_sync(0xFFFFFFFFu, sumsq, s);
+        if (lane == 0) wsum[w] = sumsq;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double total = 0.0;
+            for (uint32_t k = 0; k < WARPS; ++k) total += wsum[k];
+            partial[(int64_t)n * gridDim.x + blockIdx.x] = total;
+        }
+    }
+}
+
+// ---- A = 9, 10 ---------------------------------------------------------------------------
 template <int A, int SRC>
-__global__ void __launch_bounds__(1 << A) col_tile_kernel(const PassParams p)
+__global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassParams p)
 {
     extern __shared__ __align__(16) float smem[];  // 2^A rows x 32 columns
     constexpr int WARPS = 1 << (A - 5);
@@ -117,26 +258,28 @@ __global__ void __launch_bounds__(1 << A) col_tile_kernel(const PassParams p)
     const void* const wsrc = worker_source<SRC>(p, n);
 
     float v[32];
-    uint32_t myword = 0;  // flip word (gradient sources) or packed signs (one-plane bit source) of row lane*WARPS+w
-    const bool one_plane = (SRC == SRC_BITS) && p.P == 1;
-    {
-        const uint32_t irow = i_tile + (lane * WARPS + w) * step;
-        if (SRC == SRC_G32 || SRC == SRC_G16) myword = eps_word(p.rng, p.id0 + (uint32_t)n, irow >> 5);
-        if (one_plane) myword = bits_row_word(wsrc, irow);
-    }
+    const uint32_t irow = i_tile + (lane * WARPS + w) * step;     // row lane * WARPS + w: its words are this lane's to fetch
     // round F: rows k = r * WARPS + w  (register bits = top five row bits)
     const uint32_t i_f = i_tile + w * step + lane;
     const uint32_t step_f = step * WARPS;
+    if constexpr (SRC == SRC_BITS) {
 #pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        float x;
-        if (one_plane) {
-            x = ((__shfl_sync(0xFFFFFFFFu, myword, r) >> lane) & 1u) ? 1.f : -1.f;
-        } else {
-            x = col_load<SRC>(p, wsrc, i_f + r * step_f, d32, lane);
-            if (SRC == SRC_G32 || SRC == SRC_G16) x = flip_shifted(x, __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
+        for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
+        float weight = 2.f;
+        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
+            const uint32_t mine = bits_row_word(p, wsrc, irow, pl);
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                if ((__shfl_sync(0xFFFFFFFFu, mine, r) >> lane) & 1u) v[r] += weight;
         }
-        v[r] = x;
+    } else {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) v[r] = col_load<SRC>(p, wsrc, i_f + r * step_f, d32);
+        if (SRC == SRC_G32 || SRC == SRC_G16) {
+            const uint32_t mine = eps_word(p.rng, p.id0 + (uint32_t)n, irow >> 5);
+#pragma unroll
+            for (int r = 0; r < 32; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, mine, r), 31u - lane);
+        }
     }
     butterflies32<31>(v);
 #pragma unroll
@@ -179,44 +322,42 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) col_tile16_kernel(const PassP
     const void* const wsrc = worker_source<SRC>(p, n);
 
     float v[32];
-    // Per-row words (flip word of a gradient row, or the packed signs of a one-plane source row):
-    // lane j fetches them for rows (r = j & 15, h = j >> 4) and (r = 16 + (j & 15), h = j >> 4).
-    uint32_t word_lo = 0, word_hi = 0;
-    const bool one_plane = (SRC == SRC_BITS) && p.P == 1;
-    {
-        const uint32_t row_a = ((lane & 15u) << (A - 5)) | (w << 1) | h;
-        const uint32_t ia = i_tile + row_a * step, ib = ia + (step << (A - 1));
-        if (SRC == SRC_G32 || SRC == SRC_G16) {
-            word_lo = eps_word(p.rng, p.id0 + (uint32_t)n, ia >> 5);
-            word_hi = eps_word(p.rng, p.id0 + (uint32_t)n, ib >> 5);
-        }
-        if (one_plane) {
-            word_lo = bits_row_word(wsrc, ia);
-            word_hi = bits_row_word(wsrc, ib);
-        }
-    }
+    // Per-row words (flip word of a gradient row, or the packed signs of a source row):
+    // lane j fetches them for rows (r = j & 15, h = j >> 4) and (r = 16 + (j & 15), h = j >> 4); lanes of a
+    // half-warp (same h) read the word from lane r & 15 of their own half.
+    const uint32_t row_a = ((lane & 15u) << (A - 5)) | (w << 1) | h;
+    const uint32_t ia = i_tile + row_a * step, ib = ia + (step << (A - 1));
     // round F: rows k = (r << (A-5)) | (w << 1) | h
     const uint32_t i_f = i_tile + ((w << 1) | h) * step + c;
     const uint32_t step_f = step << (A - 5);
-    const uint32_t shamt = 31u - bitpos;
-    // a block whose last coordinate is inside the gradient needs no per-element bound check
-    const bool inside = i_tile + (((1u << A) - 1u) * step) + 15u < d32;
-    auto load_rows = [&](const uint32_t bound) {
+    if constexpr (SRC == SRC_BITS) {
 #pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            // lanes of a half-warp (same h) read the word from lane r & 15 of their own half
-            const uint32_t roww = __shfl_sync(0xFFFFFFFFu, r < 16 ? word_lo : word_hi, r & 15, 16);
-            float x;
-            if (one_plane) {
-                x = ((roww >> bitpos) & 1u) ? 1.f : -1.f;
-            } else {
-                x = col_load<SRC>(p, wsrc, i_f + r * step_f, bound, bitpos);
-                if (SRC == SRC_G32 || SRC == SRC_G16) x = flip_shifted(x, roww, shamt);
-            }
-            v[r] = x;
+        for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
+        float weight = 2.f;
+        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
+            const uint32_t word_lo = bits_row_word(p, wsrc, ia, pl), word_hi = bits_row_word(p, wsrc, ib, pl);
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                if ((__shfl_sync(0xFFFFFFFFu, r < 16 ? word_lo : word_hi, r & 15, 16) >> bitpos) & 1u) v[r] += weight;
         }
-    };
-    if (inside) load_rows(0xFFFFFFFFu); else load_rows(d32);   // the constant bound folds the checks away
+    } else {
+        // a block whose last coordinate is inside the gradient needs no per-element bound check
+        // (the constant bound folds the checks away)
+        if (i_tile + (((1u << A) - 1u) * step) + 15u < d32) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) v[r] = col_load<SRC>(p, wsrc, i_f + r * step_f, 0xFFFFFFFFu);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) v[r] = col_load<SRC>(p, wsrc, i_f + r * step_f, d32);
+        }
+        if (SRC == SRC_G32 || SRC == SRC_G16) {
+            const uint32_t word_lo = eps_word(p.rng, p.id0 + (uint32_t)n, ia >> 5);
+            const uint32_t word_hi = eps_word(p.rng, p.id0 + (uint32_t)n, ib >> 5);
+#pragma unroll
+            for (int r = 0; r < 32; ++r)
+                v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, r < 16 ? word_lo : word_hi, r & 15, 16), 31u - bitpos);
+        }
+    }
     butterflies32<31>(v);
     {
         float* const pf = smem + phys16((int)((((w << 1) | h) << 4) + c));
@@ -325,67 +466,130 @@ static cudaError_t launch_col4(const PassParams& p, cudaStream_t s, bool* launch
     return cudaGetLastError();
 }
 
-// Ten stages on fp32 gradients with the squared norm of every worker's gradient gathered on the way: run sums
-// in partial[worker][run] (*nruns_out of them per worker).  One-block-per-run form only; *launched stays false
-// where it does not apply (rows 128 KiB apart or more, rows shorter than a run, map refused).
-cudaError_t launch_col4_norm(const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nruns_out)
+template <int A, int SRC, bool NORM>
+static cudaError_t launch_col2(const PassParams& p, uint32_t blocks, double* partial, cudaStream_t s)
 {
-    constexpr int A = 10;
+    return launch<col2_kernel<A, SRC, NORM>>(dim3(blocks, (unsigned)p.nworkers), 2 << A, (size_t)(1 << A) * 256, s, 1, p,
+                                             (uint32_t)((p.dp >> A) / 64), partial);
+}
+
+// Strided pass on fp32 gradients with the squared norm of every worker's gradient gathered on the way: sums of
+// parts in partial[worker][part], *nparts_out (at most 256, what the caller's scratch holds) of them per worker.
+// *launched stays false where no kernel carries the sums: nine stages, rows 128 KiB apart or more at ten, more
+// than 256 runs per worker, map refused.
+cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nparts_out)
+{
+    constexpr int64_t kMaxParts = 256;
     *launched = false;
+    if (A >= 5 && A <= 8) {
+        const int64_t ntiles = (p.dp >> A) / 64;
+        const uint32_t blocks = (uint32_t)(ntiles < kMaxParts ? ntiles : kMaxParts);
+        *launched = true;
+        *nparts_out = (int)blocks;
+        switch (A) {
+            case 5: return launch_col2<5, SRC_G32, true>(p, blocks, partial, s);
+            case 6: return launch_col2<6, SRC_G32, true>(p, blocks, partial, s);
+            case 7: return launch_col2<7, SRC_G32, true>(p, blocks, partial, s);
+            default: return launch_col2<8, SRC_G32, true>(p, blocks, partial, s);
+        }
+    }
+    if (A != 10) return cudaSuccess;
     const uint64_t S = (uint64_t)1 << p.lo_log;
     const uint64_t rows = (uint64_t)(p.d >> p.lo_log);
     const int64_t nsegs = (p.dp >> A) / 16;
     const int64_t nruns = nsegs / 8;
-    if (p.lo_log >= 15 || S < 128 || nsegs % 8 != 0 || nruns * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
+    if (p.lo_log >= 15 || S < 128 || nsegs % 8 != 0 || nruns > kMaxParts || nruns * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
     CUtensorMap map;
     if (!make_col_tensor_map(&map, p.src, S, rows, (uint64_t)p.nworkers, (uint64_t)p.src_stride)) return cudaSuccess;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(col4_norm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col4::SMEM_BYTES)) != cudaSuccess) return e;
     col4_norm_kernel<<<(unsigned)(nruns * p.nworkers), 512, Col4::SMEM_BYTES, s>>>(p, map, (int)nruns, (uint32_t)rows, partial);
     *launched = true;
-    *nruns_out = (int)nruns;
+    *nparts_out = (int)nruns;
     return cudaGetLastError();
 }
 
-// ---- packed one-plane source, fp16 arithmetic ------------------------------------------------
-// The server's first pass starts from +-1, and after A <= 10 stages every value is an integer of
-// magnitude <= 1024, which fp16 holds exactly.  So this variant keeps two adjacent columns per
-// lane as a half2: a block owns 2^A rows x 64 columns, butterflies are HADD2 (two coordinates
+// ---- packed source, fp16 arithmetic ------------------------------------------------------------
+// A decoder's first pass starts from 2 c - K (one plane: +-1), and after A stages every value is an integer of
+// magnitude <= K 2^A, which fp16 holds exactly up to 2048.  So this variant keeps two adjacent columns per
+// lane as a half2: 64 columns per warp, butterflies are HADD2 (two coordinates
 // per instruction), and the intermediate is written as fp16 (half the bytes, still full
-// 128-byte lines per warp).  Rows of the packed source are two words; they are staged once in
-// shared memory.
-template <int A>
-__global__ void __launch_bounds__(1 << A) colh_tile_kernel(const PassParams p)
+// 128-byte lines per warp).  A row segment of the source is two words per plane: lanes fetch them, one
+// gather for every sixteen rows, and pass them by shuffle.
+// at(r): coordinate of register r = 0 .. 31, column 0 of the warp's 64
+template <typename At>
+__device__ __forceinline__ void load_planes_half2(const PassParams& p, const uint32_t* bits, uint32_t lane, __half2 (&v)[32], At at)
 {
-    extern __shared__ __align__(16) uint32_t smemh[];   // [2^A][32] half2 tile, then [2^A] word pairs
-    constexpr int ROWS = 1 << A;
-    constexpr int WARPS = 1 << (A - 5);
-    uint2* const wtab = reinterpret_cast<uint2*>(smemh + ROWS * 32);
-    const int n = blockIdx.y;
-    const int tid = threadIdx.x;
-    const uint32_t lane = tid & 31;
-    const int w = tid >> 5;
-    const int64_t seg = blockIdx.x;                               // 64-column segment id
-    const int64_t lo0 = (seg << 6) & (((int64_t)1 << p.lo_log) - 1);
-    const int64_t hi = (seg << 6) >> p.lo_log;
-    const int64_t i_tile = (hi << (p.lo_log + A)) + lo0;
-
-    {
-        const uint32_t* bits = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride;
-        wtab[tid] = __ldg(reinterpret_cast<const uint2*>(bits + ((i_tile + ((int64_t)tid << p.lo_log)) >> 5)));
+    const uint32_t sh = (2u * lane) & 31u, from = lane >> 4;
+    // words of registers (lane >> 1) and 16 + (lane >> 1), column half lane & 1
+    const uint32_t* const wa = bits + (at(lane >> 1) >> 5) + (lane & 1u);
+    const uint32_t* const wb = bits + (at(16u + (lane >> 1)) >> 5) + (lane & 1u);
+    if (p.P == 1) {
+        const uint32_t word_a = __ldg(wa), word_b = __ldg(wb);
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
+            // bit 0 -> sign of the low half, bit 1 -> sign of the high half; set bit = +1
+            const uint32_t hb = 0xBC00BC00u ^ ((x * 0x40008000u) & 0x80008000u);
+            v[r] = *reinterpret_cast<const __half2*>(&hb);
+        }
+    } else {
+        const __half2 base = __float2half2_rn((float)(-p.K));
+#pragma unroll
+        for (int r = 0; r < 32; ++r) v[r] = base;
+        uint32_t weight = 0x4000u;                               // fp16 2.0; the exponent grows plane by plane
+        for (int pl = 0; pl < p.P; ++pl, weight += 0x400u) {
+            const int64_t off = (int64_t)pl * (p.dp >> 5);
+            const uint32_t word_a = __ldg(wa + off), word_b = __ldg(wb + off);
+#pragma unroll
+            for (int r = 0; r < 32; ++r) {
+                const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
+                const uint32_t hb = ((x * 0x8001u) & 0x00010001u) * weight;
+                v[r] = __hadd2(v[r], *reinterpret_cast<const __half2*>(&hb));
+            }
+        }
     }
-    __syncthreads();
+}
+
+// A <= 5: a thread's registers hold the 2^A rows of two columns, for 2^(5-A) adjacent 64-column segments
+template <int A>
+__global__ void __launch_bounds__(256) colh_small_kernel(const PassParams p)
+{
+    constexpr uint32_t R = 1u << A;
+    constexpr int SEG_LOG = 11 - A;                               // columns of a warp: 2^(5-A) segments of 64
+    const int n = blockIdx.y;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t seg = blockIdx.x * 8u + (threadIdx.x >> 5);
+    if (seg >= (uint32_t)((p.dp >> A) >> SEG_LOG)) return;        // (whole warps)
+    const uint32_t lo0 = (seg << SEG_LOG) & ((1u << p.lo_log) - 1u);
+    const uint32_t i_tile = ((uint32_t)(((uint64_t)seg << SEG_LOG) >> p.lo_log) << (p.lo_log + A)) + lo0;
+    auto at = [&](uint32_t r) { return i_tile + ((r & (R - 1u)) << p.lo_log) + ((r >> A) << 6); };
+    __half2 v[32];
+    load_planes_half2(p, static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride, lane, v, at);
+    butterflies32<R - 1, __half2>(v);
+    __half* const dst = static_cast<__half*>(p.dst) + (int64_t)n * p.dst_stride + 2u * lane;
+#pragma unroll
+    for (int r = 0; r < 32; ++r)
+        __stcg(reinterpret_cast<unsigned int*>(dst + at((uint32_t)r)), *reinterpret_cast<const unsigned int*>(&v[r]));
+}
+
+// A = 6..9
+template <int A>
+__global__ void __launch_bounds__(1 << A, 1024 >> A) colh_tile_kernel(const PassParams p)
+{
+    extern __shared__ __align__(16) uint32_t smemh[];   // [2^A][32] half2 tile
+    constexpr int WARPS = 1 << (A - 5);
+    const int n = blockIdx.y;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t w = threadIdx.x >> 5;
+    const uint32_t seg = blockIdx.x;                              // 64-column segment id
+    const uint32_t lo0 = (seg << 6) & ((1u << p.lo_log) - 1u);
+    const uint32_t i_tile = ((uint32_t)(((uint64_t)seg << 6) >> p.lo_log) << (p.lo_log + A)) + lo0;
+    const uint32_t step = 1u << p.lo_log;
 
     __half2 v[32];
-    const uint32_t sh = (2u * lane) & 31u;
-    const uint32_t* const wsel = reinterpret_cast<const uint32_t*>(wtab) + (lane >> 4);
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const uint32_t x = (wsel[2 * (r * WARPS + w)] >> sh) & 3u;
-        // bit 0 -> sign of the low half, bit 1 -> sign of the high half; set bit = +1
-        const uint32_t hb = 0xBC00BC00u ^ ((x * 0x40008000u) & 0x80008000u);
-        v[r] = *reinterpret_cast<const __half2*>(&hb);
-    }
+    load_planes_half2(p, static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride, lane, v,
+                      [&](uint32_t r) { return i_tile + (r * WARPS + w) * step; });
     butterflies32<31, __half2>(v);
     __half2* const tile = reinterpret_cast<__half2*>(smemh);
 #pragma unroll
@@ -393,13 +597,15 @@ __global__ void __launch_bounds__(1 << A) colh_tile_kernel(const PassParams p)
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < 32; ++r) v[r] = tile[((w * 32 + r) << 5) + lane];
-    butterflies32<(A >= 10) ? 31 : ((1 << (A - 5)) - 1), __half2>(v);
-    __half2* dst = reinterpret_cast<__half2*>(static_cast<__half*>(p.dst) + (int64_t)n * p.dst_stride + i_tile) + lane;
+    butterflies32<(1 << (A - 5)) - 1, __half2>(v);
+    __half2* const dst = reinterpret_cast<__half2*>(static_cast<__half*>(p.dst) + (int64_t)n * p.dst_stride + i_tile) + lane;
+    const uint32_t i_l = (w * 32u) * (step >> 1);
 #pragma unroll
-    for (int r = 0; r < 32; ++r) dst[((int64_t)(w * 32 + r) << p.lo_log) >> 1] = v[r];
+    for (int r = 0; r < 32; ++r)
+        __stcg(reinterpret_cast<unsigned int*>(dst + i_l + r * (step >> 1)), *reinterpret_cast<const unsigned int*>(&v[r]));   // L2 only: read next by another kernel
 }
 
-// The same pass on 2^A rows x 32 columns (16 half2 lanes x one row bit per lane, like the
+// A = 10, one plane: 2^A rows x 32 columns (16 half2 lanes x one row bit per lane, like the
 // 16-column fp32 variant): half the shared memory and half the threads per block, so two blocks
 // share an SM and one block's stores overlap the other's arithmetic.  A row of the packed source
 // is one word; lane j fetches the words of rows (r = j & 15, h = j >> 4) and (16 + (j & 15), h).
@@ -459,27 +665,31 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) colh_tile32_kernel(const Pass
 template <int A>
 static cudaError_t launch_colh_one(const PassParams& p, cudaStream_t s)
 {
-    if constexpr (A >= 8) {
-        auto kern = colh_tile32_kernel<A>;
-        constexpr size_t smem = (size_t)phys16((1 << A) * 16) * 4;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers);
-        kern<<<grid, 1 << (A - 1), smem, s>>>(p);
+    if constexpr (A <= 5) {
+        const uint32_t segs = (uint32_t)(p.dp >> 11);
+        return launch<colh_small_kernel<A>>(dim3((segs + 7u) / 8u, (unsigned)p.nworkers), 256, 0, s, 1, p);
+    } else if constexpr (A <= 9) {
+        return launch<colh_tile_kernel<A>>(dim3((unsigned)((p.dp >> A) / 64), (unsigned)p.nworkers), 1 << A, (size_t)(1 << A) * 128, s, 1, p);
     } else {
-        auto kern = colh_tile_kernel<A>;
-        constexpr size_t smem = (size_t)(1 << A) * (32 * 4 + 8);
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((p.dp >> A) / 64), (unsigned)p.nworkers);
-        kern<<<grid, 1 << A, smem, s>>>(p);
+        return launch<colh_tile32_kernel<A>>(dim3((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers), 1 << (A - 1),
+                                             (size_t)phys16((1 << A) * 16) * 4, s, 1, p);
     }
-    return cudaGetLastError();
+}
+
+bool colh_applicable(int A, const PassParams& p)
+{
+    return p.P == 1 ? A <= 10 : A <= 9 && (p.K << A) <= 2048;
 }
 
 cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s)
 {
+    if (!colh_applicable(A, p)) return cudaErrorInvalidValue;
     switch (A) {
+        case 1: return launch_colh_one<1>(p, s);
+        case 2: return launch_colh_one<2>(p, s);
+        case 3: return launch_colh_one<3>(p, s);
+        case 4: return launch_colh_one<4>(p, s);
+        case 5: return launch_colh_one<5>(p, s);
         case 6: return launch_colh_one<6>(p, s);
         case 7: return launch_colh_one<7>(p, s);
         case 8: return launch_colh_one<8>(p, s);
@@ -492,45 +702,25 @@ cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s)
 template <int A, int SRC>
 static cudaError_t launch_col_one(const PassParams& p, cudaStream_t s)
 {
-    if constexpr (A <= 5) {
-        const dim3 grid((unsigned)((p.dp >> A) / 256), (unsigned)p.nworkers);
-        col_small_kernel<A, SRC><<<grid, 256, 0, s>>>(p);
-    } else if constexpr (A >= 8) {
+    if constexpr (A <= 4) {
+        return launch<col_small_kernel<A, SRC>>(dim3((unsigned)((p.dp >> A) / 256), (unsigned)p.nworkers), 256, 0, s, 1, p);
+    } else if constexpr (A <= 8) {
+        return launch_col2<A, SRC, false>(p, (uint32_t)((p.dp >> A) / 64), nullptr, s);
+    } else if constexpr (A == 9) {
+        // 32 columns: two blocks of 512 threads per SM, 128-byte row segments (0.20 ms on 2^27 coordinates against
+        // 0.24 ms with tiles of 16 columns)
+        return launch<col_tile_kernel<A, SRC>>(dim3((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers), 1 << A, (size_t)(1 << A) * 128, s, 1, p);
+    } else {
         // ten stages on fp32 gradients: the copy-engine kernels, unless the driver refuses the tensor map
-        if constexpr (A == 10 && SRC == SRC_G32) {
+        if constexpr (SRC == SRC_G32) {
             bool launched = false;
             const cudaError_t e = launch_col4(p, s, &launched);
             if (e != cudaSuccess || launched) return e;
         }
-        if constexpr (A == 10 && SRC == SRC_G16) {
-            // bf16 gradients with rows megabytes apart (the top pass of a transform longer than 2^30): 32-column
-            // tiles, so that a row visit moves 64 bytes in and 128 bytes out instead of half of that (31.2 against
-            // 35.4 ms on 8 workers of 2^31; the same tiles from packed bits were slower, 30.7 against 28.0 ms)
-            if (p.lo_log >= 20) {
-                auto wide = col_tile_kernel<A, SRC>;
-                constexpr size_t wsmem = (size_t)(1 << A) * 32 * 4;
-                cudaError_t e = cudaFuncSetAttribute(wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem);
-                if (e != cudaSuccess) return e;
-                const dim3 grid((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers);
-                wide<<<grid, 1 << A, wsmem, s>>>(p);
-                return cudaGetLastError();
-            }
-        }
-        auto kern = col_tile16_kernel<A, SRC>;
-        constexpr size_t smem = (size_t)phys16((1 << A) * 16) * 4;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((p.dp >> A) / 16), (unsigned)p.nworkers);
-        kern<<<grid, 1 << (A - 1), smem, s>>>(p);
-    } else {
-        auto kern = col_tile_kernel<A, SRC>;
-        constexpr size_t smem = (size_t)(1 << A) * 32 * 4;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers);
-        kern<<<grid, 1 << A, smem, s>>>(p);
+        // 16 columns: at 32 a block fills the SM by itself (0.26 ms against 0.22 ms on 2^27 coordinates)
+        return launch<col_tile16_kernel<A, SRC>>(dim3((unsigned)((p.dp >> A) / 16), (unsigned)p.nworkers), 1 << (A - 1),
+                                                 (size_t)phys16((1 << A) * 16) * 4, s, 1, p);
     }
-    return cudaGetLastError();
 }
 
 template <int A>

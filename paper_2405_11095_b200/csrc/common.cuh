@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 namespace fosgd {
 
 // ---- sources and sinks of a transform pass -------------------------------------------
@@ -19,7 +21,8 @@ enum Sink : int {
     SINK_WS = 0,     // fp32 intermediate (or the scaled transform output of fosgd_flatten)
     SINK_PACK1 = 1,  // dither + sign + pack, K = 1
     SINK_PACKK = 2,  // K dithers, count, P bit planes
-    SINK_FINAL = 3   // flip, sum over the workers of the launch, optional read-modify-write, scale
+    SINK_FINAL = 3,  // flip, sum over the workers of the launch, optional read-modify-write, scale
+    SINK_SINGLE = 4  // SINK_FINAL of a launch with one worker: no sums kept in registers
 };
 
 struct Rng {
@@ -138,12 +141,6 @@ __device__ __forceinline__ uint32_t eps_word(const Rng& g, uint32_t id, uint32_t
     return pick(rng_words(g, id, 0u, j >> 2), j & 3u);
 }
 
-// Dither integer from one generator word: t = 2*k24 + 1 - 2^24 (odd, |t| < 2^24, exact in fp32).
-__device__ __forceinline__ float dither_from_word(uint32_t w)
-{
-    return (float)((int)((w >> 8) << 1) - 16777215);
-}
-
 __device__ __forceinline__ float flip_by_bit(float x, uint32_t word, uint32_t bit)
 {
     return __uint_as_float(__float_as_uint(x) ^ (((word >> bit) & 1u) << 31));
@@ -245,6 +242,127 @@ __device__ __forceinline__ bool group_all(int id, int nthreads, bool ok)
     return all != 0;
 }
 
+// ---- thread-block clusters: the blocks of a cluster read each other's shared memory ----------------
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// four floats at shared-memory address `addr` (a multiple of 16) of the cluster's block `rank`
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr, uint32_t rank)
+{
+    uint32_t remote;
+    float4 q;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(q.x), "=f"(q.y), "=f"(q.z), "=f"(q.w) : "r"(remote) : "memory");
+    return q;
+}
+
+// SINK_FINAL / SINK_SINGLE: one finished sum to memory (sc = scale times amplitude)
+__device__ __forceinline__ void store_final(float* dst, float o, float sc, int overwrite)
+{
+    if (overwrite == 2) {
+        *dst = fmaf(o, sc, *dst);   // dst += scale * sum (the descent step on top of the decoder)
+    } else {
+        if (!overwrite) o += *dst;
+        *dst = o * sc;
+    }
+}
+
+__device__ __forceinline__ void store_final4(float* dst, float4 o, float sc, int overwrite)
+{
+    float4* const d4 = reinterpret_cast<float4*>(dst);
+    if (overwrite == 2) {
+        const float4 c = *d4;
+        o = make_float4(fmaf(o.x, sc, c.x), fmaf(o.y, sc, c.y), fmaf(o.z, sc, c.z), fmaf(o.w, sc, c.w));
+    } else {
+        if (!overwrite) {
+            const float4 c = *d4;
+            o.x += c.x; o.y += c.y; o.z += c.z; o.w += c.w;
+        }
+        o.x *= sc; o.y *= sc; o.z *= sc; o.w *= sc;
+    }
+    *d4 = o;
+}
+
+// The blocks of a cluster have each left their workers' sums of one tile of 2^T coordinates in shared memory at
+// `sums` (`at(e)` = word offset of coordinate e, whole groups of four together); block `rank` of `size` adds its
+// share of the coordinates over the blocks in order and stores it.  All threads of all blocks call it.
+template <int T, typename At>
+__device__ __forceinline__ void cluster_reduce_store(const PassParams& p, int64_t tile_base, const float* sums, uint32_t rank,
+                                                     uint32_t size, float sc, At at)
+{
+    cluster_sync();
+    const uint32_t share = (1u << T) / size, base = smem_u32(sums);
+    float* const dst = static_cast<float*>(p.dst) + tile_base;
+    for (uint32_t e = rank * share + 4u * threadIdx.x; e < (rank + 1u) * share; e += 4u * blockDim.x) {
+        float4 o = ld_cluster4(base + 4u * at(e), 0u);
+        for (uint32_t k = 1; k < size; ++k) {
+            const float4 q = ld_cluster4(base + 4u * at(e), k);
+            o.x += q.x; o.y += q.y; o.z += q.z; o.w += q.w;
+        }
+        const int64_t left = p.d_out - (tile_base + e);
+        if (left >= 4) {
+            store_final4(dst + e, o, sc, p.overwrite);
+        } else {
+            if (left > 0) store_final(dst + e, o.x, sc, p.overwrite);
+            if (left > 1) store_final(dst + e + 1, o.y, sc, p.overwrite);
+            if (left > 2) store_final(dst + e + 2, o.z, sc, p.overwrite);
+        }
+    }
+    cluster_sync();   // nobody leaves while its sums are being read
+}
+
+// ---- launching ---------------------------------------------------------------------------------
+// One kernel launch.  Dynamic shared memory beyond the default is allowed once per kernel and device (a driver
+// attribute, cheaper to remember than to set before every launch); cluster > 1: clusters of that many blocks in y.
+template <auto Kern, typename... Args>
+inline cudaError_t launch(dim3 grid, unsigned threads, size_t smem, cudaStream_t s, unsigned cluster, const Args&... args)
+{
+    static std::atomic<uint64_t> allowed{0};   // bit = device
+    cudaError_t e;
+    if (smem > 48 * 1024) {
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+        if (!(allowed.load(std::memory_order_acquire) & bit) || bit == 0) {
+            if ((e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+            allowed.fetch_or(bit, std::memory_order_release);
+        }
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    if (cluster > 1) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 1;
+        attr[0].val.clusterDim.y = cluster;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, Kern, args...);
+}
+
+inline cudaError_t sm_count(int* sms)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
+// Blocks (a power of two, at most the eight of a portable cluster) that share the workers of one tile, when
+// `tiles` blocks alone would leave the chip idle: as many as fit beside each other, at least two workers each.
+inline unsigned worker_split(int64_t tiles, int nworkers, int64_t resident_blocks)
+{
+    unsigned s = 1;
+    while (s < 8 && tiles * (2 * s) <= resident_blocks && nworkers >= (int)(4 * s)) s *= 2;
+    return s;
+}
+
 // ---- shared by the translation units of the C-ABI (not exported) -----------------------------
 // thread-local last CUDA error behind fosgd_last_cuda_error()
 __attribute__((visibility("hidden"))) void set_last_cuda_error(int e);
@@ -255,7 +373,8 @@ __attribute__((visibility("hidden"))) int check_decode_args(const void* bits, in
 // ---- host-visible launchers (one translation unit per family) --------------------------
 cudaError_t launch_row(int T, int src, int sink, const PassParams& p, cudaStream_t s);
 cudaError_t launch_col(int A, int src, const PassParams& p, cudaStream_t s);
-cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s);   // one-plane bits -> fp16 intermediate
+bool colh_applicable(int A, const PassParams& p);                          // every value after A stages exact in fp16
+cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s);   // packed planes -> fp16 intermediate
 bool tc_col_applicable(const PassParams& p, bool any_size);                            // ten strided stages from one plane on the tensor cores
 cudaError_t launch_tc_col(const PassParams& p, cudaStream_t s);          // one-plane bits -> fp16 intermediate
 cudaError_t tc_timeouts(int* out);
@@ -273,7 +392,7 @@ cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t wo
                               double alpha_s, double n_eff, float* lam, float* lam_s, double* partial, cudaStream_t s);
 cudaError_t launch_amplitudes_finalize(const double* partial, int M, int nparts, double alpha, double alpha_s, double n_eff,
                                        float* lam, float* lam_s, cudaStream_t s);
-cudaError_t launch_col4_norm(const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nruns_out);
+cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nparts_out);
 cudaError_t launch_block_amplitudes(const void* grads, int bf16, int64_t d, int64_t dp, int64_t worker_stride, int M,
                                     int block_log2, double alpha, double alpha_s, float* lam, float* lam_s,
                                     double* seg, cudaStream_t st);

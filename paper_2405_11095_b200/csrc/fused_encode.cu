@@ -98,17 +98,17 @@ __device__ __forceinline__ void row_role(const PassParamsRK& p, uint32_t* const 
         const float amp = amplitude_at(p, n, tile_base);
 
         float v[32];
-        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + tile_base;
+        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + tile_base + baseF;
+        static_assert(C::VB == 1, "pairs of coordinates per load");
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const float4 x = __ldcg(reinterpret_cast<const float4*>(src + (baseF | (g << (kT - 3)))));   // written by other SMs: L2
-            v[4 * g + 0] = x.x; v[4 * g + 1] = x.y; v[4 * g + 2] = x.z; v[4 * g + 3] = x.w;
+        for (int g = 0; g < 16; ++g) {
+            const float2 x = __ldcg(reinterpret_cast<const float2*>(src + round_F_offset<kT>(g)));   // written by other SMs: L2
+            v[2 * g + 0] = x.x; v[2 * g + 1] = x.y;
         }
         butterflies32<31>(v);
         store_round_F<kT>(smem, baseF, v);
         S::sync();
         round_M<kT>(smem, baseM, v);
-        S::sync();
         load_round_L(smem, baseL, v);
         butterflies32<C::ACT_L>(v);
         sink_pack1(p, n, id, tile_base + baseL, lane, v, amp);

@@ -5,22 +5,26 @@
 // 32 values in registers and the block runs three register rounds of up to five stages each,
 // exchanging through shared memory (row pitch 36 words: no bank conflicts in any round).
 //
-//   round F: register bits {0, 1, T-3, T-2, T-1}   128-bit loads, 128-bit shared stores
-//   round M: register bits {2, 3, 4, m1, m2}       (m1, m2) = (10, 11), or (T-2, T-1) if T < 12
-//   round L: register bits {5, 6, 7, 8, 9}         lane = bits 0..4, so lane r can own packed word r
+//   round F: register bits 10 .. T-1 and, up to five, the lowest (vector loads) and bits 9, 8, 7
+//   round M: register bits 0 .. 4, lane = bits 5 .. 9    (128-bit shared loads and stores)
+//   round L: register bits 5 .. 9, lane = bits 0 .. 4, so lane r can own packed word r
 //
-// A bit that two rounds hold is transformed by the first and rides along in the second.
+// A bit that two rounds hold is transformed by the first and rides along in the second.  All bits
+// above 9 are done in round F, so from then on a warp works on 1024 consecutive coordinates of its
+// own: one block-wide barrier per tile, between F and M, and none between M and L.  (Earlier form:
+// F on {0, 1, T-3 .. T-1}, M on {2, 3, 4, 10, 11} with 32-bit accesses and a second block barrier.)
 //
 // Two kernels share these rounds:
 //   row_kernel        source read by the threads themselves: gradients and packed bits (the
-//                     single-pass case, transform length <= 2^15), and fp32 intermediates whose
-//                     tile is too large for a separate landing buffer.
+//                     single-pass case, transform length <= 2^15), and fp32 intermediates on the way
+//                     to a dither sink or with a tile too large for a separate landing buffer.
 //   row_stream_kernel source = intermediate of the strided passes, fetched tile by tile with
 //                     the bulk async copy engine (cp.async.bulk + mbarrier) into a landing
 //                     buffer beside the work tile: the copy of tile k+1 starts as soon as
 //                     round F has read tile k, and runs underneath the other rounds and the sink.
 #pragma once
 #include "common.cuh"
+#include "dither.cuh"
 
 namespace fosgd {
 
@@ -71,9 +75,9 @@ __device__ __forceinline__ int deposit(int tid)
 template <int T>
 struct RowCfg {
     static constexpr int NT = 1 << (T - 5);
-    static constexpr uint32_t FMASK = 0x3u | (0x7u << (T - 3));
-    static constexpr int M1 = (T >= 12) ? 10 : T - 2;
-    static constexpr uint32_t MMASK = 0x1Cu | (0x3u << M1);
+    static constexpr int VB = (T >= 15) ? 0 : (T == 14 ? 1 : 2);      // log2 of the vector of a round-F load
+    static constexpr uint32_t FMASK = ((1u << VB) - 1u) | (((1u << (5 - VB)) - 1u) << (T - (5 - VB)));
+    static constexpr uint32_t MMASK = 0x1Fu;
     static constexpr uint32_t LMASK = 0x3E0u;
     static constexpr int ACT_M = active_mask(MMASK, FMASK);
     static constexpr int ACT_L = active_mask(LMASK, FMASK | MMASK);
@@ -106,25 +110,39 @@ __host__ __device__ constexpr int min_blocks()
 }
 
 // ---- the three rounds on the padded tile ---------------------------------------------------
+// registers g * 2^VB .. + 2^VB - 1 of round F are consecutive coordinates starting at this tile offset
+template <int T>
+__device__ __forceinline__ constexpr int round_F_offset(int g) { return reg_offset(RowCfg<T>::FMASK, g << RowCfg<T>::VB); }
+
 template <int T>
 __device__ __forceinline__ void store_round_F(float* smem, int baseF, const float (&v)[32])
 {
+    constexpr int VB = RowCfg<T>::VB;
+    float* const pf = smem + phys(baseF);   // (the lane's low coordinate bits never carry into the register bits)
 #pragma unroll
-    for (int g = 0; g < 8; ++g)
-        *reinterpret_cast<float4*>(smem + phys(baseF | (g << (T - 3)))) =
-            make_float4(v[4 * g + 0], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+    for (int g = 0; g < (32 >> VB); ++g) {
+        float* const q = pf + phys(round_F_offset<T>(g));
+        if constexpr (VB == 2) *reinterpret_cast<float4*>(q) = make_float4(v[4 * g + 0], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        else if constexpr (VB == 1) *reinterpret_cast<float2*>(q) = make_float2(v[2 * g + 0], v[2 * g + 1]);
+        else *q = v[g];
+    }
 }
 
+// this warp's 1024 coordinates: lane = bits 5..9, registers = bits 0..4
 template <int T>
 __device__ __forceinline__ void round_M(float* smem, int baseM, float (&v)[32])
 {
     using C = RowCfg<T>;
-    float* const pm = smem + phys(baseM);
+    float4* const pm = reinterpret_cast<float4*>(smem + phys(baseM));
 #pragma unroll
-    for (int r = 0; r < 32; ++r) v[r] = pm[phys(reg_offset(C::MMASK, r))];
+    for (int q = 0; q < 8; ++q) {
+        const float4 x = pm[q];
+        v[4 * q + 0] = x.x; v[4 * q + 1] = x.y; v[4 * q + 2] = x.z; v[4 * q + 3] = x.w;
+    }
     butterflies32<C::ACT_M>(v);
 #pragma unroll
-    for (int r = 0; r < 32; ++r) pm[phys(reg_offset(C::MMASK, r))] = v[r];
+    for (int q = 0; q < 8; ++q) pm[q] = make_float4(v[4 * q + 0], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+    __syncwarp();
 }
 
 __device__ __forceinline__ void load_round_L(const float* smem, int baseL, float (&v)[32])
@@ -211,19 +229,149 @@ __device__ __forceinline__ void sink_packK(const PassParamsRK& p, int n, uint32_
 
 __device__ __forceinline__ void sink_final_store(const PassParams& p, int64_t i0, const float (&accv)[32], float amp)
 {
-    float* dst = static_cast<float*>(p.dst);
+    float* const dst = static_cast<float*>(p.dst) + i0;
     const float sc = p.scale * amp;
+    const int64_t left = p.d_out - i0;
+    if (p.overwrite == 1) {
 #pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const int64_t i = i0 + (r << 5);
-        if (i < p.d_out) {
-            float o = accv[r];
-            if (p.overwrite == 2) {
-                dst[i] = fmaf(o, sc, dst[i]);   // dst += scale * sum (the descent step on top of the decoder)
+        for (int r = 0; r < 32; ++r)
+            if ((r << 5) < left) dst[r << 5] = accv[r] * sc;
+    } else {
+        // read-modify-write, eight loads in flight at a time
+#pragma unroll
+        for (int q = 0; q < 32; q += 8) {
+            float c[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) c[r] = ((q + r) << 5) < left ? dst[(q + r) << 5] : 0.f;
+#pragma unroll
+            for (int r = 0; r < 8; ++r)
+                if (((q + r) << 5) < left) dst[(q + r) << 5] = p.overwrite == 2 ? fmaf(accv[q + r], sc, c[r]) : (accv[q + r] + c[r]) * sc;
+        }
+    }
+}
+
+// the same for a tile whose workers were shared among the blocks of a cluster
+template <int T>
+__device__ __forceinline__ void split_final_store(const PassParams& p, int64_t tile_base, int baseL, float* smem,
+                                                  const float (&accv)[32], float amp)
+{
+    __syncthreads();   // the exchange tile is free
+#pragma unroll
+    for (int r = 0; r < 32; ++r) smem[baseL + (r << 5)] = accv[r];
+    cluster_reduce_store<T>(p, tile_base, smem, blockIdx.y, gridDim.y, p.scale * amp, [](uint32_t e) { return e; });
+}
+
+// ---- round F's registers from memory ----------------------------------------------------------
+// fw: flip words of the tile (gradient sources)
+template <int T, int SRC>
+__device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t tile_base, int baseF, const uint32_t* fw,
+                                            float (&v)[32])
+{
+    constexpr int VB = RowCfg<T>::VB, VN = 1 << VB;
+    const int64_t i0 = tile_base + baseF;
+    if constexpr (SRC == SRC_G32) {
+        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
+        const int64_t left = p.d - i0;    // valid elements from this thread's first coordinate on
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int o = round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if (o + VN <= left) {
+                if constexpr (VB == 2) {
+                    const float4 q = __ldcs(reinterpret_cast<const float4*>(src + o));
+                    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+                } else if constexpr (VB == 1) {
+                    const float2 q = __ldcs(reinterpret_cast<const float2*>(src + o));
+                    x[0] = q.x; x[1] = q.y;
+                } else {
+                    x[0] = __ldcs(src + o);
+                }
             } else {
-                if (!p.overwrite) o += dst[i];
-                dst[i] = o * sc;
+#pragma unroll
+                for (int k = 0; k < VN; ++k) x[k] = (o + k < left) ? src[o + k] : 0.f;
             }
+        }
+    } else if constexpr (SRC == SRC_G16) {
+        const uint16_t* const src = static_cast<const uint16_t*>(p.src) + (int64_t)n * p.src_stride + i0;
+        const int64_t left = p.d - i0;
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int o = round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if (VB > 0 && o + VN <= left) {
+                if constexpr (VB == 2) {
+                    const uint2 q = __ldcs(reinterpret_cast<const uint2*>(src + o));
+                    x[0] = __uint_as_float(q.x << 16); x[1] = __uint_as_float(q.x & 0xFFFF0000u);
+                    x[2] = __uint_as_float(q.y << 16); x[3] = __uint_as_float(q.y & 0xFFFF0000u);
+                } else if constexpr (VB == 1) {
+                    const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(src + o));
+                    x[0] = __uint_as_float(q << 16); x[1] = __uint_as_float(q & 0xFFFF0000u);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < VN; ++k) x[k] = (o + k < left) ? __uint_as_float((uint32_t)src[o + k] << 16) : 0.f;
+            }
+        }
+    } else if constexpr (SRC == SRC_WS) {
+        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int o = round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if constexpr (VB == 2) {
+                const float4 q = __ldcs(reinterpret_cast<const float4*>(src + o));
+                x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+            } else if constexpr (VB == 1) {
+                const float2 q = __ldcs(reinterpret_cast<const float2*>(src + o));
+                x[0] = q.x; x[1] = q.y;
+            } else {
+                x[0] = __ldcs(src + o);
+            }
+        }
+    } else if constexpr (SRC == SRC_WS16) {
+        const __half* const src = static_cast<const __half*>(p.src) + (int64_t)n * p.src_stride + i0;
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int o = round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if constexpr (VB == 2) {
+                const uint2 q = __ldcs(reinterpret_cast<const uint2*>(src + o));
+                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
+                const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
+                x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
+            } else if constexpr (VB == 1) {
+                const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(src + o));
+                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q));
+                x[0] = a.x; x[1] = a.y;
+            } else {
+                x[0] = __half2float(__ldcs(src + o));
+            }
+        }
+    } else {  // SRC_BITS
+        const uint32_t* const src = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride + (tile_base >> 5);
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int e0 = baseF | round_F_offset<T>(g);
+            const uint32_t pos = (uint32_t)e0 & 31u;
+            float* const x = v + g * VN;
+            if (p.P == 1) {
+                const uint32_t w = __ldg(src + (e0 >> 5)) >> pos;
+#pragma unroll
+                for (int k = 0; k < VN; ++k) x[k] = (w & (1u << k)) ? 1.f : -1.f;
+            } else {
+#pragma unroll
+                for (int k = 0; k < VN; ++k) x[k] = plane_value(src + (e0 >> 5), p.dp >> 5, p.P, p.K, pos + k);
+            }
+        }
+    }
+    if constexpr (SRC == SRC_G32 || SRC == SRC_G16) {
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const int e0 = baseF | round_F_offset<T>(g);
+            const uint32_t w = fw[e0 >> 5];
+            const uint32_t pos = (uint32_t)e0 & 31u;
+#pragma unroll
+            for (int k = 0; k < VN; ++k) v[g * VN + k] = flip_by_bit(v[g * VN + k], w, pos + k);
         }
     }
 }
@@ -241,15 +389,21 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
     const int tid = threadIdx.x;
     const uint32_t lane = tid & 31;
     const int64_t tile_base = (int64_t)blockIdx.x << T;
+    // SINK_FINAL: the blocks of a cluster (gridDim.y of them, one if the tiles alone fill the chip) take the
+    // workers in turn and add up their sums at the end
     constexpr bool kLoopWorkers = (SINK == SINK_FINAL);
-    constexpr bool kFlips = (SRC == SRC_G32 || SRC == SRC_G16 || SINK == SINK_FINAL);
-    const int n_begin = kLoopWorkers ? 0 : (int)blockIdx.y;
+    constexpr bool kFlips = (SRC == SRC_G32 || SRC == SRC_G16 || SINK == SINK_FINAL || SINK == SINK_SINGLE);
+    const int n_begin = (int)blockIdx.y;
     const int n_end = kLoopWorkers ? p.nworkers : n_begin + 1;
+    const int n_step = kLoopWorkers ? (int)gridDim.y : 1;
     // one amplitude per tile (a block of the blocked mode is at least a tile): thread 0 reads it
     // first, so that its latency hides behind the tile load, and parks it in shared memory until
     // the sink (the barriers of the exchange rounds order the two)
     __shared__ float s_amp;
-    if (tid == 0) s_amp = (!kLoopWorkers || p.amp_mode == AMP_SCALE) ? amplitude_at(p, n_begin, tile_base) : 1.f;
+    if (tid == 0) {
+        if (SINK == SINK_SINGLE) s_amp = p.amp_mode != AMP_DITHER ? amplitude_at(p, 0, tile_base) : 1.f;
+        else s_amp = (!kLoopWorkers || p.amp_mode == AMP_SCALE) ? amplitude_at(p, kLoopWorkers ? 0 : n_begin, tile_base) : 1.f;
+    }
 
     const int baseF = deposit<C::FMASK, T>(tid);
     const int baseM = deposit<C::MMASK, T>(tid);
@@ -262,7 +416,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         for (int r = 0; r < 32; ++r) accv[r] = 0.f;
     }
 
-    for (int n = n_begin; n < n_end; ++n) {
+    for (int n = n_begin; n < n_end; n += n_step) {
         const uint32_t id = p.id0 + (uint32_t)n;
         const float wamp = (kLoopWorkers && p.amp_mode == AMP_WEIGHT) ? amplitude_at(p, n, tile_base) : 1.f;
         if (kFlips) {
@@ -275,67 +429,11 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         }
 
         float v[32];
-        // ---------------- round F: load ----------------
-#pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const int e0 = baseF | (g << (T - 3));
-            const int64_t i = tile_base + e0;
-            float x0, x1, x2, x3;
-            if (SRC == SRC_G32) {
-                const float* src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride;
-                if (i + 3 < p.d) {
-                    const float4 q = __ldcs(reinterpret_cast<const float4*>(src + i));
-                    x0 = q.x; x1 = q.y; x2 = q.z; x3 = q.w;
-                } else {
-                    x0 = (i + 0 < p.d) ? src[i + 0] : 0.f;
-                    x1 = (i + 1 < p.d) ? src[i + 1] : 0.f;
-                    x2 = (i + 2 < p.d) ? src[i + 2] : 0.f;
-                    x3 = 0.f;
-                }
-            } else if (SRC == SRC_G16) {
-                const uint16_t* src = static_cast<const uint16_t*>(p.src) + (int64_t)n * p.src_stride;
-                uint32_t lo, hi;
-                if (i + 3 < p.d) {
-                    const uint2 q = __ldcs(reinterpret_cast<const uint2*>(src + i));
-                    lo = q.x; hi = q.y;
-                } else {
-                    const uint32_t h0 = (i + 0 < p.d) ? src[i + 0] : 0u;
-                    const uint32_t h1 = (i + 1 < p.d) ? src[i + 1] : 0u;
-                    const uint32_t h2 = (i + 2 < p.d) ? src[i + 2] : 0u;
-                    lo = h0 | (h1 << 16); hi = h2;
-                }
-                x0 = __uint_as_float(lo << 16); x1 = __uint_as_float(lo & 0xFFFF0000u);
-                x2 = __uint_as_float(hi << 16); x3 = __uint_as_float(hi & 0xFFFF0000u);
-            } else if (SRC == SRC_WS) {
-                const float* src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride;
-                const float4 q = __ldcs(reinterpret_cast<const float4*>(src + i));
-                x0 = q.x; x1 = q.y; x2 = q.z; x3 = q.w;
-            } else {  // SRC_BITS
-                const uint32_t* src = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride + (i >> 5);
-                const uint32_t pos = (uint32_t)i & 31u;
-                if (p.P == 1) {
-                    const uint32_t w = __ldg(src) >> pos;
-                    x0 = (w & 1u) ? 1.f : -1.f; x1 = (w & 2u) ? 1.f : -1.f;
-                    x2 = (w & 4u) ? 1.f : -1.f; x3 = (w & 8u) ? 1.f : -1.f;
-                } else {
-                    const int64_t pw = p.dp >> 5;
-                    x0 = plane_value(src, pw, p.P, p.K, pos + 0); x1 = plane_value(src, pw, p.P, p.K, pos + 1);
-                    x2 = plane_value(src, pw, p.P, p.K, pos + 2); x3 = plane_value(src, pw, p.P, p.K, pos + 3);
-                }
-            }
-            if (SRC == SRC_G32 || SRC == SRC_G16) {
-                const uint32_t w = fw[e0 >> 5];
-                const uint32_t pos = (uint32_t)e0 & 31u;
-                x0 = flip_by_bit(x0, w, pos + 0); x1 = flip_by_bit(x1, w, pos + 1);
-                x2 = flip_by_bit(x2, w, pos + 2); x3 = flip_by_bit(x3, w, pos + 3);
-            }
-            v[4 * g + 0] = x0; v[4 * g + 1] = x1; v[4 * g + 2] = x2; v[4 * g + 3] = x3;
-        }
+        load_source<T, SRC>(p, n, tile_base, baseF, fw, v);
         butterflies32<31>(v);
         store_round_F<T>(smem, baseF, v);
         __syncthreads();
         round_M<T>(smem, baseM, v);
-        __syncthreads();
         load_round_L(smem, baseL, v);
         butterflies32<C::ACT_L>(v);
 
@@ -345,13 +443,107 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
             sink_pack1(p, n, id, i0, lane, v, s_amp);
         } else if constexpr (SINK == SINK_PACKK) {
             sink_packK(p, n, id, i0, lane, v, s_amp);
+        } else if constexpr (SINK == SINK_SINGLE) {
+            const uint32_t* const fwl = fw + ((baseL - (int)lane) >> 5);
+            // (a per-worker weight rounds the sum first, as it does among several workers)
+            const float w = p.amp_mode == AMP_WEIGHT ? s_amp : 1.f;
+#pragma unroll
+            for (int r = 0; r < 32; ++r) v[r] = flip_by_bit(v[r], fwl[r], lane) * w;
+            sink_final_store(p, i0, v, p.amp_mode == AMP_WEIGHT ? 1.f : s_amp);
         } else {
             const uint32_t* const fwl = fw + ((baseL - (int)lane) >> 5);
 #pragma unroll
             for (int r = 0; r < 32; ++r) accv[r] = fmaf(flip_by_bit(v[r], fwl[r], lane), wamp, accv[r]);
         }
     }
-    if (SINK == SINK_FINAL) sink_final_store(p, i0, accv, s_amp);
+    if constexpr (SINK == SINK_FINAL) {
+        if (gridDim.y == 1) sink_final_store(p, i0, accv, s_amp);
+        else split_final_store<T>(p, tile_base, baseL, smem, accv, s_amp);
+    }
+}
+
+// =============================================================================================
+// row_packk_kernel: K > 1 dithers on few tiles, or many dithers
+// =============================================================================================
+// The generator dominates (K calls per four coordinates against three register rounds), so the block transforms its
+// tile into shared memory and its warps then share out the tile's (group of 128 coordinates, range of dithers)
+// units.  Where the tiles leave the chip idle, gridDim.y blocks transform the same tile and each dithers a part
+// of its groups: one vector of 2^13 with K = 255, a single tile, takes 8 us (without the launch 13.5) against 310
+// in one block of eight warps with all dithers of 32 coordinates to a lane; 2^20 with K = 255 0.21 ms against 0.51.
+// On a full grid row_kernel's in-register sink is the faster one up to about 24 dithers (2^24, K = 3 / 15 / 31:
+// 62 / 228 / 445 us against 84 / 244 / 416): it has eight generator calls in flight per lane and no ballots.
+constexpr int kManyDithers = 24;
+
+template <int T>
+struct PackKCfg {
+    static constexpr int THREADS = RowCfg<T>::NT < 256 ? 256 : RowCfg<T>::NT;
+    static constexpr int WARPS = THREADS / 32;
+    static constexpr int GROUPS = 1 << (T - 7);
+    static constexpr int MIN_BLOCKS = 1024 / THREADS;
+    static constexpr size_t SMEM_BYTES = RowCfg<T>::SMEM_BYTES + (size_t)WARPS * 128;   // + packed counts of up to WARPS groups
+};
+
+template <int T, int SRC>
+__global__ void __launch_bounds__(PackKCfg<T>::THREADS, PackKCfg<T>::MIN_BLOCKS) row_packk_kernel(const PassParamsRK p)
+{
+    using C = RowCfg<T>;
+    using K = PackKCfg<T>;
+    extern __shared__ __align__(16) float smem[];
+    uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);
+    uint32_t* const counts = fw + C::FLIP_WORDS + 4;
+    const int tid = threadIdx.x;
+    const uint32_t lane = tid & 31;
+    const int warp = tid >> 5;
+    const int64_t tile_base = (int64_t)blockIdx.x << T;
+    const int n = blockIdx.z;
+    const uint32_t id = p.id0 + (uint32_t)n;
+    const bool active = K::THREADS == C::NT || tid < C::NT;      // (whole warps)
+    const float dc = p.dither_c * amplitude_at(p, n, tile_base);
+
+    if (SRC == SRC_G32) {
+        if (tid < C::FLIP_WORDS / 4)
+            reinterpret_cast<uint4*>(fw)[tid] = rng_words(p.rng, id, 0u, (uint32_t)(tile_base >> 7) + (uint32_t)tid);
+        __syncthreads();
+    }
+    if (active) {
+        const int baseF = deposit<C::FMASK, T>(tid);
+        float v[32];
+        load_source<T, SRC>(p, n, tile_base, baseF, fw, v);
+        butterflies32<31>(v);
+        store_round_F<T>(smem, baseF, v);
+    }
+    __syncthreads();
+    if (active) {
+        const int baseL = deposit<C::LMASK, T>(tid);
+        float v[32];
+        round_M<T>(smem, deposit<C::MMASK, T>(tid), v);
+        load_round_L(smem, baseL, v);
+        butterflies32<C::ACT_L>(v);
+        float* const pl = smem + phys(baseL);
+#pragma unroll
+        for (int r = 0; r < 32; ++r) pl[phys(r << 5)] = v[r];
+    }
+    counts[tid] = 0u;
+    __syncthreads();
+
+    // this block's groups, and how many warps share the dithers of one (all powers of two)
+    const int ngroups = K::GROUPS / (int)gridDim.y, g_first = (int)blockIdx.y * ngroups;
+    const int share = ngroups < K::WARPS ? K::WARPS / ngroups : 1;
+    const int k0 = p.K * (warp % share) / share, k1 = p.K * (warp % share + 1) / share;
+    uint32_t* const dst = static_cast<uint32_t*>(p.dst) + (int64_t)n * p.dst_stride + (tile_base >> 5);
+    for (int j = warp / share; j < ngroups; j += K::WARPS / share) {
+        const int g = g_first + j;
+        float y[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) y[r] = smem[phys(128 * g + 32 * r) + (int)lane];
+        const uint32_t c = dither_counts(p, id, (((uint32_t)(tile_base >> 7) + (uint32_t)g) << 5) + lane, y, dc, k0, k1);
+        if (share == 1) store_count_planes(c, lane, p.P, dst + 4 * g, p.dp >> 5);
+        else atomicAdd(counts + 32 * j + (int)lane, c);
+    }
+    if (share > 1) {
+        __syncthreads();
+        if (warp < ngroups) store_count_planes(counts[32 * warp + (int)lane], lane, p.P, dst + 4 * (g_first + warp), p.dp >> 5);
+    }
 }
 
 // =============================================================================================
@@ -398,21 +590,22 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
     const int tid = threadIdx.x;
     const uint32_t lane = tid & 31;
     constexpr bool kFinal = (SINK == SINK_FINAL);
-    // SINK_FINAL: this block's tile is fixed, one amplitude scales the sum (AMP_SCALE) or every
-    // worker brings its own weight (AMP_WEIGHT); pack sinks read the amplitude of each item
-    // (parked in shared memory until the store; the barriers of the worker loop order the two)
+    // SINK_FINAL: this block's tile is fixed, one amplitude scales the sum (AMP_SCALE; parked in shared
+    // memory until the store, the barriers of the worker loop order the two) or every worker brings its
+    // own weight (AMP_WEIGHT)
     __shared__ float s_amp_final;
     if (tid == 0) s_amp_final = (kFinal && p.amp_mode == AMP_SCALE) ? amplitude_at(p, 0, (int64_t)blockIdx.x << T) : 1.f;
-    // work items: SINK_FINAL -> this block's tile for every worker in turn;
+    // work items: SINK_FINAL -> this block's tile for every worker in turn (every gridDim.y-th of them
+    //             where the blocks of a cluster share a tile's workers);
     //             otherwise  -> (worker, tile) pairs strided over the grid
-    const int64_t nitems = kFinal ? (int64_t)p.nworkers
+    const int64_t nitems = kFinal ? (int64_t)((p.nworkers - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y)
                                   : (ntiles * p.nworkers - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x;
 
     const int baseF = deposit<C::FMASK, T>(tid);
     const int baseM = deposit<C::MMASK, T>(tid);
     const int baseL = deposit<C::LMASK, T>(tid);
 
-    auto item_worker = [&](int64_t j) -> int { return kFinal ? (int)j : (int)((blockIdx.x + j * gridDim.x) / ntiles); };
+    auto item_worker = [&](int64_t j) -> int { return kFinal ? (int)(blockIdx.y + j * gridDim.y) : (int)((blockIdx.x + j * gridDim.x) / ntiles); };
     auto item_tile = [&](int64_t j) -> int64_t { return kFinal ? (int64_t)blockIdx.x : (int64_t)((blockIdx.x + j * gridDim.x) % ntiles); };
     auto item_src = [&](int64_t j) -> const char* {
         return static_cast<const char*>(p.src) + ((int64_t)item_worker(j) * p.src_stride + (item_tile(j) << T)) * kElem;
@@ -436,7 +629,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
         const int64_t tile_base = item_tile(j) << T;
         const int64_t i0 = tile_base + baseL;
         const uint32_t id = p.id0 + (uint32_t)n;
-        const float amp = (!kFinal || p.amp_mode == AMP_WEIGHT) ? amplitude_at(p, n, tile_base) : 1.f;
+        const float amp = (kFinal && p.amp_mode == AMP_WEIGHT) ? amplitude_at(p, n, tile_base) : 1.f;
 
         // bounded wait; the block then agrees on the outcome, so that it stops as a whole
         if (!__syncthreads_and(mbar_wait(bar, parity) ? 1 : 0)) {
@@ -448,23 +641,32 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
                 mbar_inval(bar);
             }
             __syncthreads();
-            return;
+            break;   // (the sums stay incomplete; the blocks of a cluster still meet at its end)
         }
         parity ^= 1u;
 
         float v[32];
         // round F reads the tile as it arrived (linear) and writes the padded exchange layout
+        constexpr int VN = 1 << C::VB;
 #pragma unroll
-        for (int g = 0; g < 8; ++g) {
-            const int e0 = baseF | (g << (T - 3));
-            if (SRC == SRC_WS) {
+        for (int g = 0; g < (32 >> C::VB); ++g) {
+            const int e0 = baseF | round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if constexpr (SRC == SRC_WS) {
+                static_assert(SRC != SRC_WS || C::VB == 2, "fp32 tiles are streamed up to 2^13");
                 const float4 q = *reinterpret_cast<const float4*>(landing + e0);
-                v[4 * g + 0] = q.x; v[4 * g + 1] = q.y; v[4 * g + 2] = q.z; v[4 * g + 3] = q.w;
+                x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
             } else {
-                const uint2 q = *reinterpret_cast<const uint2*>(reinterpret_cast<const __half*>(landing) + e0);
-                const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
-                const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
-                v[4 * g + 0] = a.x; v[4 * g + 1] = a.y; v[4 * g + 2] = b.x; v[4 * g + 3] = b.y;
+                const __half* const h = reinterpret_cast<const __half*>(landing) + e0;
+                if constexpr (C::VB == 0) {
+                    x[0] = __half2float(h[0]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < VN; k += 2) {
+                        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(h + k));
+                        x[k] = a.x; x[k + 1] = a.y;
+                    }
+                }
             }
         }
         butterflies32<31>(v);
@@ -477,24 +679,22 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
             reinterpret_cast<uint4*>(fw)[tid] = w;
         }
         round_M<T>(smem, baseM, v);
-        __syncthreads();
         load_round_L(smem, baseL, v);
         __syncthreads();   // the tile lives in registers: the work tile may be overwritten by the next round F
         butterflies32<C::ACT_L>(v);
 
         if constexpr (SINK == SINK_WS) {
             sink_ws(p, n, i0, v);
-        } else if constexpr (SINK == SINK_PACK1) {
-            sink_pack1(p, n, id, i0, lane, v, amp);
-        } else if constexpr (SINK == SINK_PACKK) {
-            sink_packK(p, n, id, i0, lane, v, amp);
         } else {
             const uint32_t* const fwl = fw + ((baseL - (int)lane) >> 5);
 #pragma unroll
             for (int r = 0; r < 32; ++r) accv[r] = fmaf(flip_by_bit(v[r], fwl[r], lane), amp, accv[r]);
         }
     }
-    if (kFinal) sink_final_store(p, ((int64_t)blockIdx.x << T) + baseL, accv, s_amp_final);
+    if constexpr (kFinal) {
+        if (gridDim.y == 1) sink_final_store(p, ((int64_t)blockIdx.x << T) + baseL, accv, s_amp_final);
+        else split_final_store<T>(p, (int64_t)blockIdx.x << T, baseL, smem, accv, s_amp_final);
+    }
 }
 
 // ---- launchers ---------------------------------------------------------------------------------
@@ -503,29 +703,36 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
 {
     using C = RowCfg<T>;
     const int64_t ntiles = p.dp >> T;
-    if constexpr ((SRC == SRC_WS || SRC == SRC_WS16) && StreamCfg<T, SRC>::kFits) {
-        auto kern = row_stream_kernel<T, SRC, SINK>;
-        constexpr size_t kSmem = StreamCfg<T, SRC>::SMEM_BYTES;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        if (e != cudaSuccess) return e;
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
+    // a few tiles with many workers each (2^13, 8 workers: one tile) would leave most SMs idle
+    const unsigned split = SINK == SINK_FINAL ? worker_split(ntiles, p.nworkers, (int64_t)sms * min_blocks<T, SINK>()) : 1u;
+    // On the way to the dither sink the fp32 tiles are read by the threads themselves: without the persistent
+    // grid the blocks of an SM drift apart and one's loads and butterflies fill the gaps of another's generator
+    // rounds (2^27 coordinates, T = 10 / 12 / 13: 0.175 / 0.187 / 0.189 ms against 0.215 / 0.213 / 0.225 ms streamed).
+    // One worker per tile leaves nothing to stream either.
+    constexpr bool kStream = (SRC == SRC_WS16 || SRC == SRC_WS) && (SINK == SINK_FINAL || SINK == SINK_WS) && StreamCfg<T, SRC>::kFits;
+    if constexpr (SINK == SINK_PACKK) {
+        // parts of the tiles' groups until the blocks fill the chip
+        unsigned parts = 1;
+        while ((int)parts < PackKCfg<T>::GROUPS && ntiles * p.nworkers * (2 * parts) <= (int64_t)sms * PackKCfg<T>::MIN_BLOCKS) parts *= 2;
+        if (parts == 1 && p.K < kManyDithers)
+            return launch<row_kernel<T, SRC, SINK>>(dim3((unsigned)ntiles, (unsigned)p.nworkers), C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p));
+        return launch<row_packk_kernel<T, SRC>>(dim3((unsigned)ntiles, parts, (unsigned)p.nworkers), PackKCfg<T>::THREADS,
+                                                PackKCfg<T>::SMEM_BYTES, s, 1, with_round_keys(p));
+    } else if constexpr (kStream) {
         int64_t blocks = ntiles;
         if (SINK != SINK_FINAL) {
-            int dev = 0, sms = 0, per_sm = 0;
-            if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-            if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, kSmem)) != cudaSuccess) return e;
-            blocks = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
+            blocks = (int64_t)sms * min_blocks<T, SINK>();
             if (blocks > ntiles * p.nworkers) blocks = ntiles * p.nworkers;
         }
-        kern<<<(unsigned)blocks, C::NT, kSmem, s>>>(kernel_params<SINK>(p), ntiles);
+        return launch<row_stream_kernel<T, SRC, SINK>>(dim3((unsigned)blocks, split), C::NT, StreamCfg<T, SRC>::SMEM_BYTES, s, split,
+                                                       kernel_params<SINK>(p), ntiles);
     } else {
-        auto kern = row_kernel<T, SRC, SINK>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((unsigned)ntiles, SINK == SINK_FINAL ? 1u : (unsigned)p.nworkers);
-        kern<<<grid, C::NT, C::SMEM_BYTES, s>>>(kernel_params<SINK>(p));
+        const dim3 grid((unsigned)ntiles, SINK == SINK_FINAL ? split : (unsigned)p.nworkers);
+        return launch<row_kernel<T, SRC, SINK>>(grid, C::NT, C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
     }
-    return cudaGetLastError();
 }
 
 template <int T>
@@ -544,6 +751,9 @@ cudaError_t launch_row_T(int src, int sink, const PassParams& p, cudaStream_t s)
     FOSGD_ROW_CASE(SRC_BITS, SINK_FINAL)
     FOSGD_ROW_CASE(SRC_WS, SINK_FINAL)
     FOSGD_ROW_CASE(SRC_WS16, SINK_FINAL)
+    FOSGD_ROW_CASE(SRC_BITS, SINK_SINGLE)
+    FOSGD_ROW_CASE(SRC_WS, SINK_SINGLE)
+    FOSGD_ROW_CASE(SRC_WS16, SINK_SINGLE)
 #undef FOSGD_ROW_CASE
     return cudaErrorInvalidValue;
 }

@@ -1,27 +1,33 @@
 // Transforms shorter than 2^10 (tiny gradients, or small blocks in blocked mode): one thread
 // block per transform, the textbook in-place butterfly sweeps in shared memory.  Every source
-// and sink of the library in one kernel; written for coverage of small sizes, not for speed.
+// and sink of the library in one kernel.  Such calls are all latency: the butterflies cost about a
+// microsecond, and the dithers are shared out over all warps (group of 128 coordinates, range of dithers), so
+// that K = 255 on one transform of 2^9 is 16 generator calls deep instead of one thread's 8160.
 #include "common.cuh"
+#include "dither.cuh"
 
 namespace fosgd {
 
-__global__ void __launch_bounds__(128) small_kernel(const PassParams p, const int L, const int src, const int sink)
+constexpr int kSmallThreads = 512;   // of the dither sinks (K > 1); 128 otherwise
+
+__global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK p, const int L, const int src, const int sink)
 {
     __shared__ float x[512];
     __shared__ float acc[512];
+    __shared__ uint32_t counts[4 * 32];
     const int n = 1 << L;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, nt = blockDim.x;
     const int64_t base = (int64_t)blockIdx.x << L;
-    const bool loop_workers = (sink == SINK_FINAL);
+    const bool loop_workers = (sink == SINK_FINAL || sink == SINK_SINGLE);
     const int w_begin = loop_workers ? 0 : (int)blockIdx.y;
     const int w_end = loop_workers ? p.nworkers : w_begin + 1;
-    for (int e = tid; e < n; e += 128) acc[e] = 0.f;
+    for (int e = tid; e < n; e += nt) acc[e] = 0.f;
 
     for (int wk = w_begin; wk < w_end; ++wk) {
         const uint32_t id = p.id0 + (uint32_t)wk;
         const float amp = amplitude_at(p, wk, base);   // one transform never spans two blocks
         __syncthreads();
-        for (int e = tid; e < n; e += 128) {
+        for (int e = tid; e < n; e += nt) {
             const int64_t i = base + e;
             float v;
             if (src == SRC_G32) {
@@ -41,7 +47,7 @@ __global__ void __launch_bounds__(128) small_kernel(const PassParams p, const in
         }
         __syncthreads();
         for (int h = 1; h < n; h <<= 1) {
-            for (int j = tid; j < n / 2; j += 128) {
+            for (int j = tid; j < n / 2; j += nt) {
                 const int idx = ((j & ~(h - 1)) << 1) | (j & (h - 1));
                 const float a = x[idx], b = x[idx + h];
                 x[idx] = a + b;
@@ -51,45 +57,43 @@ __global__ void __launch_bounds__(128) small_kernel(const PassParams p, const in
         }
         if (sink == SINK_WS) {
             float* dst = static_cast<float*>(p.dst) + (int64_t)wk * p.dst_stride;
-            for (int e = tid; e < n; e += 128) dst[base + e] = x[e] * p.scale;
+            for (int e = tid; e < n; e += nt) dst[base + e] = x[e] * p.scale;
         } else if (sink == SINK_PACK1 || sink == SINK_PACKK) {
-            uint32_t* dst = static_cast<uint32_t*>(p.dst) + (int64_t)wk * p.dst_stride;
-            for (int wj = tid; wj < n / 32; wj += 128) {
-                uint32_t planes[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                for (int b = 0; b < 32; ++b) {
-                    const int64_t i = base + wj * 32 + b;
-                    int c = 0;
-                    for (int k = 0; k < p.K; ++k) {
-                        const uint4 w4 = rng_words(p.rng, id, 1u + (uint32_t)k,
-                                                   ((uint32_t)(i >> 7) << 5) + ((uint32_t)i & 31u));
-                        const uint32_t word = pick(w4, (uint32_t)(i >> 5) & 3u);
-                        c += (fmaf(dither_from_word(word), p.dither_c * amp, x[wj * 32 + b]) >= 0.f) ? 1 : 0;
-                    }
-                    for (int pl = 0; pl < p.P; ++pl) planes[pl] |= (uint32_t)((c >> pl) & 1) << b;
-                }
-                for (int pl = 0; pl < p.P; ++pl) dst[(int64_t)pl * (p.dp >> 5) + ((base >> 5) + wj)] = planes[pl];
+            // groups of 128 coordinates: four words, or the n / 32 words of a shorter transform inside its group
+            const int warp = tid >> 5, lane = tid & 31, warps = nt / 32;
+            const int ngroups = n >= 128 ? n / 128 : 1, nr = n >= 128 ? 4 : n / 32, r_first = (int)(base >> 5) & 3;
+            const int share = warps / ngroups;                    // (both powers of two, warps >= 4)
+            const int g = warp / share, k0 = p.K * (warp % share) / share, k1 = p.K * (warp % share + 1) / share;
+            if (tid < 128) counts[tid] = 0u;
+            __syncthreads();
+            float y[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int word = 4 * g + r - (n >= 128 ? 0 : r_first);
+                y[r] = word >= 0 && word < n / 32 ? x[32 * word + lane] : 0.f;
             }
+            const uint32_t c = dither_counts(p, id, (((uint32_t)(base >> 7) + (uint32_t)g) << 5) + (uint32_t)lane, y,
+                                             p.dither_c * amp, k0, k1);
+            atomicAdd(counts + 32 * g + lane, c);
+            __syncthreads();
+            uint32_t* dst = static_cast<uint32_t*>(p.dst) + (int64_t)wk * p.dst_stride + (base >> 5);
+            if (warp < ngroups)
+                store_count_planes(counts[32 * warp + lane], (uint32_t)lane, p.P, dst + 4 * warp, p.dp >> 5, n >= 128 ? 0 : r_first, nr);
         } else {
-            for (int e = tid; e < n; e += 128) {
+            for (int e = tid; e < n; e += nt) {
                 const int64_t i = base + e;
                 const float f = flip_by_bit(x[e], eps_word(p.rng, id, (uint32_t)(i >> 5)), (uint32_t)i & 31u);
                 acc[e] = fmaf(f, p.amp_mode == AMP_WEIGHT ? amp : 1.f, acc[e]);
             }
         }
     }
-    if (sink == SINK_FINAL) {
+    if (loop_workers) {
         float* dst = static_cast<float*>(p.dst);
         const float sc = p.scale * (p.amp_mode == AMP_SCALE ? amplitude_at(p, 0, base) : 1.f);
-        for (int e = tid; e < n; e += 128) {
+        for (int e = tid; e < n; e += nt) {
             const int64_t i = base + e;
             if (i < p.d_out) {
-                float o = acc[e];
-                if (p.overwrite == 2) {
-                    dst[i] = fmaf(o, sc, dst[i]);
-                } else {
-                    if (!p.overwrite) o += dst[i];
-                    dst[i] = o * sc;
-                }
+                store_final(dst + i, acc[e], sc, p.overwrite);
             }
         }
     }
@@ -99,8 +103,7 @@ cudaError_t launch_small(int L, int src, int sink, const PassParams& p, cudaStre
 {
     if (L < 5 || L > 9) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)(p.dp >> L), sink == SINK_FINAL ? 1u : (unsigned)p.nworkers);
-    small_kernel<<<grid, 128, 0, s>>>(p, L, src, sink);
-    return cudaGetLastError();
+    return launch<small_kernel>(grid, sink == SINK_PACKK ? kSmallThreads : 128, 0, s, 1, with_round_keys(p), L, src, sink);
 }
 
 }  // namespace fosgd

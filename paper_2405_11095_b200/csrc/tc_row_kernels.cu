@@ -137,9 +137,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int W = p.nworkers;
+    // the blocks of a cluster (gridDim.y of them) take a tile's workers in turn; one block, all of them
+    const int n_first = (int)blockIdx.y, n_step = (int)gridDim.y;
+    const int W = (p.nworkers - n_first + n_step - 1) / n_step;      // workers of this block
+    const int n_end = n_first + W * n_step;
     const int my_tiles = ((int)blockIdx.x < ntiles) ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int64_t nitems = (int64_t)my_tiles * W;   // item g: this block's tile number g / W, worker g % W
+    const int64_t nitems = (int64_t)my_tiles * W;   // item g: this block's tile number g / W, its worker number g % W
 
     // where an item sits: first coordinate of its tile and its worker; advanced item by item (worker fastest)
     struct Cursor {
@@ -148,12 +151,14 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
     };
     const int64_t tile_step = (int64_t)gridDim.x << kT;
     auto advance = [&](Cursor& c) {
-        if (++c.n == W) {
-            c.n = 0;
+        c.n += n_step;
+        if (c.n == n_end) {
+            c.n = n_first;
             c.tile_base += tile_step;
         }
     };
-    const Cursor c_first{(int64_t)blockIdx.x << kT, 0};
+    const Cursor c_first{(int64_t)blockIdx.x << kT, n_first};
+    constexpr auto swizzled = [](uint32_t e) -> uint32_t { return (e & ~31u) | ((((e >> 2) ^ (e >> 7)) & 7u) << 2); };   // split sums: e's group of four
 
     if (warp == kIssueWarp) {
         // ================= the warp that issues the products =================
@@ -247,8 +252,6 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             const unsigned char* const land = smem + kOffLand + r * kTileBytes + srow * 256u + sq * 16u;
 #pragma unroll
             for (int t = 0; t < 4; ++t) pre[t] = *reinterpret_cast<const uint4*>(land + 64 * t);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar + BAR_LAND_FREE + r);
             hbutterfly(pre[0], pre[1]);   // column bit 5
             hbutterfly(pre[2], pre[3]);
             hbutterfly(pre[0], pre[2]);   // column bit 6
@@ -257,9 +260,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             unsigned char* const dst = smem + kOffB + b * kBBytes + sq * kBGroupStride + (srow >> 3) * 128u + (srow & 7u) * 16u;
 #pragma unroll
             for (int t = 0; t < 4; ++t) *reinterpret_cast<uint4*>(dst + 4 * t * kBGroupStride) = pre[t];
+            // One fence for both proxies' next accesses: the product reads the operand, the copy engine rewrites the slot.
+            // (The slot is given back only here: freed right after the loads were issued, without a fence, it was
+            // now and then refilled before the last of them had read it.)
             fence_generic_before_async();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar + BAR_B_FULL + b);
+            if (lane == 0) {
+                mbar_arrive(bar + BAR_LAND_FREE + r);
+                mbar_arrive(bar + BAR_B_FULL + b);
+            }
             return true;
         };
         // drain item g: accumulator -> registers, H_32 over the 32 columns, flip, add
@@ -289,41 +298,19 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
 #pragma unroll
                 for (int r = 0; r < 32; ++r) accv[r] += flip_top(v[r], fw << (31 - r));
             }
-            if (n == W - 1) {
+            if (n + n_step == n_end && n_step == 1) {
                 // the tile's sum is complete: scale and store 32 consecutive coordinates
                 const int64_t i0 = tile_base + jrow * 128u + cw * 32u;
                 const float sc = p.scale * (p.amp_mode == AMP_SCALE ? amplitude_at(p, 0, tile_base) : 1.f);
                 float* const dst = static_cast<float*>(p.dst) + i0;
                 if (i0 + 32 <= p.d_out) {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        float4 o = make_float4(accv[4 * q], accv[4 * q + 1], accv[4 * q + 2], accv[4 * q + 3]);
-                        float4* const d4 = reinterpret_cast<float4*>(dst) + q;
-                        if (p.overwrite == 2) {
-                            const float4 c = *d4;
-                            o = make_float4(fmaf(o.x, sc, c.x), fmaf(o.y, sc, c.y), fmaf(o.z, sc, c.z), fmaf(o.w, sc, c.w));
-                        } else {
-                            if (!p.overwrite) {
-                                const float4 c = *d4;
-                                o.x += c.x; o.y += c.y; o.z += c.z; o.w += c.w;
-                            }
-                            o.x *= sc; o.y *= sc; o.z *= sc; o.w *= sc;
-                        }
-                        *d4 = o;
-                    }
+                    for (int q = 0; q < 8; ++q)
+                        store_final4(dst + 4 * q, make_float4(accv[4 * q], accv[4 * q + 1], accv[4 * q + 2], accv[4 * q + 3]), sc, p.overwrite);
                 } else {
 #pragma unroll
-                    for (int r = 0; r < 32; ++r) {
-                        if (i0 + r < p.d_out) {
-                            float o = accv[r];
-                            if (p.overwrite == 2) {
-                                dst[r] = fmaf(o, sc, dst[r]);
-                            } else {
-                                if (!p.overwrite) o += dst[r];
-                                dst[r] = o * sc;
-                            }
-                        }
-                    }
+                    for (int r = 0; r < 32; ++r)
+                        if (i0 + r < p.d_out) store_final(dst + r, accv[r], sc, p.overwrite);
                 }
 #pragma unroll
                 for (int r = 0; r < 32; ++r) accv[r] = 0.f;
@@ -340,6 +327,23 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         }
         if (ok && nitems > 0) ok = drain_item(nitems - 1);
         if (!ok && lane == 0 && atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
+        if (n_step > 1) {
+            // This block's share of the sums into the landing slots: every copy has landed, and every warp has
+            // read its last tile (the accumulator just drained followed all warps' staging of it; after a wait that
+            // gave up the sums are incomplete anyway).  Groups of four are permuted by the row: a warp
+            // writes 32 rows 512 bytes apart.
+            float* const sums = reinterpret_cast<float*>(smem + kOffLand);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                *reinterpret_cast<float4*>(sums + swizzled(jrow * 128u + cw * 32u + 4u * q)) =
+                    make_float4(accv[4 * q], accv[4 * q + 1], accv[4 * q + 2], accv[4 * q + 3]);
+        }
+    }
+    if (n_step > 1) {
+        __syncthreads();
+        const int64_t tile_base = (int64_t)blockIdx.x << kT;
+        cluster_reduce_store<kT>(p, tile_base, reinterpret_cast<const float*>(smem + kOffLand), blockIdx.y, gridDim.y,
+                                 p.scale * (p.amp_mode == AMP_SCALE ? amplitude_at(p, 0, tile_base) : 1.f), swizzled);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -360,15 +364,14 @@ bool tc_row_applicable(const PassParams& p, int T, bool any_size)
 
 cudaError_t launch_tc_row(const PassParams& p, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(tc_row_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const int64_t ntiles = p.dp >> kT;
+    // fewer tiles than half the SMs (transforms up to 2^20): clusters of blocks share a tile's workers, one tile each
+    const unsigned split = worker_split(ntiles, p.nworkers, sms);
     const int64_t blocks = ntiles < sms ? ntiles : sms;
-    tc_row_final_kernel<<<(unsigned)blocks, kThreads, kSmemBytes, s>>>(p, (int)ntiles);
-    return cudaGetLastError();
+    return launch<tc_row_final_kernel>(dim3((unsigned)blocks, split), kThreads, kSmemBytes, s, split, p, (int)ntiles);
 }
 
 cudaError_t tcrow_timeouts(int* out) { return cudaMemcpyFromSymbol(out, g_tcrow_wait_timeouts, sizeof(int)); }
