@@ -24,8 +24,12 @@ cudaError_t row_timeouts_13(int*);
 cudaError_t row_timeouts_14(int*);
 cudaError_t row_timeouts_15(int*);
 
+// An intermediate's tile of 2^15 would fill an SM's registers by itself: its top stage is done while two blocks of
+// 2^14 read their pair (2^25, eight workers, dither sink: 0.42 ms against 0.48 with tiles of 2^15; one decoded
+// vector, updating x in place: 70 us against 84).
 cudaError_t launch_row(int T, int src, int sink, const PassParams& p, cudaStream_t s)
 {
+    if (T == 15 && (src == SRC_WS || src == SRC_WS16)) return launch_row_14(src == SRC_WS ? SRC_WS_PAIR : SRC_WS16_PAIR, sink, p, s);
     switch (T) {
         case 10: return launch_row_10(src, sink, p, s);
         case 11: return launch_row_11(src, sink, p, s);
@@ -75,7 +79,7 @@ cudaError_t traced(char kind, int size, int src, int sink, const PassParams& p, 
                   : kind == 'c' ? launch_col(size, src, p, s)
                   : kind == 'h' ? launch_colh(size, p, s)
                   : kind == 't' ? launch_tc_col(p, s)
-                  : kind == 'u' ? launch_tc_row(p, s)
+                  : kind == 'u' ? launch_tc_row(size, p, s)
                                 : launch_small(size, src, sink, p, s);
     trace_end(on, s, TraceEntry{kind, size, src, sink, p.id0 == FOSGD_SERVER_ID ? 0 : p.nworkers, decoder});
     return e;

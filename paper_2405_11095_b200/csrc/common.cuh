@@ -15,7 +15,11 @@ enum Src : int {
     SRC_G16 = 1,   // caller gradients, bf16 (exact upcast), same padding and flip
     SRC_BITS = 2,  // packed signs / count planes: q_i = 2 c_i - K
     SRC_WS = 3,    // fp32 intermediate of an earlier pass
-    SRC_WS16 = 4   // fp16 intermediate (exact small integers from a packed one-plane source)
+    SRC_WS16 = 4,  // fp16 intermediate (exact small integers from a packed source)
+    // The contiguous pass of a 2^25 transform, whose 15 stages are one more than a tile of 2^14 has: the top one is
+    // done while reading, by both tiles of a pair (each reads both halves, the second time out of L2).
+    SRC_WS_PAIR = 5,
+    SRC_WS16_PAIR = 6
 };
 enum Sink : int {
     SINK_WS = 0,     // fp32 intermediate (or the scaled transform output of fosgd_flatten)
@@ -378,8 +382,8 @@ cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s);   // packed
 bool tc_col_applicable(const PassParams& p, bool any_size);                            // ten strided stages from one plane on the tensor cores
 cudaError_t launch_tc_col(const PassParams& p, cudaStream_t s);          // one-plane bits -> fp16 intermediate
 cudaError_t tc_timeouts(int* out);
-bool tc_row_applicable(const PassParams& p, int T, bool any_size);                     // contiguous 2^14 tiles of the fp16 intermediate, seven stages on the tensor cores
-cudaError_t launch_tc_row(const PassParams& p, cudaStream_t s);          // fp16 intermediate -> flip + sum sink
+bool tc_row_applicable(const PassParams& p, int T, bool any_size);                     // contiguous 2^14 tiles of the fp16 intermediate, seven or eight stages on the tensor cores
+cudaError_t launch_tc_row(int T, const PassParams& p, cudaStream_t s);          // fp16 intermediate -> flip + sum sink
 cudaError_t tcrow_timeouts(int* out);
 // uplink encoder of a 2^24-long transform as one kernel (strided and contiguous pass side by side)
 size_t enc_fused_sync_bytes(int nworkers);                               // zeroed device words the launch needs

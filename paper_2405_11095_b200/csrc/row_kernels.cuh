@@ -269,7 +269,29 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
 {
     constexpr int VB = RowCfg<T>::VB, VN = 1 << VB;
     const int64_t i0 = tile_base + baseF;
-    if constexpr (SRC == SRC_G32) {
+    if constexpr (SRC == SRC_WS_PAIR || SRC == SRC_WS16_PAIR) {
+        // x_0 + x_1 of the pair's halves for its first tile, x_0 - x_1 for its second
+        static_assert(VB == 1, "tiles of 2^14");
+        const bool second = (tile_base >> T) & 1;
+        const int64_t at = (int64_t)n * p.src_stride + i0 - (second ? (int64_t)1 << T : 0);
+#pragma unroll
+        for (int g = 0; g < 16; ++g) {
+            const int o = round_F_offset<T>(g);
+            float2 a, b;
+            if constexpr (SRC == SRC_WS_PAIR) {
+                const float* const src = static_cast<const float*>(p.src) + at;
+                a = __ldcg(reinterpret_cast<const float2*>(src + o));
+                b = __ldcg(reinterpret_cast<const float2*>(src + o + (1 << T)));
+            } else {
+                const __half* const src = static_cast<const __half*>(p.src) + at;
+                const uint32_t qa = __ldcg(reinterpret_cast<const uint32_t*>(src + o)), qb = __ldcg(reinterpret_cast<const uint32_t*>(src + o + (1 << T)));
+                a = __half22float2(*reinterpret_cast<const __half2*>(&qa));
+                b = __half22float2(*reinterpret_cast<const __half2*>(&qb));
+            }
+            v[2 * g] = second ? a.x - b.x : a.x + b.x;
+            v[2 * g + 1] = second ? a.y - b.y : a.y + b.y;
+        }
+    } else if constexpr (SRC == SRC_G32) {
         const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
         const int64_t left = p.d - i0;    // valid elements from this thread's first coordinate on
 #pragma unroll
@@ -742,18 +764,29 @@ cudaError_t launch_row_T(int src, int sink, const PassParams& p, cudaStream_t s)
     if (src == SRC_ && sink == SINK_) return launch_row_one<T, SRC_, SINK_>(p, s);
     FOSGD_ROW_CASE(SRC_G32, SINK_WS)
     FOSGD_ROW_CASE(SRC_G16, SINK_WS)
-    FOSGD_ROW_CASE(SRC_WS, SINK_WS)
     FOSGD_ROW_CASE(SRC_G32, SINK_PACK1)
     FOSGD_ROW_CASE(SRC_G16, SINK_PACK1)
-    FOSGD_ROW_CASE(SRC_WS, SINK_PACK1)
     FOSGD_ROW_CASE(SRC_G32, SINK_PACKK)
-    FOSGD_ROW_CASE(SRC_WS, SINK_PACKK)
     FOSGD_ROW_CASE(SRC_BITS, SINK_FINAL)
-    FOSGD_ROW_CASE(SRC_WS, SINK_FINAL)
-    FOSGD_ROW_CASE(SRC_WS16, SINK_FINAL)
     FOSGD_ROW_CASE(SRC_BITS, SINK_SINGLE)
-    FOSGD_ROW_CASE(SRC_WS, SINK_SINGLE)
-    FOSGD_ROW_CASE(SRC_WS16, SINK_SINGLE)
+    if constexpr (T <= 14) {     // (an intermediate's tiles of 2^15 are pairs of 2^14)
+        FOSGD_ROW_CASE(SRC_WS, SINK_WS)
+        FOSGD_ROW_CASE(SRC_WS, SINK_PACK1)
+        FOSGD_ROW_CASE(SRC_WS, SINK_PACKK)
+        FOSGD_ROW_CASE(SRC_WS, SINK_FINAL)
+        FOSGD_ROW_CASE(SRC_WS, SINK_SINGLE)
+        FOSGD_ROW_CASE(SRC_WS16, SINK_FINAL)
+        FOSGD_ROW_CASE(SRC_WS16, SINK_SINGLE)
+    }
+    if constexpr (T == 14) {
+        FOSGD_ROW_CASE(SRC_WS_PAIR, SINK_WS)
+        FOSGD_ROW_CASE(SRC_WS_PAIR, SINK_PACK1)
+        FOSGD_ROW_CASE(SRC_WS_PAIR, SINK_PACKK)
+        FOSGD_ROW_CASE(SRC_WS_PAIR, SINK_FINAL)
+        FOSGD_ROW_CASE(SRC_WS_PAIR, SINK_SINGLE)
+        FOSGD_ROW_CASE(SRC_WS16_PAIR, SINK_FINAL)
+        FOSGD_ROW_CASE(SRC_WS16_PAIR, SINK_SINGLE)
+    }
 #undef FOSGD_ROW_CASE
     return cudaErrorInvalidValue;
 }

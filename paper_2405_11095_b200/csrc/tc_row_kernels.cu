@@ -13,6 +13,8 @@
 //   3. H_32 over column bits 0..4 runs in fp32 registers: tcgen05.ld hands every thread 32
 //      consecutive columns of one row, which is also one word of the flip vector, so the flip and
 //      the sum over the workers follow in the same registers.
+// HALVES = 2: the 15 stages of a 2^25 transform.  The top one pairs tiles of 2^14; the two products of a pair, the second
+// one added or subtracted, go into one accumulator (fp32, |D| <= 2^20), so every block stages both halves.
 // All values are integers below 2^24 in magnitude, so the result equals the plain-ALU kernel's bit
 // for bit.
 //
@@ -54,13 +56,14 @@ enum { BAR_B_FULL = 0, BAR_B_FREE = 2, BAR_ACC_FULL = 4, BAR_ACC_FREE = 6, BAR_F
 
 // instruction descriptor: D = f32 (1 << 4), A = B = fp16 (0), A K-major, B MN-major (1 << 16), N = 128, M = 128
 constexpr uint32_t kIdescF16 = (1u << 4) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+constexpr uint32_t kNegateB = 1u << 14;   // D -= A B
 
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate)
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(kIdescF16), "r"(accumulate) : "memory");
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
 // x with its sign flipped iff the top bit of w is set
@@ -83,6 +86,7 @@ __device__ __forceinline__ void hbutterfly(uint4& a, uint4& b)
 
 }  // namespace
 
+template <int HALVES>
 __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassParams p, const int ntiles)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -166,23 +170,39 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             const uint64_t adesc = umma_desc(smem_u32(smem + kOffA), kAChunkStride, kAGroupStride);
             bool ok = true;
             int64_t g = 0;
+            int tile = (int)blockIdx.x, w = 0;
             for (; g < nitems; ++g) {
                 const uint32_t b = (uint32_t)g & 1u, u = (uint32_t)(g >> 1);
-                ok = mbar_wait_or_stop(bar + BAR_B_FULL + b, u & 1u, s_stop);                        // operand staged
-                if (ok && u > 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, (u - 1u) & 1u, s_stop);   // accumulator drained
-                if (!ok) break;
-                tc_fence_after_sync();
-                const uint64_t bdesc = umma_desc(smem_u32(smem + kOffB + b * kBBytes), 128u, kBGroupStride);
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)   // K = 16 per instruction: two 16-byte chunks of A, two groups of eight rows of B
-                    umma_f16(tmem_base + b * 128u, adesc + (uint64_t)(ks * (256 >> 4)), bdesc + (uint64_t)(ks * (256 >> 4)), ks > 0 ? 1u : 0u);
-                umma_commit(bar + BAR_B_FREE + b);
+                for (int h = 0; h < HALVES && ok; ++h) {
+                    const uint32_t sb = (uint32_t)(HALVES * g + h) & 1u, su = (uint32_t)((HALVES * g + h) >> 1);
+                    ok = mbar_wait_or_stop(bar + BAR_B_FULL + sb, su & 1u, s_stop);                                     // operand staged
+                    if (ok && h == 0 && u > 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, (u - 1u) & 1u, s_stop);   // accumulator drained
+                    if (!ok) break;
+                    tc_fence_after_sync();
+                    const uint64_t bdesc = umma_desc(smem_u32(smem + kOffB + sb * kBBytes), 128u, kBGroupStride);
+                    // the pair's second half enters its first tile with a plus, its second tile with a minus
+                    const uint32_t idesc = (h == 1 && (tile & 1)) ? kIdescF16 | kNegateB : kIdescF16;
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)   // K = 16 per instruction: two 16-byte chunks of A, two groups of eight rows of B
+                        umma_f16(tmem_base + b * 128u, adesc + (uint64_t)(ks * (256 >> 4)), bdesc + (uint64_t)(ks * (256 >> 4)), idesc, h + ks > 0 ? 1u : 0u);
+                    umma_commit(bar + BAR_B_FREE + sb);
+                }
+                if (!ok) break;
                 umma_commit(bar + BAR_ACC_FULL + b);
+                if (++w == W) {
+                    w = 0;
+                    tile += (int)gridDim.x;
+                }
             }
             if (!ok) {
                 if (atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
                 // products already committed may still be running: one more bounded wait each before the tensor memory goes back
                 for (int64_t h = (g >= 2 ? g - 2 : 0); h < g; ++h) mbar_wait(bar + BAR_ACC_FULL + (h & 1), (uint32_t)(h >> 1) & 1u);
+                if (HALVES > 1) {   // (the first half of the item given up on)
+                    umma_commit(bar + BAR_ACC_FULL + (g & 1));
+                    mbar_wait(bar + BAR_ACC_FULL + (g & 1), (uint32_t)(g >> 1) & 1u);
+                }
             }
         }
     } else if (warp == kServiceWarp) {
@@ -192,11 +212,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         Cursor c_ld = c_first, c_fl = c_first;
         bool ok = true;
         int64_t issued = 0;   // lane 0: copies started
+        const int64_t nloads = HALVES * nitems;
         auto issue_load = [&](int64_t g) -> bool {
             const uint32_t r = (uint32_t)(g % kRing), u = (uint32_t)(g / kRing);
             if (u > 0 && !mbar_wait_or_stop(bar + BAR_LAND_FREE + r, (u - 1u) & 1u, s_stop)) return false;   // every warp has read the slot
-            const __half* const src = static_cast<const __half*>(p.src) + (int64_t)c_ld.n * p.src_stride + c_ld.tile_base;
-            advance(c_ld);
+            const __half* src = static_cast<const __half*>(p.src) + (int64_t)c_ld.n * p.src_stride + c_ld.tile_base;
+            if (HALVES == 2) src += (int64_t)((int)(g & 1) - (int)((c_ld.tile_base >> kT) & 1)) * (1 << kT);   // the pair's halves in turn
+            if (HALVES == 1 || (g & 1)) advance(c_ld);
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar + BAR_LAND_FULL + r)), "r"(kTileBytes) : "memory");
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"(smem_u32(smem + kOffLand + r * kTileBytes)), "l"(src), "r"(kTileBytes), "r"(smem_u32(bar + BAR_LAND_FULL + r)) : "memory");
@@ -204,10 +226,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             return true;
         };
         if (lane == 0) {
-            for (int64_t g = 0; g < kRing - 1 && g < nitems && ok; ++g) ok = issue_load(g);
+            for (int64_t g = 0; g < kRing - 1 && g < nloads && ok; ++g) ok = issue_load(g);
         }
         for (int64_t g = 0; g < nitems; ++g) {
-            if (lane == 0 && ok && g + kRing - 1 < nitems) ok = issue_load(g + kRing - 1);
+#pragma unroll
+            for (int h = 0; h < HALVES; ++h)
+                if (lane == 0 && ok && HALVES * g + h + kRing - 1 < nloads) ok = issue_load(HALVES * g + h + kRing - 1);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             const uint32_t b = (uint32_t)g & 1u, u = (uint32_t)(g >> 1);
@@ -243,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         bool ok = true;
         Cursor c_drain = c_first;
 
-        // stage item g: landed tile -> H_4 over column bits 5, 6 -> operand buffer
+        // stage landed tile g: H_4 over column bits 5, 6 -> operand buffer
         auto stage_item = [&](int64_t g) -> bool {
             const uint32_t b = (uint32_t)g & 1u, u = (uint32_t)(g >> 1);
             const uint32_t r = (uint32_t)(g % kRing), ur = (uint32_t)(g / kRing);
@@ -321,7 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
 #pragma unroll
         for (int r = 0; r < 32; ++r) accv[r] = 0.f;
         for (int64_t g = 0; g < nitems && ok; ++g) {
-            ok = stage_item(g);
+#pragma unroll
+            for (int h = 0; h < HALVES && ok; ++h) ok = stage_item(HALVES * g + h);
             if (!ok) break;
             if (g > 0) ok = drain_item(g - 1);        // underneath the product of item g
         }
@@ -356,13 +381,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
 
 // One packed plane's fp16 intermediate in contiguous tiles of 2^14, and at least three workers to sum: with one or
 // two (a single decoder, the downlink) the plain-ALU pass is the faster one (0.033 against 0.041 ms on one vector
-// of 2^24, 0.051 against 0.057 on two; 0.069 against 0.068 on three, 0.156 against 0.119 on eight).
+// of 2^24, 0.051 against 0.057 on two; 0.069 against 0.068 on three, 0.156 against 0.119 on eight).  The 15 stages of a
+// 2^25 transform: from five workers on, whose sums repay staging every tile twice (eight: 0.30 against 0.35 ms).
 bool tc_row_applicable(const PassParams& p, int T, bool any_size)
 {
-    return T == kT && p.P == 1 && (any_size || p.nworkers >= 3) && (p.dp >> kT) >= 1 && (p.dp >> kT) <= 0x7FFFFFFF;
+    if (p.P != 1 || (p.dp >> kT) < 1 || (p.dp >> kT) > 0x7FFFFFFF) return false;
+    return T == kT ? any_size || p.nworkers >= 3 : T == kT + 1 && p.nworkers > 4;
 }
 
-cudaError_t launch_tc_row(const PassParams& p, cudaStream_t s)
+cudaError_t launch_tc_row(int T, const PassParams& p, cudaStream_t s)
 {
     int sms = 0;
     const cudaError_t e = sm_count(&sms);
@@ -370,8 +397,9 @@ cudaError_t launch_tc_row(const PassParams& p, cudaStream_t s)
     const int64_t ntiles = p.dp >> kT;
     // fewer tiles than half the SMs (transforms up to 2^20): clusters of blocks share a tile's workers, one tile each
     const unsigned split = worker_split(ntiles, p.nworkers, sms);
-    const int64_t blocks = ntiles < sms ? ntiles : sms;
-    return launch<tc_row_final_kernel>(dim3((unsigned)blocks, split), kThreads, kSmemBytes, s, split, p, (int)ntiles);
+    const dim3 grid((unsigned)(ntiles < sms ? ntiles : sms), split);
+    if (T == kT) return launch<tc_row_final_kernel<1>>(grid, kThreads, kSmemBytes, s, split, p, (int)ntiles);
+    return launch<tc_row_final_kernel<2>>(grid, kThreads, kSmemBytes, s, split, p, (int)ntiles);
 }
 
 cudaError_t tcrow_timeouts(int* out) { return cudaMemcpyFromSymbol(out, g_tcrow_wait_timeouts, sizeof(int)); }
