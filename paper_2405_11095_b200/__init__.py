@@ -105,9 +105,17 @@ def _check(status: int, where: str) -> None:
         raise FosgdError(status, where)
 
 
+_torch = None
+
+
 def _stream() -> int:
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    """Handle of torch's current stream.  Read without building a torch.cuda.Stream object: that costs 3 us,
+    as much as the launch of a kernel, on every call."""
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
 
 
 def _ptr(t) -> int:

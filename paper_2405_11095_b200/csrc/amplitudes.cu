@@ -19,6 +19,7 @@ constexpr float kMinBlockAmplitude = 1e-30f;
 template <bool BF16>
 __global__ void __launch_bounds__(256) sumsq_partial_kernel(const void* grads, int64_t d, int64_t worker_stride, double* partial)
 {
+    pdl_begin();
     const int n = blockIdx.y;
     double acc = 0.0;
     // 16-byte loads over the aligned body (rows start 16-byte aligned), scalar loads over the tail
@@ -26,7 +27,7 @@ __global__ void __launch_bounds__(256) sumsq_partial_kernel(const void* grads, i
     const int64_t nv = d / V;
     const uint4* row = reinterpret_cast<const uint4*>(static_cast<const char*>(grads) + (int64_t)n * worker_stride * (BF16 ? 2 : 4));
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < nv; i += (int64_t)gridDim.x * 256) {
-        const uint4 w = __ldg(row + i);
+        const uint4 w = load_ca(row + i);
         const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -61,19 +62,22 @@ __global__ void __launch_bounds__(256) sumsq_partial_kernel(const void* grads, i
 __global__ void __launch_bounds__(256) amplitudes_finalize_kernel(const double* partial, int M, int nblocks, double alpha,
                                                                   double alpha_s, double n_eff, float* lam_out, float* lam_s_out)
 {
-    __shared__ double best[256];
+    // a warp per worker: lane-strided sums, then across lanes, always in the same order
+    __shared__ double best[8];
+    pdl_begin();
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     double mine = 0.0;
-    for (int n = threadIdx.x; n < M; n += 256) {
+    for (int n = (int)warp; n < M; n += 8) {
         double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += partial[(int64_t)n * nblocks + b];
+        for (int b = (int)lane; b < nblocks; b += 32) s += partial[(int64_t)n * nblocks + b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         mine = fmax(mine, s);
     }
-    best[threadIdx.x] = mine;
+    if (lane == 0) best[warp] = mine;
     __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) best[threadIdx.x] = fmax(best[threadIdx.x], best[threadIdx.x + s]);
-        __syncthreads();
-    }
+    if (threadIdx.x == 0)
+        for (int w = 1; w < 8; ++w) best[0] = fmax(best[0], best[w]);
     if (threadIdx.x == 0) {
         const double B = sqrt(best[0]);
         const double lam = alpha * B * sqrt(log(n_eff) / n_eff);
@@ -90,6 +94,7 @@ template <bool BF16>
 __global__ void __launch_bounds__(128) segment_sumsq_kernel(const void* grads, int64_t d, int64_t dp, int64_t worker_stride,
                                                             int s, double* seg)
 {
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31u;
     const int64_t warp_base = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) << 10;
@@ -110,11 +115,11 @@ __global__ void __launch_bounds__(128) segment_sumsq_kernel(const void* grads, i
             float x[4];
             if (i + 3 < d) {
                 if (BF16) {
-                    const uint2 w = __ldg(reinterpret_cast<const uint2*>(g16 + i));
+                    const uint2 w = load_ca(reinterpret_cast<const uint2*>(g16 + i));
                     x[0] = __uint_as_float(w.x << 16); x[1] = __uint_as_float(w.x & 0xFFFF0000u);
                     x[2] = __uint_as_float(w.y << 16); x[3] = __uint_as_float(w.y & 0xFFFF0000u);
                 } else {
-                    const float4 q = __ldg(reinterpret_cast<const float4*>(g32 + i));
+                    const float4 q = load_ca(reinterpret_cast<const float4*>(g32 + i));
                     x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
                 }
             } else {
@@ -148,6 +153,7 @@ __global__ void __launch_bounds__(128) segment_sumsq_kernel(const void* grads, i
 __global__ void __launch_bounds__(128) block_amplitudes_kernel(const double* seg, int64_t nb, int64_t segs_per_block,
                                                                int M, double alpha, double n_eff, float* lam)
 {
+    pdl_begin();
     const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31u;
     if (w >= nb * M) return;
@@ -164,6 +170,7 @@ __global__ void __launch_bounds__(128) block_amplitudes_kernel(const double* seg
 __global__ void __launch_bounds__(128) server_block_amplitudes_kernel(const float* lam, int64_t nb, int M, double alpha_s,
                                                                       double n_eff, float* lam_s)
 {
+    pdl_begin();
     const int64_t blk = (int64_t)blockIdx.x * 128 + threadIdx.x;
     if (blk >= nb) return;
     float m = 0.f;
@@ -179,37 +186,33 @@ cudaError_t launch_block_amplitudes(const void* grads, int bf16, int64_t d, int6
     const int64_t nb = dp >> block_log2;
     const double n_eff = (double)((int64_t)1 << block_log2);
     const dim3 grid((unsigned)((dp + 4095) >> 12), (unsigned)M);
-    if (bf16) segment_sumsq_kernel<true><<<grid, 128, 0, st>>>(grads, d, dp, worker_stride, s, seg);
-    else segment_sumsq_kernel<false><<<grid, 128, 0, st>>>(grads, d, dp, worker_stride, s, seg);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = bf16 ? launch<segment_sumsq_kernel<true>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg)
+                         : launch<segment_sumsq_kernel<false>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg);
     if (e != cudaSuccess) return e;
     const int64_t warps = nb * M;
-    block_amplitudes_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(seg, nb, (int64_t)1 << (block_log2 - s), M, alpha,
-                                                                        n_eff, lam);
-    e = cudaGetLastError();
+    e = launch<block_amplitudes_kernel>(dim3((unsigned)((warps + 3) / 4)), 128, 0, st, 1, (const double*)seg, nb,
+                                        (int64_t)1 << (block_log2 - s), M, alpha, n_eff, lam);
     if (e != cudaSuccess || lam_s == nullptr) return e;
-    server_block_amplitudes_kernel<<<(unsigned)((nb + 127) / 128), 128, 0, st>>>(lam, nb, M, alpha_s, n_eff, lam_s);
-    return cudaGetLastError();
+    return launch<server_block_amplitudes_kernel>(dim3((unsigned)((nb + 127) / 128)), 128, 0, st, 1, (const float*)lam, nb, M, alpha_s, n_eff, lam_s);
 }
 
 cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t worker_stride, int M, double alpha,
                               double alpha_s, double n_eff, float* lam, float* lam_s, double* partial, cudaStream_t s)
 {
-    const dim3 grid(kNormBlocks, (unsigned)M);
-    if (bf16) sumsq_partial_kernel<true><<<grid, 256, 0, s>>>(grads, d, worker_stride, partial);
-    else sumsq_partial_kernel<false><<<grid, 256, 0, s>>>(grads, d, worker_stride, partial);
-    cudaError_t e = cudaGetLastError();
+    // parts of at least 4096 coordinates: every one costs the second step a load
+    const int nparts = (int)(d >= (int64_t)kNormBlocks * 4096 ? kNormBlocks : (d + 4095) / 4096);
+    const dim3 grid((unsigned)nparts, (unsigned)M);
+    const cudaError_t e = bf16 ? launch<sumsq_partial_kernel<true>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial)
+                               : launch<sumsq_partial_kernel<false>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial);
     if (e != cudaSuccess) return e;
-    amplitudes_finalize_kernel<<<1, 256, 0, s>>>(partial, M, kNormBlocks, alpha, alpha_s, n_eff, lam, lam_s);
-    return cudaGetLastError();
+    return launch_amplitudes_finalize(partial, M, nparts, alpha, alpha_s, n_eff, lam, lam_s, s);
 }
 
-// the second step alone: amplitudes from partial sums of squares that another kernel gathered ([M][nparts])
+// the second step alone: amplitudes from partial sums of squares ([M][nparts])
 cudaError_t launch_amplitudes_finalize(const double* partial, int M, int nparts, double alpha, double alpha_s, double n_eff,
                                        float* lam, float* lam_s, cudaStream_t s)
 {
-    amplitudes_finalize_kernel<<<1, 256, 0, s>>>(partial, M, nparts, alpha, alpha_s, n_eff, lam, lam_s);
-    return cudaGetLastError();
+    return launch<amplitudes_finalize_kernel>(dim3(1), 256, 0, s, 1, partial, M, nparts, alpha, alpha_s, n_eff, lam, lam_s);
 }
 
 }  // namespace fosgd

@@ -24,9 +24,9 @@ template <int SRC>
 __device__ __forceinline__ float col_load(const PassParams& p, const void* worker_src, uint32_t i, uint32_t d32)
 {
     if (SRC == SRC_G32) {
-        return (i < d32) ? __ldcs(static_cast<const float*>(worker_src) + i) : 0.f;
+        return (i < d32) ? load_cs(static_cast<const float*>(worker_src) + i) : 0.f;
     } else if (SRC == SRC_G16) {
-        return (i < d32) ? __uint_as_float((uint32_t)__ldcs(static_cast<const uint16_t*>(worker_src) + i) << 16) : 0.f;
+        return (i < d32) ? __uint_as_float((uint32_t)load_cs(static_cast<const uint16_t*>(worker_src) + i) << 16) : 0.f;
     } else if (SRC == SRC_WS) {
         return static_cast<const float*>(worker_src)[i];
     } else {
@@ -53,7 +53,7 @@ __device__ __forceinline__ float flip_shifted(float x, uint32_t word, uint32_t s
 // 2^25 coordinates of two planes, ten stages: 174 us with every thread loading its own words).
 __device__ __forceinline__ uint32_t bits_row_word(const PassParams& p, const void* worker_src, uint32_t irow, int plane)
 {
-    return __ldg(static_cast<const uint32_t*>(worker_src) + (irow >> 5) + (int64_t)plane * (p.dp >> 5));
+    return load_ca(static_cast<const uint32_t*>(worker_src) + (irow >> 5) + (int64_t)plane * (p.dp >> 5));
 }
 
 // ---- A <= 4 -----------------------------------------------------------------------------
@@ -61,6 +61,7 @@ template <int A, int SRC>
 __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
 {
     constexpr int R = 1 << A;
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -116,6 +117,7 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
 {
     extern __shared__ __align__(16) float2 tile2[];
     constexpr uint32_t WARPS = 1u << (A - 4);
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5;
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
             for (int r = 0; r < 32; ++r) v[r] = base;
             float weight = 2.f;
             for (int pl = 0; pl < p.P; ++pl, weight += weight) {
-                const uint32_t mine = __ldg(words + (int64_t)pl * (p.dp >> 5));
+                const uint32_t mine = load_ca(words + (int64_t)pl * (p.dp >> 5));
 #pragma unroll
                 for (int r = 0; r < 16; ++r) {
                     const uint32_t x = __shfl_sync(0xFFFFFFFFu, mine, 2 * r + (int)from) >> bit;
@@ -155,10 +157,10 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
         } else if constexpr (kGrad) {
             auto load2 = [&](uint32_t i, float& x0, float& x1) {
                 if constexpr (SRC == SRC_G32) {
-                    const float2 q = __ldcs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i));
+                    const float2 q = load_cs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i));
                     x0 = q.x; x1 = q.y;
                 } else {
-                    const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i));
+                    const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i));
                     x0 = __uint_as_float(q << 16); x1 = __uint_as_float(q & 0xFFFF0000u);
                 }
             };
@@ -246,6 +248,7 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassP
 {
     extern __shared__ __align__(16) float smem[];  // 2^A rows x 32 columns
     constexpr int WARPS = 1 << (A - 5);
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5;
@@ -308,6 +311,7 @@ template <int A, int SRC>
 __global__ void __launch_bounds__(1 << (A - 1), 2) col_tile16_kernel(const PassParams p)
 {
     extern __shared__ __align__(16) float smem[];
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t c = lane & 15, h = lane >> 4;
@@ -385,6 +389,7 @@ __global__ void __launch_bounds__(512, 2) col4_kernel(const PassParams p, const 
                                                       const int nruns, const uint32_t full_rows)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
+    pdl_begin();
     col4_run<BlockSync>(p, &tmap, full_rows, (int)(blockIdx.x / (unsigned)nruns), (blockIdx.x % (unsigned)nruns) * 8u, smem_raw,
                         (int)threadIdx.x, &g_col_wait_timeouts);
 }
@@ -394,6 +399,7 @@ __global__ void __launch_bounds__(512, 2) col4_norm_kernel(const PassParams p, c
                                                            const int nruns, const uint32_t full_rows, double* const partial)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
+    pdl_begin();
     col4_run<BlockSync, true>(p, &tmap, full_rows, (int)(blockIdx.x / (unsigned)nruns), (blockIdx.x % (unsigned)nruns) * 8u, smem_raw,
                               (int)threadIdx.x, &g_col_wait_timeouts, partial + blockIdx.x);
 }
@@ -402,6 +408,7 @@ __global__ void __launch_bounds__(1024, 1) col4_duo_kernel(const PassParams p, c
                                                            const int nruns, const uint32_t full_rows)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
+    pdl_begin();
     col4_duo(p, &tmap, (uint32_t)nruns, full_rows, (uint32_t)nruns * (uint32_t)p.nworkers, smem_raw, &g_col_wait_timeouts);
 }
 
@@ -446,24 +453,18 @@ static cudaError_t launch_col4(const PassParams& p, cudaStream_t s, bool* launch
     if (S < 128 || nsegs % 8 != 0 || nruns * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
     CUtensorMap map;
     if (!make_col_tensor_map(&map, p.src, S, rows, (uint64_t)p.nworkers, (uint64_t)p.src_stride)) return cudaSuccess;
-    cudaError_t e;
+    *launched = true;
     if (p.lo_log >= 15) {
         // rows 128 KiB apart or more: the two-group persistent form (0.44 against 0.48 ms on 8 workers of 2^25)
-        if ((e = cudaFuncSetAttribute(col4_duo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col4Duo::SMEM_BYTES)) != cudaSuccess) return e;
-        int dev = 0, sms = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-        int64_t blocks = nruns * p.nworkers;
-        if (blocks > sms) blocks = sms;
-        col4_duo_kernel<<<(unsigned)blocks, 1024, Col4Duo::SMEM_BYTES, s>>>(p, map, (int)nruns, (uint32_t)rows);
-    } else {
-        // one block per run (0.83 against 0.91 ms on 32 workers of 2^24; blocks that start at different times
-        // keep the memory system evenly loaded)
-        if ((e = cudaFuncSetAttribute(col4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col4::SMEM_BYTES)) != cudaSuccess) return e;
-        col4_kernel<<<(unsigned)(nruns * p.nworkers), 512, Col4::SMEM_BYTES, s>>>(p, map, (int)nruns, (uint32_t)rows);
+        int sms = 0;
+        const cudaError_t e = sm_count(&sms);
+        if (e != cudaSuccess) return e;
+        const int64_t runs = nruns * p.nworkers;
+        return launch<col4_duo_kernel>(dim3((unsigned)(runs < sms ? runs : sms)), 1024, Col4Duo::SMEM_BYTES, s, 1, p, map, (int)nruns, (uint32_t)rows);
     }
-    *launched = true;
-    return cudaGetLastError();
+    // one block per run (0.83 against 0.91 ms on 32 workers of 2^24; blocks that start at different times
+    // keep the memory system evenly loaded)
+    return launch<col4_kernel>(dim3((unsigned)(nruns * p.nworkers)), 512, Col4::SMEM_BYTES, s, 1, p, map, (int)nruns, (uint32_t)rows);
 }
 
 template <int A, int SRC, bool NORM>
@@ -501,12 +502,9 @@ cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStr
     if (p.lo_log >= 15 || S < 128 || nsegs % 8 != 0 || nruns > kMaxParts || nruns * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
     CUtensorMap map;
     if (!make_col_tensor_map(&map, p.src, S, rows, (uint64_t)p.nworkers, (uint64_t)p.src_stride)) return cudaSuccess;
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(col4_norm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Col4::SMEM_BYTES)) != cudaSuccess) return e;
-    col4_norm_kernel<<<(unsigned)(nruns * p.nworkers), 512, Col4::SMEM_BYTES, s>>>(p, map, (int)nruns, (uint32_t)rows, partial);
     *launched = true;
     *nparts_out = (int)nruns;
-    return cudaGetLastError();
+    return launch<col4_norm_kernel>(dim3((unsigned)(nruns * p.nworkers)), 512, Col4::SMEM_BYTES, s, 1, p, map, (int)nruns, (uint32_t)rows, partial);
 }
 
 // ---- packed source, fp16 arithmetic ------------------------------------------------------------
@@ -525,7 +523,7 @@ __device__ __forceinline__ void load_planes_half2(const PassParams& p, const uin
     const uint32_t* const wa = bits + (at(lane >> 1) >> 5) + (lane & 1u);
     const uint32_t* const wb = bits + (at(16u + (lane >> 1)) >> 5) + (lane & 1u);
     if (p.P == 1) {
-        const uint32_t word_a = __ldg(wa), word_b = __ldg(wb);
+        const uint32_t word_a = load_ca(wa), word_b = load_ca(wb);
 #pragma unroll
         for (int r = 0; r < 32; ++r) {
             const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
@@ -540,7 +538,7 @@ __device__ __forceinline__ void load_planes_half2(const PassParams& p, const uin
         uint32_t weight = 0x4000u;                               // fp16 2.0; the exponent grows plane by plane
         for (int pl = 0; pl < p.P; ++pl, weight += 0x400u) {
             const int64_t off = (int64_t)pl * (p.dp >> 5);
-            const uint32_t word_a = __ldg(wa + off), word_b = __ldg(wb + off);
+            const uint32_t word_a = load_ca(wa + off), word_b = load_ca(wb + off);
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
                 const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
@@ -557,6 +555,7 @@ __global__ void __launch_bounds__(256) colh_small_kernel(const PassParams p)
 {
     constexpr uint32_t R = 1u << A;
     constexpr int SEG_LOG = 11 - A;                               // columns of a warp: 2^(5-A) segments of 64
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t seg = blockIdx.x * 8u + (threadIdx.x >> 5);
@@ -579,6 +578,7 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) colh_tile_kernel(const Pass
 {
     extern __shared__ __align__(16) uint32_t smemh[];   // [2^A][32] half2 tile
     constexpr int WARPS = 1 << (A - 5);
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t w = threadIdx.x >> 5;
@@ -613,6 +613,7 @@ template <int A>
 __global__ void __launch_bounds__(1 << (A - 1), 2) colh_tile32_kernel(const PassParams p)
 {
     extern __shared__ __align__(16) uint32_t smemh[];
+    pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t c2 = lane & 15, h = lane >> 4;
@@ -628,8 +629,8 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) colh_tile32_kernel(const Pass
     {
         const uint32_t row_a = ((lane & 15u) << (A - 5)) | (w << 1) | h;
         const uint32_t ia = i_tile + row_a * step;
-        word_lo = __ldg(bits + (ia >> 5));
-        word_hi = __ldg(bits + ((ia + (step << (A - 1))) >> 5));
+        word_lo = load_ca(bits + (ia >> 5));
+        word_hi = load_ca(bits + ((ia + (step << (A - 1))) >> 5));
     }
     __half2 v[32];
     const uint32_t sh = 2u * c2;

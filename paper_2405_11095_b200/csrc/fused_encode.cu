@@ -102,7 +102,7 @@ __device__ __forceinline__ void row_role(const PassParamsRK& p, uint32_t* const 
         static_assert(C::VB == 1, "pairs of coordinates per load");
 #pragma unroll
         for (int g = 0; g < 16; ++g) {
-            const float2 x = __ldcg(reinterpret_cast<const float2*>(src + round_F_offset<kT>(g)));   // written by other SMs: L2
+            const float2 x = load_cg(reinterpret_cast<const float2*>(src + round_F_offset<kT>(g)));   // written by other SMs: L2
             v[2 * g + 0] = x.x; v[2 * g + 1] = x.y;
         }
         butterflies32<31>(v);

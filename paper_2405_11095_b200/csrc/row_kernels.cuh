@@ -280,11 +280,11 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             float2 a, b;
             if constexpr (SRC == SRC_WS_PAIR) {
                 const float* const src = static_cast<const float*>(p.src) + at;
-                a = __ldcg(reinterpret_cast<const float2*>(src + o));
-                b = __ldcg(reinterpret_cast<const float2*>(src + o + (1 << T)));
+                a = load_cg(reinterpret_cast<const float2*>(src + o));
+                b = load_cg(reinterpret_cast<const float2*>(src + o + (1 << T)));
             } else {
                 const __half* const src = static_cast<const __half*>(p.src) + at;
-                const uint32_t qa = __ldcg(reinterpret_cast<const uint32_t*>(src + o)), qb = __ldcg(reinterpret_cast<const uint32_t*>(src + o + (1 << T)));
+                const uint32_t qa = load_cg(reinterpret_cast<const uint32_t*>(src + o)), qb = load_cg(reinterpret_cast<const uint32_t*>(src + o + (1 << T)));
                 a = __half22float2(*reinterpret_cast<const __half2*>(&qa));
                 b = __half22float2(*reinterpret_cast<const __half2*>(&qb));
             }
@@ -300,13 +300,13 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             float* const x = v + g * VN;
             if (o + VN <= left) {
                 if constexpr (VB == 2) {
-                    const float4 q = __ldcs(reinterpret_cast<const float4*>(src + o));
+                    const float4 q = load_cs(reinterpret_cast<const float4*>(src + o));
                     x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
                 } else if constexpr (VB == 1) {
-                    const float2 q = __ldcs(reinterpret_cast<const float2*>(src + o));
+                    const float2 q = load_cs(reinterpret_cast<const float2*>(src + o));
                     x[0] = q.x; x[1] = q.y;
                 } else {
-                    x[0] = __ldcs(src + o);
+                    x[0] = load_cs(src + o);
                 }
             } else {
 #pragma unroll
@@ -322,11 +322,11 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             float* const x = v + g * VN;
             if (VB > 0 && o + VN <= left) {
                 if constexpr (VB == 2) {
-                    const uint2 q = __ldcs(reinterpret_cast<const uint2*>(src + o));
+                    const uint2 q = load_cs(reinterpret_cast<const uint2*>(src + o));
                     x[0] = __uint_as_float(q.x << 16); x[1] = __uint_as_float(q.x & 0xFFFF0000u);
                     x[2] = __uint_as_float(q.y << 16); x[3] = __uint_as_float(q.y & 0xFFFF0000u);
                 } else if constexpr (VB == 1) {
-                    const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(src + o));
+                    const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(src + o));
                     x[0] = __uint_as_float(q << 16); x[1] = __uint_as_float(q & 0xFFFF0000u);
                 }
             } else {
@@ -341,13 +341,13 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             const int o = round_F_offset<T>(g);
             float* const x = v + g * VN;
             if constexpr (VB == 2) {
-                const float4 q = __ldcs(reinterpret_cast<const float4*>(src + o));
+                const float4 q = load_cs(reinterpret_cast<const float4*>(src + o));
                 x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
             } else if constexpr (VB == 1) {
-                const float2 q = __ldcs(reinterpret_cast<const float2*>(src + o));
+                const float2 q = load_cs(reinterpret_cast<const float2*>(src + o));
                 x[0] = q.x; x[1] = q.y;
             } else {
-                x[0] = __ldcs(src + o);
+                x[0] = load_cs(src + o);
             }
         }
     } else if constexpr (SRC == SRC_WS16) {
@@ -357,16 +357,16 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             const int o = round_F_offset<T>(g);
             float* const x = v + g * VN;
             if constexpr (VB == 2) {
-                const uint2 q = __ldcs(reinterpret_cast<const uint2*>(src + o));
+                const uint2 q = load_cs(reinterpret_cast<const uint2*>(src + o));
                 const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
                 const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
                 x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
             } else if constexpr (VB == 1) {
-                const uint32_t q = __ldcs(reinterpret_cast<const uint32_t*>(src + o));
+                const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(src + o));
                 const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q));
                 x[0] = a.x; x[1] = a.y;
             } else {
-                x[0] = __half2float(__ldcs(src + o));
+                x[0] = __half2float(load_cs(src + o));
             }
         }
     } else {  // SRC_BITS
@@ -377,7 +377,7 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             const uint32_t pos = (uint32_t)e0 & 31u;
             float* const x = v + g * VN;
             if (p.P == 1) {
-                const uint32_t w = __ldg(src + (e0 >> 5)) >> pos;
+                const uint32_t w = load_ca(src + (e0 >> 5)) >> pos;
 #pragma unroll
                 for (int k = 0; k < VN; ++k) x[k] = (w & (1u << k)) ? 1.f : -1.f;
             } else {
@@ -406,6 +406,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
 {
     using C = RowCfg<T>;
     extern __shared__ __align__(16) float smem[];
+    pdl_begin();
     uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);
 
     const int tid = threadIdx.x;
@@ -511,6 +512,7 @@ __global__ void __launch_bounds__(PackKCfg<T>::THREADS, PackKCfg<T>::MIN_BLOCKS)
     using C = RowCfg<T>;
     using K = PackKCfg<T>;
     extern __shared__ __align__(16) float smem[];
+    pdl_begin();
     uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);
     uint32_t* const counts = fw + C::FLIP_WORDS + 4;
     const int tid = threadIdx.x;
@@ -601,6 +603,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
 {
     using C = RowCfg<T>;
     using S = StreamCfg<T, SRC>;
+    pdl_begin();
     static_assert(SRC == SRC_WS || SRC == SRC_WS16, "streamed sources only");
     extern __shared__ __align__(16) float smem[];
     uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);

@@ -15,6 +15,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK
     __shared__ float x[512];
     __shared__ float acc[512];
     __shared__ uint32_t counts[4 * 32];
+    pdl_begin();
     const int n = 1 << L;
     const int tid = threadIdx.x, nt = blockDim.x;
     const int64_t base = (int64_t)blockIdx.x << L;

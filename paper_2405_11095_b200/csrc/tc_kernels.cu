@@ -69,6 +69,7 @@ __device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t adesc, uint64_
 __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams p, const int64_t ntiles)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
+    pdl_trigger();
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const uint32_t lane = tid & 31;
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
         *s_stop = 0;
     }
     fence_generic_before_async();   // the constant operand, for the tensor core's reads
+    pdl_wait();                     // (the set-up above needs nothing from the kernel before)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
             tile_origin(item, n, i_tile);
             const uint32_t* const bits = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride;
 #pragma unroll
-            for (int k = 0; k < 2; ++k) w[k] = __ldg(reinterpret_cast<const uint4*>(bits + ((i_tile + ((uint32_t)tid + 512u * k) * step) >> 5)));
+            for (int k = 0; k < 2; ++k) w[k] = load_ca(reinterpret_cast<const uint4*>(bits + ((i_tile + ((uint32_t)tid + 512u * k) * step) >> 5)));
         };
 
         uint4 next_bits[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
@@ -291,16 +293,13 @@ bool tc_col_applicable(const PassParams& p, bool any_size)
 cudaError_t launch_tc_col(const PassParams& p, cudaStream_t s)
 {
     if (!tc_col_applicable(p, true)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(tc_col_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes);
+    int sms = 0;
+    const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    int dev = 0, sms = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     const int64_t ntiles = p.dp >> 17;                        // 1024 rows x 128 columns each
     int64_t blocks = ntiles * p.nworkers;
     if (blocks > sms) blocks = sms;
-    tc_col_kernel<<<(unsigned)blocks, kTcThreads, kTcSmemBytes, s>>>(p, ntiles);
-    return cudaGetLastError();
+    return launch<tc_col_kernel>(dim3((unsigned)blocks), kTcThreads, kTcSmemBytes, s, 1, p, ntiles);
 }
 
 cudaError_t tc_timeouts(int* out) { return cudaMemcpyFromSymbol(out, g_tc_wait_timeouts, sizeof(int)); }

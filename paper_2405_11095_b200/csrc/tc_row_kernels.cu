@@ -90,6 +90,7 @@ template <int HALVES>
 __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassParams p, const int ntiles)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
+    pdl_trigger();
     const int tid = threadIdx.x;
     const int warp = tid >> 5;
     const uint32_t lane = tid & 31;
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         *s_stop = 0;
     }
     fence_generic_before_async();   // the constant operand, for the tensor core's reads
+    pdl_wait();                     // (the set-up above needs nothing from the kernel before)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
