@@ -50,10 +50,39 @@ __device__ __forceinline__ float flip_shifted(float x, uint32_t word, uint32_t s
 
 // Packed source: the 32 columns of a row segment are one word per plane.  Lane r fetches the
 // word of the r-th row this warp handles (one gather per warp and plane instead of 32 broadcast loads:
-// 2^25 coordinates of two planes, ten stages: 174 us with every thread loading its own words).
+// 2^25 coordinates of two planes, ten stages: 174 us with every thread loading its own words), and a bit
+// transpose across the warp (five shuffles instead of one per row) hands every lane its columns.
 __device__ __forceinline__ uint32_t bits_row_word(const PassParams& p, const void* worker_src, uint32_t irow, int plane)
 {
     return load_ca(static_cast<const uint32_t*>(worker_src) + (irow >> 5) + (int64_t)plane * (p.dp >> 5));
+}
+
+// Two adjacent columns of sixteen rows: on entry lane 16 h + r holds the word of row r that covers the columns of
+// half-warp h; on return bit r is row r of column 2 (lane & 15), bit 16 + r of the column beside it.
+__device__ __forceinline__ uint32_t column_pair_bits(uint32_t word, uint32_t lane)
+{
+    const uint32_t t = warp_transpose_bits(word, lane);
+    const uint32_t a = __shfl_sync(0xFFFFFFFFu, t, 2u * (lane & 15u)), b = __shfl_sync(0xFFFFFFFFu, t, 2u * (lane & 15u) + 1u);
+    return __byte_perm(a, b, (lane & 16u) ? 0x7632 : 0x5410);
+}
+
+// v[r] = 2 c - K of R rows from the P count planes of one column (exact): column(pl) = this lane's column of plane pl,
+// one bit per row.  fetch(pl) starts the plane's loads one plane ahead.
+template <int R, typename Fetch, typename Column>
+__device__ __forceinline__ void planes_to_values(const PassParams& p, float (&v)[32], Fetch fetch, Column column)
+{
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = (float)(-p.K);
+    auto next = fetch(0);
+    float weight = 2.f;
+    for (int pl = 0; pl < p.P; ++pl, weight += weight) {
+        const auto mine = next;
+        if (pl + 1 < p.P) next = fetch(pl + 1);
+        const uint32_t x = column(mine);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if ((x >> r) & 1u) v[r] += weight;
+    }
 }
 
 // ---- A <= 4 -----------------------------------------------------------------------------
@@ -74,16 +103,8 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
 
     float v[32];
     if constexpr (SRC == SRC_BITS) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = (float)(-p.K);
-        float weight = 2.f;
-        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
-            uint32_t mine = 0;
-            if ((int)lane < R) mine = bits_row_word(p, wsrc, (i_first - lane) + lane * step, pl);
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                if ((__shfl_sync(0xFFFFFFFFu, mine, r) >> lane) & 1u) v[r] += weight;
-        }
+        planes_to_values<R>(p, v, [&](int pl) { return (int)lane < R ? bits_row_word(p, wsrc, (i_first - lane) + lane * step, pl) : 0u; },
+                            [&](uint32_t mine) { return warp_transpose_bits(mine, lane); });
     } else {
         uint32_t myword = 0;  // flip word of row `lane` (gradient sources)
         if (SRC == SRC_G32 || SRC == SRC_G16) {
@@ -135,25 +156,16 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
         // round F: rows k = r * WARPS + w
         const uint32_t i_f = i_tile + w * step + 2u * lane;
         const uint32_t step_f = step * WARPS;
-        // the two words (flips, or packed signs) of row r belong to lanes 2 r and 2 r + 1
-        const uint32_t iw = i_tile + w * step + (lane >> 1) * step_f + 32u * (lane & 1u);
-        const uint32_t from = lane >> 4, bit = (2u * lane) & 31u;
+        // the two words (flips, or packed signs) of row r belong to lanes r and 16 + r
+        const uint32_t iw = i_tile + w * step + (lane & 15u) * step_f + 32u * (lane >> 4);
+        const uint32_t from = lane & 16u, bit = (2u * lane) & 31u;
         float v[32];
         if constexpr (SRC == SRC_BITS) {
-            const uint32_t* const words = static_cast<const uint32_t*>(wsrc) + (iw >> 5);
-            const float base = (float)(-p.K);
+            float u[32];    // the sixteen rows of the lane's first column, then those of its second
+            planes_to_values<32>(p, u, [&](int pl) { return bits_row_word(p, wsrc, iw, pl); },
+                                 [&](uint32_t mine) { return column_pair_bits(mine, lane); });
 #pragma unroll
-            for (int r = 0; r < 32; ++r) v[r] = base;
-            float weight = 2.f;
-            for (int pl = 0; pl < p.P; ++pl, weight += weight) {
-                const uint32_t mine = load_ca(words + (int64_t)pl * (p.dp >> 5));
-#pragma unroll
-                for (int r = 0; r < 16; ++r) {
-                    const uint32_t x = __shfl_sync(0xFFFFFFFFu, mine, 2 * r + (int)from) >> bit;
-                    if (x & 1u) v[2 * r] += weight;               // 2 c - K, bit by bit (exact)
-                    if (x & 2u) v[2 * r + 1] += weight;
-                }
-            }
+            for (int r = 0; r < 16; ++r) { v[2 * r] = u[r]; v[2 * r + 1] = u[16 + r]; }
         } else if constexpr (kGrad) {
             auto load2 = [&](uint32_t i, float& x0, float& x1) {
                 if constexpr (SRC == SRC_G32) {
@@ -185,7 +197,7 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
             const uint32_t sh = 31u - bit;
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
-                const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, 2 * r + (int)from);
+                const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, r + (int)from);
                 v[2 * r] = flip_shifted(v[2 * r], word, sh);
                 v[2 * r + 1] = flip_shifted(v[2 * r + 1], word, sh - 1u);
             }
@@ -266,15 +278,8 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassP
     const uint32_t i_f = i_tile + w * step + lane;
     const uint32_t step_f = step * WARPS;
     if constexpr (SRC == SRC_BITS) {
-#pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
-        float weight = 2.f;
-        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
-            const uint32_t mine = bits_row_word(p, wsrc, irow, pl);
-#pragma unroll
-            for (int r = 0; r < 32; ++r)
-                if ((__shfl_sync(0xFFFFFFFFu, mine, r) >> lane) & 1u) v[r] += weight;
-        }
+        planes_to_values<32>(p, v, [&](int pl) { return bits_row_word(p, wsrc, irow, pl); },
+                             [&](uint32_t mine) { return warp_transpose_bits(mine, lane); });
     } else {
 #pragma unroll
         for (int r = 0; r < 32; ++r) v[r] = col_load<SRC>(p, wsrc, i_f + r * step_f, d32);
@@ -335,15 +340,12 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) col_tile16_kernel(const PassP
     const uint32_t i_f = i_tile + ((w << 1) | h) * step + c;
     const uint32_t step_f = step << (A - 5);
     if constexpr (SRC == SRC_BITS) {
-#pragma unroll
-        for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
-        float weight = 2.f;
-        for (int pl = 0; pl < p.P; ++pl, weight += weight) {
-            const uint32_t word_lo = bits_row_word(p, wsrc, ia, pl), word_hi = bits_row_word(p, wsrc, ib, pl);
-#pragma unroll
-            for (int r = 0; r < 32; ++r)
-                if ((__shfl_sync(0xFFFFFFFFu, r < 16 ? word_lo : word_hi, r & 15, 16) >> bitpos) & 1u) v[r] += weight;
-        }
+        planes_to_values<32>(p, v, [&](int pl) { return make_uint2(bits_row_word(p, wsrc, ia, pl), bits_row_word(p, wsrc, ib, pl)); },
+                             [&](uint2 mine) {
+                                 const uint32_t a = __shfl_sync(0xFFFFFFFFu, warp_transpose_bits(mine.x, lane), bitpos);
+                                 const uint32_t b = __shfl_sync(0xFFFFFFFFu, warp_transpose_bits(mine.y, lane), bitpos);
+                                 return __byte_perm(a, b, h ? 0x7632 : 0x5410);
+                             });
     } else {
         // a block whose last coordinate is inside the gradient needs no per-element bound check
         // (the constant bound folds the checks away)
@@ -513,36 +515,44 @@ cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStr
 // lane as a half2: 64 columns per warp, butterflies are HADD2 (two coordinates
 // per instruction), and the intermediate is written as fp16 (half the bytes, still full
 // 128-byte lines per warp).  A row segment of the source is two words per plane: lanes fetch them, one
-// gather for every sixteen rows, and pass them by shuffle.
+// gather for every sixteen rows, and a bit transpose hands every lane its columns.
+// rows 0..15 (a) and 16..31 (b) of two adjacent columns, one bit each as column_pair_bits leaves them, as +-1
+__device__ __forceinline__ void signs_to_half2(uint32_t a, uint32_t b, __half2 (&v)[32])
+{
+#pragma unroll
+    for (int r = 0; r < 32; ++r) {
+        // bit r -> sign of the low half, bit 16 + r -> sign of the high half; set bit = +1
+        const uint32_t hb = 0xBC00BC00u ^ (((r < 16 ? a : b) << (15 - (r & 15))) & 0x80008000u);
+        v[r] = *reinterpret_cast<const __half2*>(&hb);
+    }
+}
+
 // at(r): coordinate of register r = 0 .. 31, column 0 of the warp's 64
 template <typename At>
 __device__ __forceinline__ void load_planes_half2(const PassParams& p, const uint32_t* bits, uint32_t lane, __half2 (&v)[32], At at)
 {
-    const uint32_t sh = (2u * lane) & 31u, from = lane >> 4;
-    // words of registers (lane >> 1) and 16 + (lane >> 1), column half lane & 1
-    const uint32_t* const wa = bits + (at(lane >> 1) >> 5) + (lane & 1u);
-    const uint32_t* const wb = bits + (at(16u + (lane >> 1)) >> 5) + (lane & 1u);
+    // words of registers (lane & 15) and 16 + (lane & 15), column half lane >> 4
+    const uint32_t* const wa = bits + (at(lane & 15u) >> 5) + (lane >> 4);
+    const uint32_t* const wb = bits + (at(16u + (lane & 15u)) >> 5) + (lane >> 4);
     if (p.P == 1) {
         const uint32_t word_a = load_ca(wa), word_b = load_ca(wb);
-#pragma unroll
-        for (int r = 0; r < 32; ++r) {
-            const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
-            // bit 0 -> sign of the low half, bit 1 -> sign of the high half; set bit = +1
-            const uint32_t hb = 0xBC00BC00u ^ ((x * 0x40008000u) & 0x80008000u);
-            v[r] = *reinterpret_cast<const __half2*>(&hb);
-        }
+        signs_to_half2(column_pair_bits(word_a, lane), column_pair_bits(word_b, lane), v);
     } else {
         const __half2 base = __float2half2_rn((float)(-p.K));
 #pragma unroll
         for (int r = 0; r < 32; ++r) v[r] = base;
+        uint32_t next_a = load_ca(wa), next_b = load_ca(wb);
         uint32_t weight = 0x4000u;                               // fp16 2.0; the exponent grows plane by plane
         for (int pl = 0; pl < p.P; ++pl, weight += 0x400u) {
-            const int64_t off = (int64_t)pl * (p.dp >> 5);
-            const uint32_t word_a = load_ca(wa + off), word_b = load_ca(wb + off);
+            const uint32_t a = column_pair_bits(next_a, lane), b = column_pair_bits(next_b, lane);
+            if (pl + 1 < p.P) {
+                const int64_t off = (int64_t)(pl + 1) * (p.dp >> 5);
+                next_a = load_ca(wa + off);
+                next_b = load_ca(wb + off);
+            }
 #pragma unroll
             for (int r = 0; r < 32; ++r) {
-                const uint32_t x = (__shfl_sync(0xFFFFFFFFu, r < 16 ? word_a : word_b, 2 * (r & 15) + (int)from) >> sh) & 3u;
-                const uint32_t hb = ((x * 0x8001u) & 0x00010001u) * weight;
+                const uint32_t hb = (((r < 16 ? a : b) >> (r & 15)) & 0x00010001u) * weight;
                 v[r] = __hadd2(v[r], *reinterpret_cast<const __half2*>(&hb));
             }
         }
@@ -633,14 +643,7 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) colh_tile32_kernel(const Pass
         word_hi = load_ca(bits + ((ia + (step << (A - 1))) >> 5));
     }
     __half2 v[32];
-    const uint32_t sh = 2u * c2;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        const uint32_t roww = __shfl_sync(0xFFFFFFFFu, r < 16 ? word_lo : word_hi, r & 15, 16);
-        const uint32_t x = (roww >> sh) & 3u;
-        const uint32_t hb = 0xBC00BC00u ^ ((x * 0x40008000u) & 0x80008000u);
-        v[r] = *reinterpret_cast<const __half2*>(&hb);
-    }
+    signs_to_half2(column_pair_bits(word_lo, lane), column_pair_bits(word_hi, lane), v);
     butterflies32<31, __half2>(v);
     __half2* const tile = reinterpret_cast<__half2*>(smemh);
     {

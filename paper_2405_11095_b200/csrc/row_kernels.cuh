@@ -262,8 +262,8 @@ __device__ __forceinline__ void split_final_store(const PassParams& p, int64_t t
 }
 
 // ---- round F's registers from memory ----------------------------------------------------------
-// fw: flip words of the tile (gradient sources)
-template <int T, int SRC>
+// fw: flip words of the tile (gradient sources).  ONE_PLANE: a packed source known to have a single plane.
+template <int T, int SRC, bool ONE_PLANE = false>
 __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t tile_base, int baseF, const uint32_t* fw,
                                             float (&v)[32])
 {
@@ -370,19 +370,28 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             }
         }
     } else {  // SRC_BITS
-        const uint32_t* const src = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride + (tile_base >> 5);
+        // plane by plane (one of them: +-1), a word per group of consecutive coordinates; no unrolling over the planes: a
+        // short vector runs through this code once, and fetching the instructions would cost more than they do
+        const uint32_t* src = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride + ((tile_base + baseF) >> 5);
+        const uint32_t pos = (uint32_t)baseF & 31u;      // (the groups are whole words apart)
+        constexpr int NG = 32 >> VB;
+        uint32_t w[NG];
+        if constexpr (ONE_PLANE) {
 #pragma unroll
-        for (int g = 0; g < (32 >> VB); ++g) {
-            const int e0 = baseF | round_F_offset<T>(g);
-            const uint32_t pos = (uint32_t)e0 & 31u;
-            float* const x = v + g * VN;
-            if (p.P == 1) {
-                const uint32_t w = load_ca(src + (e0 >> 5)) >> pos;
+            for (int g = 0; g < NG; ++g) w[g] = load_ca(src + (round_F_offset<T>(g) >> 5)) >> pos;
 #pragma unroll
-                for (int k = 0; k < VN; ++k) x[k] = (w & (1u << k)) ? 1.f : -1.f;
-            } else {
+            for (int r = 0; r < 32; ++r) v[r] = ((w[r >> VB] >> (r & (VN - 1))) & 1u) ? 1.f : -1.f;
+        } else {
 #pragma unroll
-                for (int k = 0; k < VN; ++k) x[k] = plane_value(src + (e0 >> 5), p.dp >> 5, p.P, p.K, pos + k);
+            for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
+            float weight = 2.f;
+#pragma unroll 1
+            for (int pl = 0; pl < p.P; ++pl, weight += weight, src += p.dp >> 5) {
+#pragma unroll
+                for (int g = 0; g < NG; ++g) w[g] = load_ca(src + (round_F_offset<T>(g) >> 5)) >> pos;
+#pragma unroll
+                for (int r = 0; r < 32; ++r)
+                    if ((w[r >> VB] >> (r & (VN - 1))) & 1u) v[r] += weight;
             }
         }
     }
@@ -452,7 +461,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         }
 
         float v[32];
-        load_source<T, SRC>(p, n, tile_base, baseF, fw, v);
+        load_source<T, SRC, kLoopWorkers>(p, n, tile_base, baseF, fw, v);   // (uplink planes come one to a worker)
         butterflies32<31>(v);
         store_round_F<T>(smem, baseF, v);
         __syncthreads();
