@@ -1,6 +1,7 @@
 """Python binding of libfosgd (FO-SGD gradient-compression round trip on one B200).
 
-Argument marshalling only: every step of the path runs in the library's CUDA kernels.
+Argument marshalling only (in native code, csrc/binding.c, for the calls that a program makes in its loop): every
+step of the path runs in the library's CUDA kernels.
 Tensors are torch CUDA tensors used as device buffers; the calls enqueue work on torch's
 current stream and return without synchronising.  There is no CPU fallback: the first call
 into the package without a built ``libfosgd.so`` raises ImportError.
@@ -105,17 +106,40 @@ def _check(status: int, where: str) -> None:
         raise FosgdError(status, where)
 
 
-_torch = None
+_calls = None      # the native module, once it is bound to the loaded library
+
+# order of the function table of csrc/binding.c
+_NATIVE_FUNCTIONS = ("fosgd_encode", "fosgd_flatten", "fosgd_decode", "fosgd_server_aggregate", "fosgd_downlink_decode",
+                     "fosgd_amplitudes", "fosgd_encode_dev", "fosgd_server_aggregate_dev", "fosgd_downlink_decode_dev",
+                     "fosgd_downlink_encode", "fosgd_downlink_apply", "fosgd_encode_measured")
+
+
+def _bind():
+    """The native marshalling module (csrc/binding.c: a call costs 1 us there and 3 us through ctypes), bound to the
+    loaded library and to torch's current device and stream."""
+    global _calls
+    import torch
+    torch.cuda.current_device()      # brings CUDA up, or says why there is none
+    L = lib()
+    try:
+        from . import _native as n
+    except ImportError as e:
+        raise ImportError(f"{_HERE}/_native.so is missing: build it with `python -m paper_2405_11095_b200.build`") from e
+    n.bind(tuple(C.cast(getattr(L, f), C.c_void_p).value for f in _NATIVE_FUNCTIONS), torch._C._cuda_getDevice,
+           torch._C._cuda_getCurrentRawStream, torch.float32, torch.bfloat16)
+    _calls = n
+    return n
+
+
+def _failed(status: int, where: str, grads=None) -> None:
+    if grads is not None:
+        _dtype_code(grads)           # names an unsupported type
+    _check(status, where)
 
 
 def _stream() -> int:
-    """Handle of torch's current stream.  Read without building a torch.cuda.Stream object: that costs 3 us,
-    as much as the launch of a kernel, on every call."""
-    global _torch
-    if _torch is None:
-        import torch
-        _torch = torch
-    return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
+    import torch
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _ptr(t) -> int:
@@ -163,26 +187,25 @@ def workspace_bytes(op: int, d: int, M: int = 1, dtype: int = F32, block_log2: i
 
 def encode(grads, d, bits, lam, seed, step, worker_id0=0, block_log2=0, ws=None, worker_stride=None):
     """fosgd_encode: grads [M, >=d] (fp32/bf16, row stride = worker_stride) -> bits [M, d'/32] int32."""
-    M = grads.shape[0] if grads.dim() == 2 else 1
-    stride = worker_stride if worker_stride is not None else (grads.stride(0) if grads.dim() == 2 else d)
-    _check(_lib.fosgd_encode(_ptr(grads), _dtype_code(grads), d, stride, M, worker_id0, seed, step, lam,
-                             block_log2, _ptr(bits), _ptr(ws), _nbytes(ws), _stream()), "fosgd_encode")
+    st = (_calls or _bind()).encode(grads, d, bits, lam, seed, step, worker_id0, block_log2, ws, worker_stride)
+    if st:
+        _failed(st, "fosgd_encode", grads)
     return bits
 
 
 def flatten(grads, d, out, seed, step, worker_id0=0, block_log2=0, ws=None, worker_stride=None):
     """fosgd_flatten: out [M, d'] fp32 = H D_eps x."""
-    M = grads.shape[0] if grads.dim() == 2 else 1
-    stride = worker_stride if worker_stride is not None else (grads.stride(0) if grads.dim() == 2 else d)
-    _check(_lib.fosgd_flatten(_ptr(grads), _dtype_code(grads), d, stride, M, worker_id0, seed, step,
-                              block_log2, _ptr(out), _ptr(ws), _nbytes(ws), _stream()), "fosgd_flatten")
+    st = (_calls or _bind()).flatten(grads, d, out, seed, step, worker_id0, block_log2, ws, worker_stride)
+    if st:
+        _failed(st, "fosgd_flatten", grads)
     return out
 
 
 def decode(bits, d, out, lam, seed, step, worker_id, block_log2=0, ws=None):
     """fosgd_decode: bits [d'/32] -> out [d] fp32."""
-    _check(_lib.fosgd_decode(_ptr(bits), d, worker_id, seed, step, lam, block_log2, _ptr(out), _ptr(ws),
-                             _nbytes(ws), _stream()), "fosgd_decode")
+    st = (_calls or _bind()).decode(bits, d, out, lam, seed, step, worker_id, block_log2, ws)
+    if st:
+        _failed(st, "fosgd_decode")
     return out
 
 
@@ -200,18 +223,18 @@ def decode_noalloc(bits, d, out, lam, seed, step, worker_id, block_log2=0):
 def server_aggregate(bits, d, acc, lam, seed, step, N_total=None, worker_id0=0, flags=AGG_BEGIN | AGG_END,
                      lam_s=0.0, K=1, down_bits=None, block_log2=0, ws=None):
     """fosgd_server_aggregate: bits [M, d'/32] -> acc [d'] fp32 (and down_bits [P, d'/32] on END)."""
-    M = bits.shape[0] if bits.dim() == 2 else 1
-    _check(_lib.fosgd_server_aggregate(_ptr(bits), d, M, worker_id0, M if N_total is None else N_total,
-                                       seed, step, lam, block_log2, _ptr(acc), flags, lam_s, K,
-                                       _ptr(down_bits), _ptr(ws), _nbytes(ws), _stream()),
-           "fosgd_server_aggregate")
+    st = (_calls or _bind()).server_aggregate(bits, d, acc, lam, seed, step, N_total, worker_id0, flags, lam_s, K,
+                                             down_bits, block_log2, ws)
+    if st:
+        _failed(st, "fosgd_server_aggregate")
     return acc
 
 
 def downlink_decode(down_bits, d, out, lam_s, seed, step, K=1, block_log2=0, ws=None):
     """fosgd_downlink_decode: down_bits [P, d'/32] -> out [d] fp32."""
-    _check(_lib.fosgd_downlink_decode(_ptr(down_bits), d, seed, step, lam_s, K, block_log2, _ptr(out),
-                                      _ptr(ws), _nbytes(ws), _stream()), "fosgd_downlink_decode")
+    st = (_calls or _bind()).downlink_decode(down_bits, d, out, lam_s, seed, step, K, block_log2, ws)
+    if st:
+        _failed(st, "fosgd_downlink_decode")
     return out
 
 
@@ -219,22 +242,19 @@ def amplitudes(grads, d, lam, lam_s=None, alpha=2.0, alpha_s=2.0, block_log2=0, 
                worker_stride=None):
     """fosgd_amplitudes: device tensors lam ([1], or [M, d' >> b] with per_block) and lam_s ([1] or
     [d' >> b], optional) <- the amplitudes of the gradients' own norms."""
-    M = grads.shape[0] if grads.dim() == 2 else 1
-    stride = worker_stride if worker_stride is not None else (grads.stride(0) if grads.dim() == 2 else d)
-    _check(_lib.fosgd_amplitudes(_ptr(grads), _dtype_code(grads), d, stride, M, alpha, alpha_s, block_log2,
-                                 int(per_block), _ptr(lam), _ptr(lam_s), _ptr(ws), _nbytes(ws), _stream()),
-           "fosgd_amplitudes")
+    st = (_calls or _bind()).amplitudes(grads, d, lam, lam_s, alpha, alpha_s, block_log2, per_block, ws, worker_stride)
+    if st:
+        _failed(st, "fosgd_amplitudes", grads)
     return lam, lam_s
 
 
 def encode_dev(grads, d, bits, lam, seed, step, worker_id0=0, block_log2=0, per_block=False, ws=None,
                worker_stride=None):
     """fosgd_encode_dev: fosgd_encode with the amplitude(s) read from the device tensor `lam`."""
-    M = grads.shape[0] if grads.dim() == 2 else 1
-    stride = worker_stride if worker_stride is not None else (grads.stride(0) if grads.dim() == 2 else d)
-    _check(_lib.fosgd_encode_dev(_ptr(grads), _dtype_code(grads), d, stride, M, worker_id0, seed, step,
-                                 _ptr(lam), int(per_block), block_log2, _ptr(bits), _ptr(ws), _nbytes(ws), _stream()),
-           "fosgd_encode_dev")
+    st = (_calls or _bind()).encode_dev(grads, d, bits, lam, seed, step, worker_id0, block_log2, per_block, ws,
+                                       worker_stride)
+    if st:
+        _failed(st, "fosgd_encode_dev", grads)
     return bits
 
 
@@ -242,49 +262,46 @@ def encode_measured(grads, d, bits, lam, lam_s, seed, step, alpha=2.0, alpha_s=2
                     amp_ws=None, worker_stride=None):
     """fosgd_encode_measured: amplitudes(...) and encode_dev(...) in one call (one amplitude for all workers);
     the gradients are read once where the encoder's first pass can carry the norm.  lam, lam_s: device [1]."""
-    M = grads.shape[0] if grads.dim() == 2 else 1
-    stride = worker_stride if worker_stride is not None else (grads.stride(0) if grads.dim() == 2 else d)
-    _check(_lib.fosgd_encode_measured(_ptr(grads), _dtype_code(grads), d, stride, M, worker_id0, seed, step, alpha, alpha_s,
-                                      block_log2, _ptr(lam), _ptr(lam_s), _ptr(bits), _ptr(ws), _nbytes(ws), _ptr(amp_ws),
-                                      _nbytes(amp_ws), _stream()), "fosgd_encode_measured")
+    st = (_calls or _bind()).encode_measured(grads, d, bits, lam, lam_s, seed, step, alpha, alpha_s, worker_id0, block_log2,
+                                            ws, amp_ws, worker_stride)
+    if st:
+        _failed(st, "fosgd_encode_measured", grads)
     return bits
 
 
 def server_aggregate_dev(bits, d, acc, lam, seed, step, N_total=None, worker_id0=0, flags=AGG_BEGIN | AGG_END,
                          lam_s=None, K=1, down_bits=None, block_log2=0, per_block=False, ws=None):
     """fosgd_server_aggregate_dev: amplitudes read from the device tensors `lam` and `lam_s`."""
-    M = bits.shape[0] if bits.dim() == 2 else 1
-    _check(_lib.fosgd_server_aggregate_dev(_ptr(bits), d, M, worker_id0, M if N_total is None else N_total,
-                                           seed, step, _ptr(lam), _ptr(lam_s), int(per_block), block_log2, _ptr(acc),
-                                           flags, K, _ptr(down_bits), _ptr(ws), _nbytes(ws), _stream()),
-           "fosgd_server_aggregate_dev")
+    st = (_calls or _bind()).server_aggregate_dev(bits, d, acc, lam, seed, step, N_total, worker_id0, flags, lam_s, K,
+                                                 down_bits, block_log2, per_block, ws)
+    if st:
+        _failed(st, "fosgd_server_aggregate_dev")
     return acc
 
 
 def downlink_decode_dev(down_bits, d, out, lam_s, seed, step, K=1, block_log2=0, per_block=False, ws=None):
     """fosgd_downlink_decode_dev: lambda^s read from the device tensor `lam_s`."""
-    _check(_lib.fosgd_downlink_decode_dev(_ptr(down_bits), d, seed, step, _ptr(lam_s), int(per_block), K, block_log2,
-                                          _ptr(out), _ptr(ws), _nbytes(ws), _stream()), "fosgd_downlink_decode_dev")
+    st = (_calls or _bind()).downlink_decode_dev(down_bits, d, out, lam_s, seed, step, K, block_log2, per_block, ws)
+    if st:
+        _failed(st, "fosgd_downlink_decode_dev")
     return out
 
 
 def downlink_encode(gbar, d, down_bits, lam_s, seed, step, K=1, block_log2=0, per_block=False, ws=None):
     """fosgd_downlink_encode: the server's encoder on a finished average gbar [d'] -> down_bits
     [P, d'/32].  lam_s: a float, or a device tensor in either layout of `amplitudes`."""
-    dev = None if isinstance(lam_s, (int, float)) else lam_s
-    _check(_lib.fosgd_downlink_encode(_ptr(gbar), d, seed, step, 0.0 if dev is not None else float(lam_s), _ptr(dev),
-                                      int(per_block), K, block_log2, _ptr(down_bits), _ptr(ws), _nbytes(ws),
-                                      _stream()), "fosgd_downlink_encode")
+    st = (_calls or _bind()).downlink_encode(gbar, d, down_bits, lam_s, seed, step, K, block_log2, per_block, ws)
+    if st:
+        _failed(st, "fosgd_downlink_encode")
     return down_bits
 
 
 def downlink_apply(down_bits, d, x, lam_s, seed, step, step_size, K=1, block_log2=0, per_block=False, ws=None):
     """fosgd_downlink_apply: x <- x - step_size * D(down_bits) (eq. (4.2) fused into the downlink
     decoder).  lam_s: a float, or a device tensor in either layout of `amplitudes`."""
-    dev = None if isinstance(lam_s, (int, float)) else lam_s
-    _check(_lib.fosgd_downlink_apply(_ptr(down_bits), d, seed, step, 0.0 if dev is not None else float(lam_s),
-                                     _ptr(dev), int(per_block), K, block_log2, float(step_size), _ptr(x),
-                                     _ptr(ws), _nbytes(ws), _stream()), "fosgd_downlink_apply")
+    st = (_calls or _bind()).downlink_apply(down_bits, d, x, lam_s, seed, step, step_size, K, block_log2, per_block, ws)
+    if st:
+        _failed(st, "fosgd_downlink_apply")
     return x
 
 

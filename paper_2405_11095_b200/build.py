@@ -5,11 +5,13 @@ import concurrent.futures as cf
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 SO = os.path.join(HERE, "libfosgd.so")
+NATIVE_SO = os.path.join(HERE, "_native.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
@@ -33,12 +35,25 @@ def _units():
 
 
 def _newest_source() -> float:
-    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
+    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != "binding.c"]
     paths.append(os.path.join(HERE, "..", "include", "fosgd.h"))
     return max(os.path.getmtime(p) for p in paths)
 
 
+def build_binding(force: bool = False) -> str:
+    """The native half of the Python binding (a CPython extension, host code only)."""
+    src = os.path.join(CSRC, "binding.c")
+    newest = max(os.path.getmtime(p) for p in (src, os.path.join(HERE, "..", "include", "fosgd.h")))
+    if force or not os.path.exists(NATIVE_SO) or os.path.getmtime(NATIVE_SO) < newest:
+        tmp = NATIVE_SO + f".tmp{os.getpid()}"
+        subprocess.run(["gcc", "-std=gnu11", "-O2", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"], "-o", tmp, src],
+                       check=True)
+        os.replace(tmp, NATIVE_SO)
+    return NATIVE_SO
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_binding(force)
     if not force and os.path.exists(SO) and os.path.getmtime(SO) >= _newest_source():
         return SO
     os.makedirs(OBJ, exist_ok=True)
