@@ -4,15 +4,25 @@
 
 namespace fosgd {
 
-// shared-memory matrix descriptor, no swizzle: start address, leading and stride byte offsets in
-// units of 16 bytes, descriptor version 1.  K-major operand: leading = bytes between core matrices
-// (8 rows x 16 bytes) along K, stride = between groups of eight rows; MN-major operand: leading =
-// bytes between groups of eight K-rows, stride = between 16-byte column groups.
+// Shared-memory matrix descriptors: start address and strides in units of 16 bytes, descriptor version 1.
+//   K-major operand, no swizzle: core matrices of 8 rows x 16 bytes; leading = bytes between them along K,
+//   stride = bytes between groups of eight rows.
 __device__ __forceinline__ uint64_t umma_desc(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes)
 {
     return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) |
            ((uint64_t)(sbo_bytes >> 4) << 32) | ((uint64_t)1 << 46);
 }
+
+//   MN-major operand, 128-byte swizzle: rows k of 128 bytes (64 fp16 or 128 8-bit columns), eight rows to an atom of
+//   1024 bytes, the 16-byte chunks of a row permuted by k & 7 (swizzled_row_chunk); leading = bytes between blocks of 128
+//   bytes' worth of columns, stride = bytes between groups of eight rows. 
+__device__ __forceinline__ uint64_t umma_desc_mn128(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes)
+{
+    return umma_desc(smem_addr, lbo_bytes, sbo_bytes) | ((uint64_t)2 << 61);
+}
+
+// byte offset of 16-byte chunk c of row k inside a block of rows of 128 bytes
+__device__ __forceinline__ uint32_t swizzled_row_chunk(uint32_t k, uint32_t c) { return k * 128u + ((c ^ (k & 7u)) << 4); }
 
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -42,6 +52,23 @@ __device__ __forceinline__ bool mbar_wait_or_stop(uint64_t* bar, uint32_t parity
     }
     return false;
 }
+
+// Position in a ring of N buffers: the buffer's index, and the parity of the phase that its "full" barrier completes
+// when the buffer is filled for the current round.  A wait for its "free" barrier takes the other parity (which a fresh
+// barrier satisfies at once: the first round finds every buffer free).  Counters of 32 bits that roll over: with
+// 64-bit item numbers and their remainders the one-thread roles of a pipeline spent a thousand cycles per item.
+template <uint32_t N>
+struct RingPos {
+    uint32_t i = 0, full = 0;
+    __device__ __forceinline__ uint32_t free() const { return full ^ 1u; }
+    __device__ __forceinline__ void next()
+    {
+        if (++i == N) {
+            i = 0;
+            full ^= 1u;
+        }
+    }
+};
 
 // 32 consecutive accumulator columns of this thread's lane.  The load is asynchronous: it and its wait
 // are one statement, so that the compiler never sees the destination registers as live while the load is

@@ -41,11 +41,11 @@ constexpr int kThreads = (kFlipWarp + 1) * 32;             // 736: 80 registers 
 constexpr int kAcc = 3;                                    // accumulators (128 columns of tensor memory each) and flip buffers in turn
 constexpr int kRing = 3;                                   // landing slots for whole tiles (bulk copies in flight)
 constexpr uint32_t kTileBytes = 2u << kT;                  // one fp16 tile
-constexpr uint32_t kBGroupStride = 16 * 128 + 32;          // bytes between groups of eight columns of B (+32: staging stores hit distinct banks)
 constexpr uint32_t kAColumns = 64;                         // H_128 as fp16 in tensor memory: lane = row, two k per 32-bit column
 constexpr uint32_t kTmemColumns = 512;                     // kAcc accumulators of 128 columns, then H_128
 constexpr uint32_t kOffB = 0;                              // two operand buffers
-constexpr uint32_t kBBytes = 16 * kBGroupStride;
+constexpr uint32_t kBBlock = 128 * 128;                    // 64 columns x 128 rows k of an operand buffer
+constexpr uint32_t kBBytes = 2 * kBBlock;
 constexpr uint32_t kOffFlips = kOffB + 2 * kBBytes;        // kAcc buffers of 128 rows x 4 flip words
 constexpr uint32_t kOffLand = kOffFlips + kAcc * 2048;     // kRing landing slots
 constexpr uint32_t kOffBar = kOffLand + kRing * kTileBytes;   // mbarriers, stop word, tensor-memory base
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
     const int W = (p.nworkers - n_first + n_step - 1) / n_step;      // workers of this block
     const int n_end = n_first + W * n_step;
     const int my_tiles = ((int)blockIdx.x < ntiles) ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
-    const int64_t nitems = (int64_t)my_tiles * W;   // item g: this block's tile number g / W, its worker number g % W
+    const int nitems = my_tiles * W;                // item g: this block's tile number g / W, its worker number g % W
 
     // where an item sits: first coordinate of its tile and its worker; advanced item by item (worker fastest)
     struct Cursor {
@@ -179,23 +179,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         // ================= the warp that issues the products =================
         if (lane == 0) {
             bool ok = true;
-            int64_t g = 0;
+            int g = 0;
             int tile = (int)blockIdx.x, w = 0;
-            for (; g < nitems; ++g) {
-                const uint32_t b = (uint32_t)(g % kAcc), u = (uint32_t)(g / kAcc);
+            RingPos<kAcc> acc;
+            RingPos<2> op;
+            for (; g < nitems; ++g, acc.next()) {
+                const uint32_t b = acc.i;
 #pragma unroll
-                for (int h = 0; h < HALVES && ok; ++h) {
-                    const uint32_t sb = (uint32_t)(HALVES * g + h) & 1u, su = (uint32_t)((HALVES * g + h) >> 1);
-                    ok = mbar_wait_or_stop(bar + BAR_B_FULL + sb, su & 1u, s_stop);                                     // operand staged
-                    if (ok && h == 0 && u > 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, (u - 1u) & 1u, s_stop);   // accumulator drained
+                for (int h = 0; h < HALVES && ok; ++h, op.next()) {
+                    const uint32_t sb = op.i;
+                    ok = mbar_wait_or_stop(bar + BAR_B_FULL + sb, op.full, s_stop);                          // operand staged
+                    if (ok && h == 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, acc.free(), s_stop);    // accumulator drained
                     if (!ok) break;
                     tc_fence_after_sync();
-                    const uint64_t bdesc = umma_desc(smem_u32(smem + kOffB + sb * kBBytes), 128u, kBGroupStride);
+                    const uint64_t bdesc = umma_desc_mn128(smem_u32(smem + kOffB + sb * kBBytes), kBBlock, 1024u);
                     // the pair's second half enters its first tile with a plus, its second tile with a minus
                     const uint32_t idesc = (h == 1 && (tile & 1)) ? kIdescF16 | kNegateB : kIdescF16;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks)   // K = 16 per instruction: eight columns of A, two groups of eight rows of B
-                        umma_f16(tmem_base + b * 128u, tmem_a + 8u * ks, bdesc + (uint64_t)(ks * (256 >> 4)), idesc, h + ks > 0 ? 1u : 0u);
+                        umma_f16(tmem_base + b * 128u, tmem_a + 8u * ks, bdesc + (uint64_t)(ks * (2048 >> 4)), idesc, h + ks > 0 ? 1u : 0u);
                     umma_commit(bar + BAR_B_FREE + sb);
                 }
                 if (!ok) break;
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             if (!ok) {
                 if (atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
                 // products already committed may still be running: one more bounded wait each before the tensor memory goes back
-                for (int64_t h = (g >= kAcc ? g - kAcc : 0); h < g; ++h) mbar_wait(bar + BAR_ACC_FULL + (h % kAcc), (uint32_t)(h / kAcc) & 1u);
+                for (int h = (g >= kAcc ? g - kAcc : 0); h < g; ++h) mbar_wait(bar + BAR_ACC_FULL + (h % kAcc), (uint32_t)(h / kAcc) & 1u);
                 if (HALVES > 1) {   // (the first half of the item given up on)
                     umma_commit(bar + BAR_ACC_FULL + (g % kAcc));
                     mbar_wait(bar + BAR_ACC_FULL + (g % kAcc), (uint32_t)(g / kAcc) & 1u);
@@ -220,11 +222,12 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         if (lane == 0) {
             Cursor c = c_first;
             bool ok = true;
-            int64_t g = 0;        // copies started
-            const int64_t nloads = HALVES * nitems;
-            for (; g < nloads; ++g) {
-                const uint32_t r = (uint32_t)(g % kRing), u = (uint32_t)(g / kRing);
-                if (u > 0 && !mbar_wait_or_stop(bar + BAR_LAND_FREE + r, (u - 1u) & 1u, s_stop)) {   // every staging warp has read the slot
+            int g = 0;        // copies started
+            const int nloads = HALVES * nitems;
+            RingPos<kRing> slot;
+            for (; g < nloads; ++g, slot.next()) {
+                const uint32_t r = slot.i;
+                if (!mbar_wait_or_stop(bar + BAR_LAND_FREE + r, slot.free(), s_stop)) {   // every staging warp has read the slot
                     ok = false;
                     break;
                 }
@@ -238,17 +241,18 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
             if (!ok && atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
             // copies started but possibly not landed yet: one more bounded wait each, so that the engine is not
             // left writing into shared memory that the next block of this SM may own
-            for (int64_t h = (g >= kRing ? g - kRing : 0); h < g; ++h)
+            for (int h = (g >= kRing ? g - kRing : 0); h < g; ++h)
                 mbar_wait(bar + BAR_LAND_FULL + (h % kRing), (uint32_t)(h / kRing) & 1u);
         }
     } else if (warp == kFlipWarp) {
         // ================= flip words: four generator calls per lane and item, 128 rows x 128 flips =================
         Cursor c = c_first;
         bool ok = true;
-        for (int64_t g = 0; g < nitems; ++g) {
-            const uint32_t b = (uint32_t)(g % kAcc), u = (uint32_t)(g / kAcc);
+        RingPos<kAcc> acc;
+        for (int g = 0; g < nitems; ++g, acc.next()) {
+            const uint32_t b = acc.i;
             // the drain of item g - kAcc has read its flip words (every warp reads them before it frees the accumulator)
-            if (u > 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, (u - 1u) & 1u, s_stop);
+            ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + b, acc.free(), s_stop);
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (!ok) break;
             const uint32_t id = p.id0 + (uint32_t)c.n, c0 = (uint32_t)(c.tile_base >> 7);
@@ -266,23 +270,25 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         if (!ok && lane == 0 && atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
     } else if (warp >= kFirstStageWarp && warp < kIssueWarp) {
         // ================= staging: landed tile -> H_4 over column bits 5, 6 -> operand buffer =================
-        const uint32_t st = (uint32_t)tid - kFirstStageWarp * 32u, sq = st & 3u;     // rows (st >> 2) + 8 kStageWarps i, column chunks sq + 4 t
-        const int64_t nloads = HALVES * nitems;
+        const uint32_t st = (uint32_t)tid - kFirstStageWarp * 32u, sq = st & 3u;     // column chunks sq + 4 t of rows row0 + 8 kStageWarps i
+        // The eight lanes of a 128-bit access have rows k and k + 4.  Reading, the two rows start 256 bytes multiples apart: the
+        // second one reads its chunks with column bit 5 swapped, so that together they cover all banks (its differences
+        // come out negated).  Writing, the operand's swizzle keeps the two apart.
+        const uint32_t odd = (st >> 2) & 1u, row0 = ((st >> 5) << 3) | (odd << 2) | ((st >> 3) & 3u), negate = odd ? 0x80008000u : 0u;
+        const int nloads = HALVES * nitems;
         bool ok = true;
-        for (int64_t g = 0; g < nloads; ++g) {
-            const uint32_t b = (uint32_t)g & 1u, u = (uint32_t)(g >> 1);
-            const uint32_t r = (uint32_t)(g % kRing), ur = (uint32_t)(g / kRing);
-            ok = mbar_wait_or_stop(bar + BAR_LAND_FULL + r, ur & 1u, s_stop);                              // the tile has landed
-            if (ok && u > 0) ok = mbar_wait_or_stop(bar + BAR_B_FREE + b, (u - 1u) & 1u, s_stop);          // product g - 2 has read the buffer
+        RingPos<kRing> slot;
+        RingPos<2> op;
+        for (int g = 0; g < nloads; ++g, slot.next(), op.next()) {
+            const uint32_t b = op.i, r = slot.i;
+            ok = mbar_wait_or_stop(bar + BAR_LAND_FULL + r, slot.full, s_stop);                            // the tile has landed
+            if (ok) ok = mbar_wait_or_stop(bar + BAR_B_FREE + b, op.free(), s_stop);                       // product g - 2 has read the buffer
             if (!ok) break;
 #pragma unroll
             for (int i = 0; i < 16 / kStageWarps; ++i) {
-                const uint32_t srow = (st >> 2) + 8u * kStageWarps * i;
+                const uint32_t srow = row0 + 8u * kStageWarps * i;
                 uint4 pre[4];
                 const unsigned char* const land = smem + kOffLand + r * kTileBytes + srow * 256u + sq * 16u;
-                // The eight lanes of a 128-bit access read two rows 256 bytes apart: odd rows read their chunks with
-                // column bit 5 swapped, so that the two cover all banks; their differences come out negated.
-                const uint32_t odd = (st >> 2) & 1u, negate = odd ? 0x80008000u : 0u;
 #pragma unroll
                 for (int t = 0; t < 4; ++t) pre[t] = *reinterpret_cast<const uint4*>(land + 64u * ((uint32_t)t ^ odd));
                 hbutterfly(pre[0], pre[1]);   // column bit 5
@@ -291,9 +297,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
                 pre[3] = make_uint4(pre[3].x ^ negate, pre[3].y ^ negate, pre[3].z ^ negate, pre[3].w ^ negate);
                 hbutterfly(pre[0], pre[2]);   // column bit 6
                 hbutterfly(pre[1], pre[3]);
-                unsigned char* const dst = smem + kOffB + b * kBBytes + sq * kBGroupStride + (srow >> 3) * 128u + (srow & 7u) * 16u;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) *reinterpret_cast<uint4*>(dst + 4 * t * kBGroupStride) = pre[t];
+                for (int t = 0; t < 4; ++t)
+                    *reinterpret_cast<uint4*>(smem + kOffB + b * kBBytes + (t >> 1) * kBBlock + swizzled_row_chunk(srow, sq + 4u * (t & 1))) = pre[t];
             }
             // One fence for both proxies' next accesses: the product reads the operand, the copy engine rewrites the slot.
             // (The slot is given back only here: freed right after the loads were issued, without a fence, it was
@@ -315,14 +321,15 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
         Cursor c_drain = c_first;
 
         // drain item g: accumulator -> registers, H_32 over the 32 columns, flip, add
-        auto drain_item = [&](int64_t g) -> bool {
-            const uint32_t b = (uint32_t)(g % kAcc), u = (uint32_t)(g / kAcc);
+        RingPos<kAcc> acc;
+        auto drain_item = [&]() -> bool {
+            const uint32_t b = acc.i;
             const int n = c_drain.n;
             const int64_t tile_base = c_drain.tile_base;
             advance(c_drain);
-            if (!mbar_wait_or_stop(bar + BAR_ACC_FULL + b, u & 1u, s_stop)) return false;
+            if (!mbar_wait_or_stop(bar + BAR_ACC_FULL + b, acc.full, s_stop)) return false;
             tc_fence_after_sync();
-            if (!mbar_wait_or_stop(bar + BAR_FLIPS + b, u & 1u, s_stop)) return false;
+            if (!mbar_wait_or_stop(bar + BAR_FLIPS + b, acc.full, s_stop)) return false;
             const uint32_t fw = reinterpret_cast<const uint32_t*>(smem + kOffFlips + b * 2048u)[cw * 128u + jrow];
             const float wamp = (p.amp_mode == AMP_WEIGHT) ? amplitude_at(p, n, tile_base) : 1.f;
             uint32_t raw[32];
@@ -363,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
 
 #pragma unroll
         for (int r = 0; r < 32; ++r) accv[r] = 0.f;
-        for (int64_t g = 0; g < nitems && ok; ++g) ok = drain_item(g);
+        for (int g = 0; g < nitems && ok; ++g, acc.next()) ok = drain_item();
         if (!ok && lane == 0 && atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tcrow_wait_timeouts, 1);
         if (n_step > 1) {
             // This block's share of the sums into the landing slots: every copy has landed and been read (the last
