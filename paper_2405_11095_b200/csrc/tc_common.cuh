@@ -70,14 +70,6 @@ struct RingPos {
     }
 };
 
-// sixteen 32-bit columns of this thread's lane
-__device__ __forceinline__ void tmem_store16(uint32_t taddr, const uint32_t (&w)[16])
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-                 ::"r"(taddr), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]),
-                   "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]) : "memory");
-}
-
 // 32 consecutive accumulator columns of this thread's lane.  The load is asynchronous: it and its wait
 // are one statement, so that the compiler never sees the destination registers as live while the load is
 // still in flight (a version that started the load earlier, underneath the staging of the next item, had

@@ -8,8 +8,8 @@
 //      kept non-negative by a bias (a + b, a - b + c), so no carry crosses a byte.
 //   2. H_128 over the low seven row bits is a 128 x 128 x 128 integer matrix product per value t'
 //      of the top bits: D_t'[j][n] = sum_k H_128[j][k] Z_t'[k][n] with 8-bit operands in shared
-//      memory (B = Z_t', the bytes as the expansion left them: n contiguous, i.e. MN-major, 128-byte swizzle)
-//      and tensor memory (A = H_128), and 32-bit accumulators in tensor memory: tcgen05.mma.kind::i8, four
+//      memory (A = H_128, K-major; B = Z_t', the bytes as the expansion left them: n contiguous,
+//      i.e. MN-major) and 32-bit accumulators in tensor memory: tcgen05.mma.kind::i8, four
 //      instructions of K = 32 per product, issued by one thread, completion through an mbarrier.
 //   3. The accumulators come back with tcgen05.ld (a thread = one output row j of a lane quarter,
 //      32 columns per load), become fp16 (all values are even integers of magnitude <= 1024) and
@@ -39,36 +39,34 @@ namespace {
 constexpr int kWorkerWarps = 16;
 constexpr int kWorkers = kWorkerWarps * 32;
 constexpr int kTcThreads = kWorkers + 32;
-constexpr int kAcc = 3;                                       // accumulators (128 columns of tensor memory each) in turn
-constexpr uint32_t kAColumns = 32;                            // H_128 as int8 in tensor memory: lane = row, four k per 32-bit column
-constexpr uint32_t kBOperandBytes = 128 * 128;                // rows k of 128 bytes, 128-byte swizzle
-constexpr uint32_t kOffB = 0;                                 // eight B operands
+constexpr uint32_t kBOperandBytes = 8 * 2064;                 // eight column groups of 16, 2048 B each + 16 B so that they sit on different banks
+constexpr uint32_t kOffA = 0;                                 // H_128 as int8, K-major core matrices: 16 KiB
+constexpr uint32_t kOffB = 16384;                             // eight B operands
 constexpr uint32_t kOffBits = kOffB + 8 * kBOperandBytes;     // the tile's packed rows: 1024 x 16 B
-constexpr uint32_t kOffBar = kOffBits + 16384;                // mbarriers, stop word, tensor-memory base address
+constexpr uint32_t kOffBar = kOffBits + 16384;                // eleven mbarriers, stop word, tensor-memory base address
 constexpr uint32_t kPatchPitch = 64;                          // bytes per row of a warp's output patch: 32 fp16; the 16-byte chunks of a row are
                                                               // permuted by (row >> 1) & 3, which keeps both the row-wise writes and the
                                                               // eight-rows-by-64-bytes reads off each other's banks
 constexpr uint32_t kOffPatch = kOffBar + 128;                 // one patch of 32 rows per worker warp
 constexpr uint32_t kTcSmemBytes = kOffPatch + kWorkerWarps * 32 * kPatchPitch;
 
-enum { BAR_B_FULL = 0, BAR_B_DONE = 1, BAR_BITS = 2, BAR_ACC_FULL = 3, BAR_ACC_FREE = 3 + kAcc };
+enum { BAR_B_FULL = 0, BAR_B_DONE = 1, BAR_ACC_FULL = 2, BAR_ACC_FREE = 6, BAR_BITS = 10 };
 
 // instruction descriptor: D = s32 (2 << 4), A = B = signed 8-bit (1 << 7, 1 << 10), A K-major, B MN-major
 // (1 << 16), N = 128 (N / 8 << 17), M = 128 (M / 16 << 24)
 constexpr uint32_t kIdescI8 = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (16u << 17) | (8u << 24);
 
-// A from tensor memory
-__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t accumulate)
+__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(kIdescI8), "r"(accumulate) : "memory");
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(kIdescI8), "r"(accumulate) : "memory");
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams p, const uint32_t ntiles)
+__global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams p, const int64_t ntiles)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     pdl_trigger();
@@ -80,6 +78,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
     uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffBar + 100);
 
     // ---- once per block: the constant operand, barriers, tensor memory ----
+    if (tid < kWorkers) {
+        // A[m][k] = (-1)^popcount(m & k): row m, 32 of its k per thread; core matrix = 8 rows x 16 bytes
+        const uint32_t m = (uint32_t)tid >> 2, kc0 = ((uint32_t)tid & 3u) * 2u;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            uint32_t w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                w[q] = 0;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const uint32_t k = (kc0 + c) * 16u + 4u * q + b;
+                    w[q] |= ((__popc(m & k) & 1) ? 0xFFu : 0x01u) << (8 * b);
+                }
+            }
+            *reinterpret_cast<uint4*>(smem + kOffA + (m & 7u) * 16u + (m >> 3) * 1024u + (kc0 + c) * 128u) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+    }
     if (warp == kWorkerWarps) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -89,59 +105,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
         mbar_init(bar + BAR_B_DONE, 1);
         mbar_init(bar + BAR_BITS, kWorkerWarps);
 #pragma unroll
-        for (int a = 0; a < kAcc; ++a) {
+        for (int a = 0; a < 4; ++a) {
             mbar_init(bar + BAR_ACC_FULL + a, 1);
             mbar_init(bar + BAR_ACC_FREE + a, kWorkerWarps);
         }
         *s_stop = 0;
     }
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    const uint32_t tmem_base = *tmem_slot;
-    const uint32_t tmem_a = tmem_base + kAcc * 128u;
-    if (warp < 4) {
-        // A[m][k] = (-1)^popcount(m & k): a warp writes the 32 rows of its lane quarter
-        const uint32_t m = (uint32_t)tid;
-        uint32_t w[16];
-#pragma unroll 1
-        for (uint32_t c0 = 0; c0 < kAColumns; c0 += 16) {
-#pragma unroll
-            for (uint32_t c = 0; c < 16; ++c) {
-                w[c] = 0;
-#pragma unroll
-                for (uint32_t b = 0; b < 4; ++b) w[c] |= ((__popc(m & (4u * (c0 + c) + b)) & 1) ? 0xFFu : 0x01u) << (8 * b);
-            }
-            tmem_store16(tmem_a + (((uint32_t)warp * 32u) << 16) + c0, w);
-        }
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    }
+    fence_generic_before_async();   // the constant operand, for the tensor core's reads
     pdl_wait();                     // (the set-up above needs nothing from the kernel before)
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
 
     const uint32_t step = 1u << p.lo_log;
-    const uint32_t total = ntiles * (uint32_t)p.nworkers;     // (at most 2^14 x 65535)
-    const int nitems = blockIdx.x < total ? (int)((total - blockIdx.x + gridDim.x - 1u) / gridDim.x) : 0;
+    const int64_t total = ntiles * p.nworkers;
+    const int64_t nitems = ((int64_t)blockIdx.x < total) ? (total - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
 
     if (warp == kWorkerWarps) {
         // ================= the warp that issues the products =================
         if (lane == 0) {
+            const uint64_t adesc = umma_desc(smem_u32(smem + kOffA), 128u, 1024u);
             bool ok = true;
             int64_t issued = 0;   // products committed so far (eight per tile)
-            RingPos<kAcc> acc;
-            for (int g = 0; g < nitems && ok; ++g) {
+            for (int64_t g = 0; g < nitems && ok; ++g) {
                 ok = mbar_wait_or_stop(bar + BAR_B_FULL, (uint32_t)g & 1u, s_stop);                 // the tile's eight operands are staged
-                for (int t = 0; t < 8 && ok; ++t, acc.next()) {
-                    ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + acc.i, acc.free(), s_stop);   // drained
+                for (int t = 0; t < 8 && ok; ++t) {
+                    const uint32_t a = (uint32_t)t & 3u, u = (uint32_t)(2 * g) + ((uint32_t)t >> 2);   // accumulator and how often it has been used
+                    if (u > 0) ok = mbar_wait_or_stop(bar + BAR_ACC_FREE + a, (u - 1u) & 1u, s_stop);   // drained
                     if (!ok) break;
                     tc_fence_after_sync();
-                    const uint64_t bdesc = umma_desc_mn128(smem_u32(smem + kOffB + (uint32_t)t * kBOperandBytes), kBOperandBytes, 1024u);
+                    const uint64_t bdesc = umma_desc(smem_u32(smem + kOffB + (uint32_t)t * kBOperandBytes), 128u, 2064u);
 #pragma unroll
-                    for (int ks = 0; ks < 4; ++ks)   // K = 32 per instruction: eight columns of A, four groups of eight rows of B
-                        umma_i8(tmem_base + acc.i * 128u, tmem_a + 8u * ks, bdesc + (uint64_t)(ks * (4096 >> 4)), ks > 0 ? 1u : 0u);
-                    umma_commit(bar + BAR_ACC_FULL + acc.i);
+                    for (int ks = 0; ks < 4; ++ks)   // K = 32 per instruction: two core matrices of A, four k-groups of B
+                        umma_i8(tmem_base + a * 128u, adesc + (uint64_t)(ks * (256 >> 4)), bdesc + (uint64_t)(ks * (512 >> 4)), ks > 0 ? 1u : 0u);
+                    umma_commit(bar + BAR_ACC_FULL + a);
                     ++issued;
                 }
                 if (ok) umma_commit(bar + BAR_B_DONE);
@@ -149,8 +147,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
             if (!ok) {
                 if (atomicExch((int*)s_stop, 1) == 0) atomicAdd(&g_tc_wait_timeouts, 1);
                 // products already committed may still be running: one more bounded wait each before the tensor memory goes back
-                for (int64_t h = (issued >= kAcc ? issued - kAcc : 0); h < issued; ++h)
-                    mbar_wait(bar + BAR_ACC_FULL + (h % kAcc), (uint32_t)(h / kAcc) & 1u);
+                for (int64_t h = (issued >= 4 ? issued - 4 : 0); h < issued; ++h)
+                    mbar_wait(bar + BAR_ACC_FULL + (h & 3), (uint32_t)(h >> 2) & 1u);
             }
         }
     } else {
@@ -162,15 +160,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
         unsigned char* const patch = smem + kOffPatch + (uint32_t)warp * 32u * kPatchPitch;
         bool ok = true;
 
-        auto tile_origin = [&](uint32_t item, int& n, uint32_t& i_tile) {
+        auto tile_origin = [&](int64_t item, int& n, uint32_t& i_tile) {
             n = (int)(item / ntiles);
-            const uint32_t tile = item - (uint32_t)n * ntiles;
+            const uint32_t tile = (uint32_t)(item % ntiles);
             const uint32_t col0 = (tile << 7) & (step - 1u);
             const uint32_t hi = (tile << 7) >> p.lo_log;
             i_tile = (hi << (p.lo_log + 10)) + col0;                        // row 0, column 0 of the tile
         };
         // this thread's two packed rows (tid and tid + 512) of an item: 16 bytes = 128 columns each
-        auto load_bits = [&](uint32_t item, uint4 (&w)[2]) {
+        auto load_bits = [&](int64_t item, uint4 (&w)[2]) {
             int n;
             uint32_t i_tile;
             tile_origin(item, n, i_tile);
@@ -179,11 +177,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
             for (int k = 0; k < 2; ++k) w[k] = load_ca(reinterpret_cast<const uint4*>(bits + ((i_tile + ((uint32_t)tid + 512u * k) * step) >> 5)));
         };
 
-        RingPos<kAcc> acc;
         uint4 next_bits[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
         if (nitems > 0) load_bits(blockIdx.x, next_bits);
-        for (int g = 0; g < nitems && ok; ++g) {
-            const uint32_t item = blockIdx.x + (uint32_t)g * gridDim.x;
+        for (int64_t g = 0; g < nitems && ok; ++g) {
+            const int64_t item = (int64_t)blockIdx.x + g * gridDim.x;
             int n;
             uint32_t i_tile;
             tile_origin(item, n, i_tile);
@@ -229,7 +226,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
                 }
 #pragma unroll
                 for (int t = 0; t < 8; ++t)
-                    *reinterpret_cast<uint4*>(smem + kOffB + (uint32_t)t * kBOperandBytes + swizzled_row_chunk(kr, cg)) =
+                    *reinterpret_cast<uint4*>(smem + kOffB + (uint32_t)t * kBOperandBytes + cg * 2064u + (kr >> 3) * 128u + (kr & 7u) * 16u) =
                         make_uint4(x[t][0], x[t][1], x[t][2], x[t][3]);
             }
             fence_generic_before_async();
@@ -239,9 +236,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_col_kernel(const PassParams 
             // ---- drain the eight accumulators: fp16 through the warp's patch to global memory ----
             __half* const dst = static_cast<__half*>(p.dst) + (int64_t)n * p.dst_stride + i_tile + cw * 32u;
 #pragma unroll 1
-            for (int t = 0; t < 8; ++t, acc.next()) {
-                const uint32_t a = acc.i;
-                if (!mbar_wait_or_stop(bar + BAR_ACC_FULL + a, acc.full, s_stop)) { ok = false; break; }
+            for (int t = 0; t < 8; ++t) {
+                const uint32_t a = (uint32_t)t & 3u, u = (uint32_t)(2 * g) + ((uint32_t)t >> 2);
+                if (!mbar_wait_or_stop(bar + BAR_ACC_FULL + a, u & 1u, s_stop)) { ok = false; break; }
                 tc_fence_after_sync();
                 uint32_t v[32];
                 tmem_load32(tmem_base + ((lq * 32u) << 16) + a * 128u + cw * 32u, v);
@@ -302,7 +299,7 @@ cudaError_t launch_tc_col(const PassParams& p, cudaStream_t s)
     const int64_t ntiles = p.dp >> 17;                        // 1024 rows x 128 columns each
     int64_t blocks = ntiles * p.nworkers;
     if (blocks > sms) blocks = sms;
-    return launch<tc_col_kernel>(dim3((unsigned)blocks), kTcThreads, kTcSmemBytes, s, 1, p, (uint32_t)ntiles);
+    return launch<tc_col_kernel>(dim3((unsigned)blocks), kTcThreads, kTcSmemBytes, s, 1, p, ntiles);
 }
 
 cudaError_t tc_timeouts(int* out) { return cudaMemcpyFromSymbol(out, g_tc_wait_timeouts, sizeof(int)); }

@@ -141,7 +141,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
                 const uint32_t lo = (__popc(m & k) & 1) ? 0xBC00u : 0x3C00u;
                 w[c] = lo | ((lo ^ ((m & 1u) << 15)) << 16);      // k + 1 differs from k in bit 0 alone
             }
-            tmem_store16(tmem_a + (((uint32_t)warp * 32u) << 16) + c0, w);
+            asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+                         ::"r"(tmem_a + (((uint32_t)warp * 32u) << 16) + c0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]),
+                           "r"(w[6]), "r"(w[7]), "r"(w[8]), "r"(w[9]), "r"(w[10]), "r"(w[11]), "r"(w[12]), "r"(w[13]), "r"(w[14]), "r"(w[15]) : "memory");
         }
         asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
