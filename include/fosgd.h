@@ -213,6 +213,15 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
                           float* lambda_s_dev, uint32_t* bits, void* ws, size_t ws_bytes, void* amp_ws,
                           size_t amp_ws_bytes, fosgd_stream stream);
 
+/* The same for one amplitude per worker and block of the blocked mode (block_log2 >= 5): fosgd_amplitudes with per_block = 1
+ * and fosgd_encode_dev in one call.  lambda_dev: [M][d' >> block_log2], lambda_s_dev: [d' >> block_log2] (nullable).  Where one
+ * thread block transforms a whole block of the gradient (2^10 .. 2^15), or the strided pass can carry the sums (2^16 .. 2^22,
+ * `ws` holding all M workers), the gradients are read once.  amp_ws: scratch of FOSGD_OP_BLOCK_AMPLITUDES. */
+int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_t worker_stride, int M, uint32_t worker_id0,
+                                 uint64_t seed, uint64_t step, double alpha, double alpha_s, int block_log2, float* lambda_dev,
+                                 float* lambda_s_dev, uint32_t* bits, void* ws, size_t ws_bytes, void* amp_ws,
+                                 size_t amp_ws_bytes, fosgd_stream stream);
+
 /* fosgd_decode without a scratch argument (the paper has no counterpart; it computes exactly
  * what fosgd_decode computes).  For callers that must not allocate device memory where they
  * decode (no allocator reachable from their code, cudaMalloc banned because it synchronises,

@@ -28,7 +28,7 @@ EXPORTS = ("fosgd_padded_dim", "fosgd_planes", "fosgd_lambda", "fosgd_lambda_ser
            "fosgd_trace_label", "fosgd_decode_noalloc", "fosgd_async_timeouts", "fosgd_amplitudes",
            "fosgd_encode_dev", "fosgd_server_aggregate_dev", "fosgd_downlink_decode_dev", "fosgd_downlink_apply",
            "fosgd_downlink_encode", "fosgd_probe_issue_rate", "fosgd_set_tensor_core_pass",
-           "fosgd_set_fused_encoder", "fosgd_encode_measured")
+           "fosgd_set_fused_encoder", "fosgd_encode_measured", "fosgd_encode_measured_blocks")
 
 
 class FosgdError(RuntimeError):
@@ -72,6 +72,7 @@ def _load() -> C.CDLL:
     L.fosgd_set_tensor_core_pass.argtypes, L.fosgd_set_tensor_core_pass.restype = [cint], cint
     L.fosgd_set_fused_encoder.argtypes, L.fosgd_set_fused_encoder.restype = [cint], cint
     L.fosgd_encode_measured.argtypes = [vp, cint, i64, i64, cint, u32, u64, u64, dbl, dbl, cint, vp, vp, vp, vp, sz, vp, sz, vp]
+    L.fosgd_encode_measured_blocks.argtypes = L.fosgd_encode_measured.argtypes
     L.fosgd_strerror.argtypes, L.fosgd_strerror.restype = [cint], C.c_char_p
     L.fosgd_last_cuda_error.restype = cint
     L.fosgd_version.restype = C.c_char_p
@@ -111,7 +112,7 @@ _calls = None      # the native module, once it is bound to the loaded library
 # order of the function table of csrc/binding.c
 _NATIVE_FUNCTIONS = ("fosgd_encode", "fosgd_flatten", "fosgd_decode", "fosgd_server_aggregate", "fosgd_downlink_decode",
                      "fosgd_amplitudes", "fosgd_encode_dev", "fosgd_server_aggregate_dev", "fosgd_downlink_decode_dev",
-                     "fosgd_downlink_encode", "fosgd_downlink_apply", "fosgd_encode_measured")
+                     "fosgd_downlink_encode", "fosgd_downlink_apply", "fosgd_encode_measured", "fosgd_encode_measured_blocks")
 
 
 def _bind():
@@ -266,6 +267,17 @@ def encode_measured(grads, d, bits, lam, lam_s, seed, step, alpha=2.0, alpha_s=2
                                             ws, amp_ws, worker_stride)
     if st:
         _failed(st, "fosgd_encode_measured", grads)
+    return bits
+
+
+def encode_measured_blocks(grads, d, bits, lam, lam_s, seed, step, alpha=2.0, alpha_s=2.0, worker_id0=0, block_log2=0,
+                           ws=None, amp_ws=None, worker_stride=None):
+    """fosgd_encode_measured_blocks: amplitudes(..., per_block=True) and encode_dev(..., per_block=True) in one call;
+    the gradients are read once where the encoder can carry the norms.  lam: [M, d' >> b], lam_s: [d' >> b]."""
+    st = (_calls or _bind()).encode_measured_blocks(grads, d, bits, lam, lam_s, seed, step, alpha, alpha_s, worker_id0,
+                                                   block_log2, ws, amp_ws, worker_stride)
+    if st:
+        _failed(st, "fosgd_encode_measured_blocks", grads)
     return bits
 
 

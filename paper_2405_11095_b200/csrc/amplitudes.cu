@@ -14,7 +14,6 @@
 namespace fosgd {
 
 constexpr int kNormBlocks = 256;
-constexpr float kMinBlockAmplitude = 1e-30f;
 
 template <bool BF16>
 __global__ void __launch_bounds__(256) sumsq_partial_kernel(const void* grads, int64_t d, int64_t worker_stride, double* partial)
@@ -162,8 +161,6 @@ __global__ void __launch_bounds__(128) block_amplitudes_kernel(const double* seg
     for (int64_t k = lane; k < segs_per_block; k += 32) acc += row[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-    // floor: a block of zeros keeps a positive amplitude, so that its sign bits are still
-    // decided by the dither (and decode to ~0) instead of by the sign of a zero
     if (lane == 0) lam[w] = fmaxf((float)(alpha * sqrt(acc) * sqrt(log(n_eff) / n_eff)), kMinBlockAmplitude);
 }
 
@@ -184,16 +181,27 @@ cudaError_t launch_block_amplitudes(const void* grads, int bf16, int64_t d, int6
 {
     const int s = block_log2 < 10 ? block_log2 : 10;
     const int64_t nb = dp >> block_log2;
-    const double n_eff = (double)((int64_t)1 << block_log2);
     const dim3 grid((unsigned)((dp + 4095) >> 12), (unsigned)M);
     cudaError_t e = bf16 ? launch<segment_sumsq_kernel<true>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg)
                          : launch<segment_sumsq_kernel<false>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg);
     if (e != cudaSuccess) return e;
+    return launch_block_amplitudes_finalize(seg, (int64_t)1 << (block_log2 - s), nb, M, block_log2, alpha, alpha_s, lam, lam_s, st);
+}
+
+cudaError_t launch_block_amplitudes_finalize(const double* seg, int64_t parts, int64_t nb, int M, int block_log2, double alpha,
+                                             double alpha_s, float* lam, float* lam_s, cudaStream_t st)
+{
     const int64_t warps = nb * M;
-    e = launch<block_amplitudes_kernel>(dim3((unsigned)((warps + 3) / 4)), 128, 0, st, 1, (const double*)seg, nb,
-                                        (int64_t)1 << (block_log2 - s), M, alpha, n_eff, lam);
+    const cudaError_t e = launch<block_amplitudes_kernel>(dim3((unsigned)((warps + 3) / 4)), 128, 0, st, 1, seg, nb, parts, M, alpha,
+                                                          (double)((int64_t)1 << block_log2), lam);
     if (e != cudaSuccess || lam_s == nullptr) return e;
-    return launch<server_block_amplitudes_kernel>(dim3((unsigned)((nb + 127) / 128)), 128, 0, st, 1, (const float*)lam, nb, M, alpha_s, n_eff, lam_s);
+    return launch_server_amplitudes(lam, nb, M, block_log2, alpha_s, lam_s, st);
+}
+
+cudaError_t launch_server_amplitudes(const float* lam, int64_t nb, int M, int block_log2, double alpha_s, float* lam_s, cudaStream_t st)
+{
+    return launch<server_block_amplitudes_kernel>(dim3((unsigned)((nb + 127) / 128)), 128, 0, st, 1, lam, nb, M, alpha_s,
+                                                  (double)((int64_t)1 << block_log2), lam_s);
 }
 
 cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t worker_stride, int M, double alpha,

@@ -13,7 +13,7 @@
 #include "../../include/fosgd.h"
 
 enum { FN_ENCODE, FN_FLATTEN, FN_DECODE, FN_AGGREGATE, FN_DOWN_DECODE, FN_AMPLITUDES, FN_ENCODE_DEV, FN_AGGREGATE_DEV,
-       FN_DOWN_DECODE_DEV, FN_DOWN_ENCODE, FN_DOWN_APPLY, FN_ENCODE_MEASURED, FN_COUNT };
+       FN_DOWN_DECODE_DEV, FN_DOWN_ENCODE, FN_DOWN_APPLY, FN_ENCODE_MEASURED, FN_ENCODE_MEASURED_BLOCKS, FN_COUNT };
 
 static void* g_fn[FN_COUNT];
 static PyObject *g_get_device, *g_get_stream, *g_float32, *g_bfloat16;
@@ -310,7 +310,7 @@ CALLABLE(encode_dev)
 }
 
 /* grads d bits lam lam_s seed step alpha alpha_s worker_id0 block_log2 ws amp_ws worker_stride */
-CALLABLE(encode_measured)
+static PyObject* measured(PyObject* const* a, Py_ssize_t n, int fn)
 {
     ENTER(14)
     const int64_t d = I64(1);
@@ -327,8 +327,11 @@ CALLABLE(encode_measured)
     void* const aws = PTR(12);
     const size_t awsn = nbytes(c, a[12]);
     const fosgd_stream s = stream(c);
-    CALL(FN(FN_ENCODE_MEASURED, fosgd_encode_measured)(g.p, g.dtype, d, g.stride, g.M, id0, seed, step, alpha, alpha_s, b, lam, lam_s, bits, ws, wsn, aws, awsn, s))
+    CALL(FN(fn, fosgd_encode_measured)(g.p, g.dtype, d, g.stride, g.M, id0, seed, step, alpha, alpha_s, b, lam, lam_s, bits, ws, wsn, aws, awsn, s))
 }
+
+CALLABLE(encode_measured) { return measured(a, n, FN_ENCODE_MEASURED); }
+CALLABLE(encode_measured_blocks) { return measured(a, n, FN_ENCODE_MEASURED_BLOCKS); }
 
 /* addresses (a tuple in the order of FN_*), current-device function, current-stream function, float32, bfloat16 */
 CALLABLE(bind)
@@ -357,7 +360,7 @@ CALLABLE(bind)
 static PyMethodDef methods[] = {METHOD(bind), METHOD(encode), METHOD(flatten), METHOD(decode), METHOD(server_aggregate),
                                 METHOD(server_aggregate_dev), METHOD(downlink_decode), METHOD(downlink_decode_dev),
                                 METHOD(downlink_encode), METHOD(downlink_apply), METHOD(amplitudes), METHOD(encode_dev),
-                                METHOD(encode_measured), {NULL, NULL, 0, NULL}};
+                                METHOD(encode_measured), METHOD(encode_measured_blocks), {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", NULL, -1, methods, NULL, NULL, NULL, NULL};
 
 PyMODINIT_FUNC PyInit__native(void)

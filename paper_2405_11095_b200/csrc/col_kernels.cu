@@ -86,8 +86,9 @@ __device__ __forceinline__ void planes_to_values(const PassParams& p, float (&v)
 }
 
 // ---- A <= 4 -----------------------------------------------------------------------------
-template <int A, int SRC>
-__global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
+// NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
+template <int A, int SRC, bool NORM>
+__global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, double* const partial)
 {
     constexpr int R = 1 << A;
     pdl_begin();
@@ -115,6 +116,21 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p)
         if (SRC == SRC_G32 || SRC == SRC_G16) {
 #pragma unroll
             for (int r = 0; r < R; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
+        }
+    }
+    if constexpr (NORM) {
+        __shared__ double wsum[8];
+        float sq = 0.f;
+#pragma unroll
+        for (int r = 0; r < R; ++r) sq = fmaf(v[r], v[r], sq);
+        double sum = (double)sq;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        if (lane == 0) wsum[threadIdx.x >> 5] = sum;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int k = 1; k < 8; ++k) sum += wsum[k];
+            partial[(int64_t)n * gridDim.x + blockIdx.x] = sum;
         }
     }
 #pragma unroll
@@ -509,6 +525,33 @@ cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStr
     return launch<col4_norm_kernel>(dim3((unsigned)(nruns * p.nworkers)), 512, Col4::SMEM_BYTES, s, 1, p, map, (int)nruns, (uint32_t)rows, partial);
 }
 
+template <int SRC>
+static cudaError_t launch_col_block_norm_src(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int64_t* parts)
+{
+    *launched = true;
+    if (A == 4) {
+        *parts = (p.dp >> A) / 256;
+        return launch<col_small_kernel<4, SRC, true>>(dim3((unsigned)*parts, (unsigned)p.nworkers), 256, 0, s, 1, p, partial);
+    }
+    *parts = (p.dp >> A) / 64;
+    switch (A) {
+        case 5: return launch_col2<5, SRC, true>(p, (uint32_t)*parts, partial, s);
+        case 6: return launch_col2<6, SRC, true>(p, (uint32_t)*parts, partial, s);
+        case 7: return launch_col2<7, SRC, true>(p, (uint32_t)*parts, partial, s);
+        case 8: return launch_col2<8, SRC, true>(p, (uint32_t)*parts, partial, s);
+    }
+    *launched = false;
+    return cudaSuccess;
+}
+
+// Tiles never span two transforms and a transform's tiles are numbered one after the other, so a block's sums are
+// adjacent.  (At most one sum per 2^11 coordinates: what the scratch of the separate norm pass holds twice over.)
+cudaError_t launch_col_block_norm(int A, int src, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int64_t* parts_per_worker)
+{
+    return src == SRC_G16 ? launch_col_block_norm_src<SRC_G16>(A, p, partial, s, launched, parts_per_worker)
+                          : launch_col_block_norm_src<SRC_G32>(A, p, partial, s, launched, parts_per_worker);
+}
+
 // ---- packed source, fp16 arithmetic ------------------------------------------------------------
 // A decoder's first pass starts from 2 c - K (one plane: +-1), and after A stages every value is an integer of
 // magnitude <= K 2^A, which fp16 holds exactly up to 2048.  So this variant keeps two adjacent columns per
@@ -707,7 +750,7 @@ template <int A, int SRC>
 static cudaError_t launch_col_one(const PassParams& p, cudaStream_t s)
 {
     if constexpr (A <= 4) {
-        return launch<col_small_kernel<A, SRC>>(dim3((unsigned)((p.dp >> A) / 256), (unsigned)p.nworkers), 256, 0, s, 1, p);
+        return launch<col_small_kernel<A, SRC, false>>(dim3((unsigned)((p.dp >> A) / 256), (unsigned)p.nworkers), 256, 0, s, 1, p, nullptr);
     } else if constexpr (A <= 8) {
         return launch_col2<A, SRC, false>(p, (uint32_t)((p.dp >> A) / 64), nullptr, s);
     } else if constexpr (A == 9) {

@@ -57,6 +57,10 @@ struct PassParams {
     int64_t amp_stride;
     int amp_shift;
     int amp_mode;        // AMP_DITHER, AMP_SCALE or AMP_WEIGHT
+    // Single-pass encoder that measures its own amplitudes (a block of the blocked mode is one tile): worker n's block k
+    // gets amp_out[n * amp_stride + k] = max(amp_factor * norm of the block, kMinBlockAmplitude).  Null otherwise.
+    float* amp_out;
+    double amp_factor;
     Rng rng;
 };
 
@@ -65,6 +69,10 @@ enum AmpMode {
     AMP_SCALE = 1,   // SINK_FINAL multiplies its scale by worker 0's entry (one amplitude for all workers)
     AMP_WEIGHT = 2   // SINK_FINAL weights every worker's contribution by that worker's entry
 };
+
+// floor of a measured block amplitude: a block of zeros keeps a positive one, so that its sign bits are still decided by
+// the dither (and decode to ~0) instead of by the sign of a zero
+constexpr float kMinBlockAmplitude = 1e-30f;
 
 // The parameter block of the kernels with a dither sink: PassParams plus the ten round keys of the
 // generator (Weyl sequence of the key), computed once on the host.  As kernel parameters they sit in
@@ -441,6 +449,13 @@ cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t wo
 cudaError_t launch_amplitudes_finalize(const double* partial, int M, int nparts, double alpha, double alpha_s, double n_eff,
                                        float* lam, float* lam_s, cudaStream_t s);
 cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nparts_out);
+// strided pass that also leaves every tile's sum of squares in partial[worker][tile]; *launched stays false where no kernel
+// carries them
+cudaError_t launch_col_block_norm(int A, int src, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int64_t* parts_per_worker);
+// block amplitudes from sums of squares ([M * nb][parts]); lam == nullptr: the server's from finished lam_in alone
+cudaError_t launch_block_amplitudes_finalize(const double* seg, int64_t parts, int64_t nb, int M, int block_log2, double alpha,
+                                             double alpha_s, float* lam, float* lam_s, cudaStream_t st);
+cudaError_t launch_server_amplitudes(const float* lam, int64_t nb, int M, int block_log2, double alpha_s, float* lam_s, cudaStream_t st);
 cudaError_t launch_block_amplitudes(const void* grads, int bf16, int64_t d, int64_t dp, int64_t worker_stride, int M,
                                     int block_log2, double alpha, double alpha_s, float* lam, float* lam_s,
                                     double* seg, cudaStream_t st);

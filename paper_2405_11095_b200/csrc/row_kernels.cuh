@@ -424,6 +424,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
     // SINK_FINAL: the blocks of a cluster (gridDim.y of them, one if the tiles alone fill the chip) take the
     // workers in turn and add up their sums at the end
     constexpr bool kLoopWorkers = (SINK == SINK_FINAL);
+    constexpr bool kMeasures = (SRC == SRC_G32 || SRC == SRC_G16) && SINK == SINK_PACK1;
     constexpr bool kFlips = (SRC == SRC_G32 || SRC == SRC_G16 || SINK == SINK_FINAL || SINK == SINK_SINGLE);
     const int n_begin = (int)blockIdx.y;
     const int n_end = kLoopWorkers ? p.nworkers : n_begin + 1;
@@ -462,6 +463,29 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
 
         float v[32];
         load_source<T, SRC, kLoopWorkers>(p, n, tile_base, baseF, fw, v);   // (uplink planes come one to a worker)
+        if constexpr (kMeasures) {
+            if (p.amp_out != nullptr) {
+                // the tile is a whole block: its norm (fp32 within a thread, fp64 across threads, fixed order) sets its
+                // amplitude (readers are behind the barrier of the exchange rounds)
+                __shared__ double wsum[C::NT / 32];
+                float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                for (int r = 0; r < 32; r += 2) {
+                    s0 = fmaf(v[r], v[r], s0);
+                    s1 = fmaf(v[r + 1], v[r + 1], s1);
+                }
+                double sum = (double)(s0 + s1);
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+                if (lane == 0) wsum[tid >> 5] = sum;
+                __syncthreads();
+                if (tid == 0) {
+                    for (int k = 1; k < C::NT / 32; ++k) sum += wsum[k];
+                    s_amp = fmaxf((float)(p.amp_factor * sqrt(sum)), kMinBlockAmplitude);
+                    p.amp_out[(int64_t)n * p.amp_stride + blockIdx.x] = s_amp;
+                }
+            }
+        }
         butterflies32<31>(v);
         store_round_F<T>(smem, baseF, v);
         __syncthreads();

@@ -65,11 +65,12 @@ def round_trip(codec, grads, d, buf: RoundTripBuffers, lam, lam_s, seed, step, *
     final_down = buf.down if world == 1 else None
     dev_amp = amps is not None
     pb = dev_amp and amps.per_block
-    # one amplitude for all workers, one rank, all workers resident: the encoder measures the norms itself
-    # (fosgd_encode_measured reads the gradients once where its first pass can carry the sums)
-    measured_encode = (dev_amp and not amps.per_block and world == 1 and chunks == 1 and encode_streams <= 1
-                       and hasattr(codec, "encode_measured"))
-    if dev_amp and not measured_encode:
+    # one rank, all workers resident: the encoder measures the norms itself
+    # (fosgd_encode_measured and _blocks read the gradients once where the encoder can carry the sums)
+    measured_encode = None
+    if dev_amp and world == 1 and chunks == 1 and encode_streams <= 1:
+        measured_encode = getattr(codec, "encode_measured_blocks" if pb else "encode_measured", None)
+    if dev_amp and measured_encode is None:
         # every distinct gradient is a row of `grads` (streamed workers cycle through the rows)
         codec.amplitudes(grads, d, amps.lam, amps.lam_s, alpha=amps.alpha, alpha_s=amps.alpha_s,
                          block_log2=block_log2, per_block=pb, ws=amps.ws, worker_stride=worker_stride)
@@ -85,10 +86,10 @@ def round_trip(codec, grads, d, buf: RoundTripBuffers, lam, lam_s, seed, step, *
         if encode_streams > 1 and rows >= encode_streams:
             _encode_on_streams(codec, grads, d, buf, lam, seed, step, first, block_log2, worker_stride,
                                amps, encode_streams)
-        elif measured_encode:
-            codec.encode_measured(grads, d, buf.bits, amps.lam, amps.lam_s, seed, step, alpha=amps.alpha,
-                                  alpha_s=amps.alpha_s, worker_id0=first, block_log2=block_log2, ws=buf.ws,
-                                  amp_ws=amps.ws, worker_stride=worker_stride)
+        elif measured_encode is not None:
+            measured_encode(grads, d, buf.bits, amps.lam, amps.lam_s, seed, step, alpha=amps.alpha, alpha_s=amps.alpha_s,
+                            worker_id0=first, block_log2=block_log2, ws=buf.ws, amp_ws=amps.ws,
+                            worker_stride=worker_stride)
         elif dev_amp:
             codec.encode_dev(grads, d, buf.bits, amps.lam, seed, step, worker_id0=first, block_log2=block_log2,
                              per_block=pb, ws=buf.ws, worker_stride=worker_stride)
