@@ -652,6 +652,8 @@ int fosgd_downlink_apply(const uint32_t* down_bits, int64_t d, uint64_t seed, ui
     return downlink_impl(down_bits, d, seed, step, lam_s, K, block_log2, x, ws, ws_bytes, stream, -(double)step_size);
 }
 
+static double block_amplitude_factor(double alpha, int L) { return alpha * sqrt(log((double)((int64_t)1 << L)) / (double)((int64_t)1 << L)); }
+
 int fosgd_amplitudes(const void* grads, int dtype, int64_t d, int64_t worker_stride, int M, double alpha,
                      double alpha_s, int block_log2, int per_block, float* lambda_dev, float* lambda_s_dev,
                      void* ws, size_t ws_bytes, fosgd_stream stream)
@@ -670,7 +672,16 @@ int fosgd_amplitudes(const void* grads, int dtype, int64_t d, int64_t worker_str
     if (!aligned16(ws)) return FOSGD_EALIGN;
     const bool on = g_trace_events != nullptr && g_trace_count < g_trace_capacity && g_trace_count < kTraceMax;
     if (on) cudaEventRecord(g_trace_events[2 * g_trace_count], (cudaStream_t)stream);
-    const cudaError_t e =
+    cudaError_t e;
+    if (per_block && block_log2 >= 10 && block_log2 <= 15) {
+        // a block is a tile: the same sums, in the same order, as the encoder that measures its own blocks
+        PassParams p{};
+        p.src = grads; p.src_stride = worker_stride; p.d = d; p.dp = g.dp; p.nworkers = M;
+        p.amp_out = lambda_dev; p.amp_stride = g.dp >> block_log2; p.amp_factor = block_amplitude_factor(alpha, block_log2);
+        e = launch_row(block_log2, dtype == FOSGD_BF16 ? SRC_G16 : SRC_G32, SINK_NORM, p, (cudaStream_t)stream);
+        if (e == cudaSuccess && lambda_s_dev != nullptr)
+            e = launch_server_amplitudes(lambda_dev, p.amp_stride, M, block_log2, alpha_s, lambda_s_dev, (cudaStream_t)stream);
+    } else e =
         per_block ? launch_block_amplitudes(grads, dtype == FOSGD_BF16, d, g.dp, worker_stride, M, block_log2, alpha,
                                             alpha_s, lambda_dev, lambda_s_dev, static_cast<double*>(ws),
                                             (cudaStream_t)stream)
@@ -772,7 +783,7 @@ int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_
         p.dst = bits; p.dst_stride = g.dp >> 5;
         p.amp_dev = nullptr;
         p.amp_out = lambda_dev;
-        p.amp_factor = alpha * sqrt(log((double)((int64_t)1 << g.L)) / (double)((int64_t)1 << g.L));
+        p.amp_factor = block_amplitude_factor(alpha, g.L);
         e = traced('r', pl.T, src, SINK_PACK1, p, s);
         if (e == cudaSuccess && lambda_s_dev != nullptr) {
             const bool on = trace_begin(s);

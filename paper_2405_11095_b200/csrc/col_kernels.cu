@@ -183,31 +183,47 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
 #pragma unroll
             for (int r = 0; r < 16; ++r) { v[2 * r] = u[r]; v[2 * r + 1] = u[16 + r]; }
         } else if constexpr (kGrad) {
-            auto load2 = [&](uint32_t i, float& x0, float& x1) {
-                if constexpr (SRC == SRC_G32) {
-                    const float2 q = load_cs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i));
-                    x0 = q.x; x1 = q.y;
-                } else {
-                    const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i));
-                    x0 = __uint_as_float(q << 16); x1 = __uint_as_float(q & 0xFFFF0000u);
-                }
-            };
             // a tile whose last coordinate is inside the gradient: all sixteen loads in flight, no checks
-            if (i_tile + ((1u << A) - 1u) * step + 63u < d32) {
+            const bool whole = i_tile + ((1u << A) - 1u) * step + 63u < d32;
+            if constexpr (SRC == SRC_G32) {
+                auto load2 = [&](int r) {
+                    const float2 q = load_cs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f));
+                    v[2 * r] = q.x; v[2 * r + 1] = q.y;
+                };
+                if (whole) {
 #pragma unroll
-                for (int r = 0; r < 16; ++r) load2(i_f + r * step_f, v[2 * r], v[2 * r + 1]);
+                    for (int r = 0; r < 16; ++r) load2(r);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) {
+                        v[2 * r] = v[2 * r + 1] = 0.f;
+                        if (i_f + r * step_f + 1u < d32) load2(r);
+                    }
+                }
             } else {
+                // raw pairs first: widening each one where it is loaded would make the checked loads wait for one another
+                // (2^32 padded coordinates, seven stages, 61% of the rows inside the gradient: 5.34 ms so)
+                uint32_t q[16];
+                auto load2 = [&](int r) { return load_cs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i_f + r * step_f)); };
+                if (whole) {
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) q[r] = load2(r);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) {
+                        q[r] = 0u;
+                        if (i_f + r * step_f + 1u < d32) q[r] = load2(r);
+                    }
+                }
 #pragma unroll
                 for (int r = 0; r < 16; ++r) {
-                    const uint32_t i = i_f + r * step_f;
-                    v[2 * r] = v[2 * r + 1] = 0.f;
-                    if (i + 1u < d32) load2(i, v[2 * r], v[2 * r + 1]);
+                    v[2 * r] = __uint_as_float(q[r] << 16); v[2 * r + 1] = __uint_as_float(q[r] & 0xFFFF0000u);
                 }
-                if (d32 & 1u) {       // an odd length ends inside a pair
+            }
+            if (!whole && (d32 & 1u)) {       // an odd length ends inside a pair
 #pragma unroll
-                    for (int r = 0; r < 16; ++r)
-                        if (i_f + r * step_f + 1u == d32) v[2 * r] = col_load<SRC>(p, wsrc, d32 - 1u, d32);
-                }
+                for (int r = 0; r < 16; ++r)
+                    if (i_f + r * step_f + 1u == d32) v[2 * r] = col_load<SRC>(p, wsrc, d32 - 1u, d32);
             }
             const uint32_t mine = eps_word(p.rng, p.id0 + (uint32_t)n, iw >> 5);
             const uint32_t sh = 31u - bit;

@@ -26,7 +26,8 @@ enum Sink : int {
     SINK_PACK1 = 1,  // dither + sign + pack, K = 1
     SINK_PACKK = 2,  // K dithers, count, P bit planes
     SINK_FINAL = 3,  // flip, sum over the workers of the launch, optional read-modify-write, scale
-    SINK_SINGLE = 4  // SINK_FINAL of a launch with one worker: no sums kept in registers
+    SINK_SINGLE = 4, // SINK_FINAL of a launch with one worker: no sums kept in registers
+    SINK_NORM = 6    // no transform: the amplitudes of blocks of one tile each (amp_out)
 };
 
 struct Rng {

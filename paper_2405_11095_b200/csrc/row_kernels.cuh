@@ -262,6 +262,109 @@ __device__ __forceinline__ void split_final_store(const PassParams& p, int64_t t
 }
 
 // ---- round F's registers from memory ----------------------------------------------------------
+// A tile of the gradient, zeros beyond its end.  WHOLE: the end lies elsewhere.  bf16 is widened after the last load:
+// behind the bounds checks each widening would otherwise make the next load wait.
+template <int T, int SRC, bool WHOLE>
+__device__ __forceinline__ void load_gradient_tile(const PassParams& p, int n, int64_t i0, float (&v)[32])
+{
+    constexpr int VB = RowCfg<T>::VB, VN = 1 << VB, NG = 32 >> VB;
+    const int64_t left = p.d - i0;    // valid elements from this thread's first coordinate on
+    if constexpr (SRC == SRC_G32) {
+        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            const int o = round_F_offset<T>(g);
+            float* const x = v + g * VN;
+            if (WHOLE || o + VN <= left) {
+                if constexpr (VB == 2) {
+                    const float4 q = load_cs(reinterpret_cast<const float4*>(src + o));
+                    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+                } else if constexpr (VB == 1) {
+                    const float2 q = load_cs(reinterpret_cast<const float2*>(src + o));
+                    x[0] = q.x; x[1] = q.y;
+                } else {
+                    x[0] = load_cs(src + o);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < VN; ++k) x[k] = (o + k < left) ? src[o + k] : 0.f;
+            }
+        }
+    } else {
+        const uint16_t* const src = static_cast<const uint16_t*>(p.src) + (int64_t)n * p.src_stride + i0;
+        constexpr int NW = VB == 2 ? 2 : 1;     // 32-bit words of a group
+        uint32_t q[NG * NW];
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            const int o = round_F_offset<T>(g);
+            uint32_t* const x = q + g * NW;
+            if (WHOLE || o + VN <= left) {
+                if constexpr (VB == 2) {
+                    const uint2 two = load_cs(reinterpret_cast<const uint2*>(src + o));
+                    x[0] = two.x; x[1] = two.y;
+                } else if constexpr (VB == 1) {
+                    x[0] = load_cs(reinterpret_cast<const uint32_t*>(src + o));
+                } else {
+                    x[0] = load_cs(src + o);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < NW; ++k) x[k] = 0u;
+#pragma unroll
+                for (int k = 0; k < VN; ++k)
+                    if (o + k < left) x[k >> 1] |= (uint32_t)src[o + k] << (16 * (k & 1));
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+            const uint32_t w = VB == 0 ? q[r] : q[r >> 1];
+            v[r] = __uint_as_float((VB > 0 && (r & 1)) ? w & 0xFFFF0000u : w << 16);
+        }
+    }
+}
+
+template <int T, int SRC>
+__device__ __forceinline__ void load_gradient(const PassParams& p, int n, int64_t tile_base, int baseF, float (&v)[32])
+{
+    if (tile_base + ((int64_t)1 << T) <= p.d) load_gradient_tile<T, SRC, true>(p, n, tile_base + baseF, v);
+    else load_gradient_tile<T, SRC, false>(p, n, tile_base + baseF, v);
+}
+
+// The tile is a whole block of the gradient: its norm sets the block's amplitude, in *s_amp after the next barrier and in
+// the table.  One order of the sum for every caller: fp32 within a thread, fp64 across threads.
+template <int T>
+__device__ __forceinline__ void measure_block(const PassParams& p, int n, int tid, const float (&v)[32], float* s_amp)
+{
+    __shared__ double wsum[RowCfg<T>::NT / 32];
+    float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < 32; r += 2) {
+        s0 = fmaf(v[r], v[r], s0);
+        s1 = fmaf(v[r + 1], v[r + 1], s1);
+    }
+    double sum = (double)(s0 + s1);
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    if ((tid & 31) == 0) wsum[tid >> 5] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        for (int k = 1; k < RowCfg<T>::NT / 32; ++k) sum += wsum[k];
+        *s_amp = fmaxf((float)(p.amp_factor * sqrt(sum)), kMinBlockAmplitude);
+        p.amp_out[(int64_t)n * p.amp_stride + blockIdx.x] = *s_amp;
+    }
+}
+
+// the amplitudes alone, for the callers whose encoder does not measure them
+template <int T, int SRC>
+__global__ void __launch_bounds__(1 << (T - 5), 1 << (15 - T)) row_norm_kernel(const PassParams p)
+{
+    __shared__ float s_amp;
+    pdl_begin();
+    float v[32];
+    load_gradient<T, SRC>(p, blockIdx.y, (int64_t)blockIdx.x << T, deposit<RowCfg<T>::FMASK, T>(threadIdx.x), v);
+    measure_block<T>(p, blockIdx.y, threadIdx.x, v, &s_amp);
+}
+
 // fw: flip words of the tile (gradient sources).  ONE_PLANE: a packed source known to have a single plane.
 template <int T, int SRC, bool ONE_PLANE = false>
 __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t tile_base, int baseF, const uint32_t* fw,
@@ -291,49 +394,8 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
             v[2 * g] = second ? a.x - b.x : a.x + b.x;
             v[2 * g + 1] = second ? a.y - b.y : a.y + b.y;
         }
-    } else if constexpr (SRC == SRC_G32) {
-        const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
-        const int64_t left = p.d - i0;    // valid elements from this thread's first coordinate on
-#pragma unroll
-        for (int g = 0; g < (32 >> VB); ++g) {
-            const int o = round_F_offset<T>(g);
-            float* const x = v + g * VN;
-            if (o + VN <= left) {
-                if constexpr (VB == 2) {
-                    const float4 q = load_cs(reinterpret_cast<const float4*>(src + o));
-                    x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-                } else if constexpr (VB == 1) {
-                    const float2 q = load_cs(reinterpret_cast<const float2*>(src + o));
-                    x[0] = q.x; x[1] = q.y;
-                } else {
-                    x[0] = load_cs(src + o);
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < VN; ++k) x[k] = (o + k < left) ? src[o + k] : 0.f;
-            }
-        }
-    } else if constexpr (SRC == SRC_G16) {
-        const uint16_t* const src = static_cast<const uint16_t*>(p.src) + (int64_t)n * p.src_stride + i0;
-        const int64_t left = p.d - i0;
-#pragma unroll
-        for (int g = 0; g < (32 >> VB); ++g) {
-            const int o = round_F_offset<T>(g);
-            float* const x = v + g * VN;
-            if (VB > 0 && o + VN <= left) {
-                if constexpr (VB == 2) {
-                    const uint2 q = load_cs(reinterpret_cast<const uint2*>(src + o));
-                    x[0] = __uint_as_float(q.x << 16); x[1] = __uint_as_float(q.x & 0xFFFF0000u);
-                    x[2] = __uint_as_float(q.y << 16); x[3] = __uint_as_float(q.y & 0xFFFF0000u);
-                } else if constexpr (VB == 1) {
-                    const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(src + o));
-                    x[0] = __uint_as_float(q << 16); x[1] = __uint_as_float(q & 0xFFFF0000u);
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < VN; ++k) x[k] = (o + k < left) ? __uint_as_float((uint32_t)src[o + k] << 16) : 0.f;
-            }
-        }
+    } else if constexpr (SRC == SRC_G32 || SRC == SRC_G16) {
+        load_gradient<T, SRC>(p, n, tile_base, baseF, v);
     } else if constexpr (SRC == SRC_WS) {
         const float* const src = static_cast<const float*>(p.src) + (int64_t)n * p.src_stride + i0;
 #pragma unroll
@@ -464,27 +526,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         float v[32];
         load_source<T, SRC, kLoopWorkers>(p, n, tile_base, baseF, fw, v);   // (uplink planes come one to a worker)
         if constexpr (kMeasures) {
-            if (p.amp_out != nullptr) {
-                // the tile is a whole block: its norm (fp32 within a thread, fp64 across threads, fixed order) sets its
-                // amplitude (readers are behind the barrier of the exchange rounds)
-                __shared__ double wsum[C::NT / 32];
-                float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                for (int r = 0; r < 32; r += 2) {
-                    s0 = fmaf(v[r], v[r], s0);
-                    s1 = fmaf(v[r + 1], v[r + 1], s1);
-                }
-                double sum = (double)(s0 + s1);
-#pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-                if (lane == 0) wsum[tid >> 5] = sum;
-                __syncthreads();
-                if (tid == 0) {
-                    for (int k = 1; k < C::NT / 32; ++k) sum += wsum[k];
-                    s_amp = fmaxf((float)(p.amp_factor * sqrt(sum)), kMinBlockAmplitude);
-                    p.amp_out[(int64_t)n * p.amp_stride + blockIdx.x] = s_amp;
-                }
-            }
+            if (p.amp_out != nullptr) measure_block<T>(p, n, tid, v, &s_amp);   // (its readers are behind the exchange's barrier)
         }
         butterflies32<31>(v);
         store_round_F<T>(smem, baseF, v);
@@ -798,6 +840,11 @@ cudaError_t launch_row_T(int src, int sink, const PassParams& p, cudaStream_t s)
 {
 #define FOSGD_ROW_CASE(SRC_, SINK_) \
     if (src == SRC_ && sink == SINK_) return launch_row_one<T, SRC_, SINK_>(p, s);
+    if (sink == SINK_NORM) {
+        const dim3 grid((unsigned)(p.dp >> T), (unsigned)p.nworkers);
+        return src == SRC_G16 ? launch<row_norm_kernel<T, SRC_G16>>(grid, 1 << (T - 5), 0, s, 1, p)
+                              : launch<row_norm_kernel<T, SRC_G32>>(grid, 1 << (T - 5), 0, s, 1, p);
+    }
     FOSGD_ROW_CASE(SRC_G32, SINK_WS)
     FOSGD_ROW_CASE(SRC_G16, SINK_WS)
     FOSGD_ROW_CASE(SRC_G32, SINK_PACK1)
