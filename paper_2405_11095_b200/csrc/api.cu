@@ -105,8 +105,8 @@ struct Plan {
 // 10 + 12 0.40; 2^20: 6 + 14 against 10 + 10 0.36 and 0.39 ms, and one vector of 2^20 0.018 against 0.043 ms,
 // because ten stages make only eight runs of tiles); below 2^20 the tile shrinks so that the contiguous pass still has blocks for the chip.
 // Two strided passes: eight stages each while T stays within 10..14 (2^27: 8 + 8 + 11 1.03 ms per two workers,
-// 6 + 10 + 11 1.10, 3 + 10 + 14 1.18); 2^31: 7 + 10 + 14 8.9 ms per worker against 10 + 10 + 11 10.5 ms, whose
-// top pass visits 1024 rows megabytes apart for 64 bytes each.
+// 6 + 10 + 11 1.10, 3 + 10 + 14 1.18); 2^31, top pass first: 8 + 9 + 14 8.24 ms per worker, 7 + 10 + 14 8.85,
+// 9 + 8 + 14 8.73, 8 + 8 + 15 8.72, 10 + 7 + 14 (whose top pass visits 1024 rows megabytes apart) 12.7.
 //
 // Decoder.  Every value is an exact integer, so the cut is free to follow the call: `workers` summed, P planes.
 //   five workers or more, up to 2^24: tiles of 2^14, whose contiguous pass runs on the tensor cores (2^20, 128
@@ -115,7 +115,11 @@ struct Plan {
 //   three or four from 2^20 on: ten strided stages (on the tensor cores if there are tiles enough), short tiles;
 //   one or two, or several planes: the plain-ALU pass is fastest on short tiles (one vector of 2^30: T = 10 1.5 ms, T = 14
 //     1.95), the first pass up to eight stages (six below 2^20, to leave the contiguous pass blocks for the chip);
-//   two strided passes: the same for fp32 (2^31: T = 11 2.8 ms per worker, T = 14 4.2).
+//   two strided passes: T = 12, where the contiguous pass still keeps pace with memory, the top pass nine stages (or eight:
+//     ten on the tensor cores lose their speed where rows lie megabytes apart), the middle pass what is left, up to
+//     nine.  Top + middle + T, per worker: 2^31 9 + 9 + 13 6.3 ms (10 + 10 + 11 7.2, 8 + 9 + 14 6.9), 2^30 9 + 9 + 12 3.1
+//     (10 + 10 + 10 3.5), 2^28 9 + 7 + 12 0.73 (9 + 9 + 10 0.78), 2^26 8 + 6 + 12 0.18 (8 + 8 + 10 0.19).  Several planes
+//     have a top pass of eight at any length (2^31, K = 15: 8 + 9 + 14 9.3 ms, 9 + 9 + 13 12.2, 10 + 10 + 11 13.4).
 Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1)
 {
     Plan pl{};
@@ -134,10 +138,9 @@ Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1)
         else pl.T = L == 18 ? 11 : (L < 18 ? 12 : (L == 19 ? 13 : 14));
         pl.A[0] = L - pl.T;
     } else {
-        pl.T = decoder ? (L > 30 ? L - 20 : 10) : (L > 30 ? 14 : L - 16);
-        const int rest = L - pl.T;
-        pl.A[0] = decoder ? rest / 2 : (rest > 16 ? 10 : 8);
-        pl.A[1] = rest - pl.A[0];
+        pl.A[1] = decoder && P == 1 && L >= 28 ? 9 : 8;
+        pl.T = decoder ? (L - pl.A[1] <= 21 ? 12 : L - pl.A[1] - 9) : (L > 30 ? 14 : L - 16);
+        pl.A[0] = L - pl.T - pl.A[1];
     }
     pl.lo[0] = pl.T;
     pl.lo[1] = pl.T + pl.A[0];
