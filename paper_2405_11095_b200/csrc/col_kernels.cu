@@ -91,7 +91,7 @@ template <int A, int SRC, bool NORM>
 __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, double* const partial)
 {
     constexpr int R = 1 << A;
-    pdl_begin();
+    pdl_trigger();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31;
     const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -102,15 +102,16 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
     const uint32_t d32 = (uint32_t)p.d;
     const void* const wsrc = worker_source<SRC>(p, n);
 
+    uint32_t myword = 0;  // flip word of row `lane` (gradient sources; from the generator alone)
+    if (SRC == SRC_G32 || SRC == SRC_G16) {
+        if ((int)lane < R) myword = eps_word(p.rng, p.id0 + (uint32_t)n, ((i_first - lane) + lane * step) >> 5);
+    }
+    pdl_wait();
     float v[32];
     if constexpr (SRC == SRC_BITS) {
         planes_to_values<R>(p, v, [&](int pl) { return (int)lane < R ? bits_row_word(p, wsrc, (i_first - lane) + lane * step, pl) : 0u; },
                             [&](uint32_t mine) { return warp_transpose_bits(mine, lane); });
     } else {
-        uint32_t myword = 0;  // flip word of row `lane` (gradient sources)
-        if (SRC == SRC_G32 || SRC == SRC_G16) {
-            if ((int)lane < R) myword = eps_word(p.rng, p.id0 + (uint32_t)n, ((i_first - lane) + lane * step) >> 5);
-        }
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = col_load<SRC>(p, wsrc, i_first + r * step, d32);
         if (SRC == SRC_G32 || SRC == SRC_G16) {

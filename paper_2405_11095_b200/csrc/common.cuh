@@ -297,6 +297,16 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr, uint32_t rank)
     return q;
 }
 
+// the double at shared-memory address `addr` of the cluster's block `rank`
+__device__ __forceinline__ double ld_cluster_double(uint32_t addr, uint32_t rank)
+{
+    uint32_t remote;
+    double q;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(q) : "r"(remote) : "memory");
+    return q;
+}
+
 // SINK_FINAL / SINK_SINGLE: one finished sum to memory (sc = scale times amplitude)
 __device__ __forceinline__ void store_final(float* dst, float o, float sc, int overwrite)
 {

@@ -84,6 +84,8 @@ struct RowCfg {
     static constexpr int TILE_WORDS = phys(1 << T);
     static constexpr int FLIP_WORDS = (1 << T) / 32;
     static constexpr size_t SMEM_BYTES = (size_t)(TILE_WORDS + FLIP_WORDS) * 4 + 16;  // + mbarrier
+    static constexpr size_t EARLY_AT = (SMEM_BYTES + 15) / 16 * 16;                   // the dither words of EARLY
+    static constexpr size_t EARLY_SMEM_BYTES = EARLY_AT + ((size_t)4 << T);
     static_assert(((FMASK | MMASK | LMASK) & ((1u << T) - 1)) == ((1u << T) - 1), "bits uncovered");
 };
 
@@ -162,8 +164,10 @@ __device__ __forceinline__ void sink_ws(const PassParams& p, int n, int64_t i0, 
 
 // Sign bits are shifted into a per-lane mask (bit r = sign of register r), then the 32 x 32 bit
 // matrix is transposed across the warp so that lane r owns packed word r.
+// EARLY: the words were left at early[0], early[stride], ..
+template <bool EARLY = false>
 __device__ __forceinline__ void sink_pack1(const PassParamsRK& p, int n, uint32_t id, int64_t i0, uint32_t lane,
-                                           const float (&v)[32], float amp)
+                                           const float (&v)[32], float amp, const uint4* early = nullptr, int stride = 0)
 {
     const uint32_t cbase = ((uint32_t)(i0 >> 7) << 5) + lane;
     const float dc = p.dither_c * amp;
@@ -171,7 +175,7 @@ __device__ __forceinline__ void sink_pack1(const PassParamsRK& p, int n, uint32_
     uint32_t neg = 0;
 #pragma unroll
     for (int m = 7; m >= 0; --m) {
-        const uint4 w = rng_words_dither(p, id, 1u, cbase + 32u * m);
+        const uint4 w = EARLY ? early[m * stride] : rng_words_dither(p, id, 1u, cbase + 32u * m);
         const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
         for (int q = 3; q >= 0; --q) {
@@ -472,12 +476,15 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
 // =============================================================================================
 // row_kernel: sources read by the threads themselves (single-pass transforms)
 // =============================================================================================
-template <int T, int SRC, int SINK>
+// EARLY: what comes from the generator alone, the first worker's flips and the dither words of SINK_PACK1, is made before the
+// wait for the kernel in front (the words kept in shared memory), where a chain of short kernels hides it: server and
+// downlink of 2^17, four workers, 16.6 -> 13.8 us, an encode of eight times 2^13 3.6 -> 2.7, of four times 2^16 6.7 -> 4.9.
+template <int T, int SRC, int SINK, bool EARLY>
 __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kernel(const typename KernelParams<SINK>::type p)
 {
     using C = RowCfg<T>;
     extern __shared__ __align__(16) float smem[];
-    pdl_begin();
+    pdl_trigger();
     uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);
 
     const int tid = threadIdx.x;
@@ -491,6 +498,20 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
     const int n_begin = (int)blockIdx.y;
     const int n_end = kLoopWorkers ? p.nworkers : n_begin + 1;
     const int n_step = kLoopWorkers ? (int)gridDim.y : 1;
+    auto flip_words = [&](uint32_t id) {
+        if (tid < C::FLIP_WORDS / 4) {
+            const uint4 w = rng_words(p.rng, id, 0u, (uint32_t)(tile_base >> 7) + (uint32_t)tid);
+            reinterpret_cast<uint4*>(fw)[tid] = w;
+        }
+    };
+    if (EARLY && kFlips) flip_words(p.id0 + (uint32_t)n_begin);
+    uint4* const early = reinterpret_cast<uint4*>(reinterpret_cast<char*>(smem) + C::EARLY_AT) + tid;
+    if constexpr (EARLY && SINK == SINK_PACK1) {
+        const uint32_t cbase = ((uint32_t)((tile_base + deposit<C::LMASK, T>(tid)) >> 7) << 5) + lane;
+#pragma unroll 2
+        for (int m = 0; m < 8; ++m) early[m * C::NT] = rng_words_dither(p, p.id0 + (uint32_t)n_begin, 1u, cbase + 32u * m);
+    }
+    pdl_wait();
     // one amplitude per tile (a block of the blocked mode is at least a tile): thread 0 reads it
     // first, so that its latency hides behind the tile load, and parks it in shared memory until
     // the sink (the barriers of the exchange rounds order the two)
@@ -515,11 +536,8 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         const uint32_t id = p.id0 + (uint32_t)n;
         const float wamp = (kLoopWorkers && p.amp_mode == AMP_WEIGHT) ? amplitude_at(p, n, tile_base) : 1.f;
         if (kFlips) {
-            if (kLoopWorkers) __syncthreads();  // previous worker's readers of fw and of the tile
-            if (tid < C::FLIP_WORDS / 4) {
-                const uint4 w = rng_words(p.rng, id, 0u, (uint32_t)(tile_base >> 7) + (uint32_t)tid);
-                reinterpret_cast<uint4*>(fw)[tid] = w;
-            }
+            if (kLoopWorkers && !(EARLY && n == n_begin)) __syncthreads();  // previous worker's readers of fw and of the tile
+            if (!EARLY || n != n_begin) flip_words(id);
             __syncthreads();
         }
 
@@ -538,7 +556,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         if constexpr (SINK == SINK_WS) {
             sink_ws(p, n, i0, v);
         } else if constexpr (SINK == SINK_PACK1) {
-            sink_pack1(p, n, id, i0, lane, v, s_amp);
+            sink_pack1<EARLY>(p, n, id, i0, lane, v, s_amp, early, C::NT);
         } else if constexpr (SINK == SINK_PACKK) {
             sink_packK(p, n, id, i0, lane, v, s_amp);
         } else if constexpr (SINK == SINK_SINGLE) {
@@ -678,7 +696,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
 {
     using C = RowCfg<T>;
     using S = StreamCfg<T, SRC>;
-    pdl_begin();
+    pdl_trigger();
     static_assert(SRC == SRC_WS || SRC == SRC_WS16, "streamed sources only");
     extern __shared__ __align__(16) float smem[];
     uint32_t* const fw = reinterpret_cast<uint32_t*>(smem + C::TILE_WORDS);
@@ -690,6 +708,12 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
     const int tid = threadIdx.x;
     const uint32_t lane = tid & 31;
     constexpr bool kFinal = (SINK == SINK_FINAL);
+    auto flip_words = [&](uint32_t id, int64_t tile_base) {
+        if (tid < C::FLIP_WORDS / 4)
+            reinterpret_cast<uint4*>(fw)[tid] = rng_words(p.rng, id, 0u, (uint32_t)(tile_base >> 7) + (uint32_t)tid);
+    };
+    if (kFinal) flip_words(p.id0 + blockIdx.y, (int64_t)blockIdx.x << T);
+    pdl_wait();        // (the flips come from the generator alone)
     // SINK_FINAL: this block's tile is fixed, one amplitude scales the sum (AMP_SCALE; parked in shared
     // memory until the store, the barriers of the worker loop order the two) or every worker brings its
     // own weight (AMP_WEIGHT)
@@ -774,10 +798,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
         fence_generic_before_async();   // (the landing buffer is only read by the threads, never written)
         __syncthreads();   // round F complete: the landing buffer is free, nobody is in the previous item
         if (tid == 0 && j + 1 < nitems) bulk_load(landing, item_src(j + 1), kTileBytes, bar);
-        if (kFinal && tid < C::FLIP_WORDS / 4) {
-            const uint4 w = rng_words(p.rng, id, 0u, (uint32_t)(tile_base >> 7) + (uint32_t)tid);
-            reinterpret_cast<uint4*>(fw)[tid] = w;
-        }
+        if (kFinal && j > 0) flip_words(id, tile_base);
         round_M<T>(smem, baseM, v);
         load_round_L(smem, baseL, v);
         __syncthreads();   // the tile lives in registers: the work tile may be overwritten by the next round F
@@ -818,7 +839,7 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
         unsigned parts = 1;
         while ((int)parts < PackKCfg<T>::GROUPS && ntiles * p.nworkers * (2 * parts) <= (int64_t)sms * PackKCfg<T>::MIN_BLOCKS) parts *= 2;
         if (parts == 1 && p.K < kManyDithers)
-            return launch<row_kernel<T, SRC, SINK>>(dim3((unsigned)ntiles, (unsigned)p.nworkers), C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p));
+            return launch<row_kernel<T, SRC, SINK, false>>(dim3((unsigned)ntiles, (unsigned)p.nworkers), C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p));
         return launch<row_packk_kernel<T, SRC>>(dim3((unsigned)ntiles, parts, (unsigned)p.nworkers), PackKCfg<T>::THREADS,
                                                 PackKCfg<T>::SMEM_BYTES, s, 1, with_round_keys(p));
     } else if constexpr (kStream) {
@@ -831,7 +852,14 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
                                                        kernel_params<SINK>(p), ntiles);
     } else {
         const dim3 grid((unsigned)ntiles, SINK == SINK_FINAL ? split : (unsigned)p.nworkers);
-        return launch<row_kernel<T, SRC, SINK>>(grid, C::NT, C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
+        if constexpr (SINK != SINK_WS && (T <= 12 || ((SRC == SRC_G32 || SRC == SRC_G16 || SRC == SRC_BITS) && T <= 14))) {
+            // one block per SM at most, which finds room beside those of the kernel in front: the early form (above).  Behind
+            // a strided pass only up to 2^12: with the larger tiles' shared memory the chain lost more than it gained (four
+            // workers of 300007, server and downlink: 26.6 -> 28.3 us; of 2^17, tiles of 2^12: 16.6 -> 13.8)
+            if (ntiles * grid.y <= sms)
+                return launch<row_kernel<T, SRC, SINK, true>>(grid, C::NT, SINK == SINK_PACK1 ? C::EARLY_SMEM_BYTES : C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
+        }
+        return launch<row_kernel<T, SRC, SINK, false>>(grid, C::NT, C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
     }
 }
 

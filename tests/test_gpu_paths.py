@@ -134,6 +134,27 @@ def test_encoder_on_ragged_lengths(F, L, dtype):
     assert_bits_near_ties(to_np_words(bits[1]), ref, margin, lam, 1)
 
 
+@pytest.mark.parametrize("d,M", [(1000, 148), (1000, 149), (1 << 16, 9), (1 << 16, 10), (10_000, 148), (10_000, 149)])
+def test_encoder_of_as_many_blocks_as_processors(F, d, M):
+    """Dither words made before or after the wait for the kernel in front (up to a block per processor, 148 of them): the
+    first and last worker against the oracle, and the same words from single-worker calls."""
+    seed, step = 29, d
+    grads = gradients(d, M, torch.float32)
+    dp = F.padded_dim(d)
+    ws = torch.empty(max(16, M * F.workspace_bytes(F.OP_ENCODE, d)), dtype=torch.uint8, device=DEV)
+    bits, one = torch.zeros(2, M, dp // 32, dtype=torch.int32, device=DEV)
+    x = grads[:, :d].cpu().double().numpy()
+    lam = oracle.lam(float(np.linalg.norm(x[M - 1])), 2.0, dp)
+    F.encode(grads, d, bits, lam, seed, step, ws=ws, worker_stride=grads.shape[1])
+    for n in (0, 1, M - 1):
+        F.encode(grads[n], d, one[n], lam, seed, step, worker_id0=n, ws=ws, worker_stride=grads.shape[1])
+    torch.cuda.synchronize()
+    for n in (0, 1, M - 1):
+        assert torch.equal(bits[n], one[n])
+        ref, margin = oracle.encode(x[n], seed, step, n, lam, want_margin=True)
+        assert_bits_near_ties(to_np_words(bits[n]), ref, margin, lam, 1)
+
+
 @pytest.mark.parametrize("d,b,M", [
     (700, 0, 9), (9000, 0, 2), (9000, 0, 33),        # one tile: up to eight blocks of a cluster share the workers
     (40_000, 0, 5), (300_000, 0, 7), (300_000, 14, 3),
