@@ -224,6 +224,12 @@ bool fused_encoder_enabled() { return g_fused_encoder.load(std::memory_order_rel
 
 // Enqueue one source -> sink transform for p.nworkers workers.  Workers are processed in
 // chunks of as many as the scratch buffer holds; SINK_FINAL accumulates chunk after chunk.
+// Decoders of a few short vectors (2^16 .. 2^18) in one kernel: the top five stages as counts of packed bits (SRC_BITS_TOP).
+// Short calls are a chain of launches, and this is one fewer: server and downlink of 2^16, one worker, 8.0 -> 6.9 us, four
+// 12.2 -> 11.3; 2^17, four, 13.7 -> 12.2; 2^18, four, 17.5 -> 15.6.  Above 2^20 coordinates in all the counting itself takes
+// longer than the strided pass (2^18, eight workers, 18.9 -> 24.6), and so it does on longer vectors (2^19, one, 15.4 -> 18.3).
+bool top_counts_applicable(int L, int64_t dp, int workers) { return L >= 16 && L <= 18 && dp * workers <= (int64_t)1 << 20; }
+
 int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, size_t ws_bytes,
                   cudaStream_t s)
 {
@@ -236,6 +242,10 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
         return FOSGD_OK;
     }
     if (ws == nullptr || ws_bytes < g.ws_per_worker) return FOSGD_EWORKSPACE;
+    if (src == SRC_BITS && sink == SINK_FINAL && p.P == 1 && top_counts_applicable(pl.L, g.dp, p.nworkers)) {
+        FOSGD_CUDA_OK(traced('r', pl.L - kTopStages, SRC_BITS_TOP, p.nworkers == 1 ? (int)SINK_SINGLE : sink, p, s));
+        return FOSGD_OK;
+    }
     const size_t cap = ws_bytes / g.ws_per_worker;
     const int total = p.nworkers;
     int chunk = (int)(cap < (size_t)total ? cap : (size_t)total);
@@ -885,7 +895,7 @@ int fosgd_trace_count(void) { return g_trace_count; }
 const char* fosgd_trace_label(int k)
 {
     if (k < 0 || k >= g_trace_count) return "";
-    static const char* const srcs[] = {"f32", "bf16", "bits", "ws", "ws16"};
+    static const char* const srcs[] = {"f32", "bf16", "bits", "ws", "ws16", "ws", "ws16", "bits"};
     static const char* const sinks[] = {"ws", "pack1", "packK", "final", "final", "ws16", "amp"};
     const TraceEntry& t = g_trace_log[k];
     char who[16];

@@ -19,8 +19,11 @@ enum Src : int {
     // The contiguous pass of a 2^25 transform, whose 15 stages are one more than a tile of 2^14 has: the top one is
     // done while reading, by both tiles of a pair (each reads both halves, the second time out of L2).
     SRC_WS_PAIR = 5,
-    SRC_WS16_PAIR = 6
+    SRC_WS16_PAIR = 6,
+    // One plane of a transform of 2^(T + kTopStages): the top stages are counts of packed bits, made while reading
+    SRC_BITS_TOP = 7
 };
+constexpr int kTopStages = 5;
 enum Sink : int {
     SINK_WS = 0,     // fp32 intermediate (or the scaled transform output of fosgd_flatten)
     SINK_PACK1 = 1,  // dither + sign + pack, K = 1

@@ -85,6 +85,8 @@ struct RowCfg {
     static constexpr int FLIP_WORDS = (1 << T) / 32;
     static constexpr size_t SMEM_BYTES = (size_t)(TILE_WORDS + FLIP_WORDS) * 4 + 16;  // + mbarrier
     static constexpr size_t EARLY_AT = (SMEM_BYTES + 15) / 16 * 16;                   // the dither words of EARLY
+    static constexpr size_t TOP_AT = EARLY_AT;                                        // the planes of SRC_BITS_TOP
+    static constexpr size_t TOP_SMEM_BYTES = TOP_AT + (size_t)(kTopStages + 1) * NT * 4;
     static constexpr size_t EARLY_SMEM_BYTES = EARLY_AT + ((size_t)4 << T);
     static_assert(((FMASK | MMASK | LMASK) & ((1u << T) - 1)) == ((1u << T) - 1), "bits uncovered");
 };
@@ -370,6 +372,53 @@ __global__ void __launch_bounds__(1 << (T - 5), 1 << (15 - T)) row_norm_kernel(c
 }
 
 // fw: flip words of the tile (gradient sources).  ONE_PLANE: a packed source known to have a single plane.
+// SRC_BITS_TOP.  Entry j of tile t after the top stages is sum_s (-1)^popc(s & t) x_s(j) over the 2^5 segments s of the
+// transform, x = 2 b - 1: the number of set bits among b_s(j) ^ parity(s & t).  The thread counts 32 entries at once, one
+// packed word per segment, by a tree of bit-sliced adders, and leaves the six planes of the counts at top[0], top[NT], ..
+template <int K>
+__device__ __forceinline__ void add_planes(uint32_t (&a)[6], const uint32_t (&b)[6])   // a += b, planes 0 .. K - 1 each
+{
+    uint32_t carry = a[0] & b[0];
+    a[0] ^= b[0];
+#pragma unroll
+    for (int k = 1; k < K; ++k) {
+        const uint32_t x = a[k], y = b[k];
+        a[k] = x ^ y ^ carry;
+        carry = (x & y) | (carry & (x | y));
+    }
+    a[K] = carry;
+}
+template <int K>
+__device__ __forceinline__ void count_words(const uint32_t* w, uint32_t (&sum)[6])      // planes of the count of 2^K words
+{
+    if constexpr (K == 0) {
+        sum[0] = w[0];
+    } else {
+        uint32_t other[6];
+        count_words<K - 1>(w, sum);
+        count_words<K - 1>(w + (1 << (K - 1)), other);
+        add_planes<K>(sum, other);
+    }
+}
+template <int T>
+__device__ __forceinline__ void count_segments(const PassParams& p, int n, int tid, uint32_t* top)
+{
+    constexpr int NT = RowCfg<T>::NT;
+    const uint32_t t = blockIdx.x & 31u;
+    // bit s = parity(s & t)
+    const uint32_t odd = ((t & 1u) ? 0xAAAAAAAAu : 0u) ^ ((t & 2u) ? 0xCCCCCCCCu : 0u) ^ ((t & 4u) ? 0xF0F0F0F0u : 0u) ^
+                         ((t & 8u) ? 0xFF00FF00u : 0u) ^ ((t & 16u) ? 0xFFFF0000u : 0u);
+    const uint32_t* const src = static_cast<const uint32_t*>(p.src) + (int64_t)n * p.src_stride + (int64_t)(blockIdx.x >> 5) * (32 * NT) + tid;
+    uint32_t w[32], sum[6];
+#pragma unroll
+    for (int s = 0; s < 32; ++s) w[s] = load_ca(src + s * NT);
+#pragma unroll
+    for (int s = 0; s < 32; ++s) w[s] ^= (odd >> s) & 1u ? 0xFFFFFFFFu : 0u;
+    count_words<kTopStages>(w, sum);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) top[k * NT + tid] = sum[k];
+}
+
 template <int T, int SRC, bool ONE_PLANE = false>
 __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t tile_base, int baseF, const uint32_t* fw,
                                             float (&v)[32])
@@ -433,6 +482,23 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
                 x[0] = a.x; x[1] = a.y;
             } else {
                 x[0] = __half2float(load_cs(src + o));
+            }
+        }
+    } else if constexpr (SRC == SRC_BITS_TOP) {
+        const uint32_t* const top = fw + (RowCfg<T>::TOP_AT - RowCfg<T>::TILE_WORDS * 4) / 4 + (baseF >> 5);
+        const uint32_t pos = (uint32_t)baseF & 31u;
+#pragma unroll
+        for (int g = 0; g < (32 >> VB); ++g) {
+            const uint32_t* const at = top + (round_F_offset<T>(g) >> 5);
+#pragma unroll
+            for (int k = 0; k < VN; ++k) v[g * VN + k] = -32.f;
+            float weight = 2.f;
+#pragma unroll
+            for (int pl = 0; pl < 6; ++pl, weight += weight) {
+                const uint32_t w = at[pl * RowCfg<T>::NT] >> pos;
+#pragma unroll
+                for (int k = 0; k < VN; ++k)
+                    if ((w >> k) & 1u) v[g * VN + k] += weight;
             }
         }
     } else {  // SRC_BITS
@@ -538,6 +604,7 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
         if (kFlips) {
             if (kLoopWorkers && !(EARLY && n == n_begin)) __syncthreads();  // previous worker's readers of fw and of the tile
             if (!EARLY || n != n_begin) flip_words(id);
+            if constexpr (SRC == SRC_BITS_TOP) count_segments<T>(p, n, tid, reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smem) + C::TOP_AT));
             __syncthreads();
         }
 
@@ -852,14 +919,15 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
                                                        kernel_params<SINK>(p), ntiles);
     } else {
         const dim3 grid((unsigned)ntiles, SINK == SINK_FINAL ? split : (unsigned)p.nworkers);
-        if constexpr (SINK != SINK_WS && (T <= 12 || ((SRC == SRC_G32 || SRC == SRC_G16 || SRC == SRC_BITS) && T <= 14))) {
+        constexpr size_t kBytes = SRC == SRC_BITS_TOP ? C::TOP_SMEM_BYTES : C::SMEM_BYTES;
+        if constexpr (SINK != SINK_WS && (T <= 12 || ((SRC == SRC_G32 || SRC == SRC_G16 || SRC == SRC_BITS || SRC == SRC_BITS_TOP) && T <= 14))) {
             // one block per SM at most, which finds room beside those of the kernel in front: the early form (above).  Behind
             // a strided pass only up to 2^12: with the larger tiles' shared memory the chain lost more than it gained (four
             // workers of 300007, server and downlink: 26.6 -> 28.3 us; of 2^17, tiles of 2^12: 16.6 -> 13.8)
             if (ntiles * grid.y <= sms)
-                return launch<row_kernel<T, SRC, SINK, true>>(grid, C::NT, SINK == SINK_PACK1 ? C::EARLY_SMEM_BYTES : C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
+                return launch<row_kernel<T, SRC, SINK, true>>(grid, C::NT, SINK == SINK_PACK1 ? C::EARLY_SMEM_BYTES : kBytes, s, split, kernel_params<SINK>(p));
         }
-        return launch<row_kernel<T, SRC, SINK, false>>(grid, C::NT, C::SMEM_BYTES, s, split, kernel_params<SINK>(p));
+        return launch<row_kernel<T, SRC, SINK, false>>(grid, C::NT, kBytes, s, split, kernel_params<SINK>(p));
     }
 }
 
@@ -880,6 +948,10 @@ cudaError_t launch_row_T(int src, int sink, const PassParams& p, cudaStream_t s)
     FOSGD_ROW_CASE(SRC_G32, SINK_PACKK)
     FOSGD_ROW_CASE(SRC_BITS, SINK_FINAL)
     FOSGD_ROW_CASE(SRC_BITS, SINK_SINGLE)
+    if constexpr (T >= 16 - kTopStages && T <= 18 - kTopStages) {
+        FOSGD_ROW_CASE(SRC_BITS_TOP, SINK_FINAL)
+        FOSGD_ROW_CASE(SRC_BITS_TOP, SINK_SINGLE)
+    }
     if constexpr (T <= 14) {     // (an intermediate's tiles of 2^15 are pairs of 2^14)
         FOSGD_ROW_CASE(SRC_WS, SINK_WS)
         FOSGD_ROW_CASE(SRC_WS, SINK_PACK1)

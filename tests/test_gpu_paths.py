@@ -157,7 +157,9 @@ def test_encoder_of_as_many_blocks_as_processors(F, d, M):
 
 @pytest.mark.parametrize("d,b,M", [
     (700, 0, 9), (9000, 0, 2), (9000, 0, 33),        # one tile: up to eight blocks of a cluster share the workers
-    (40_000, 0, 5), (300_000, 0, 7), (300_000, 14, 3),
+    (40_000, 0, 5), (40_000, 0, 1), (40_000, 0, 16), (40_000, 0, 17),     # top stages as counts of bits, up to 2^20 in all
+    (100_000, 16, 3), (1 << 17, 0, 8), (200_000, 18, 2), ((1 << 18) - 1, 0, 4),
+    (300_000, 0, 7), (300_000, 14, 3),
     (1 << 20, 0, 3), (1 << 20, 0, 128),              # ten strided stages; 64 tiles for the tensor-core pass, workers split
     (3 << 20, 20, 11), ((1 << 21) - 9, 0, 64),       # items that do not divide among the blocks
     ((1 << 25) - 5, 0, 2), ((1 << 25) - 5, 0, 5),    # pairs of halves, without and with the tensor-core pass
