@@ -895,7 +895,10 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
     const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
     // a few tiles with many workers each (2^13, 8 workers: one tile) would leave most SMs idle
-    const unsigned split = SINK == SINK_FINAL ? worker_split(ntiles, p.nworkers, (int64_t)sms * min_blocks<T, SINK>()) : 1u;
+    // (one worker per block instead of two where a decode is little but latency: four vectors of 2^16 7.0 -> 5.1 us, of
+    // 2^17 7.9 -> 6.1; of 2^18 11.3 -> 13.1)
+    const int share = SRC == SRC_BITS_TOP && T <= 12 ? 2 * p.nworkers : p.nworkers;
+    const unsigned split = SINK == SINK_FINAL ? worker_split(ntiles, share, (int64_t)sms * min_blocks<T, SINK>()) : 1u;
     // On the way to the dither sink the fp32 tiles are read by the threads themselves: without the persistent
     // grid the blocks of an SM drift apart and one's loads and butterflies fill the gaps of another's generator
     // rounds (2^27 coordinates, T = 10 / 12 / 13: 0.175 / 0.187 / 0.189 ms against 0.215 / 0.213 / 0.225 ms streamed).
