@@ -79,6 +79,7 @@ cudaError_t traced(char kind, int size, int src, int sink, const PassParams& p, 
                   : kind == 'c' ? launch_col(size, src, p, s)
                   : kind == 'h' ? launch_colh(size, p, s)
                   : kind == 't' ? launch_tc_col(p, s)
+                  : kind == 'e' ? launch_cluster_encode(src, p, s)
                   : kind == 'u' ? launch_tc_row(size, p, s)
                                 : launch_small(size, src, sink, p, s);
     trace_end(on, s, TraceEntry{kind, size, src, sink, p.id0 == FOSGD_SERVER_ID ? 0 : p.nworkers, decoder});
@@ -96,7 +97,7 @@ struct Plan {
     int lo[2];   // lowest index bit of each strided pass
 };
 
-// The cut depends on L and the direction alone, never on the number of workers: the encoder's fp32 sums, and
+// The cut depends on the vector and the direction alone, never on the number of workers: the encoder's fp32 sums, and
 // with them its packed signs, are the same however the workers are batched.
 //
 // Encoder.  A strided pass costs its memory traffic up to eight stages (0.17 ms per 2^27 coordinates, nine 0.20,
@@ -244,6 +245,10 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
     if (ws == nullptr || ws_bytes < g.ws_per_worker) return FOSGD_EWORKSPACE;
     if (src == SRC_BITS && sink == SINK_FINAL && p.P == 1 && top_counts_applicable(pl.L, g.dp, p.nworkers)) {
         FOSGD_CUDA_OK(traced('r', pl.L - kTopStages, SRC_BITS_TOP, p.nworkers == 1 ? (int)SINK_SINGLE : sink, p, s));
+        return FOSGD_OK;
+    }
+    if ((src == SRC_G32 || src == SRC_G16) && sink == SINK_PACK1 && cluster_encode_applicable(pl.L, g.dp)) {
+        FOSGD_CUDA_OK(traced('e', pl.L, src, sink, p, s));
         return FOSGD_OK;
     }
     const size_t cap = ws_bytes / g.ws_per_worker;
@@ -726,9 +731,10 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
     if (g.plan.ncol > 0 && (ws == nullptr || ws_bytes < g.ws_per_worker)) return FOSGD_EWORKSPACE;
     const Plan& pl = g.plan;
     cudaStream_t s = (cudaStream_t)stream;
-    // One pass over the gradients where the strided pass can carry the sums: fp32, a single strided pass, and scratch for all M workers at once (the amplitude is a maximum over all of them, so every
-    // strided pass must be over before the first dither).
-    if (dtype == FOSGD_F32 && pl.ncol == 1 && ws_bytes / g.ws_per_worker >= (size_t)M) {
+    // One pass over the gradients where the strided pass can carry the sums: fp32, a single strided pass, and scratch
+    // for all M workers at once (the amplitude is a maximum over all of them, so every strided pass must be over before
+    // the first dither).  The one-kernel encoder of blocks of 2^16 has no such point: the two calls one after the other.
+    if (dtype == FOSGD_F32 && pl.ncol == 1 && !cluster_encode_applicable(pl.L, g.dp) && ws_bytes / g.ws_per_worker >= (size_t)M) {
         PassParams pc{};
         pc.src = grads; pc.src_stride = worker_stride; pc.d = d; pc.dp = g.dp;
         pc.dst = ws; pc.dst_stride = g.dp; pc.lo_log = pl.lo[0];
@@ -791,13 +797,13 @@ int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_
     p.P = 1; p.K = 1; p.nworkers = M; p.id0 = worker_id0; p.rng = make_rng(seed, step);
     set_amp(&p, Amp{1.f, lambda_dev, nb, block_log2}, AMP_DITHER);
     p.dither_c = (float)(g.rootn / 16777216.0);
-    if (pl.ncol == 0 && pl.L >= 10) {
+    if ((pl.ncol == 0 && pl.L >= 10) || (cluster_encode_applicable(pl.L, g.dp) && ws != nullptr)) {
         // one kernel per block anyway: it measures what it transforms
         p.dst = bits; p.dst_stride = g.dp >> 5;
         p.amp_dev = nullptr;
         p.amp_out = lambda_dev;
         p.amp_factor = block_amplitude_factor(alpha, g.L);
-        e = traced('r', pl.T, src, SINK_PACK1, p, s);
+        e = traced(pl.ncol == 0 ? 'r' : 'e', pl.ncol == 0 ? pl.T : pl.L, src, SINK_PACK1, p, s);
         if (e == cudaSuccess && lambda_s_dev != nullptr) {
             const bool on = trace_begin(s);
             e = launch_server_amplitudes(lambda_dev, nb, M, block_log2, alpha_s, lambda_s_dev, s);
@@ -902,7 +908,7 @@ const char* fosgd_trace_label(int k)
     if (t.workers > 0) snprintf(who, sizeof who, "%d", t.workers);
     else snprintf(who, sizeof who, "srv");
     snprintf(g_trace_label, sizeof g_trace_label, "%s%d:%s->%s@%s",
-             t.kind == 'r' ? "row" : (t.kind == 'c' ? (t.decoder ? "dcol" : "col") : (t.kind == 'h' ? "colh" : (t.kind == 'n' ? "norm" : (t.kind == 't' ? "tc" : (t.kind == 'u' ? "tcrow" : (t.kind == 'f' ? "fused" : "small")))))),
+             t.kind == 'r' ? "row" : (t.kind == 'c' ? (t.decoder ? "dcol" : "col") : (t.kind == 'h' ? "colh" : (t.kind == 'n' ? "norm" : (t.kind == 't' ? "tc" : (t.kind == 'u' ? "tcrow" : (t.kind == 'f' ? "fused" : (t.kind == 'e' ? "cluster" : "small"))))))),
              t.size, srcs[t.src], sinks[t.sink], who);
     return g_trace_label;
 }

@@ -442,6 +442,9 @@ __attribute__((visibility("hidden"))) int check_decode_args(const void* bits, in
 
 // ---- host-visible launchers (one translation unit per family) --------------------------
 cudaError_t launch_row(int T, int src, int sink, const PassParams& p, cudaStream_t s);
+// one-plane encoder of blocks of 2^16 in one kernel (cluster_encode.cu)
+bool cluster_encode_applicable(int L, int64_t dp);
+cudaError_t launch_cluster_encode(int src, const PassParams& p, cudaStream_t s);
 cudaError_t launch_col(int A, int src, const PassParams& p, cudaStream_t s);
 bool colh_applicable(int A, const PassParams& p);                          // every value after A stages exact in fp16
 cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s);   // packed planes -> fp16 intermediate

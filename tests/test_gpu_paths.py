@@ -34,6 +34,7 @@ def gradients(d, M, dtype, pad=8, seed=0):
     (3 * (1 << 16) + 9, 3, 16),        # strided passes that carry the sums: up to 2^22 (eight stages)
     (2 * (1 << 17) - 3, 2, 17),
     ((1 << 18) + 4099, 2, 18),
+    ((9 << 16) + 31, 2, 16),           # a cluster of thread blocks holds the block
     (2 * (1 << 20), 2, 20),
     ((1 << 22) + 12345, 2, 22),
     ((1 << 23) - 1, 2, 23),
@@ -134,7 +135,7 @@ def test_encoder_on_ragged_lengths(F, L, dtype):
     assert_bits_near_ties(to_np_words(bits[1]), ref, margin, lam, 1)
 
 
-@pytest.mark.parametrize("d,M", [(1000, 148), (1000, 149), (1 << 16, 9), (1 << 16, 10), (10_000, 148), (10_000, 149)])
+@pytest.mark.parametrize("d,M", [(1000, 148), (1000, 149), (1 << 16, 18), ((1 << 16) - 5, 19), (10_000, 148), (10_000, 149)])
 def test_encoder_of_as_many_blocks_as_processors(F, d, M):
     """Dither words made before or after the wait for the kernel in front (up to a block per processor, 148 of them): the
     first and last worker against the oracle, and the same words from single-worker calls."""
@@ -153,6 +154,30 @@ def test_encoder_of_as_many_blocks_as_processors(F, d, M):
         assert torch.equal(bits[n], one[n])
         ref, margin = oracle.encode(x[n], seed, step, n, lam, want_margin=True)
         assert_bits_near_ties(to_np_words(bits[n]), ref, margin, lam, 1)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d,M", [(1 << 19, 3), ((1 << 19) + 1, 1), ((9 << 16) - 2345, 2), ((7 << 16) + 1, 2), ((7 << 16) - 3, 2)])
+def test_encoder_of_blocks_of_2p16(F, d, M, dtype):
+    """The one-kernel form (from eight blocks on) and the two-kernel form against the oracle, and batches against single
+    workers word for word."""
+    seed, step, b = 31, 2, 16
+    grads = gradients(d, M, dtype)
+    dp, stride = F.padded_dim(d, b), grads.shape[1]
+    ws = torch.empty(M * F.workspace_bytes(F.OP_ENCODE, d, block_log2=b), dtype=torch.uint8, device=DEV)
+    bits, one = torch.zeros(2, M, dp // 32, dtype=torch.int32, device=DEV)
+    x = grads[:, :d].double().cpu().numpy()
+    lam = oracle.lam(float(np.linalg.norm(x[M - 1])) / 3, 2.0, 1 << b)
+    with F.PassTrace() as tr:
+        F.encode(grads, d, bits, lam, seed, step, worker_id0=3, block_log2=b, ws=ws, worker_stride=stride)
+    torch.cuda.synchronize()
+    assert any(lab.startswith("cluster") for lab in tr.labels) == (dp >= 1 << 19), tr.labels
+    for n in range(M):
+        F.encode(grads[n], d, one[n], lam, seed, step, worker_id0=3 + n, block_log2=b, ws=ws, worker_stride=stride)
+    torch.cuda.synchronize()
+    assert torch.equal(bits, one)
+    ref, margin = oracle.encode(x[M - 1], seed, step, 2 + M, lam, block_log2=b, want_margin=True)
+    assert_bits_near_ties(to_np_words(bits[M - 1]), ref, margin, lam, 1)
 
 
 @pytest.mark.parametrize("d,b,M", [
