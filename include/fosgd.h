@@ -203,8 +203,8 @@ int fosgd_downlink_apply(const uint32_t* down_bits, int64_t d, uint64_t seed, ui
  * usual case that the gradients just encoded are the ones whose norm sets the amplitude (Theorem 5.5 with
  * B = max_n ||g_n||_2 over the M workers of the call).  lambda_dev (and lambda_s_dev, nullable) receive the
  * amplitudes as fosgd_amplitudes writes them; the packed signs are those of fosgd_encode_dev with that lambda.
- * Where the first strided pass of the encoder can carry the sums (fp32 gradients, transform length 2^20 ..
- * 2^24 in global or blocked mode, `ws` holding all M workers) the gradients are read once instead of twice;
+ * Where the strided pass of the encoder can carry the sums (fp32 gradients, transform lengths 2^17 .. 2^22, 2^24
+ * and 2^25 in global or blocked mode, `ws` holding all M workers) the gradients are read once instead of twice;
  * elsewhere the call runs the two calls one after the other.  The sums are added in a fixed order, so the
  * amplitudes are reproducible, but in another order than fosgd_amplitudes uses: the two may differ in the
  * last bit.  amp_ws: scratch of fosgd_workspace_bytes(FOSGD_OP_AMPLITUDES, ..., M, ...) bytes. */
@@ -261,18 +261,18 @@ const char* fosgd_trace_label(int k);   /* e.g. "col10:f32->ws@4", "row14:ws->pa
                                            workers of the launch, or "srv" for the server's own vector on the downlink); valid until the next call */
 
 /* Which passes of a decoder that starts from one packed plane (fosgd_decode, fosgd_server_aggregate,
- * the downlink decoder with K = 1; transform lengths 2^20 .. 2^25) run on the tensor cores.  The
+ * the downlink decoder with K = 1; transform lengths 2^16 .. 2^25, the ten-stage passes of longer ones) run on the tensor cores.  The
  * recursion H_k = H_1 (x) H_{k-1} below Def. 3.4 makes every Kronecker factor H_128 a legal 128 x 128
  * matrix product, and on the decode side all operands are exact small integers (Def. 3.8: q_i = +-1).
  *   FOSGD_TC_STRIDED     the ten strided stages as H_8 on packed bytes plus a 128 x 128 x 128 8-bit integer
  *                        product per block (tcgen05 kind::i8), instead of packed fp16 arithmetic on the
  *                        plain ALUs (launches of fewer than 256 tiles of 2^17 coordinates stay on the
  *                        plain ALUs: too few tiles to repay a block's set-up);
- *   FOSGD_TC_CONTIGUOUS  the contiguous pass on tiles of 2^14 (transform length 2^24) as H_4 in packed
+ *   FOSGD_TC_CONTIGUOUS  the contiguous pass on tiles of 2^14 (or pairs of them, length 2^25) as H_4 in packed
  *                        fp16 while staging, a 128 x 128 x 128 fp16 product with fp32 accumulators in tensor
  *                        memory per tile and worker (tcgen05 kind::f16), and H_32, flip and the sum over
  *                        the workers in registers, instead of fp32 butterflies on the plain ALUs (launches
- *                        that sum fewer than three workers stay on the plain ALUs, which are faster there).
+ *                        of a few workers, or of few tiles, stay on the plain ALUs, which are faster there).
  *   FOSGD_TC_ANY_SIZE    apply the chosen passes also to launches below the size thresholds named above.
  * Either way the results are the same bit for bit (all values are integers below 2^24 in magnitude).
  * Default: FOSGD_TC_STRIDED | FOSGD_TC_CONTIGUOUS (each measured faster than its plain-ALU kernel on a B200).  Process-wide; returns the

@@ -21,11 +21,16 @@
 // A block keeps a tile position and walks the workers (sums in registers), then moves to its next tile.  Its
 // warps are specialised, so that nobody waits for two things in turn: a load warp keeps whole tiles (32 KiB, contiguous)
 // arriving through the bulk copy engine into a ring of three landing slots; four staging warps turn landed tiles
-// into the operand layout in one of two operand buffers; one warp issues the products into four accumulators in
+// into the operand layout in one of two operand buffers; one warp issues the products into three accumulators in
 // turn; one warp makes the flip words; sixteen drain warps take the accumulators through the register stages.
 // (With sixteen warps that staged an item and then drained the one before, an item took 1.6 us, twice what its 350
 // instructions per warp or its shared-memory traffic cost.)  Synchronisation is by mbarriers only (slot landed / read,
 // operand full / free, accumulator full / free, flips ready); every wait is bounded.
+//
+// 2^24 x 32: 0.305 ms (0.357 with warps that staged and drained in turn, 0.324 before the operand was 128-byte swizzled
+// and the ring positions 32-bit), 2^25 x 8 0.265.  Bound by the staging warps' chain (without product and drain the rest
+// alone takes 0.225 ms) and the shared-memory port; eight staging warps, four accumulators or ring slots, and flips
+// made by the staging warps all measured slower or the same.
 #include "tc_common.cuh"
 
 namespace fosgd {
@@ -400,8 +405,8 @@ __global__ void __launch_bounds__(kThreads, 1) tc_row_final_kernel(const PassPar
 
 // One packed plane's fp16 intermediate in contiguous tiles of 2^14, and at least three workers to sum: with one or
 // two (a single decoder, the downlink) the plain-ALU pass is the faster one (0.033 against 0.041 ms on one vector
-// of 2^24, 0.051 against 0.057 on two; 0.069 against 0.068 on three, 0.156 against 0.119 on eight).  The 15 stages of a
-// 2^25 transform: from five workers on, whose sums repay staging every tile twice (eight: 0.30 against 0.35 ms).
+// of 2^24, 0.051 against 0.057 on two; 0.069 against 0.068 on three, 0.156 against 0.101 on eight).  The 15 stages of a
+// 2^25 transform: from five workers on, whose sums repay staging every tile twice (eight: 0.27 against 0.35 ms).
 bool tc_row_applicable(const PassParams& p, int T, bool any_size)
 {
     if (p.P != 1 || (p.dp >> kT) < 1 || (p.dp >> kT) > 0x7FFFFFFF) return false;
