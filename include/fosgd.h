@@ -261,7 +261,7 @@ const char* fosgd_trace_label(int k);   /* e.g. "col10:f32->ws@4", "row14:ws->pa
                                            workers of the launch, or "srv" for the server's own vector on the downlink); valid until the next call */
 
 /* Which passes of a decoder that starts from one packed plane (fosgd_decode, fosgd_server_aggregate,
- * the downlink decoder with K = 1; transform lengths 2^16 .. 2^25, the ten-stage passes of longer ones) run on the tensor cores.  The
+ * the downlink decoder with K = 1; transform lengths 2^18 .. 2^25) run on the tensor cores.  The
  * recursion H_k = H_1 (x) H_{k-1} below Def. 3.4 makes every Kronecker factor H_128 a legal 128 x 128
  * matrix product, and on the decode side all operands are exact small integers (Def. 3.8: q_i = +-1).
  *   FOSGD_TC_STRIDED     the ten strided stages as H_8 on packed bytes plus a 128 x 128 x 128 8-bit integer

@@ -274,7 +274,7 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
     // A packed one-plane source through two strided passes (transform length above 2^25): the first pass's output
     // is still exact in fp16, so with room for it beside the fp32 intermediate (6 instead of 4 bytes per
     // coordinate and worker) the first pass writes half the bytes in 256-byte rows and the second reads half.
-    bool half_first = (src == SRC_BITS && p.P == 1 && pl.ncol == 2 && pl.A[1] >= 6 && pl.A[1] <= 10 &&
+    bool half_first = (src == SRC_BITS && p.P == 1 && pl.ncol == 2 &&
                        ws_bytes >= g.ws_per_worker + g.ws_per_worker / 2);
     if (half_first) {
         const size_t cap16 = ws_bytes / (g.ws_per_worker + g.ws_per_worker / 2);
@@ -323,8 +323,7 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
             pc.dst = ws16;
             pc.dst_stride = g.dp;
             pc.lo_log = pl.lo[1];
-            if (pl.A[1] == 10 && tc_enabled() && tc_col_applicable(pc, tc_any_size())) FOSGD_CUDA_OK(traced('t', pl.A[1], SRC_BITS, 5, pc, s));
-            else FOSGD_CUDA_OK(traced('h', pl.A[1], SRC_BITS, 5, pc, s));
+            FOSGD_CUDA_OK(traced('h', pl.A[1], SRC_BITS, 5, pc, s));
             PassParams pm = q;
             pm.src = ws16;
             pm.src_stride = g.dp;

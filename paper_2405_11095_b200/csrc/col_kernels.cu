@@ -794,9 +794,11 @@ static cudaError_t launch_col_A(int src, const PassParams& p, cudaStream_t s)
         case SRC_G32: return launch_col_one<A, SRC_G32>(p, s);
         case SRC_G16: return launch_col_one<A, SRC_G16>(p, s);
         case SRC_BITS: return launch_col_one<A, SRC_BITS>(p, s);
-        case SRC_WS: return launch_col_one<A, SRC_WS>(p, s);
+        case SRC_WS:         // the second of two strided passes
+            if constexpr (A >= 6 && A <= 9) return launch_col_one<A, SRC_WS>(p, s);
+            break;
         case SRC_WS16:
-            if constexpr (A >= 6) return launch_col_one<A, SRC_WS16>(p, s);   // (second strided pass of a long decoder)
+            if constexpr (A >= 6 && A <= 9) return launch_col_one<A, SRC_WS16>(p, s);
             break;
     }
     return cudaErrorInvalidValue;
