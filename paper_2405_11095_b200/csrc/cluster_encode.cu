@@ -101,14 +101,8 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK_PACK1>()) clu
     else load_rows<T, SRC, false>(p, n, vec_base + column, v);
 
     double sum = 0.0;
-    if (p.amp_out != nullptr) {       // the vector is a block that sets its own amplitude (sum: fp32 in a thread, fp64 across)
-        float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-        for (int r = 0; r < 32; r += 2) {
-            s0 = fmaf(v[r], v[r], s0);
-            s1 = fmaf(v[r + 1], v[r + 1], s1);
-        }
-        sum = (double)(s0 + s1);
+    if (p.amp_out != nullptr) {       // the vector is a block that sets its own amplitude
+        sum = sum_of_squares(v);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         if (lane == 0) wsum[tid >> 5] = sum;

@@ -60,8 +60,7 @@ struct Col4 {
 // One run: tiles seg0 .. seg0 + 7 (16-column segments of the matrix view) of worker n, by the 512 threads
 // of a block or group (tid = 0 .. 511).  timeouts: device counter bumped when a bounded wait gave up;
 // the return value says whether the run completed (the same for all threads).
-// NORM: also add up the squares of the run's gradient entries (fp32 within a tile, fp64 across tiles and threads,
-// fixed order) and leave the sum in *run_sumsq, so that a norm needs no second pass over the gradients.
+// NORM: also add up the squares of the run's gradient entries (fp64, fixed order) and leave the sum in *run_sumsq, so that a norm needs no second pass over the gradients.
 template <typename S, bool NORM = false>
 __device__ __forceinline__ bool col4_run(const PassParams& p, const CUtensorMap* tmap, const uint32_t full_rows, const int n,
                                          const uint32_t seg0, unsigned char* smem_raw, const int tid, int* timeouts,
@@ -149,15 +148,7 @@ __device__ __forceinline__ bool col4_run(const PassParams& p, const CUtensorMap*
                 v[4 * g + 0] = flip_at(q.x, w, sh); v[4 * g + 1] = flip_at(q.y, w, sh - 1u);
                 v[4 * g + 2] = flip_at(q.z, w, sh - 2u); v[4 * g + 3] = flip_at(q.w, w, sh - 3u);
             }
-            if (NORM) {
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-                for (int g = 0; g < 8; ++g) {
-                    s0 = fmaf(v[4 * g + 0], v[4 * g + 0], s0); s1 = fmaf(v[4 * g + 1], v[4 * g + 1], s1);
-                    s2 = fmaf(v[4 * g + 2], v[4 * g + 2], s2); s3 = fmaf(v[4 * g + 3], v[4 * g + 3], s3);
-                }
-                sumsq += (double)((s0 + s1) + (s2 + s3));
-            }
+            if (NORM) sumsq += sum_of_squares(v);
             butterflies32<28>(v);
 #pragma unroll
             for (int g = 0; g < 8; ++g) {

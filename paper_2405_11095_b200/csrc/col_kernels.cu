@@ -121,10 +121,7 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
     }
     if constexpr (NORM) {
         __shared__ double wsum[8];
-        float sq = 0.f;
-#pragma unroll
-        for (int r = 0; r < R; ++r) sq = fmaf(v[r], v[r], sq);
-        double sum = (double)sq;
+        double sum = sum_of_squares<R>(v);
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
         if (lane == 0) wsum[threadIdx.x >> 5] = sum;
@@ -149,7 +146,7 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
 // reaches), where tiles of 16 columns (64-byte segments) took 0.21 ms; with rows megabytes apart (the top pass
 // of a 2^31 transform) the segment width decides: 5.8 ms with 64 bytes per row visit at A = 8, 2.9 ms with 256.
 // NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
-// (fp32 within a thread's tile, fp64 beyond, fixed order); blocks then take tiles gridDim.x apart.
+// (fp64, fixed order); blocks then take tiles gridDim.x apart.
 template <int A, int SRC, bool NORM>
 __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams p, const uint32_t ntiles, double* const partial)
 {
@@ -248,13 +245,7 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
             }
         }
         if constexpr (NORM) {
-            float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                s0 = fmaf(v[2 * r], v[2 * r], s0);
-                s1 = fmaf(v[2 * r + 1], v[2 * r + 1], s1);
-            }
-            sumsq += (double)(s0 + s1);
+            sumsq += sum_of_squares(v);
         }
         butterflies32<30>(v);
         if (NORM) __syncthreads();                                 // readers of the previous tile

@@ -74,6 +74,20 @@ enum AmpMode {
     AMP_WEIGHT = 2   // SINK_FINAL weights every worker's contribution by that worker's entry
 };
 
+// Sum of squares of the first N of a thread's values, in fp64 from the first product on (a square of fp32 is exact there): an fp32 square is
+// zero below 4e-23 and infinite above 1.8e19, where gradients still have a norm.  Two chains, to halve the latency.
+template <int N = 32>
+__device__ __forceinline__ double sum_of_squares(const float (&v)[32])
+{
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int r = 0; r < N; r += 2) {
+        s0 = fma((double)v[r], (double)v[r], s0);
+        s1 = fma((double)v[r + 1], (double)v[r + 1], s1);
+    }
+    return s0 + s1;
+}
+
 // floor of a measured block amplitude: a block of zeros keeps a positive one, so that its sign bits are still decided by
 // the dither (and decode to ~0) instead of by the sign of a zero
 constexpr float kMinBlockAmplitude = 1e-30f;

@@ -337,18 +337,12 @@ __device__ __forceinline__ void load_gradient(const PassParams& p, int n, int64_
 }
 
 // The tile is a whole block of the gradient: its norm sets the block's amplitude, in *s_amp after the next barrier and in
-// the table.  One order of the sum for every caller: fp32 within a thread, fp64 across threads.
+// the table.  One order of the sum (fp64) for every caller.
 template <int T>
 __device__ __forceinline__ void measure_block(const PassParams& p, int n, int tid, const float (&v)[32], float* s_amp)
 {
     __shared__ double wsum[RowCfg<T>::NT / 32];
-    float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-    for (int r = 0; r < 32; r += 2) {
-        s0 = fmaf(v[r], v[r], s0);
-        s1 = fmaf(v[r + 1], v[r + 1], s1);
-    }
-    double sum = (double)(s0 + s1);
+    double sum = sum_of_squares(v);
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
     if ((tid & 31) == 0) wsum[tid >> 5] = sum;
