@@ -714,7 +714,7 @@ __global__ void __launch_bounds__(PackKCfg<T>::THREADS, PackKCfg<T>::MIN_BLOCKS)
         float y[4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) y[r] = smem[phys(128 * g + 32 * r) + (int)lane];
-        const uint32_t c = dither_counts(p, id, (((uint32_t)(tile_base >> 7) + (uint32_t)g) << 5) + lane, y, dc, k0, k1);
+        const uint32_t c = dither_counts<true>(p, id, (((uint32_t)(tile_base >> 7) + (uint32_t)g) << 5) + lane, y, dc, k0, k1);
         if (share == 1) store_count_planes(c, lane, p.P, dst + 4 * g, p.dp >> 5);
         else atomicAdd(counts + 32 * j + (int)lane, c);
     }

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK
                 const int word = 4 * g + r - (n >= 128 ? 0 : r_first);
                 y[r] = word >= 0 && word < n / 32 ? x[32 * word + lane] : 0.f;
             }
-            const uint32_t c = dither_counts(p, id, (((uint32_t)(base >> 7) + (uint32_t)g) << 5) + (uint32_t)lane, y,
+            const uint32_t c = dither_counts<false>(p, id, (((uint32_t)(base >> 7) + (uint32_t)g) << 5) + (uint32_t)lane, y,
                                              p.dither_c * amp, k0, k1);
             atomicAdd(counts + 32 * g + lane, c);
             __syncthreads();
