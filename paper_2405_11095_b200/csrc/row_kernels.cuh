@@ -622,10 +622,10 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_kerne
             sink_packK(p, n, id, i0, lane, v, s_amp);
         } else if constexpr (SINK == SINK_SINGLE) {
             const uint32_t* const fwl = fw + ((baseL - (int)lane) >> 5);
-            // (a per-worker weight rounds the sum first, as it does among several workers)
+            // (as the first of several workers: a weight rounds the term before the scale, and added to zero a flipped zero is +0)
             const float w = p.amp_mode == AMP_WEIGHT ? s_amp : 1.f;
 #pragma unroll
-            for (int r = 0; r < 32; ++r) v[r] = flip_by_bit(v[r], fwl[r], lane) * w;
+            for (int r = 0; r < 32; ++r) v[r] = fmaf(flip_by_bit(v[r], fwl[r], lane), w, 0.f);
             sink_final_store(p, i0, v, p.amp_mode == AMP_WEIGHT ? 1.f : s_amp);
         } else {
             const uint32_t* const fwl = fw + ((baseL - (int)lane) >> 5);
