@@ -47,6 +47,18 @@ static int64_t taken(Args* c, PyObject* r)
     return v;
 }
 
+/* whatever int(o) and float(o) take: numpy's truth values for a switch, say */
+static int64_t made_int(Args* c, PyObject* o) { return c->bad ? 0 : PyLong_Check(o) ? as_int(c, o) : taken(c, PyNumber_Long(o)); }
+static double made_double(Args* c, PyObject* o)
+{
+    if (c->bad) return 0.0;
+    PyObject* const r = PyNumber_Float(o);
+    if (r == NULL) { c->bad = 1; return 0.0; }
+    const double v = PyFloat_AS_DOUBLE(r);
+    Py_DECREF(r);
+    return v;
+}
+
 static int64_t method0(Args* c, PyObject* t, PyObject* name) { return c->bad ? 0 : taken(c, PyObject_CallMethodNoArgs(t, name)); }
 static int64_t method_of_0(Args* c, PyObject* t, PyObject* name) { return c->bad ? 0 : taken(c, PyObject_CallMethodOneArg(t, name, g_zero)); }
 
@@ -105,6 +117,7 @@ static const float* device_amplitude(Args* c, PyObject* o, float* value)
 #define U64(K) ((uint64_t)as_int(c, a[K]))
 #define F32(K) ((float)as_double(c, a[K]))
 #define F64(K) (as_double(c, a[K]))
+#define SWITCH(K) ((int)made_int(c, a[K]))
 #define PTR(K) (ptr(c, a[K]))
 #define CALL(EXPR)                       \
     if (c->bad) return NULL;             \
@@ -202,7 +215,7 @@ CALLABLE(server_aggregate_dev)
     const float* const lam_s = PTR(9);
     const int K = I32(10);
     uint32_t* const down = PTR(11);
-    const int b = I32(12), pb = I32(13);
+    const int b = I32(12), pb = SWITCH(13);
     void* const ws = PTR(14);
     const size_t wsn = nbytes(c, a[14]);
     const fosgd_stream s = stream(c);
@@ -234,7 +247,7 @@ CALLABLE(downlink_decode_dev)
     float* const out = PTR(2);
     const float* const lam_s = PTR(3);
     const uint64_t seed = U64(4), step = U64(5);
-    const int K = I32(6), b = I32(7), pb = I32(8);
+    const int K = I32(6), b = I32(7), pb = SWITCH(8);
     void* const ws = PTR(9);
     const size_t wsn = nbytes(c, a[9]);
     const fosgd_stream s = stream(c);
@@ -251,7 +264,7 @@ CALLABLE(downlink_encode)
     float value;
     const float* const dev = device_amplitude(c, a[3], &value);
     const uint64_t seed = U64(4), step = U64(5);
-    const int K = I32(6), b = I32(7), pb = I32(8);
+    const int K = I32(6), b = I32(7), pb = SWITCH(8);
     void* const ws = PTR(9);
     const size_t wsn = nbytes(c, a[9]);
     const fosgd_stream s = stream(c);
@@ -268,8 +281,8 @@ CALLABLE(downlink_apply)
     float value;
     const float* const dev = device_amplitude(c, a[3], &value);
     const uint64_t seed = U64(4), step = U64(5);
-    const float step_size = F32(6);
-    const int K = I32(7), b = I32(8), pb = I32(9);
+    const float step_size = (float)made_double(c, a[6]);
+    const int K = I32(7), b = I32(8), pb = SWITCH(9);
     void* const ws = PTR(10);
     const size_t wsn = nbytes(c, a[10]);
     const fosgd_stream s = stream(c);
@@ -285,7 +298,7 @@ CALLABLE(amplitudes)
     float* const lam = PTR(2);
     float* const lam_s = PTR(3);
     const double alpha = F64(4), alpha_s = F64(5);
-    const int b = I32(6), pb = I32(7);
+    const int b = I32(6), pb = SWITCH(7);
     void* const ws = PTR(8);
     const size_t wsn = nbytes(c, a[8]);
     const fosgd_stream s = stream(c);
@@ -302,7 +315,7 @@ CALLABLE(encode_dev)
     const float* const lam = PTR(3);
     const uint64_t seed = U64(4), step = U64(5);
     const uint32_t id0 = U32(6);
-    const int b = I32(7), pb = I32(8);
+    const int b = I32(7), pb = SWITCH(8);
     void* const ws = PTR(9);
     const size_t wsn = nbytes(c, a[9]);
     const fosgd_stream s = stream(c);
