@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import concurrent.futures as cf
 import os
+import shutil
 import subprocess
 import sys
 import sysconfig
@@ -11,7 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 SO = os.path.join(HERE, "libfosgd.so")
-NATIVE_SO = os.path.join(HERE, "_native.so")
+# named after the interpreter whose headers it is built against: another one in the same tree neither finds it nor takes it for its own
+NATIVE_SO = os.path.join(HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
@@ -40,14 +42,21 @@ def _newest_source() -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
-def build_binding(force: bool = False) -> str:
-    """The native half of the Python binding (a CPython extension, host code only)."""
+def build_binding(force: bool = False):
+    """The native half of the Python binding (a CPython extension, host code only).  None where this machine has no C compiler or
+    no headers of this interpreter: the calls then go through ctypes (_marshal.py)."""
     src = os.path.join(CSRC, "binding.c")
+    unversioned = os.path.join(HERE, "_native.so")      # the name of earlier builds, which any interpreter would load
+    if os.path.exists(unversioned):
+        os.remove(unversioned)
+    include = sysconfig.get_paths()["include"]
+    if shutil.which("gcc") is None or not os.path.exists(os.path.join(include, "Python.h")):
+        print(f"no gcc or no {include}/Python.h: the Python calls go through ctypes", file=sys.stderr)
+        return None
     newest = max(os.path.getmtime(p) for p in (src, os.path.join(HERE, "..", "include", "fosgd.h")))
     if force or not os.path.exists(NATIVE_SO) or os.path.getmtime(NATIVE_SO) < newest:
         tmp = NATIVE_SO + f".tmp{os.getpid()}"
-        subprocess.run(["gcc", "-std=gnu11", "-O2", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"], "-o", tmp, src],
-                       check=True)
+        subprocess.run(["gcc", "-std=gnu11", "-O2", "-fPIC", "-shared", "-I", include, "-o", tmp, src], check=True)
         os.replace(tmp, NATIVE_SO)
     return NATIVE_SO
 
