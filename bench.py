@@ -103,9 +103,12 @@ def measured_peaks():
 
 # --------------------------------------------------------------------------- clocks
 class ClockSampler:
+    """Clocks from the end of the constructor, which waits for nvidia-smi's first sample (it takes up to a second to start), to stop()."""
+
     def __init__(self, gpu_index: int):
         self.path = f"/tmp/fosgd_clocks_{os.getpid()}_{time.monotonic_ns()}.csv"
         self.proc = None
+        self.begin = 0
         try:
             self.out = open(self.path, "w")
             self.proc = subprocess.Popen(["nvidia-smi", f"--query-gpu={CLOCK_QUERY}", "--format=csv,noheader,nounits",
@@ -113,6 +116,11 @@ class ClockSampler:
                                          stderr=subprocess.DEVNULL)
         except OSError:
             self.proc = None
+            return
+        until = time.monotonic() + 5.0
+        while os.path.getsize(self.path) == 0 and self.proc.poll() is None and time.monotonic() < until:
+            time.sleep(0.01)
+        self.begin = os.path.getsize(self.path)      # what was sampled before the region
 
     def stop(self):
         if self.proc is None:
@@ -126,6 +134,7 @@ class ClockSampler:
         sm, smax, reasons = [], [], set()
         names = ["hw_slowdown", "hw_thermal_slowdown", "sw_thermal_slowdown", "sw_power_cap"]
         with open(self.path) as f:
+            f.seek(self.begin)
             for line in f:
                 parts = [x.strip() for x in line.split(",")]
                 if len(parts) < 9:
@@ -380,7 +389,7 @@ def run_workload(env, args, w, steps, warmup, min_seconds, want_e2e):
                     order.append(lab)
                 per[lab][0] += ms
                 per[lab][1] += 1
-        if timed_ms >= 1e3 * min_seconds or nblocks >= 500:
+        if timed_ms >= 1e3 * min_seconds:      # (the same sum on every rank)
             break
     clocks = sampler.stop() if sampler else None
     ms_per_step = statistics.median(block_ms) / K
