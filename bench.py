@@ -60,6 +60,8 @@ def parse_args():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--no-legs", action="store_true", help="skip the extra workloads, the K > 1 downlink table and the issue-rate probe")
+    ap.add_argument("--details", default=None, metavar="FILE",
+                    help="also write the whole record (all digits, every figure of the further workloads) to FILE")
     ap.add_argument("--e2e-pieces", type=int, default=16,
                     help="end-to-end leg: pieces the host-to-device copy is cut into (compute overlaps the later ones)")
     return ap.parse_args()
@@ -543,6 +545,43 @@ def analyse(rec, peaks, peak_kind, alu_peak, alu_peak_kind, world):
     return paths, roofline, path_roofline
 
 
+def rounded(x, digits=5):
+    """The same structure with its floats to `digits` significant digits."""
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    if isinstance(x, list):
+        return [rounded(v, digits) for v in x]
+    return float(f"{x:.{digits}g}") if isinstance(x, float) else x
+
+
+def printed(record):
+    """The record as it is printed: short enough for a reader that keeps a few kilobytes of the output.  The metric, its times and
+    the roofline's own figures keep their digits; of the tables the times and fractions stay, rounded."""
+    def kept(d, *keys):
+        return {k: d[k] for k in keys if k in d}
+
+    line = dict(record)
+    line["kernels"] = rounded({k: kept(v, "launches_per_step", "ms_per_launch") for k, v in record["kernels"].items()})
+    line["paths"] = rounded({k: kept(v, "ms", "algorithmic_GBps", "frac_of_hbm_peak") for k, v in record["paths"].items()}, 4)
+    line["roofline"] = {k: v for k, v in record["roofline"].items() if k not in ("algorithmic_bytes_are", "frac_of_nominal_8TBps")}
+    line["roofline"]["per_kernel"] = rounded({k: kept(v, "frac", "implementation_frac")
+                                              for k, v in record["roofline"]["per_kernel"].items()}, 4)
+    line["path_roofline"] = rounded({k: v for k, v in record["path_roofline"].items() if k != "note"})
+    line["block_ms_min_median_max"] = rounded(record["block_ms_min_median_max"])
+    if "alu_probe" in record:
+        line["alu_probe"] = rounded(kept(record["alu_probe"], "lane_ops_per_s", "seconds_timed"))
+    if "downlink_K" in record:
+        line["downlink_K"] = rounded({K: kept(v, "server_downlink_encode_ms", "worker_downlink_decode_ms")
+                                      for K, v in record["downlink_K"].items()})
+    if "legs" in record:
+        line["legs"] = {name: rounded(dict(kept(leg, "value", "ms_per_step", "steps", "repeats", "async_wait_timeouts"),
+                                           clocks=kept(leg["clocks"], "sm_mhz", "reasons"),
+                                           path_ms={k: v["ms"] for k, v in leg["paths"].items()},
+                                           roofline=kept(leg["roofline"], "kernel", "frac", "implementation_frac")))
+                        for name, leg in record["legs"].items()}
+    return line
+
+
 def probe_alu(env):
     """Measured issue rates of the plain ALUs (lane operations per second), each kind timed for
     about a third of a second with the SM clock sampled alongside."""
@@ -662,7 +701,10 @@ def main():
     if not args.no_cpu_baseline and world == 1:
         line["cpu_baseline"] = {k: v for k, v in oracle_sample(w, args.block_log2, 2, 0).items()
                                 if k in ("value", "unit", "cores", "kind", "sample")}
-    print(json.dumps(line))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f)
+    print(json.dumps(printed(line)))
     if world > 1:
         dist.destroy_process_group()
 
