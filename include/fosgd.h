@@ -261,19 +261,23 @@ const char* fosgd_trace_label(int k);   /* e.g. "col10:f32->ws@4", "row14:ws->pa
                                            workers of the launch, or "srv" for the server's own vector on the downlink); valid until the next call */
 
 /* Which passes of a decoder that starts from one packed plane (fosgd_decode, fosgd_server_aggregate,
- * the downlink decoder with K = 1; transform lengths 2^18 .. 2^25) run on the tensor cores.  The
+ * the downlink decoder with K = 1; transform lengths 2^16 .. 2^25) run on the tensor cores.  The
  * recursion H_k = H_1 (x) H_{k-1} below Def. 3.4 makes every Kronecker factor H_128 a legal 128 x 128
  * matrix product, and on the decode side all operands are exact small integers (Def. 3.8: q_i = +-1).
  *   FOSGD_TC_STRIDED     the ten strided stages as H_8 on packed bytes plus a 128 x 128 x 128 8-bit integer
  *                        product per block (tcgen05 kind::i8), instead of packed fp16 arithmetic on the
- *                        plain ALUs (launches of fewer than 256 tiles of 2^17 coordinates stay on the
- *                        plain ALUs: too few tiles to repay a block's set-up);
+ *                        plain ALUs.  Lengths that are cut so: 2^24 and 2^25, and 2^20 .. 2^23 for three or four
+ *                        workers; of those, launches of at least 256 tiles of 2^17 coordinates (fewer do not repay
+ *                        a block's set-up);
  *   FOSGD_TC_CONTIGUOUS  the contiguous pass on tiles of 2^14 (or pairs of them, length 2^25) as H_4 in packed
  *                        fp16 while staging, a 128 x 128 x 128 fp16 product with fp32 accumulators in tensor
  *                        memory per tile and worker (tcgen05 kind::f16), and H_32, flip and the sum over
- *                        the workers in registers, instead of fp32 butterflies on the plain ALUs (launches
- *                        of a few workers, or of few tiles, stay on the plain ALUs, which are faster there).
- *   FOSGD_TC_ANY_SIZE    apply the chosen passes also to launches below the size thresholds named above.
+ *                        the workers in registers, instead of fp32 butterflies on the plain ALUs.  Launches of
+ *                        at least five workers and 128 (tile, worker) items at 2^16 .. 2^23, of three workers at
+ *                        2^24 and five at 2^25 (below, the plain ALUs are faster);
+ *   FOSGD_TC_ANY_SIZE    apply the chosen passes also below these thresholds: the strided one at 2^20 .. 2^25, the
+ *                        contiguous one at 2^16 .. 2^24 (at 2^20 .. 2^23 a transform takes one of them: the strided one
+ *                        where both are chosen).  The five workers of 2^25 stay a condition.
  * Either way the results are the same bit for bit (all values are integers below 2^24 in magnitude).
  * Default: FOSGD_TC_STRIDED | FOSGD_TC_CONTIGUOUS (each measured faster than its plain-ALU kernel on a B200).  Process-wide; returns the
  * previous mask. */

@@ -121,7 +121,8 @@ struct Plan {
 //     nine.  Top + middle + T, per worker: 2^31 9 + 9 + 13 6.3 ms (10 + 10 + 11 7.2, 8 + 9 + 14 6.9), 2^30 9 + 9 + 12 3.1
 //     (10 + 10 + 10 3.5), 2^28 9 + 7 + 12 0.73 (9 + 9 + 10 0.78), 2^26 8 + 6 + 12 0.18 (8 + 8 + 10 0.19).  Several planes
 //     have a top pass of eight at any length (2^31, K = 15: 8 + 9 + 14 9.3 ms, 9 + 9 + 13 12.2, 10 + 10 + 11 13.4).
-Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1)
+// FOSGD_TC_ANY_SIZE in `tc`, the mask of the chosen tensor-core passes: the cut that lets them run, whatever the number of workers.
+Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1, int tc = 0)
 {
     Plan pl{};
     pl.L = L;
@@ -132,7 +133,10 @@ Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1)
     }
     pl.ncol = L <= 25 ? 1 : 2;
     if (pl.ncol == 1) {
+        const int forced = decoder && P == 1 && (tc & FOSGD_TC_ANY_SIZE) ? tc : 0;
         if (L == 25) pl.T = 15;
+        else if ((forced & FOSGD_TC_STRIDED) && L >= 20) pl.T = L - 10;
+        else if (forced & FOSGD_TC_CONTIGUOUS) pl.T = 14;
         else if (decoder && workers > 4 && P == 1 && (dp >> 14) * workers >= 128) pl.T = 14;
         else if (decoder && workers > 2 && P == 1 && L >= 20) pl.T = L - 10;
         else if (decoder) pl.T = L < 20 ? L - 6 : (L <= 22 ? (L - 8 < 12 ? 12 : L - 8) : (L == 23 && P == 1 ? 13 : 14));
@@ -215,9 +219,6 @@ Rng make_rng(uint64_t seed, uint64_t step)
 // which passes of a decoder whose source is one packed plane run on the tensor cores (FOSGD_TC_* bits;
 // both by default: each measured faster than its plain-ALU kernel)
 std::atomic<int> g_tensor_core_pass{FOSGD_TC_STRIDED | FOSGD_TC_CONTIGUOUS};
-bool tc_enabled() { return (g_tensor_core_pass.load(std::memory_order_relaxed) & FOSGD_TC_STRIDED) != 0; }
-bool tc_row_enabled() { return (g_tensor_core_pass.load(std::memory_order_relaxed) & FOSGD_TC_CONTIGUOUS) != 0; }
-bool tc_any_size() { return (g_tensor_core_pass.load(std::memory_order_relaxed) & FOSGD_TC_ANY_SIZE) != 0; }
 // whether an encoder of ten strided stages + a 2^14 tile runs as the one-kernel form or as two kernels (default:
 // measured on a B200 the two kernels are the faster form)
 std::atomic<int> g_fused_encoder{0};
@@ -234,7 +235,9 @@ bool top_counts_applicable(int L, int64_t dp, int workers) { return L >= 16 && L
 int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, size_t ws_bytes,
                   cudaStream_t s)
 {
-    const Plan pl = sink == SINK_FINAL ? make_plan(g.L, true, g.dp, p.nworkers, p.P) : g.plan;
+    const int tc = g_tensor_core_pass.load(std::memory_order_relaxed);
+    const bool tc_any_size = (tc & FOSGD_TC_ANY_SIZE) != 0;
+    const Plan pl = sink == SINK_FINAL ? make_plan(g.L, true, g.dp, p.nworkers, p.P, tc) : g.plan;
     cudaError_t e = cudaSuccess;
 #define FOSGD_CUDA_OK(call) do { e = (call); if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; } } while (0)
     if (pl.ncol == 0) {
@@ -243,7 +246,8 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
         return FOSGD_OK;
     }
     if (ws == nullptr || ws_bytes < g.ws_per_worker) return FOSGD_EWORKSPACE;
-    if (src == SRC_BITS && sink == SINK_FINAL && p.P == 1 && top_counts_applicable(pl.L, g.dp, p.nworkers)) {
+    if (src == SRC_BITS && sink == SINK_FINAL && p.P == 1 && top_counts_applicable(pl.L, g.dp, p.nworkers) &&
+        !(tc_any_size && (tc & FOSGD_TC_CONTIGUOUS))) {
         FOSGD_CUDA_OK(traced('r', pl.L - kTopStages, SRC_BITS_TOP, p.nworkers == 1 ? (int)SINK_SINGLE : sink, p, s));
         return FOSGD_OK;
     }
@@ -314,7 +318,7 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
             pc.dst_stride = g.dp;
             pc.lo_log = pl.lo[0];
             // ten stages: H_8 on packed bytes + H_128 on the tensor cores, same fp16 intermediate
-            tensor_pass = pl.A[0] == 10 && tc_enabled() && tc_col_applicable(pc, tc_any_size());
+            tensor_pass = pl.A[0] == 10 && (tc & FOSGD_TC_STRIDED) && tc_col_applicable(pc, tc_any_size);
             if (tensor_pass) FOSGD_CUDA_OK(traced('t', pl.A[0], SRC_BITS, 5, pc, s));
             else FOSGD_CUDA_OK(traced('h', pl.A[0], SRC_BITS, 5, pc, s));
         } else if (half_first) {
@@ -354,7 +358,7 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
         } else {
             pr.dst = dst0 + (size_t)n0 * (size_t)p.dst_stride * sink_elem_bytes(sink);
         }
-        if (half_path && sink == SINK_FINAL && tc_row_enabled() && tc_row_applicable(pr, pl.T, tc_any_size()))
+        if (half_path && sink == SINK_FINAL && (tc & FOSGD_TC_CONTIGUOUS) && tc_row_applicable(pr, pl.T, tc_any_size))
             FOSGD_CUDA_OK(traced('u', pl.T, SRC_WS16, sink, pr, s));
         else
             FOSGD_CUDA_OK(traced('r', pl.T, half_path ? (int)SRC_WS16 : (int)SRC_WS,
