@@ -63,3 +63,46 @@ def test_any_size(F, L, blocks, M):
         assert ran(labels) == (strided, contiguous), (mask, labels)
         assert torch.equal(acc, plain), mask
     assert F.async_timeouts() == 0
+
+
+DEFAULT = 3     # both passes, with their thresholds
+
+
+@pytest.mark.parametrize("d,b,M", [
+    ((9 << 16) - 1, 16, 15), ((5 << 17) + 9, 17, 7), ((1 << 18) - 1, 0, 9), (3 << 18, 18, 6), ((1 << 19) + 7, 19, 5), (1 << 20, 0, 128),
+    (3 << 20, 20, 11), ((1 << 21) - 9, 0, 64), ((1 << 22) + 5, 22, 5), ((1 << 23) - 77, 0, 5), ((1 << 24) - 1, 0, 3), ((1 << 24) + 3, 24, 6),
+    ((1 << 25) - 5, 0, 5), ((1 << 25) - 5, 0, 8), ((1 << 25) + 12345, 25, 6),
+])
+def test_contiguous_pass_of_every_length(F, d, b, M):
+    """The averaged decoder by default, against the plain ALUs: the plain average, the average in two calls with an addition in between, scratch for
+    five workers at a time, and (in blocks) an amplitude per worker and block, alone and by chunks."""
+    seed, step = 13, M
+    dp = F.padded_dim(d, b)
+    bits = planes(M, dp, d % 1009 + M)
+    need = F.workspace_bytes(F.OP_AGGREGATE, d, M=M, block_log2=b)
+    ws = torch.empty(M * need, dtype=torch.uint8, device=DEV)
+    few = ws[: min(M, 5) * need]
+    lam = torch.rand(M, dp >> b, generator=torch.Generator(device=DEV).manual_seed(M), device=DEV) + 0.5 if b else None
+
+    def run():
+        outs = [torch.full((dp,), 7.0, device=DEV) for _ in range(5 if b else 3)]
+        F.server_aggregate(bits, d, outs[0], 0.25, seed, step, worker_id0=1, block_log2=b, ws=ws)
+        k = max(M - 5, M // 2)
+        F.server_aggregate(bits[:k], d, outs[1], 0.25, seed, step, N_total=M, worker_id0=1, flags=F.AGG_BEGIN, block_log2=b, ws=ws)
+        F.server_aggregate(bits[k:], d, outs[1], 0.25, seed, step, N_total=M, worker_id0=1 + k, flags=F.AGG_END, block_log2=b, ws=ws)
+        F.server_aggregate(bits, d, outs[2], 0.25, seed, step, worker_id0=1, block_log2=b, ws=few)
+        if b:
+            F.server_aggregate_dev(bits, d, outs[3], lam, seed, step, worker_id0=1, block_log2=b, per_block=True, ws=ws)
+            F.server_aggregate_dev(bits, d, outs[4], lam, seed, step, worker_id0=1, block_log2=b, per_block=True, ws=few)
+        return outs
+
+    plain, labels = with_mask(F, 0, run)
+    assert ran(labels) == (False, False), labels
+    outs, labels = with_mask(F, DEFAULT, run)
+    T = 15 if (b or (dp - 1).bit_length()) == 25 else 14
+    assert sum(x.startswith(f"tcrow{T}") for x in labels) >= 2, labels
+    for k, (x, y) in enumerate(zip(outs, plain)):
+        # (a weight rounds each worker's term, and the sum over the workers is rounded in the order of the blocks that share them)
+        assert torch.equal(x, y) if k < 3 else float((x - y).norm()) <= 1e-6 * float(y.norm()), k
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    assert F.async_timeouts() == 0
