@@ -800,7 +800,7 @@ int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_
     p.P = 1; p.K = 1; p.nworkers = M; p.id0 = worker_id0; p.rng = make_rng(seed, step);
     set_amp(&p, Amp{1.f, lambda_dev, nb, block_log2}, AMP_DITHER);
     p.dither_c = (float)(g.rootn / 16777216.0);
-    if ((pl.ncol == 0 && pl.L >= 10) || (cluster_encode_applicable(pl.L, g.dp) && ws != nullptr)) {
+    if ((pl.ncol == 0 && pl.L >= 10) || cluster_encode_applicable(pl.L, g.dp)) {
         // one kernel per block anyway: it measures what it transforms
         p.dst = bits; p.dst_stride = g.dp >> 5;
         p.amp_dev = nullptr;

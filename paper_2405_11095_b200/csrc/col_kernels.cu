@@ -66,13 +66,13 @@ __device__ __forceinline__ uint32_t column_pair_bits(uint32_t word, uint32_t lan
     return __byte_perm(a, b, (lane & 16u) ? 0x7632 : 0x5410);
 }
 
-// v[r] = 2 c - K of R rows from the P count planes of one column (exact): column(pl) = this lane's column of plane pl,
+// v[r] = 2 c - K of 32 rows from the P count planes of one column (exact): column(pl) = this lane's column of plane pl,
 // one bit per row.  fetch(pl) starts the plane's loads one plane ahead.
-template <int R, typename Fetch, typename Column>
+template <typename Fetch, typename Column>
 __device__ __forceinline__ void planes_to_values(const PassParams& p, float (&v)[32], Fetch fetch, Column column)
 {
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = (float)(-p.K);
+    for (int r = 0; r < 32; ++r) v[r] = (float)(-p.K);
     auto next = fetch(0);
     float weight = 2.f;
     for (int pl = 0; pl < p.P; ++pl, weight += weight) {
@@ -80,16 +80,17 @@ __device__ __forceinline__ void planes_to_values(const PassParams& p, float (&v)
         if (pl + 1 < p.P) next = fetch(pl + 1);
         const uint32_t x = column(mine);
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+        for (int r = 0; r < 32; ++r)
             if ((x >> r) & 1u) v[r] += weight;
     }
 }
 
-// ---- A <= 4 -----------------------------------------------------------------------------
+// ---- A = 4, from gradients ----------------------------------------------------------------
 // NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
 template <int A, int SRC, bool NORM>
 __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, double* const partial)
 {
+    static_assert(SRC == SRC_G32 || SRC == SRC_G16, "a decoder's first pass of so few stages is colh_small_kernel");
     constexpr int R = 1 << A;
     pdl_trigger();
     const int n = blockIdx.y;
@@ -102,23 +103,14 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
     const uint32_t d32 = (uint32_t)p.d;
     const void* const wsrc = worker_source<SRC>(p, n);
 
-    uint32_t myword = 0;  // flip word of row `lane` (gradient sources; from the generator alone)
-    if (SRC == SRC_G32 || SRC == SRC_G16) {
-        if ((int)lane < R) myword = eps_word(p.rng, p.id0 + (uint32_t)n, ((i_first - lane) + lane * step) >> 5);
-    }
+    uint32_t myword = 0;  // flip word of row `lane` (from the generator alone)
+    if ((int)lane < R) myword = eps_word(p.rng, p.id0 + (uint32_t)n, ((i_first - lane) + lane * step) >> 5);
     pdl_wait();
     float v[32];
-    if constexpr (SRC == SRC_BITS) {
-        planes_to_values<R>(p, v, [&](int pl) { return (int)lane < R ? bits_row_word(p, wsrc, (i_first - lane) + lane * step, pl) : 0u; },
-                            [&](uint32_t mine) { return warp_transpose_bits(mine, lane); });
-    } else {
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = col_load<SRC>(p, wsrc, i_first + r * step, d32);
-        if (SRC == SRC_G32 || SRC == SRC_G16) {
+    for (int r = 0; r < R; ++r) v[r] = col_load<SRC>(p, wsrc, i_first + r * step, d32);
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
-        }
-    }
+    for (int r = 0; r < R; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
     if constexpr (NORM) {
         __shared__ double wsum[8];
         double sum = sum_of_squares<R>(v);
@@ -176,7 +168,7 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
         float v[32];
         if constexpr (SRC == SRC_BITS) {
             float u[32];    // the sixteen rows of the lane's first column, then those of its second
-            planes_to_values<32>(p, u, [&](int pl) { return bits_row_word(p, wsrc, iw, pl); },
+            planes_to_values(p, u, [&](int pl) { return bits_row_word(p, wsrc, iw, pl); },
                                  [&](uint32_t mine) { return column_pair_bits(mine, lane); });
 #pragma unroll
             for (int r = 0; r < 16; ++r) { v[2 * r] = u[r]; v[2 * r + 1] = u[16 + r]; }
@@ -302,7 +294,7 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassP
     const uint32_t i_f = i_tile + w * step + lane;
     const uint32_t step_f = step * WARPS;
     if constexpr (SRC == SRC_BITS) {
-        planes_to_values<32>(p, v, [&](int pl) { return bits_row_word(p, wsrc, irow, pl); },
+        planes_to_values(p, v, [&](int pl) { return bits_row_word(p, wsrc, irow, pl); },
                              [&](uint32_t mine) { return warp_transpose_bits(mine, lane); });
     } else {
 #pragma unroll
@@ -364,7 +356,7 @@ __global__ void __launch_bounds__(1 << (A - 1), 2) col_tile16_kernel(const PassP
     const uint32_t i_f = i_tile + ((w << 1) | h) * step + c;
     const uint32_t step_f = step << (A - 5);
     if constexpr (SRC == SRC_BITS) {
-        planes_to_values<32>(p, v, [&](int pl) { return make_uint2(bits_row_word(p, wsrc, ia, pl), bits_row_word(p, wsrc, ib, pl)); },
+        planes_to_values(p, v, [&](int pl) { return make_uint2(bits_row_word(p, wsrc, ia, pl), bits_row_word(p, wsrc, ib, pl)); },
                              [&](uint2 mine) {
                                  const uint32_t a = __shfl_sync(0xFFFFFFFFu, warp_transpose_bits(mine.x, lane), bitpos);
                                  const uint32_t b = __shfl_sync(0xFFFFFFFFu, warp_transpose_bits(mine.y, lane), bitpos);
@@ -733,14 +725,13 @@ static cudaError_t launch_colh_one(const PassParams& p, cudaStream_t s)
 
 bool colh_applicable(int A, const PassParams& p)
 {
-    return p.P == 1 ? A <= 10 : A <= 9 && (p.K << A) <= 2048;
+    return p.P == 1 ? A >= 2 && A <= 10 : A >= 2 && A <= 9 && (p.K << A) <= 2048;
 }
 
 cudaError_t launch_colh(int A, const PassParams& p, cudaStream_t s)
 {
     if (!colh_applicable(A, p)) return cudaErrorInvalidValue;
     switch (A) {
-        case 1: return launch_colh_one<1>(p, s);
         case 2: return launch_colh_one<2>(p, s);
         case 3: return launch_colh_one<3>(p, s);
         case 4: return launch_colh_one<4>(p, s);
@@ -784,7 +775,9 @@ static cudaError_t launch_col_A(int src, const PassParams& p, cudaStream_t s)
     switch (src) {
         case SRC_G32: return launch_col_one<A, SRC_G32>(p, s);
         case SRC_G16: return launch_col_one<A, SRC_G16>(p, s);
-        case SRC_BITS: return launch_col_one<A, SRC_BITS>(p, s);
+        case SRC_BITS:       // what launch_colh does not take: many planes, or two strided passes without scratch for fp16
+            if constexpr (A == 6 || A >= 8) return launch_col_one<A, SRC_BITS>(p, s);
+            break;
         case SRC_WS:         // the second of two strided passes
             if constexpr (A >= 6 && A <= 9) return launch_col_one<A, SRC_WS>(p, s);
             break;
@@ -798,9 +791,6 @@ static cudaError_t launch_col_A(int src, const PassParams& p, cudaStream_t s)
 cudaError_t launch_col(int A, int src, const PassParams& p, cudaStream_t s)
 {
     switch (A) {
-        case 1: return launch_col_A<1>(src, p, s);
-        case 2: return launch_col_A<2>(src, p, s);
-        case 3: return launch_col_A<3>(src, p, s);
         case 4: return launch_col_A<4>(src, p, s);
         case 5: return launch_col_A<5>(src, p, s);
         case 6: return launch_col_A<6>(src, p, s);

@@ -449,14 +449,13 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
         for (int g = 0; g < (32 >> VB); ++g) {
             const int o = round_F_offset<T>(g);
             float* const x = v + g * VN;
+            static_assert(SRC != SRC_WS || VB >= 1, "an intermediate's tiles of 2^15 are pairs of 2^14");
             if constexpr (VB == 2) {
                 const float4 q = load_cs(reinterpret_cast<const float4*>(src + o));
                 x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
-            } else if constexpr (VB == 1) {
+            } else {
                 const float2 q = load_cs(reinterpret_cast<const float2*>(src + o));
                 x[0] = q.x; x[1] = q.y;
-            } else {
-                x[0] = load_cs(src + o);
             }
         }
     } else if constexpr (SRC == SRC_WS16) {
@@ -470,12 +469,10 @@ __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t 
                 const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q.x));
                 const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&q.y));
                 x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
-            } else if constexpr (VB == 1) {
+            } else {
                 const uint32_t q = load_cs(reinterpret_cast<const uint32_t*>(src + o));
                 const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&q));
                 x[0] = a.x; x[1] = a.y;
-            } else {
-                x[0] = __half2float(load_cs(src + o));
             }
         }
     } else if constexpr (SRC == SRC_BITS_TOP) {
@@ -843,14 +840,11 @@ __global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_strea
                 x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
             } else {
                 const __half* const h = reinterpret_cast<const __half*>(landing) + e0;
-                if constexpr (C::VB == 0) {
-                    x[0] = __half2float(h[0]);
-                } else {
+                static_assert(C::VB >= 1, "an intermediate's tiles of 2^15 are pairs of 2^14");
 #pragma unroll
-                    for (int k = 0; k < VN; k += 2) {
-                        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(h + k));
-                        x[k] = a.x; x[k + 1] = a.y;
-                    }
+                for (int k = 0; k < VN; k += 2) {
+                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(h + k));
+                    x[k] = a.x; x[k + 1] = a.y;
                 }
             }
         }
