@@ -3,6 +3,8 @@
 // and sink of the library in one kernel.  Such calls are all latency: the butterflies cost about a
 // microsecond, and the dithers are shared out over all warps (group of 128 coordinates, range of dithers), so
 // that K = 255 on one transform of 2^9 is 16 generator calls deep instead of one thread's 8160.
+#include <type_traits>
+
 #include "common.cuh"
 #include "dither.cuh"
 
@@ -10,16 +12,20 @@ namespace fosgd {
 
 constexpr int kSmallThreads = 512;   // of the dither sinks (K > 1); 128 otherwise
 
-__global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK p, const int L, const int src, const int sink)
+// PACK: the dither sinks.  The others are compiled without them, with a constant number of threads: many short blocks are bound by
+// instructions and by how many of them fit an SM (2^22 coordinates in blocks of 32, decode: 229 us in one kernel, 121 without).
+// OVERLAP: launched while the kernel in front drains (grids that are not do not pay for the wait).
+template <bool PACK, bool OVERLAP>
+__global__ void __launch_bounds__(PACK ? kSmallThreads : 128)
+small_kernel(const std::conditional_t<PACK, PassParamsRK, PassParams> p, const int L, const int src, const int sink)
 {
     __shared__ float x[512];
     __shared__ float acc[512];
-    __shared__ uint32_t counts[4 * 32];
-    pdl_begin();
+    if constexpr (OVERLAP) pdl_begin();
     const int n = 1 << L;
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, nt = PACK ? (int)blockDim.x : 128;
     const int64_t base = (int64_t)blockIdx.x << L;
-    const bool loop_workers = (sink == SINK_FINAL || sink == SINK_SINGLE);
+    const bool loop_workers = !PACK && sink == SINK_FINAL;
     const int w_begin = loop_workers ? 0 : (int)blockIdx.y;
     const int w_end = loop_workers ? p.nworkers : w_begin + 1;
     for (int e = tid; e < n; e += nt) acc[e] = 0.f;
@@ -56,11 +62,9 @@ __global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK
             }
             __syncthreads();
         }
-        if (sink == SINK_WS) {
-            float* dst = static_cast<float*>(p.dst) + (int64_t)wk * p.dst_stride;
-            for (int e = tid; e < n; e += nt) dst[base + e] = x[e] * p.scale;
-        } else if (sink == SINK_PACK1 || sink == SINK_PACKK) {
+        if constexpr (PACK) {
             // groups of 128 coordinates: four words, or the n / 32 words of a shorter transform inside its group
+            __shared__ uint32_t counts[4 * 32];
             const int warp = tid >> 5, lane = tid & 31, warps = nt / 32;
             const int ngroups = n >= 128 ? n / 128 : 1, nr = n >= 128 ? 4 : n / 32, r_first = (int)(base >> 5) & 3;
             const int share = warps / ngroups;                    // (both powers of two, warps >= 4)
@@ -80,6 +84,9 @@ __global__ void __launch_bounds__(kSmallThreads) small_kernel(const PassParamsRK
             uint32_t* dst = static_cast<uint32_t*>(p.dst) + (int64_t)wk * p.dst_stride + (base >> 5);
             if (warp < ngroups)
                 store_count_planes(counts[32 * warp + lane], (uint32_t)lane, p.P, dst + 4 * warp, p.dp >> 5, n >= 128 ? 0 : r_first, nr);
+        } else if (sink == SINK_WS) {
+            float* dst = static_cast<float*>(p.dst) + (int64_t)wk * p.dst_stride;
+            for (int e = tid; e < n; e += nt) dst[base + e] = x[e] * p.scale;
         } else {
             for (int e = tid; e < n; e += nt) {
                 const int64_t i = base + e;
@@ -104,7 +111,13 @@ cudaError_t launch_small(int L, int src, int sink, const PassParams& p, cudaStre
 {
     if (L < 5 || L > 9) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)(p.dp >> L), sink == SINK_FINAL ? 1u : (unsigned)p.nworkers);
-    return launch<small_kernel>(grid, sink == SINK_PACKK ? kSmallThreads : 128, 0, s, 1, with_round_keys(p), L, src, sink);
+    const unsigned threads = sink == SINK_PACKK ? kSmallThreads : 128;
+    // blocks that walk several workers last: where the grid is neither small nor full, those that start early crowd on the
+    // SMs that have room (2^17 coordinates in blocks of 2^8, eight workers: 28 us overlapped, 21 not)
+    const int64_t limit = sink == SINK_FINAL && p.nworkers > 1 ? 1 << 14 : kOverlapThreads;
+    if (sink == SINK_PACK1 || sink == SINK_PACKK)
+        return launch_either<small_kernel<true, true>, small_kernel<true, false>>(grid, threads, s, limit, with_round_keys(p), L, src, sink);
+    return launch_either<small_kernel<false, true>, small_kernel<false, false>>(grid, threads, s, limit, p, L, src, sink);
 }
 
 }  // namespace fosgd
