@@ -448,13 +448,22 @@ inline cudaError_t sm_count(int* sms)
 }
 
 // Blocks (a power of two, at most the eight of a portable cluster) that share the workers of one tile, when
-// `tiles` blocks alone would leave the chip idle: as many as fit beside each other, at least two workers each.
+// `tiles` blocks alone would leave the chip idle: as many as fit beside each other, at least two workers each.  Starting
+// clusters has its price, so that more than 1024 blocks take at least four workers each and there are never more than 2048
+// (2^20 cut into tiles of 2^10, four workers: 19 us by pairs, 13 alone; 2^21 in blocks of 2^10, 16: 59 and 53; in blocks of
+// 2^11, eight: 25 and 31).
 inline unsigned worker_split(int64_t tiles, int nworkers, int64_t resident_blocks)
 {
     unsigned s = 1;
-    while (s < 8 && tiles * (2 * s) <= resident_blocks && nworkers >= (int)(4 * s)) s *= 2;
+    while (s < 8 && tiles * (2 * s) <= resident_blocks && nworkers >= (int)(4 * s) &&
+           (tiles * (2 * s) <= 1024 || (tiles * (2 * s) <= 2048 && nworkers >= (int)(8 * s)))) s *= 2;
     return s;
 }
+
+// A grid of more than a block per SM and less than a wave, launched while the kernel in front drains, crowds on the SMs that
+// have room at that moment and takes longer than it gains, where its blocks take long (row_stream_kernel, two workers of 2^20 16.5 us and
+// 10.5 launched the ordinary way; three 21.3 and 12.9; 15 dithers of 2^20 in tiles of 2^11 55 and 30).
+inline bool crowds(int64_t threads) { return threads > 1 << 14 && threads < 1 << 17; }
 
 // ---- shared by the translation units of the C-ABI (not exported) -----------------------------
 // thread-local last CUDA error behind fosgd_last_cuda_error()

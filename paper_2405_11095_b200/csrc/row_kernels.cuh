@@ -906,8 +906,10 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
             blocks = (int64_t)sms * min_blocks<T, SINK>();
             if (blocks > ntiles * p.nworkers) blocks = ntiles * p.nworkers;
         }
-        return launch<row_stream_kernel<T, SRC, SINK>>(dim3((unsigned)blocks, split), C::NT, StreamCfg<T, SRC>::SMEM_BYTES, s, split,
-                                                       kernel_params<SINK>(p), ntiles);
+        const dim3 grid((unsigned)blocks, split);
+        if (SINK == SINK_FINAL && crowds(blocks * split * C::NT))
+            return launch<row_stream_kernel<T, SRC, SINK>, false>(grid, C::NT, StreamCfg<T, SRC>::SMEM_BYTES, s, split, kernel_params<SINK>(p), ntiles);
+        return launch<row_stream_kernel<T, SRC, SINK>>(grid, C::NT, StreamCfg<T, SRC>::SMEM_BYTES, s, split, kernel_params<SINK>(p), ntiles);
     } else {
         const dim3 grid((unsigned)ntiles, SINK == SINK_FINAL ? split : (unsigned)p.nworkers);
         constexpr size_t kBytes = SRC == SRC_BITS_TOP ? C::TOP_SMEM_BYTES : C::SMEM_BYTES;
@@ -918,6 +920,9 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
             if (ntiles * grid.y <= sms)
                 return launch<row_kernel<T, SRC, SINK, true>>(grid, C::NT, SINK == SINK_PACK1 ? C::EARLY_SMEM_BYTES : kBytes, s, split, kernel_params<SINK>(p));
         }
+        // (not for clusters, which are placed together, nor for tiles of 2^14 and 2^15, whose set-up the overlap hides)
+        if (SINK == SINK_FINAL && T <= 13 && split == 1 && crowds(ntiles * C::NT))
+            return launch<row_kernel<T, SRC, SINK, false>, false>(grid, C::NT, kBytes, s, split, kernel_params<SINK>(p));
         return launch<row_kernel<T, SRC, SINK, false>>(grid, C::NT, kBytes, s, split, kernel_params<SINK>(p));
     }
 }
