@@ -896,8 +896,20 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
         // parts of the tiles' groups until the blocks fill the chip
         unsigned parts = 1;
         while ((int)parts < PackKCfg<T>::GROUPS && ntiles * p.nworkers * (2 * parts) <= (int64_t)sms * PackKCfg<T>::MIN_BLOCKS) parts *= 2;
-        if (parts == 1 && p.K < kManyDithers)
-            return launch<row_kernel<T, SRC, SINK, false>>(dim3((unsigned)ntiles, (unsigned)p.nworkers), C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p));
+        // large tiles on more than half the SMs: transforming each twice costs more than it spreads (128 tiles of 2^14, K = 3 / 15:
+        // 15.9 / 40.5 us by two blocks each, 12.4 / 35.1 by one; of 2^13 11.0 / 23.5 and 8.4 / 22.8, but K = 23 30.0 and 33.0)
+        const bool whole = 2 * ntiles * p.nworkers > sms && (T == 14 || (T == 13 && p.K <= 16));
+        // (on several waves of tiles of 2^10 and 2^11, which leave most threads of row_packk_kernel out of the transform, up to 28 dithers:
+        // 2^24 in blocks of 2^10, K = 24, 341 us in registers, 363 shared; 2^21 58 and 48)
+        const int64_t threads = ntiles * p.nworkers * C::NT;
+        const int many = T <= 11 && threads >= 1 << 18 ? 28 : kManyDithers;
+        if (p.K < many && (parts == 1 || whole)) {
+            const dim3 grid((unsigned)ntiles, (unsigned)p.nworkers);
+            // (short tiles with more than a few dithers crowd up to 2^17 threads: 2^22, K = 15, 66 us and 62)
+            return crowds(threads) || (T <= 12 && p.K >= kThresholdDithers && threads == 1 << 17)
+                       ? launch<row_kernel<T, SRC, SINK, false>, false>(grid, C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p))
+                       : launch<row_kernel<T, SRC, SINK, false>>(grid, C::NT, C::SMEM_BYTES, s, 1, kernel_params<SINK>(p));
+        }
         return launch<row_packk_kernel<T, SRC>>(dim3((unsigned)ntiles, parts, (unsigned)p.nworkers), PackKCfg<T>::THREADS,
                                                 PackKCfg<T>::SMEM_BYTES, s, 1, with_round_keys(p));
     } else if constexpr (kStream) {
