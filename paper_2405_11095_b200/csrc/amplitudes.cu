@@ -88,12 +88,12 @@ __global__ void __launch_bounds__(256) amplitudes_finalize_kernel(const double* 
 // ---- one amplitude per worker and block ----------------------------------------------------
 // Each warp sums the squares of 1024 consecutive coordinates in 32 coalesced steps and emits the
 // sum of every segment of 2^s of them, s = min(b, 10): the block sums themselves for b <= 10,
-// partials of 1024 coordinates for larger blocks.
-template <bool BF16>
+// partials of 1024 coordinates for larger blocks.  (OVERLAP: launched while the kernel in front drains.)
+template <bool BF16, bool OVERLAP>
 __global__ void __launch_bounds__(128) segment_sumsq_kernel(const void* grads, int64_t d, int64_t dp, int64_t worker_stride,
                                                             int s, double* seg)
 {
-    pdl_begin();
+    if constexpr (OVERLAP) pdl_begin();
     const int n = blockIdx.y;
     const uint32_t lane = threadIdx.x & 31u;
     const int64_t warp_base = ((int64_t)blockIdx.x * 4 + (threadIdx.x >> 5)) << 10;
@@ -149,10 +149,11 @@ __global__ void __launch_bounds__(128) segment_sumsq_kernel(const void* grads, i
 
 // One warp per (worker, block): adds the block's segment sums lane-strided, then across lanes,
 // always in the same order.
+template <bool OVERLAP>
 __global__ void __launch_bounds__(128) block_amplitudes_kernel(const double* seg, int64_t nb, int64_t segs_per_block,
                                                                int M, double alpha, double n_eff, float* lam)
 {
-    pdl_begin();
+    if constexpr (OVERLAP) pdl_begin();
     const int64_t w = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     const uint32_t lane = threadIdx.x & 31u;
     if (w >= nb * M) return;
@@ -182,8 +183,8 @@ cudaError_t launch_block_amplitudes(const void* grads, int bf16, int64_t d, int6
     const int s = block_log2 < 10 ? block_log2 : 10;
     const int64_t nb = dp >> block_log2;
     const dim3 grid((unsigned)((dp + 4095) >> 12), (unsigned)M);
-    cudaError_t e = bf16 ? launch<segment_sumsq_kernel<true>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg)
-                         : launch<segment_sumsq_kernel<false>>(grid, 128, 0, st, 1, grads, d, dp, worker_stride, s, seg);
+    cudaError_t e = bf16 ? launch_either<segment_sumsq_kernel<true, true>, segment_sumsq_kernel<true, false>>(grid, 128, st, kOverlapThreads, grads, d, dp, worker_stride, s, seg)
+                         : launch_either<segment_sumsq_kernel<false, true>, segment_sumsq_kernel<false, false>>(grid, 128, st, kOverlapThreads, grads, d, dp, worker_stride, s, seg);
     if (e != cudaSuccess) return e;
     return launch_block_amplitudes_finalize(seg, (int64_t)1 << (block_log2 - s), nb, M, block_log2, alpha, alpha_s, lam, lam_s, st);
 }
@@ -192,8 +193,8 @@ cudaError_t launch_block_amplitudes_finalize(const double* seg, int64_t parts, i
                                              double alpha_s, float* lam, float* lam_s, cudaStream_t st)
 {
     const int64_t warps = nb * M;
-    const cudaError_t e = launch<block_amplitudes_kernel>(dim3((unsigned)((warps + 3) / 4)), 128, 0, st, 1, seg, nb, parts, M, alpha,
-                                                          (double)((int64_t)1 << block_log2), lam);
+    const cudaError_t e = launch_either<block_amplitudes_kernel<true>, block_amplitudes_kernel<false>>(
+        dim3((unsigned)((warps + 3) / 4)), 128, st, kOverlapThreads, seg, nb, parts, M, alpha, (double)((int64_t)1 << block_log2), lam);
     if (e != cudaSuccess || lam_s == nullptr) return e;
     return launch_server_amplitudes(lam, nb, M, block_log2, alpha_s, lam_s, st);
 }

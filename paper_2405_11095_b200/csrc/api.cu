@@ -694,8 +694,11 @@ int fosgd_amplitudes(const void* grads, int dtype, int64_t d, int64_t worker_str
     const bool on = g_trace_events != nullptr && g_trace_count < g_trace_capacity && g_trace_count < kTraceMax;
     if (on) cudaEventRecord(g_trace_events[2 * g_trace_count], (cudaStream_t)stream);
     cudaError_t e;
-    if (per_block && block_log2 >= 10 && block_log2 <= 15) {
-        // a block is a tile: the same sums, in the same order, as the encoder that measures its own blocks
+    // Blocks of 2^10 (a warp to a thread block) and 2^15 (one thread block to an SM, narrow loads) are the segments' kernel's on long
+    // inputs: 16 x 2^23 bf16 140 and 107 us by tiles, 118 and 88 by segments; 2^20 the other way round, 6 and 9 us (a launch fewer).
+    const bool tiles = block_log2 >= 10 && block_log2 <= 15 && ((block_log2 > 10 && block_log2 < 15) || g.dp * M <= (int64_t)1 << 24);
+    if (per_block && tiles) {
+        // a block is a tile: one kernel
         PassParams p{};
         p.src = grads; p.src_stride = worker_stride; p.d = d; p.dp = g.dp; p.nworkers = M;
         p.amp_out = lambda_dev; p.amp_stride = g.dp >> block_log2; p.amp_factor = block_amplitude_factor(alpha, block_log2);

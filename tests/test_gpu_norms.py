@@ -38,6 +38,7 @@ def norms(grads, d, dp, b):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("d,M,b", [
     (3 * 512 - 7, 2, 9), (9 * 1024 + 1, 2, 10), (5 * (1 << 13) - 3, 3, 13), (3 * (1 << 15) + 77, 2, 15),
+    ((1 << 24) + 5, 1, 10), ((1 << 24) + 5, 1, 15),   # long inputs: by segments, where shorter ones go by tiles
     (3 * (1 << 16) + 9, 2, 16),                    # the strided pass carries the sums: four stages, ..
     ((9 << 16) + 31, 2, 16),                       # a cluster of thread blocks holds the block
     (3 * (1 << 17) - 3, 2, 17), (3 << 20, 2, 20), ((1 << 22) + 12345, 2, 22), ((1 << 23) - 1, 2, 23),   # .. up to eight; none
