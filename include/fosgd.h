@@ -203,11 +203,11 @@ int fosgd_downlink_apply(const uint32_t* down_bits, int64_t d, uint64_t seed, ui
  * usual case that the gradients just encoded are the ones whose norm sets the amplitude (Theorem 5.5 with
  * B = max_n ||g_n||_2 over the M workers of the call).  lambda_dev (and lambda_s_dev, nullable) receive the
  * amplitudes as fosgd_amplitudes writes them; the packed signs are those of fosgd_encode_dev with that lambda.
- * Where the strided pass of the encoder can carry the sums (fp32 gradients, transform lengths 2^17 .. 2^22, 2^24
- * and 2^25 in global or blocked mode, `ws` holding all M workers) the gradients are read once instead of twice;
- * elsewhere the call runs the two calls one after the other.  The sums are added in a fixed order, so the
+ * Where the strided pass of the encoder can carry the sums (fp32 gradients, transform lengths 2^17 .. 2^24
+ * in global or blocked mode, `ws` holding all M workers) the gradients are read once instead of twice;
+ * elsewhere the call runs the two calls one after the other.  The sums are fp64 and added in a fixed order, so the
  * amplitudes are reproducible, but in another order than fosgd_amplitudes uses: the two may differ in the
- * last bit.  amp_ws: scratch of fosgd_workspace_bytes(FOSGD_OP_AMPLITUDES, ..., M, ...) bytes. */
+ * last bit.  `bits` may hold sums until the signs are written.  amp_ws: scratch of fosgd_workspace_bytes(FOSGD_OP_AMPLITUDES, ..., M, ...) bytes. */
 int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worker_stride, int M, uint32_t worker_id0,
                           uint64_t seed, uint64_t step, double alpha, double alpha_s, int block_log2, float* lambda_dev,
                           float* lambda_s_dev, uint32_t* bits, void* ws, size_t ws_bytes, void* amp_ws,
@@ -216,7 +216,8 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
 /* The same for one amplitude per worker and block of the blocked mode (block_log2 >= 5): fosgd_amplitudes with per_block = 1
  * and fosgd_encode_dev in one call.  lambda_dev: [M][d' >> block_log2], lambda_s_dev: [d' >> block_log2] (nullable).  Where one
  * thread block transforms a whole block of the gradient (2^10 .. 2^15), or the strided pass can carry the sums (2^16 .. 2^22,
- * `ws` holding all M workers), the gradients are read once.  amp_ws: scratch of FOSGD_OP_BLOCK_AMPLITUDES. */
+ * `ws` holding all M workers), the gradients are read once; the amplitudes may then differ from fosgd_amplitudes' in the last
+ * bit.  amp_ws: scratch of FOSGD_OP_BLOCK_AMPLITUDES. */
 int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_t worker_stride, int M, uint32_t worker_id0,
                                  uint64_t seed, uint64_t step, double alpha, double alpha_s, int block_log2, float* lambda_dev,
                                  float* lambda_s_dev, uint32_t* bits, void* ws, size_t ws_bytes, void* amp_ws,

@@ -58,6 +58,26 @@ __global__ void __launch_bounds__(256) sumsq_partial_kernel(const void* grads, i
     if (threadIdx.x == 0) partial[(int64_t)n * gridDim.x + blockIdx.x] = red[0];
 }
 
+// [M][nparts] sums to [M][gridDim.x]: block k adds its share of consecutive parts, lane-strided, then across lanes and warps
+__global__ void __launch_bounds__(128) sum_parts_kernel(const double* parts, int64_t nparts, double* sums)
+{
+    __shared__ double wsum[4];
+    pdl_begin();
+    const double* const row = parts + (int64_t)blockIdx.y * nparts;
+    double acc = 0.0;
+    for (int64_t i = nparts * blockIdx.x / gridDim.x + threadIdx.x; i < nparts * (blockIdx.x + 1) / gridDim.x; i += 128) acc += row[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+    if ((threadIdx.x & 31u) == 0) wsum[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) sums[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]);
+}
+
+cudaError_t launch_sum_parts(const double* parts, int64_t nparts, int M, double* sums, int nsums, cudaStream_t s)
+{
+    return launch<sum_parts_kernel>(dim3((unsigned)nsums, (unsigned)M), 128, 0, s, 1, parts, nparts, sums);
+}
+
 __global__ void __launch_bounds__(256) amplitudes_finalize_kernel(const double* partial, int M, int nblocks, double alpha,
                                                                   double alpha_s, double n_eff, float* lam_out, float* lam_s_out)
 {

@@ -748,7 +748,7 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
         bool launched = false;
         int nruns = 0;
         bool on = trace_begin(s);
-        cudaError_t e = launch_col_norm(pl.A[0], pc, static_cast<double*>(amp_ws), s, &launched, &nruns);
+        cudaError_t e = launch_col_norm(pl.A[0], pc, static_cast<double*>(amp_ws), reinterpret_cast<double*>(bits), s, &launched, &nruns);
         if (launched) trace_end(on, s, TraceEntry{'c', pl.A[0], SRC_G32, SINK_WS, M, false});
         if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; }
         if (launched) {

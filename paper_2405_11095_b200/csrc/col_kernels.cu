@@ -85,6 +85,21 @@ __device__ __forceinline__ void planes_to_values(const PassParams& p, float (&v)
     }
 }
 
+// the sum over a block of W warps, lanes first, to partial[worker * gridDim.x + block]
+template <uint32_t W>
+__device__ __forceinline__ void leave_block_sum(double sum, double* partial)
+{
+    __shared__ double wsum[W];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+    if ((threadIdx.x & 31u) == 0) wsum[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (uint32_t k = 1; k < W; ++k) sum += wsum[k];
+        partial[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = sum;
+    }
+}
+
 // ---- A = 4, from gradients ----------------------------------------------------------------
 // NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
 template <int A, int SRC, bool NORM>
@@ -111,18 +126,7 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
     for (int r = 0; r < R; ++r) v[r] = col_load<SRC>(p, wsrc, i_first + r * step, d32);
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, myword, r), 31u - lane);
-    if constexpr (NORM) {
-        __shared__ double wsum[8];
-        double sum = sum_of_squares<R>(v);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        if (lane == 0) wsum[threadIdx.x >> 5] = sum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int k = 1; k < 8; ++k) sum += wsum[k];
-            partial[(int64_t)n * gridDim.x + blockIdx.x] = sum;
-        }
-    }
+    if constexpr (NORM) leave_block_sum<8>(sum_of_squares<R>(v), partial);
 #pragma unroll
     for (int r = R; r < 32; ++r) v[r] = 0.f;
     butterflies32<R - 1>(v);
@@ -137,10 +141,9 @@ __global__ void __launch_bounds__(256) col_small_kernel(const PassParams p, doub
 // Bound by memory: 2^27 coordinates of fp32 gradients take 0.17 ms at A = 8 (6.3 TB/s of the 6.5 a plain copy
 // reaches), where tiles of 16 columns (64-byte segments) took 0.21 ms; with rows megabytes apart (the top pass
 // of a 2^31 transform) the segment width decides: 5.8 ms with 64 bytes per row visit at A = 8, 2.9 ms with 256.
-// NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block]
-// (fp64, fixed order); blocks then take tiles gridDim.x apart.
+// NORM: also leave the sum of squares of each block's gradient entries in partial[worker * gridDim.x + block] (fp64, fixed order)
 template <int A, int SRC, bool NORM>
-__global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams p, const uint32_t ntiles, double* const partial)
+__global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams p, double* const partial)
 {
     extern __shared__ __align__(16) float2 tile2[];
     constexpr uint32_t WARPS = 1u << (A - 4);
@@ -153,126 +156,111 @@ __global__ void __launch_bounds__(2 << A, 512 >> A) col2_kernel(const PassParams
     const void* const wsrc = worker_source<SRC>(p, n);
     float* const dst = static_cast<float*>(p.dst) + (int64_t)n * p.dst_stride;
     constexpr bool kGrad = SRC == SRC_G32 || SRC == SRC_G16;
+    const uint32_t seg = blockIdx.x;                              // 64-column segment id
     double sumsq = 0.0;
-
-    for (uint32_t seg = blockIdx.x; seg < ntiles; seg += gridDim.x) {
-        const uint32_t lo0 = (seg << 6) & (step - 1u);
-        const uint32_t hi = (uint32_t)(((uint64_t)seg << 6) >> p.lo_log);
-        const uint32_t i_tile = (hi << (p.lo_log + A)) + lo0;     // row 0, column 0 of the tile
-        // round F: rows k = r * WARPS + w
-        const uint32_t i_f = i_tile + w * step + 2u * lane;
-        const uint32_t step_f = step * WARPS;
-        // the two words (flips, or packed signs) of row r belong to lanes r and 16 + r
-        const uint32_t iw = i_tile + w * step + (lane & 15u) * step_f + 32u * (lane >> 4);
-        const uint32_t from = lane & 16u, bit = (2u * lane) & 31u;
-        float v[32];
-        if constexpr (SRC == SRC_BITS) {
-            float u[32];    // the sixteen rows of the lane's first column, then those of its second
-            planes_to_values(p, u, [&](int pl) { return bits_row_word(p, wsrc, iw, pl); },
-                                 [&](uint32_t mine) { return column_pair_bits(mine, lane); });
+    const uint32_t lo0 = (seg << 6) & (step - 1u);
+    const uint32_t hi = (uint32_t)(((uint64_t)seg << 6) >> p.lo_log);
+    const uint32_t i_tile = (hi << (p.lo_log + A)) + lo0;     // row 0, column 0 of the tile
+    // round F: rows k = r * WARPS + w
+    const uint32_t i_f = i_tile + w * step + 2u * lane;
+    const uint32_t step_f = step * WARPS;
+    // the two words (flips, or packed signs) of row r belong to lanes r and 16 + r
+    const uint32_t iw = i_tile + w * step + (lane & 15u) * step_f + 32u * (lane >> 4);
+    const uint32_t from = lane & 16u, bit = (2u * lane) & 31u;
+    float v[32];
+    if constexpr (SRC == SRC_BITS) {
+        float u[32];    // the sixteen rows of the lane's first column, then those of its second
+        planes_to_values(p, u, [&](int pl) { return bits_row_word(p, wsrc, iw, pl); },
+                             [&](uint32_t mine) { return column_pair_bits(mine, lane); });
 #pragma unroll
-            for (int r = 0; r < 16; ++r) { v[2 * r] = u[r]; v[2 * r + 1] = u[16 + r]; }
-        } else if constexpr (kGrad) {
-            // a tile whose last coordinate is inside the gradient: all sixteen loads in flight, no checks
-            const bool whole = i_tile + ((1u << A) - 1u) * step + 63u < d32;
-            if constexpr (SRC == SRC_G32) {
-                auto load2 = [&](int r) {
-                    const float2 q = load_cs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f));
-                    v[2 * r] = q.x; v[2 * r + 1] = q.y;
-                };
-                if (whole) {
+        for (int r = 0; r < 16; ++r) { v[2 * r] = u[r]; v[2 * r + 1] = u[16 + r]; }
+    } else if constexpr (kGrad) {
+        // a tile whose last coordinate is inside the gradient: all sixteen loads in flight, no checks
+        const bool whole = i_tile + ((1u << A) - 1u) * step + 63u < d32;
+        if constexpr (SRC == SRC_G32) {
+            auto load2 = [&](int r) {
+                const float2 q = load_cs(reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f));
+                v[2 * r] = q.x; v[2 * r + 1] = q.y;
+            };
+            if (whole) {
 #pragma unroll
-                    for (int r = 0; r < 16; ++r) load2(r);
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) {
-                        v[2 * r] = v[2 * r + 1] = 0.f;
-                        if (i_f + r * step_f + 1u < d32) load2(r);
-                    }
-                }
+                for (int r = 0; r < 16; ++r) load2(r);
             } else {
-                // raw pairs first: widening each one where it is loaded would make the checked loads wait for one another
-                // (2^32 padded coordinates, seven stages, 61% of the rows inside the gradient: 5.34 ms so)
-                uint32_t q[16];
-                auto load2 = [&](int r) { return load_cs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i_f + r * step_f)); };
-                if (whole) {
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) q[r] = load2(r);
-                } else {
-#pragma unroll
-                    for (int r = 0; r < 16; ++r) {
-                        q[r] = 0u;
-                        if (i_f + r * step_f + 1u < d32) q[r] = load2(r);
-                    }
-                }
 #pragma unroll
                 for (int r = 0; r < 16; ++r) {
-                    v[2 * r] = __uint_as_float(q[r] << 16); v[2 * r + 1] = __uint_as_float(q[r] & 0xFFFF0000u);
+                    v[2 * r] = v[2 * r + 1] = 0.f;
+                    if (i_f + r * step_f + 1u < d32) load2(r);
                 }
             }
-            if (!whole && (d32 & 1u)) {       // an odd length ends inside a pair
-#pragma unroll
-                for (int r = 0; r < 16; ++r)
-                    if (i_f + r * step_f + 1u == d32) v[2 * r] = col_load<SRC>(p, wsrc, d32 - 1u, d32);
-            }
-            const uint32_t mine = eps_word(p.rng, p.id0 + (uint32_t)n, iw >> 5);
-            const uint32_t sh = 31u - bit;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, r + (int)from);
-                v[2 * r] = flip_shifted(v[2 * r], word, sh);
-                v[2 * r + 1] = flip_shifted(v[2 * r + 1], word, sh - 1u);
-            }
-        } else if constexpr (SRC == SRC_WS) {
-#pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const float2 q = *reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f);
-                v[2 * r] = q.x; v[2 * r + 1] = q.y;
-            }
         } else {
+            // raw pairs first: widening each one where it is loaded would make the checked loads wait for one another
+            // (2^32 padded coordinates, seven stages, 61% of the rows inside the gradient: 5.34 ms so)
+            uint32_t q[16];
+            auto load2 = [&](int r) { return load_cs(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(wsrc) + i_f + r * step_f)); };
+            if (whole) {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) q[r] = load2(r);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    q[r] = 0u;
+                    if (i_f + r * step_f + 1u < d32) q[r] = load2(r);
+                }
+            }
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
-                const float2 q = __half22float2(*reinterpret_cast<const __half2*>(static_cast<const __half*>(wsrc) + i_f + r * step_f));
-                v[2 * r] = q.x; v[2 * r + 1] = q.y;
+                v[2 * r] = __uint_as_float(q[r] << 16); v[2 * r + 1] = __uint_as_float(q[r] & 0xFFFF0000u);
             }
         }
-        if constexpr (NORM) {
-            sumsq += sum_of_squares(v);
-        }
-        butterflies32<30>(v);
-        if (NORM) __syncthreads();                                 // readers of the previous tile
+        if (!whole && (d32 & 1u)) {       // an odd length ends inside a pair
 #pragma unroll
-        for (int r = 0; r < 16; ++r) tile2[((r * WARPS + w) << 5) + lane] = make_float2(v[2 * r], v[2 * r + 1]);
-        __syncthreads();
-        // round L: rows k = w * 16 + r (the low A - 4 bits are new)
+            for (int r = 0; r < 16; ++r)
+                if (i_f + r * step_f + 1u == d32) v[2 * r] = col_load<SRC>(p, wsrc, d32 - 1u, d32);
+        }
+        const uint32_t mine = eps_word(p.rng, p.id0 + (uint32_t)n, iw >> 5);
+        const uint32_t sh = 31u - bit;
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
-            const float2 q = tile2[((w * 16u + r) << 5) + lane];
+            const uint32_t word = __shfl_sync(0xFFFFFFFFu, mine, r + (int)from);
+            v[2 * r] = flip_shifted(v[2 * r], word, sh);
+            v[2 * r + 1] = flip_shifted(v[2 * r + 1], word, sh - 1u);
+        }
+    } else if constexpr (SRC == SRC_WS) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const float2 q = *reinterpret_cast<const float2*>(static_cast<const float*>(wsrc) + i_f + r * step_f);
             v[2 * r] = q.x; v[2 * r + 1] = q.y;
         }
-        butterflies32<((1 << (A - 4)) - 1) << 1>(v);
-        const uint32_t i_l = i_tile + (w * 16u) * step + 2u * lane;
+    } else {
 #pragma unroll
-        for (int r = 0; r < 16; ++r)
-            __stcg(reinterpret_cast<float2*>(dst + i_l + r * step), make_float2(v[2 * r], v[2 * r + 1]));   // L2 only: read next by another kernel
-    }
-    if constexpr (NORM) {
-        __shared__ double wsum[WARPS];
-#pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) sumsq += __shfl_xor_sync(0xFFFFFFFFu, sumsq, s);
-        if (lane == 0) wsum[w] = sumsq;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double total = 0.0;
-            for (uint32_t k = 0; k < WARPS; ++k) total += wsum[k];
-            partial[(int64_t)n * gridDim.x + blockIdx.x] = total;
+        for (int r = 0; r < 16; ++r) {
+            const float2 q = __half22float2(*reinterpret_cast<const __half2*>(static_cast<const __half*>(wsrc) + i_f + r * step_f));
+            v[2 * r] = q.x; v[2 * r + 1] = q.y;
         }
     }
+    if constexpr (NORM) sumsq = sum_of_squares(v);
+    butterflies32<30>(v);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) tile2[((r * WARPS + w) << 5) + lane] = make_float2(v[2 * r], v[2 * r + 1]);
+    __syncthreads();
+    // round L: rows k = w * 16 + r (the low A - 4 bits are new)
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const float2 q = tile2[((w * 16u + r) << 5) + lane];
+        v[2 * r] = q.x; v[2 * r + 1] = q.y;
+    }
+    butterflies32<((1 << (A - 4)) - 1) << 1>(v);
+    const uint32_t i_l = i_tile + (w * 16u) * step + 2u * lane;
+#pragma unroll
+    for (int r = 0; r < 16; ++r)
+        __stcg(reinterpret_cast<float2*>(dst + i_l + r * step), make_float2(v[2 * r], v[2 * r + 1]));   // L2 only: read next by another kernel
+    if constexpr (NORM) leave_block_sum<WARPS>(sumsq, partial);
 }
 
 // ---- A = 9, 10 ---------------------------------------------------------------------------
-template <int A, int SRC>
-__global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassParams p)
+// NORM: as in col2_kernel
+template <int A, int SRC, bool NORM>
+__global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassParams p, double* const partial)
 {
     extern __shared__ __align__(16) float smem[];  // 2^A rows x 32 columns
     constexpr int WARPS = 1 << (A - 5);
@@ -305,6 +293,8 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassP
             for (int r = 0; r < 32; ++r) v[r] = flip_shifted(v[r], __shfl_sync(0xFFFFFFFFu, mine, r), 31u - lane);
         }
     }
+    double sumsq = 0.0;
+    if constexpr (NORM) sumsq = sum_of_squares(v);
     butterflies32<31>(v);
 #pragma unroll
     for (int r = 0; r < 32; ++r) smem[((r * WARPS + w) << 5) + lane] = v[r];
@@ -317,6 +307,7 @@ __global__ void __launch_bounds__(1 << A, 1024 >> A) col_tile_kernel(const PassP
     const uint32_t i_l = i_tile + (w * 32) * step + lane;
 #pragma unroll
     for (int r = 0; r < 32; ++r) __stcg(dst + i_l + r * step, v[r]);   // L2 only: read next by another kernel
+    if constexpr (NORM) leave_block_sum<WARPS>(sumsq, partial);
 }
 
 // ---- A > 5, 16-column tiles ----------------------------------------------------------------
@@ -486,43 +477,49 @@ static cudaError_t launch_col4(const PassParams& p, cudaStream_t s, bool* launch
 }
 
 template <int A, int SRC, bool NORM>
-static cudaError_t launch_col2(const PassParams& p, uint32_t blocks, double* partial, cudaStream_t s)
+static cudaError_t launch_col2(const PassParams& p, double* partial, cudaStream_t s)
 {
-    return launch<col2_kernel<A, SRC, NORM>>(dim3(blocks, (unsigned)p.nworkers), 2 << A, (size_t)(1 << A) * 256, s, 1, p,
-                                             (uint32_t)((p.dp >> A) / 64), partial);
+    return launch<col2_kernel<A, SRC, NORM>>(dim3((unsigned)((p.dp >> A) / 64), (unsigned)p.nworkers), 2 << A, (size_t)(1 << A) * 256, s, 1, p, partial);
+}
+
+template <int A, int SRC, bool NORM>
+static cudaError_t launch_col_tile(const PassParams& p, double* partial, cudaStream_t s)
+{
+    return launch<col_tile_kernel<A, SRC, NORM>>(dim3((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers), 1 << A, (size_t)(1 << A) * 128, s, 1, p, partial);
 }
 
 // Strided pass on fp32 gradients with the squared norm of every worker's gradient gathered on the way: sums of
-// parts in partial[worker][part], *nparts_out (at most 256, what the caller's scratch holds) of them per worker.
-// *launched stays false where no kernel carries the sums: nine stages, rows 128 KiB apart or more at ten, more
-// than 256 runs per worker, map refused.
-cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nparts_out)
+// parts in sums[worker][part], *nparts_out (at most 256, what the caller's scratch holds) of them per worker.  A pass of more
+// parts leaves them in `room` (8 bytes per 2^11 coordinates at most: the packed words that the next kernel writes take 2^8), for a second
+// kernel to add up.  (Blocks that walk tiles 256 apart instead: one worker of 2^25 in blocks of 2^20 187 us, the norm pass of its own 139.)
+// *launched stays false where no kernel carries the sums: four stages, rows 128 KiB apart or more at ten, map refused.
+cudaError_t launch_col_norm(int A, const PassParams& p, double* sums, double* room, cudaStream_t s, bool* launched, int* nparts_out)
 {
     constexpr int64_t kMaxParts = 256;
     *launched = false;
-    if (A >= 5 && A <= 8) {
-        const int64_t ntiles = (p.dp >> A) / 64;
-        const uint32_t blocks = (uint32_t)(ntiles < kMaxParts ? ntiles : kMaxParts);
-        *launched = true;
-        *nparts_out = (int)blocks;
+    const int64_t parts = A == 10 ? ((p.dp >> A) / 16) / 8 : (p.dp >> A) / (A == 9 ? 32 : 64);      // runs, tiles
+    double* const partial = parts > kMaxParts ? room : sums;
+    cudaError_t e;
+    if (A == 10) {
+        const uint64_t S = (uint64_t)1 << p.lo_log;
+        const uint64_t rows = (uint64_t)(p.d >> p.lo_log);
+        if (p.lo_log >= 15 || S < 128 || ((p.dp >> A) / 16) % 8 != 0 || parts * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
+        CUtensorMap map;
+        if (!make_col_tensor_map(&map, p.src, S, rows, (uint64_t)p.nworkers, (uint64_t)p.src_stride)) return cudaSuccess;
+        e = launch<col4_norm_kernel>(dim3((unsigned)(parts * p.nworkers)), 512, Col4::SMEM_BYTES, s, 1, p, map, (int)parts, (uint32_t)rows, partial);
+    } else {
         switch (A) {
-            case 5: return launch_col2<5, SRC_G32, true>(p, blocks, partial, s);
-            case 6: return launch_col2<6, SRC_G32, true>(p, blocks, partial, s);
-            case 7: return launch_col2<7, SRC_G32, true>(p, blocks, partial, s);
-            default: return launch_col2<8, SRC_G32, true>(p, blocks, partial, s);
+            case 5: e = launch_col2<5, SRC_G32, true>(p, partial, s); break;
+            case 6: e = launch_col2<6, SRC_G32, true>(p, partial, s); break;
+            case 7: e = launch_col2<7, SRC_G32, true>(p, partial, s); break;
+            case 8: e = launch_col2<8, SRC_G32, true>(p, partial, s); break;
+            case 9: e = launch_col_tile<9, SRC_G32, true>(p, partial, s); break;
+            default: return cudaSuccess;
         }
     }
-    if (A != 10) return cudaSuccess;
-    const uint64_t S = (uint64_t)1 << p.lo_log;
-    const uint64_t rows = (uint64_t)(p.d >> p.lo_log);
-    const int64_t nsegs = (p.dp >> A) / 16;
-    const int64_t nruns = nsegs / 8;
-    if (p.lo_log >= 15 || S < 128 || nsegs % 8 != 0 || nruns > kMaxParts || nruns * p.nworkers > 0x7FFFFFFF) return cudaSuccess;
-    CUtensorMap map;
-    if (!make_col_tensor_map(&map, p.src, S, rows, (uint64_t)p.nworkers, (uint64_t)p.src_stride)) return cudaSuccess;
     *launched = true;
-    *nparts_out = (int)nruns;
-    return launch<col4_norm_kernel>(dim3((unsigned)(nruns * p.nworkers)), 512, Col4::SMEM_BYTES, s, 1, p, map, (int)nruns, (uint32_t)rows, partial);
+    *nparts_out = (int)(parts > kMaxParts ? kMaxParts : parts);
+    return e == cudaSuccess && parts > kMaxParts ? launch_sum_parts(room, parts, p.nworkers, sums, (int)kMaxParts, s) : e;
 }
 
 template <int SRC>
@@ -535,10 +532,10 @@ static cudaError_t launch_col_block_norm_src(int A, const PassParams& p, double*
     }
     *parts = (p.dp >> A) / 64;
     switch (A) {
-        case 5: return launch_col2<5, SRC, true>(p, (uint32_t)*parts, partial, s);
-        case 6: return launch_col2<6, SRC, true>(p, (uint32_t)*parts, partial, s);
-        case 7: return launch_col2<7, SRC, true>(p, (uint32_t)*parts, partial, s);
-        case 8: return launch_col2<8, SRC, true>(p, (uint32_t)*parts, partial, s);
+        case 5: return launch_col2<5, SRC, true>(p, partial, s);
+        case 6: return launch_col2<6, SRC, true>(p, partial, s);
+        case 7: return launch_col2<7, SRC, true>(p, partial, s);
+        case 8: return launch_col2<8, SRC, true>(p, partial, s);
     }
     *launched = false;
     return cudaSuccess;
@@ -751,11 +748,11 @@ static cudaError_t launch_col_one(const PassParams& p, cudaStream_t s)
     if constexpr (A <= 4) {
         return launch<col_small_kernel<A, SRC, false>>(dim3((unsigned)((p.dp >> A) / 256), (unsigned)p.nworkers), 256, 0, s, 1, p, nullptr);
     } else if constexpr (A <= 8) {
-        return launch_col2<A, SRC, false>(p, (uint32_t)((p.dp >> A) / 64), nullptr, s);
+        return launch_col2<A, SRC, false>(p, nullptr, s);
     } else if constexpr (A == 9) {
         // 32 columns: two blocks of 512 threads per SM, 128-byte row segments (0.20 ms on 2^27 coordinates against
         // 0.24 ms with tiles of 16 columns)
-        return launch<col_tile_kernel<A, SRC>>(dim3((unsigned)((p.dp >> A) / 32), (unsigned)p.nworkers), 1 << A, (size_t)(1 << A) * 128, s, 1, p);
+        return launch_col_tile<A, SRC, false>(p, nullptr, s);
     } else {
         // ten stages on fp32 gradients: the copy-engine kernels, unless the driver refuses the tensor map
         if constexpr (SRC == SRC_G32) {

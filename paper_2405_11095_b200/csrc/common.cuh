@@ -497,7 +497,8 @@ cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t wo
                               double alpha_s, double n_eff, float* lam, float* lam_s, double* partial, cudaStream_t s);
 cudaError_t launch_amplitudes_finalize(const double* partial, int M, int nparts, double alpha, double alpha_s, double n_eff,
                                        float* lam, float* lam_s, cudaStream_t s);
-cudaError_t launch_col_norm(int A, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int* nparts_out);
+cudaError_t launch_col_norm(int A, const PassParams& p, double* sums, double* room, cudaStream_t s, bool* launched, int* nparts_out);
+cudaError_t launch_sum_parts(const double* parts, int64_t nparts, int M, double* sums, int nsums, cudaStream_t s);
 // strided pass that also leaves every tile's sum of squares in partial[worker][tile]; *launched stays false where no kernel
 // carries them
 cudaError_t launch_col_block_norm(int A, int src, const PassParams& p, double* partial, cudaStream_t s, bool* launched, int64_t* parts_per_worker);

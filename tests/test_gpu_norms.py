@@ -94,3 +94,26 @@ def test_one_amplitude_at_the_ends_of_the_range(F, L, scale):
         assert abs(float(lam) - ref) <= RTOL * ref, (workers, float(lam), ref)
         ref_s = 2.0 * ref * np.sqrt(np.log(n))
         assert abs(float(lam_s) - ref_s) <= RTOL * ref_s
+
+
+@pytest.mark.parametrize("d,b,M", [
+    ((5 << 17) + 1, 17, 3), ((3 << 18) - 1, 18, 2), ((3 << 20) - 5, 20, 2), ((3 << 22) - 7, 22, 1), ((1 << 23) - 3, 0, 2), ((3 << 23) + 1, 23, 1),
+    ((3 << 24) - 9, 24, 1),
+    ((1 << 20) + 1, 20, 1), (4 << 16, 16, 2),           # up to 256 sums; no kernel that carries them
+])
+def test_one_amplitude_of_a_long_vector(F, d, b, M):
+    """More sums per worker than the scratch of the norms holds (256): they wait in the output and are added up there, and
+    the packed words come out whole."""
+    dp, n = F.padded_dim(d, b), float(F.transform_len(d, b))
+    grads = scaled(M, d, torch.float32, lambda w, i: torch.full_like(i, 1) + (i == 12345).long())     # one entry of 1e20
+    stride = grads.shape[1]
+    ref = 2.0 * max(float(grads[w, :d].double().norm()) for w in range(M)) * np.sqrt(np.log(n) / n)
+    amp_ws = torch.empty(F.workspace_bytes(F.OP_AMPLITUDES, d, M=M), dtype=torch.uint8, device=DEV)
+    ws = torch.empty(M * F.workspace_bytes(F.OP_ENCODE, d, block_log2=b), dtype=torch.uint8, device=DEV)
+    lam, lam_s = torch.full((2, 1), 7.0, device=DEV)
+    bits, again = torch.zeros(2, M, dp // 32, dtype=torch.int32, device=DEV)
+    F.encode_measured(grads, d, bits, lam, lam_s, 5, 1, alpha=2.0, alpha_s=2.0, block_log2=b, ws=ws, amp_ws=amp_ws, worker_stride=stride)
+    F.encode_dev(grads, d, again, lam, 5, 1, block_log2=b, ws=ws, worker_stride=stride)
+    torch.cuda.synchronize()
+    assert torch.equal(bits, again)
+    assert abs(float(lam) - ref) <= RTOL * ref
