@@ -114,6 +114,7 @@ struct Plan {
 //     workers: 0.10 ms against 0.17 .. 0.20 on the plain ALUs at any tile); the first pass takes what is left.
 //     From 128 (tile, worker) items: below, setting up the blocks costs more (2^16, four workers: 15 against 11 us);
 //   three or four from 2^20 on: ten strided stages (on the tensor cores if there are tiles enough), short tiles;
+//   two in three or more blocks of 2^22: ten stages and T = 12 (eight blocks 120 us, 8 + 14 130; one block 24 and 22);
 //   one or two, or several planes: the plain-ALU pass is fastest on short tiles (one vector of 2^30: T = 10 1.5 ms, T = 14
 //     1.95), the first pass up to eight stages (six below 2^20, to leave the contiguous pass blocks for the chip);
 //   two strided passes: T = 12, where the contiguous pass still keeps pace with memory, the top pass nine stages (or eight:
@@ -139,6 +140,7 @@ Plan make_plan(int L, bool decoder, int64_t dp = 0, int workers = 1, int P = 1, 
         else if (forced & FOSGD_TC_CONTIGUOUS) pl.T = 14;
         else if (decoder && workers > 4 && P == 1 && (dp >> 14) * workers >= 128) pl.T = 14;
         else if (decoder && workers > 2 && P == 1 && L >= 20) pl.T = L - 10;
+        else if (decoder && workers == 2 && P == 1 && L == 22 && dp > (int64_t)1 << 23) pl.T = 12;
         else if (decoder) pl.T = L < 20 ? L - 6 : (L <= 22 ? (L - 8 < 12 ? 12 : L - 8) : (L == 23 && P == 1 ? 13 : 14));
         else pl.T = L == 18 ? 11 : (L < 18 ? 12 : (L == 19 ? 13 : 14));
         pl.A[0] = L - pl.T;
