@@ -113,6 +113,15 @@ __host__ __device__ constexpr int min_blocks()
     return 1 << (15 - T);
 }
 
+// The streamed form of that sink spills twice as much at 64 (112 bytes), in its loop: three blocks to an SM in place of four,
+// at 80 registers (two workers of 2^23 in 16 blocks 332 -> 322 us, four of 2^20 in 32 150 -> 140, three of 2^27 349 -> 304).
+template <int T, int SINK>
+__host__ __device__ constexpr int stream_blocks()
+{
+    if constexpr (SINK == SINK_FINAL && T <= 13) return 3 << (13 - T);
+    else return min_blocks<T, SINK>();
+}
+
 // ---- the three rounds on the padded tile ---------------------------------------------------
 // registers g * 2^VB .. + 2^VB - 1 of round F are consecutive coordinates starting at this tile offset
 template <int T>
@@ -750,7 +759,7 @@ struct StreamCfg {
 };
 
 template <int T, int SRC, int SINK>
-__global__ void __launch_bounds__(1 << (T - 5), min_blocks<T, SINK>()) row_stream_kernel(const typename KernelParams<SINK>::type p, const int64_t ntiles)
+__global__ void __launch_bounds__(1 << (T - 5), stream_blocks<T, SINK>()) row_stream_kernel(const typename KernelParams<SINK>::type p, const int64_t ntiles)
 {
     using C = RowCfg<T>;
     using S = StreamCfg<T, SRC>;
@@ -882,16 +891,16 @@ cudaError_t launch_row_one(const PassParams& p, cudaStream_t s)
     int sms = 0;
     const cudaError_t e = sm_count(&sms);
     if (e != cudaSuccess) return e;
-    // a few tiles with many workers each (2^13, 8 workers: one tile) would leave most SMs idle
-    // (one worker per block instead of two where a decode is little but latency: four vectors of 2^16 7.0 -> 5.1 us, of
-    // 2^17 7.9 -> 6.1; of 2^18 11.3 -> 13.1)
-    const int share = SRC == SRC_BITS_TOP && T <= 12 ? 2 * p.nworkers : p.nworkers;
-    const unsigned split = SINK == SINK_FINAL ? worker_split(ntiles, share, (int64_t)sms * min_blocks<T, SINK>()) : 1u;
     // On the way to the dither sink the fp32 tiles are read by the threads themselves: without the persistent
     // grid the blocks of an SM drift apart and one's loads and butterflies fill the gaps of another's generator
     // rounds (2^27 coordinates, T = 10 / 12 / 13: 0.175 / 0.187 / 0.189 ms against 0.215 / 0.213 / 0.225 ms streamed).
     // One worker per tile leaves nothing to stream either.
     constexpr bool kStream = (SRC == SRC_WS16 || SRC == SRC_WS) && (SINK == SINK_FINAL || SINK == SINK_WS) && StreamCfg<T, SRC>::kFits;
+    // a few tiles with many workers each (2^13, 8 workers: one tile) would leave most SMs idle
+    // (one worker per block instead of two where a decode is little but latency: four vectors of 2^16 7.0 -> 5.1 us, of
+    // 2^17 7.9 -> 6.1; of 2^18 11.3 -> 13.1)
+    const int share = SRC == SRC_BITS_TOP && T <= 12 ? 2 * p.nworkers : p.nworkers;
+    const unsigned split = SINK == SINK_FINAL ? worker_split(ntiles, share, (int64_t)sms * (kStream ? stream_blocks<T, SINK>() : min_blocks<T, SINK>())) : 1u;
     if constexpr (SINK == SINK_PACKK) {
         // parts of the tiles' groups until the blocks fill the chip
         unsigned parts = 1;
