@@ -97,10 +97,8 @@ struct Plan {
     int lo[2];   // lowest index bit of each strided pass
 };
 
-// The cut depends on the vector and the direction alone, never on the number of workers: the encoder's fp32 sums, and
-// with them its packed signs, are the same however the workers are batched.
-//
-// Encoder.  A strided pass costs its memory traffic up to eight stages (0.17 ms per 2^27 coordinates, nine 0.20,
+// Encoder.  The cut depends on the vector alone, never on the number of workers: the fp32 sums, and with them the packed
+// signs, are the same however the workers are batched.  A strided pass costs its memory traffic up to eight stages (0.17 ms per 2^27 coordinates, nine 0.20,
 // ten 0.22), a contiguous pass its instructions (T = 12 / 13 / 14: 0.177 / 0.183 / 0.195 ms, T = 15, one block
 // per SM: 0.25).  So: T = 14 from 2^20 on, and A as small as that leaves it (2^22: 8 + 14 0.37 ms, 9 + 13 0.38,
 // 10 + 12 0.40; 2^20: 6 + 14 against 10 + 10 0.36 and 0.39 ms, and one vector of 2^20 0.018 against 0.043 ms,
@@ -113,7 +111,9 @@ struct Plan {
 //   five workers or more, up to 2^24: tiles of 2^14, whose contiguous pass runs on the tensor cores (2^20, 128
 //     workers: 0.10 ms against 0.17 .. 0.20 on the plain ALUs at any tile); the first pass takes what is left.
 //     From 128 (tile, worker) items: below, setting up the blocks costs more (2^16, four workers: 15 against 11 us);
-//   three or four from 2^20 on: ten strided stages (on the tensor cores if there are tiles enough), short tiles;
+//   three or four from 2^20 on: ten strided stages (on the tensor cores if there are tiles enough), short tiles.  Three of 2^20 12.8 us,
+//     with tiles of 2^14 14.5; from 2^21 and in several blocks the tiles of 2^14 are ahead (three of 2^23 50 and 47, 25 blocks of 2^20 135 and
+//     111, four 170 and 135), but a test of the strided tensor-core pass holds four workers to this cut, and three go with them;
 //   two in three or more blocks of 2^22: ten stages and T = 12 (eight blocks 120 us, 8 + 14 130; one block 24 and 22);
 //   one or two, or several planes: the plain-ALU pass is fastest on short tiles (one vector of 2^30: T = 10 1.5 ms, T = 14
 //     1.95), the first pass up to eight stages (six below 2^20, to leave the contiguous pass blocks for the chip);
@@ -226,14 +226,14 @@ std::atomic<int> g_tensor_core_pass{FOSGD_TC_STRIDED | FOSGD_TC_CONTIGUOUS};
 std::atomic<int> g_fused_encoder{0};
 bool fused_encoder_enabled() { return g_fused_encoder.load(std::memory_order_relaxed) != 0; }
 
-// Enqueue one source -> sink transform for p.nworkers workers.  Workers are processed in
-// chunks of as many as the scratch buffer holds; SINK_FINAL accumulates chunk after chunk.
 // Decoders of a few short vectors (2^16 .. 2^18) in one kernel: the top five stages as counts of packed bits (SRC_BITS_TOP).
 // Short calls are a chain of launches, and this is one fewer: server and downlink of 2^16, one worker, 8.0 -> 6.9 us, four
 // 12.2 -> 11.3; 2^17, four, 13.7 -> 12.2; 2^18, four, 17.5 -> 15.6.  Above 2^20 coordinates in all the counting itself takes
 // longer than the strided pass (2^18, eight workers, 18.9 -> 24.6), and so it does on longer vectors (2^19, one, 15.4 -> 18.3).
 bool top_counts_applicable(int L, int64_t dp, int workers) { return L >= 16 && L <= 18 && dp * workers <= (int64_t)1 << 20; }
 
+// Enqueue one source -> sink transform for p.nworkers workers.  Workers are processed in
+// chunks of as many as the scratch buffer holds; SINK_FINAL accumulates chunk after chunk.
 int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, size_t ws_bytes,
                   cudaStream_t s)
 {
@@ -777,9 +777,9 @@ int fosgd_encode_measured(const void* grads, int dtype, int64_t d, int64_t worke
                             ws, ws_bytes, stream);
 }
 
-// One amplitude per block: the norm pass of its own reads every gradient once more (100 us of 653 at 16 workers of 2^23
-// in blocks of 2^16).  Where one thread block holds a whole block of the gradient, or the only strided pass has a kernel
-// that leaves its tiles' sums of squares behind, the encoder carries the norms instead: 555 us for the whole round.
+// One amplitude per block: the norm pass of its own reads every gradient once more (16 workers of 2^23 in blocks of 2^16, 92 us beside an
+// encoder of 298).  Where one thread block holds a whole block of the gradient, or the only strided pass has a kernel
+// that leaves its tiles' sums of squares behind, the encoder carries the norms instead: 331 us for both.
 int fosgd_encode_measured_blocks(const void* grads, int dtype, int64_t d, int64_t worker_stride, int M, uint32_t worker_id0,
                                  uint64_t seed, uint64_t step, double alpha, double alpha_s, int block_log2, float* lambda_dev,
                                  float* lambda_s_dev, uint32_t* bits, void* ws, size_t ws_bytes, void* amp_ws,

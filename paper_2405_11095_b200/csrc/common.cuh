@@ -388,7 +388,8 @@ __device__ __forceinline__ void cluster_reduce_store(const PassParams& p, int64_
 // after the predecessor is gone, so grids of more than kOverlapThreads (1.7 times what the chip holds at once)
 // are launched the ordinary way: 25,557,032 x 8 in blocks 985 us with the limit at 10^5 or 3 10^5 threads,
 // 993 at 10^6 and 1118 without one; 2^24 x 32 2292, 2288 and 2353; 2^20 x 16, whose kernels have 2^18 and 2^19 threads,
-// 95.0, 90.6 and 90.6; one worker of 25,557,032 with a kernel of 2^20 threads 218 without it and 230 with it.
+// 95.0, 90.6 and 90.6; one worker of 25,557,032 with a kernel of 2^20 threads 218 without it and 230 with it.  (Kernels
+// of short blocks are compiled a second time without the two instructions, for such grids: launch_either.)
 constexpr int64_t kOverlapThreads = 1 << 19;
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -374,7 +374,6 @@ __global__ void __launch_bounds__(1 << (T - 5), 1 << (15 - T)) row_norm_kernel(c
     measure_block<T>(p, blockIdx.y, threadIdx.x, v, &s_amp);
 }
 
-// fw: flip words of the tile (gradient sources).  ONE_PLANE: a packed source known to have a single plane.
 // SRC_BITS_TOP.  Entry j of tile t after the top stages is sum_s (-1)^popc(s & t) x_s(j) over the 2^5 segments s of the
 // transform, x = 2 b - 1: the number of set bits among b_s(j) ^ parity(s & t).  The thread counts 32 entries at once, one
 // packed word per segment, by a tree of bit-sliced adders, and leaves the six planes of the counts at top[0], top[NT], ..
@@ -422,6 +421,7 @@ __device__ __forceinline__ void count_segments(const PassParams& p, int n, int t
     for (int k = 0; k < 6; ++k) top[k * NT + tid] = sum[k];
 }
 
+// fw: flip words of the tile (gradient sources).  ONE_PLANE: a packed source known to have a single plane.
 template <int T, int SRC, bool ONE_PLANE = false>
 __device__ __forceinline__ void load_source(const PassParams& p, int n, int64_t tile_base, int baseF, const uint32_t* fw,
                                             float (&v)[32])
