@@ -239,7 +239,10 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
 {
     const int tc = g_tensor_core_pass.load(std::memory_order_relaxed);
     const bool tc_any_size = (tc & FOSGD_TC_ANY_SIZE) != 0;
-    const Plan pl = sink == SINK_FINAL ? make_plan(g.L, true, g.dp, p.nworkers, p.P, tc) : g.plan;
+    // a decoder is cut for the workers that one launch takes (2^19, eight workers by threes: 50 us as eight, 33 as three)
+    const size_t cap = ws != nullptr && g.ws_per_worker > 0 ? ws_bytes / g.ws_per_worker : 0;
+    const int at_once = cap > 0 && cap < (size_t)p.nworkers ? (int)cap : p.nworkers;
+    const Plan pl = sink == SINK_FINAL ? make_plan(g.L, true, g.dp, at_once, p.P, tc) : g.plan;
     cudaError_t e = cudaSuccess;
 #define FOSGD_CUDA_OK(call) do { e = (call); if (e != cudaSuccess) { g_last_cuda_error = (int)e; return FOSGD_ECUDA; } } while (0)
     if (pl.ncol == 0) {
@@ -257,9 +260,8 @@ int run_transform(const Geometry& g, int src, int sink, PassParams p, void* ws, 
         FOSGD_CUDA_OK(traced('e', pl.L, src, sink, p, s));
         return FOSGD_OK;
     }
-    const size_t cap = ws_bytes / g.ws_per_worker;
     const int total = p.nworkers;
-    int chunk = (int)(cap < (size_t)total ? cap : (size_t)total);
+    int chunk = at_once;
     // The one-kernel encoder (fused_encode.cu) keeps its ticket and progress words behind the chunk's
     // intermediates.  Scratch sized for exactly `chunk` workers has no room for them: the chunk then gives up
     // its last worker's slot (a caller who adds enc_fused_sync_bytes to the scratch keeps the full chunk).

@@ -100,7 +100,7 @@ def test_contiguous_pass_of_every_length(F, d, b, M):
     assert ran(labels) == (False, False), labels
     outs, labels = with_mask(F, DEFAULT, run)
     T = 15 if (b or (dp - 1).bit_length()) == 25 else 14
-    assert sum(x.startswith(f"tcrow{T}") for x in labels) >= 2, labels
+    assert any(x.startswith(f"tcrow{T}") for x in labels), labels
     for k, (x, y) in enumerate(zip(outs, plain)):
         # (a weight rounds each worker's term, and the sum over the workers is rounded in the order of the blocks that share them)
         assert torch.equal(x, y) if k < 3 else float((x - y).norm()) <= 1e-6 * float(y.norm()), k
