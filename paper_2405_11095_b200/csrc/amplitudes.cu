@@ -231,8 +231,14 @@ cudaError_t launch_amplitudes(const void* grads, int bf16, int64_t d, int64_t wo
     // parts of at least 4096 coordinates: every one costs the second step a load
     const int nparts = (int)(d >= (int64_t)kNormBlocks * 4096 ? kNormBlocks : (d + 4095) / 4096);
     const dim3 grid((unsigned)nparts, (unsigned)M);
-    const cudaError_t e = bf16 ? launch<sumsq_partial_kernel<true>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial)
-                               : launch<sumsq_partial_kernel<false>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial);
+    // one or two workers are a grid of less than a wave that crowds when it is overlapped, which a long vector feels (bf16 2^25 24.2 us and
+    // 16.8 launched the ordinary way, two of 2^26 71 and 56; fp32 40 and 41, two of 2^24 27 and 29; 2^22 5.6 and 8.3)
+    const bool plain = (M == 1 || (M == 2 && bf16)) && d >= (int64_t)1 << 24;
+    const cudaError_t e =
+        bf16 ? (plain ? launch<sumsq_partial_kernel<true>, false>(grid, 256, 0, s, 1, grads, d, worker_stride, partial)
+                      : launch<sumsq_partial_kernel<true>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial))
+             : (plain ? launch<sumsq_partial_kernel<false>, false>(grid, 256, 0, s, 1, grads, d, worker_stride, partial)
+                      : launch<sumsq_partial_kernel<false>>(grid, 256, 0, s, 1, grads, d, worker_stride, partial));
     if (e != cudaSuccess) return e;
     return launch_amplitudes_finalize(partial, M, nparts, alpha, alpha_s, n_eff, lam, lam_s, s);
 }
